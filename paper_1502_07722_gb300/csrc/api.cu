@@ -12,6 +12,7 @@
 namespace gbpic {
 int tile_window(int T);
 int energy_blocks(const Ctx& c);
+void swap_currents(Ctx& c);
 void sort_species_impl(Ctx& c, int s, cudaStream_t st, int from_b, int64_t* launches);
 }  // namespace gbpic
 
@@ -30,6 +31,7 @@ constexpr int kMaxEnergyBlocks = 1024;
 struct Layout {
     int32_t dims, nx, ny, nz, T, ntx, nty, ntz, ntiles, nkeys, nsp, jy_bits;
     int64_t count_limit;
+    bool twin;
     size_t nn;
     int64_t cap[2], n0[2];
     size_t total;
@@ -101,8 +103,10 @@ int derive_layout(const pic_config* cfg, Layout& L)
     const int arrays = L.dims == 3 ? 7 : 6;
     for (int s = 0; s < 2; s++) t += 2 * arrays * align256(4 * (size_t)L.cap[s]) + align256(4 * (size_t)(L.ntiles + 1));
     t += 6 * align256(4 * L.nn) + 5 * align256(8 * L.nn);
+    L.twin = L.dims == 2 && full;         // the field update's second set of field and current grids
+    if (L.twin) t += 6 * align256(4 * L.nn) + 3 * align256(8 * L.nn);
     const size_t plane = (size_t)L.nx * L.ny;
-    t += align256(4 * 8 * plane) + 2 * align256(4 * plane) + align256(8);
+    t += (L.dims == 3 ? align256(4 * 8 * plane) : 0) + 2 * align256(4 * plane) + align256(8);
     t += 2 * align256(4 * ((size_t)L.nkeys + 1));
     t += align256(4 * (((size_t)L.nkeys + 2047) / 2048 + 1));
     t += align256(8 * 5 * (size_t)kMaxEnergyBlocks) + align256(8 * 8) + align256(32);
@@ -182,15 +186,45 @@ int sort_all(pic_ctx* h)
 
 int redeposit(Ctx& c)
 {
+    c.prepared = 0;
     if (c.dims == 3) launch_deposit_density3(c, c.rho[c.cur], c.stream);
     else launch_deposit_density(c, c.rho[c.cur], c.stream);
     CK(cudaGetLastError());
     return PIC_OK;
 }
 
+// The currents a step deposits into start clear (the transport stage has none) and the next node
+// density from the current one (the particle kernel adds the changes). In 2D the field update of
+// the step before has done both.
+int prepare_step(Ctx& c)
+{
+    const bool twin = c.Jn[0] != nullptr;
+    if (!c.prepared) {
+        u64** J = twin ? c.Jn : c.J;
+        CopySeg prep[4] = {{c.rho[c.cur], c.rho[1 - c.cur], 8 * c.nn}};
+        int n = 1;
+        if (c.cfg.mode == PIC_MODE_FULL)
+            for (int q = 0; q < 3; q++) prep[n++] = CopySeg{nullptr, J[q], 8 * c.nn};
+        c.nlaunch[3] += launch_copy_segments(c, prep, n, c.stream);
+        CK(cudaGetLastError());
+    }
+    if (twin) swap_currents(c);
+    c.prepared = 0;
+    return PIC_OK;
+}
+
 }  // namespace
 
 namespace gbpic {
+
+void swap_currents(Ctx& c)
+{
+    for (int q = 0; q < 3; q++) {
+        u64* p = c.J[q];
+        c.J[q] = c.Jn[q];
+        c.Jn[q] = p;
+    }
+}
 
 StepArgs make_step_args(Ctx& c)
 {
@@ -311,8 +345,12 @@ int pic_init(const pic_config* cfg, void* workspace, size_t workspace_bytes, voi
     for (int q = 0; q < 6; q++) c.F[q] = cv.take<float>(L.nn);
     for (int q = 0; q < 3; q++) c.J[q] = cv.take<u64>(L.nn);
     for (int q = 0; q < 2; q++) c.rho[q] = cv.take<u64>(L.nn);
+    if (L.twin) {
+        for (int q = 0; q < 6; q++) c.Fn[q] = cv.take<float>(L.nn);
+        for (int q = 0; q < 3; q++) c.Jn[q] = cv.take<u64>(L.nn);
+    }
     const size_t plane = (size_t)L.nx * L.ny;
-    c.mur_save = cv.take<float>(8 * plane);
+    c.mur_save = d3 ? cv.take<float>(8 * plane) : nullptr;
     c.ant_c = cv.take<float>(plane);
     c.ant_s = cv.take<float>(plane);
     c.ant = cv.take<float>(2);
@@ -384,7 +422,7 @@ int pic_init(const pic_config* cfg, void* workspace, size_t workspace_bytes, voi
     for (int q = 0; q < 6; q++) ok &= cudaMemsetAsync(c.F[q], 0, 4 * L.nn, c.stream) == cudaSuccess;
     for (int q = 0; q < 3; q++) ok &= cudaMemsetAsync(c.J[q], 0, 8 * L.nn, c.stream) == cudaSuccess;
     for (int q = 0; q < 2; q++) ok &= cudaMemsetAsync(c.rho[q], 0, 8 * L.nn, c.stream) == cudaSuccess;
-    ok &= cudaMemsetAsync(c.mur_save, 0, 4 * 8 * plane, c.stream) == cudaSuccess;
+    if (d3) ok &= cudaMemsetAsync(c.mur_save, 0, 4 * 8 * plane, c.stream) == cudaSuccess;
     ok &= cudaMemsetAsync(c.red_out, 0, 8 * sizeof(double), c.stream) == cudaSuccess;   // incl. the injected-energy sum
     ok &= cudaMemsetAsync(c.status, 0, 32, c.stream) == cudaSuccess;
     if (!ok) {
@@ -427,15 +465,9 @@ int pic_step(pic_ctx* h, int32_t nsteps)
             int r = sort_all(h);
             if (r) return r;
         }
-        {
-            // clear the currents; the next node density starts from the current one (the particle
-            // kernel adds the changes)
-            const CopySeg prep[4] = {{nullptr, c.J[0], 8 * c.nn}, {nullptr, c.J[1], 8 * c.nn},
-                                     {nullptr, c.J[2], 8 * c.nn}, {c.rho[c.cur], c.rho[1 - c.cur], 8 * c.nn}};
-            c.nlaunch[3] += launch_copy_segments(c, prep, 4, c.stream);
-            CK(cudaGetLastError());
-        }
-        int r = ev_begin(h, 0);
+        int r = prepare_step(c);
+        if (r) return r;
+        r = ev_begin(h, 0);
         if (r) return r;
         if (c.dims == 3) launch_particle_step3(c, c.stream);
         else launch_particle_step(c, make_step_args(c), c.stream);
@@ -443,6 +475,7 @@ int pic_step(pic_ctx* h, int32_t nsteps)
         if (r) return r;
         c.nlaunch[0]++;
         c.nlaunch[3]++;
+        c.cur = 1 - c.cur;
         if (c.cfg.mode == PIC_MODE_FULL) {
             r = ev_begin(h, 1);
             if (r) return r;
@@ -454,7 +487,8 @@ int pic_step(pic_ctx* h, int32_t nsteps)
             c.nlaunch[3] += c.nlaunch[1] - before;
         }
         CK(cudaGetLastError());
-        c.cur = 1 - c.cur;
+        // the 2D field update has prepared the next step
+        c.prepared = c.Jn[0] != nullptr;
         c.step++;
         c.steps_since_sort++;
     }
@@ -821,6 +855,7 @@ int pic_checkpoint_restore(pic_ctx* h, const void* buf, int32_t on_host)
     for (int s = 0; s < c.nsp; s++) c.sp[s].n = hd.n[s];
     int r = ckpt_copy(h, (char*)const_cast<void*>(buf), false, on_host != 0);
     if (r) return r;
+    c.prepared = 0;
     c.step = hd.step;
     c.steps_since_sort = hd.steps_since_sort;
     CK(cudaStreamSynchronize(c.stream));

@@ -1,11 +1,11 @@
 // Batched intensity sweep: several independent slabs (uneven sizes, particle counts and laser
 // intensities) advanced together. Each slab is an ordinary context (pic_init on a slice of the
 // batch workspace); a step of the whole batch is
-//   k_prepare_batch      clear the currents, start the next node density from the current one
 //   k_particles_batch    one persistent launch over the tiles of every slab
-//   field kernels        one launch each for all slabs (blockIdx.z = slab), antenna on the device
-// and is recorded once as a CUDA graph per parity of the double-buffered node density, then
-// replayed. The per-slab arguments live in device memory (copied into a constant-memory table in
+//   k_fields_batch       the field update of every slab, which also prepares the next step (clears
+//                        its currents, starts its node density, evaluates its antenna scalars)
+// (the transport stage has k_prepare_batch in front instead) and is recorded once as a CUDA graph
+// per parity of the double-buffered grids, then replayed. The per-slab arguments live in device memory (copied into a constant-memory table in
 // front of the particle kernel), so a cell sort (host-driven, every
 // sort_every steps) only refreshes them; the graphs stay valid.
 #include <cstring>
@@ -17,18 +17,23 @@
 namespace gbpic {
 void sort_species_impl(Ctx& c, int s, cudaStream_t st, int from_b, int64_t* launches);
 int max_batch_slabs();
+void swap_currents(Ctx& c);
 
 constexpr int kMaxSlabs = 48;    // the constant-memory argument table of the batched particle kernel
 static_assert(kMaxSlabs <= kMaxFieldSlabs, "every slab's field arguments fit the batched field kernels' parameters");
 
+// Clears the currents a step deposits into (the transport stage has none) and starts the next node
+// density from the current one.
 __global__ void k_prepare_batch(const StepArgs* __restrict__ args)
 {
     const StepArgs& a = args[blockIdx.y];
     const size_t nn = (size_t)(a.nz + 1) * a.nx;
     for (size_t j = blockIdx.x * (size_t)blockDim.x + threadIdx.x; j < nn; j += (size_t)gridDim.x * blockDim.x) {
-        a.J[0][j] = 0;
-        a.J[1][j] = 0;
-        a.J[2][j] = 0;
+        if (a.full) {
+            a.J[0][j] = 0;
+            a.J[1][j] = 0;
+            a.J[2][j] = 0;
+        }
         a.rho_next[j] = a.rho_cur[j];
     }
 }
@@ -45,10 +50,10 @@ struct pic_batch {
     size_t max_nn;
     int64_t step;
     StepArgs* args_dev;          // [2][n]: parity 0 (density in buffer 0) and parity 1
-    FieldBatch fields;           // every slab's field arguments (host copy, passed by value)
+    FieldBatch fields[2];        // every slab's field arguments per parity (host copy, passed by value)
     AntennaParams* ap_dev;       // [n]
     long long* step_dev;         // [n]
-    float* ant_dev;              // [n][2]
+    float* ant_dev;              // [2][n][2]: the antenna scalars of a step of each parity
     int* tile_base_dev;          // [n + 1]
     cudaGraphExec_t graph[2];
     int captured;
@@ -66,20 +71,37 @@ size_t a256(size_t x) { return (x + 255) & ~(size_t)255; }
 size_t batch_tail_bytes(int n)
 {
     return a256(sizeof(StepArgs) * 2 * n) + a256(sizeof(AntennaParams) * n) + a256(8 * (size_t)n) +
-           a256(8 * (size_t)n) + a256(4 * ((size_t)n + 1));
+           a256(16 * (size_t)n) + a256(4 * ((size_t)n + 1));
 }
 
+// The other parity of a slab's double-buffered grids (density; with fields also the fields and the
+// currents, which a step swaps too).
+void flip_parity(Ctx& c)
+{
+    c.cur = 1 - c.cur;
+    if (!c.Jn[0]) return;
+    swap_currents(c);
+    for (int q = 0; q < 6; q++) {
+        float* f = c.F[q];
+        c.F[q] = c.Fn[q];
+        c.Fn[q] = f;
+    }
+}
+
+// Arguments of a step that starts at parity p: the particle kernel deposits into the cleared
+// currents Jn and the field update then reads them (as J).
 int upload_args(pic_batch* b)
 {
     std::vector<StepArgs> h(2 * b->n);
     for (int s = 0; s < b->n; s++) {
         Ctx& c = b->slab[s]->c;
-        const int cur = c.cur;
-        for (int p = 0; p < 2; p++) {
-            c.cur = p;
-            h[p * b->n + s] = make_step_args(c);
+        for (int k = 0; k < 2; k++) {
+            const int p = c.cur;
+            StepArgs& a = h[p * b->n + s];
+            a = make_step_args(c);
+            for (int q = 0; q < 3 && c.Jn[0]; q++) a.J[q] = c.Jn[q];
+            flip_parity(c);
         }
-        c.cur = cur;
     }
     if (cudaMemcpyAsync(b->args_dev, h.data(), sizeof(StepArgs) * h.size(), cudaMemcpyHostToDevice, b->st) !=
         cudaSuccess)
@@ -87,17 +109,36 @@ int upload_args(pic_batch* b)
     return cudaStreamSynchronize(b->st) == cudaSuccess ? PIC_OK : PIC_ECUDA;
 }
 
+void enqueue_prepare(pic_batch* b, int parity)
+{
+    dim3 pg((unsigned)((b->max_nn + 1023) / 1024 > 4096 ? 4096 : (b->max_nn + 1023) / 1024), b->n);
+    k_prepare_batch<<<pg, 256, 0, b->st>>>(b->args_dev + parity * b->n);
+}
+
 void enqueue_step(pic_batch* b, int parity)
 {
     const StepArgs* args = b->args_dev + parity * b->n;
-    dim3 pg((unsigned)((b->max_nn + 1023) / 1024 > 4096 ? 4096 : (b->max_nn + 1023) / 1024), b->n);
-    k_prepare_batch<<<pg, 256, 0, b->st>>>(args);
+    if (!b->full) enqueue_prepare(b, parity);
     if (b->timing) cudaEventRecord(b->ev[0], b->st);
     launch_particle_step_batch(args, b->tile_base_dev, b->n, b->total_tiles, b->full, b->pot, b->maxW, b->nsm, b->st);
     if (b->timing) cudaEventRecord(b->ev[1], b->st);
     if (b->full)
-        launch_fields_batch(b->fields, b->ap_dev, b->step_dev, b->ant_dev, b->st);
+        launch_fields_batch(b->fields[parity], b->ap_dev, b->step_dev, b->ant_dev + (1 - parity) * 2 * b->n, b->st);
     if (b->timing) cudaEventRecord(b->ev[2], b->st);
+}
+
+// The fields' update prepares the step after it; the first step, and one after a slab's state was
+// written from outside (a checkpoint, new particles), is prepared here.
+void prepare(pic_batch* b)
+{
+    if (!b->full) return;
+    bool ready = true;
+    for (int s = 0; s < b->n; s++) ready &= b->slab[s]->c.prepared != 0;
+    if (ready) return;
+    const int parity = b->slab[0]->c.cur;
+    enqueue_prepare(b, parity);
+    launch_antenna_batch(b->ap_dev, b->step_dev, b->ant_dev + parity * 2 * b->n, b->n, b->st);
+    b->nlaunch[3] += 2;
 }
 
 int capture(pic_batch* b)
@@ -181,16 +222,31 @@ int pic_batch_init(const pic_config* cfgs, int32_t n, void* workspace, size_t by
     b->step_dev = reinterpret_cast<long long*>(p);
     p += a256(8 * (size_t)n);
     b->ant_dev = reinterpret_cast<float*>(p);
-    p += a256(8 * (size_t)n);
+    p += a256(16 * (size_t)n);
     b->tile_base_dev = reinterpret_cast<int*>(p);
     std::vector<AntennaParams> ap(n);
-    b->fields.n = n;
     for (int s = 0; s < n; s++) {
-        b->fields.f[s] = make_field_args(b->slab[s]->c);
-        b->fields.f[s].ant = b->ant_dev + 2 * s;     // the batch's per-slab antenna scalars
-        ap[s] = make_antenna_params(b->slab[s]->c);
+        Ctx& c = b->slab[s]->c;
+        ap[s] = make_antenna_params(c);
+        if (!c.Jn[0]) continue;
+        for (int k = 0; k < 2; k++) {
+            // the update of a step of this parity follows its moves: the density and the currents
+            // are the other buffers, the fields not yet
+            const int par = c.cur;
+            c.cur = 1 - c.cur;
+            swap_currents(c);
+            FieldArgs& f = b->fields[par].f[s];
+            f = make_field_args(c);
+            f.ant = b->ant_dev + par * 2 * n + 2 * s;
+            c.cur = par;
+            swap_currents(c);
+            flip_parity(c);
+        }
     }
-    field_row_blocks(b->fields);
+    for (int par = 0; par < 2; par++) {
+        b->fields[par].n = n;
+        if (b->full) field_row_blocks(b->fields[par]);
+    }
     bool ok = cudaMemcpyAsync(b->ap_dev, ap.data(), sizeof(AntennaParams) * n, cudaMemcpyHostToDevice, b->st) ==
                   cudaSuccess &&
               cudaMemcpyAsync(b->tile_base_dev, tile_base.data(), 4 * (size_t)(n + 1), cudaMemcpyHostToDevice,
@@ -230,6 +286,7 @@ int pic_batch_step(pic_batch* b, int32_t nsteps)
 {
     if (!b || nsteps < 0) return PIC_EINVAL;
     if (b->sticky) return b->sticky;
+    if (nsteps > 0) prepare(b);
     for (int it = 0; it < nsteps; it++) {
         if (b->sort_every > 0 && b->steps_since_sort >= b->sort_every) {
             if (b->timing) cudaEventRecord(b->ev[3], b->st);
@@ -259,19 +316,20 @@ int pic_batch_step(pic_batch* b, int32_t nsteps)
             b->ms[0] += m0;
             b->ms[1] += m1;
             b->nlaunch[0] += 1;
-            b->nlaunch[1] += b->full ? 6 : 0;
-            b->nlaunch[3] += 2 + (b->full ? 6 : 0);
+            b->nlaunch[1] += b->full ? 1 : 0;
+            b->nlaunch[3] += 2;
         } else {
             if (!b->captured) {
                 const int r = capture(b);
                 if (r) return r;
             }
             if (cudaGraphLaunch(b->graph[parity], b->st) != cudaSuccess) return PIC_ECUDA;
-            b->nlaunch[3] += 2 + (b->full ? 6 : 0);
+            b->nlaunch[3] += 2;
         }
         for (int s = 0; s < b->n; s++) {
             Ctx& c = b->slab[s]->c;
-            c.cur = 1 - c.cur;
+            flip_parity(c);
+            c.prepared = c.Jn[0] != nullptr;
             c.step++;
         }
         b->step++;

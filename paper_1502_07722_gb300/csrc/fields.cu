@@ -4,16 +4,32 @@
 // half step. x is periodic; the tangential E components on the wall rows z = 0 and z = nz take
 // the first-order Mur absorbing condition.
 //
-// The same node functions serve one simulation (one launch per kernel) and a batch of
-// simulations (one launch per kernel for all of them, blockIdx.z = simulation).
+// The whole update is one kernel. It reads one set of the six field grids and writes the other (the
+// context swaps them), so a warp may recompute its neighbours' intermediate values from the old
+// ones; the same pass clears the current grids the next step deposits into (the other set) and
+// starts the next node density from the current one.
+//
+// What bounds it: memory traffic on the large grids, the launch on the small ones. Against three
+// in-place passes (B half, E, B half) with a copy/clear kernel and a one-thread antenna kernel, a
+// node moves 112 bytes instead of 172 and a step has two launches instead of six.
+#include <cmath>
+
 #include "pic_internal.cuh"
 
 namespace gbpic {
 
-// Antenna amplitude of one step (FP64 on the device, one thread):
+// A warp owns kCols columns (plus one to the left and two to the right that it recomputes) and walks
+// up a segment of rows with the last rows' values in registers: the x neighbours come by shuffle, the
+// z neighbours from the row before, and no barrier or shared memory is needed. The next row's loads
+// are issued one row ahead.
+constexpr int kCols = 29, kFieldThreads = 128;
+
+// Antenna amplitude of one step (FP64):
 //   E_x += 2 (c dt / dx) E0 env(t) amp(x) sin(w (t - t_ant) + phi(x))
 // split as ant[0] * amp cos(phi) + ant[1] * amp sin(phi) with ant = A (sin, cos)(w (t - t_ant)).
-__device__ __forceinline__ void antenna_scalars(const AntennaParams& p, long long step, float* ant)
+// A single simulation evaluates it on the host with the launch's arguments (one thread of the GPU
+// took 5.3 us for it); a batch, whose steps are replayed from a graph, on the device.
+__host__ __device__ inline void antenna_scalars(const AntennaParams& p, long long step, float* ant)
 {
     float s = 0.0f, c = 0.0f;
     if (p.on) {
@@ -27,155 +43,187 @@ __device__ __forceinline__ void antenna_scalars(const AntennaParams& p, long lon
     ant[1] = c;
 }
 
-__global__ void k_antenna(AntennaParams p, long long step, float* ant) { antenna_scalars(p, step, ant); }
+__device__ __forceinline__ int wrap_col(int i, int nx)
+{
+    if (i < 0) i += nx;
+    while (i >= nx) i -= nx;       // a warp wider than the grid wraps more than once
+    return i;
+}
 
-// batched: slab s reads its own step counter, advances it after the step (k_step_done)
+struct V3 {
+    float x, y, z;
+};
+struct J3 {
+    u64 x, y, z;
+};
+__device__ __forceinline__ V3 load3(const float* const F[3], size_t c, bool in)
+{
+    return in ? V3{__ldg(F[0] + c), __ldg(F[1] + c), __ldg(F[2] + c)} : V3{0.0f, 0.0f, 0.0f};
+}
+__device__ __forceinline__ J3 load3(const u64* const J[3], size_t c, bool in)
+{
+    return in ? J3{__ldg(J[0] + c), __ldg(J[1] + c), __ldg(J[2] + c)} : J3{0, 0, 0};
+}
+__device__ __forceinline__ float right(float v) { return __shfl_down_sync(0xffffffffu, v, 1); }
+__device__ __forceinline__ float left(float v) { return __shfl_up_sync(0xffffffffu, v, 1); }
+
+// The update of rows k0 .. k1 - 1 of the columns i0 .. i0 + kCols - 1 by one warp. Lane l holds column
+// i0 + l - 1; lanes 1 .. kCols write. At row r the warp knows E(r), E(r + 1) (old), takes B(r) to the
+// half step, E(r) to the new step, and finishes row r - 1 (its second half step of B needs the new
+// E(r)). Rows 0 and nz of the new tangential E follow from the new row beside them (Mur).
+__device__ __forceinline__ void field_rows(const FieldArgs& f, int i0, int k0, int k1, float a0, float a1)
+{
+    const int nx = f.nx, nz = f.nz, lane = threadIdx.x & 31;
+    const int gi = wrap_col(i0 + lane - 1, nx);
+    const bool own = lane >= 1 && lane <= kCols && i0 + lane - 1 < nx;
+    const float* const Ep[3] = {f.F[0], f.F[1], f.F[2]};
+    const float* const Bp[3] = {f.F[3], f.F[4], f.F[5]};
+    const float antc = f.antc[gi], ants = f.ants[gi];
+    const int r0 = k0 > 0 ? k0 - 1 : 0;
+    size_t c = (size_t)r0 * nx + gi;
+    V3 e = load3(Ep, c, true), en = load3(Ep, c + nx, true);      // old E of rows r, r + 1
+    V3 bl = load3(Bp, c, true);
+    J3 jl = load3(f.J, c, true);
+    V3 ep = {0, 0, 0}, bp = {0, 0, 0}, np = {0, 0, 0};           // row r - 1: old E, half-step B, new E
+    for (int r = r0; r <= k1; r++, c += nx) {
+        if (r > nz) {
+            // the wall row nz (the last segment): its B is finished below from np alone
+            break;
+        }
+        // one row ahead
+        const V3 e2 = load3(Ep, c + 2 * (size_t)nx, r + 2 <= nz && r < k1);
+        const V3 b2 = load3(Bp, c + nx, r + 1 <= nz && r < k1);
+        const J3 j2 = load3(f.J, c + nx, r + 1 <= nz && r < k1);
+        // B(r) to the half step (Bx, By have nz rows)
+        V3 b = bl;
+        const float eyr = right(e.y), ezr = right(e.z);
+        if (r < nz) {
+            b.x += f.h_b * (en.y - e.y);
+            b.y += f.h_b * ((ezr - e.z) - (en.x - e.x));
+        }
+        b.z -= f.h_b * (eyr - e.y);
+        // E(r) to the new step
+        const float byl = left(b.y), bzl = left(b.z);
+        V3 n = e;
+        if (r > 0 && r < nz) {
+            float v = e.x - f.h_e * (b.y - bp.y) - f.cj * (float)(long long)jl.x;
+            if (r == f.k_ant) v += antc * a0 + ants * a1;
+            n.x = v;
+            n.y = e.y + f.h_e * ((b.x - bp.x) - (b.z - bzl)) - f.cjy * (float)(long long)jl.y;
+        }
+        if (r < nz) n.z += f.h_e * (b.y - byl) - f.cj * (float)(long long)jl.z;
+        if (r == 1) {
+            np.x = e.x + f.mur * (n.x - ep.x);
+            np.y = e.y + f.mur * (n.y - ep.y);
+        } else if (r == nz) {
+            n.x = ep.x + f.mur * (np.x - e.x);
+            n.y = ep.y + f.mur * (np.y - e.y);
+        }
+        if (r == f.k_flux && r >= k0 && r < k1) {            // uniform over the warp
+            // (Ex By - Ey Bx) at the half step
+            float s = own ? 0.25f * ((e.x + n.x) * (bp.y + b.y) - (e.y + n.y) * (bp.x + b.x)) : 0.0f;
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (lane == 0 && s != 0.0f) atomicAdd(f.flux, (double)s);
+        }
+        // finish row r - 1
+        const float npyr = right(np.y), npzr = right(np.z);
+        if (r > k0 && own) {
+            const size_t q = c - nx;
+            f.G[0][q] = np.x;
+            f.G[1][q] = np.y;
+            f.G[2][q] = np.z;
+            f.G[3][q] = bp.x + f.h_b * (n.y - np.y);
+            f.G[4][q] = bp.y + f.h_b * ((npzr - np.z) - (n.x - np.x));
+            f.G[5][q] = bp.z - f.h_b * (npyr - np.y);
+        }
+        // the next step's currents and node density
+        if (r >= k0 && r < k1 && own) {
+            f.Z[0][c] = 0;
+            f.Z[1][c] = 0;
+            f.Z[2][c] = 0;
+            f.rho_next[c] = f.rho[c];
+        }
+        ep = e;
+        bp = b;
+        np = n;
+        e = en;
+        en = e2;
+        bl = b2;
+        jl = j2;
+    }
+    if (k1 == nz + 1) {
+        const float npyr = right(np.y);
+        if (own) {
+            const size_t q = (size_t)nz * nx + gi;
+            f.G[0][q] = np.x;
+            f.G[1][q] = np.y;
+            f.G[2][q] = np.z;
+            f.G[3][q] = bp.x;
+            f.G[4][q] = bp.y;
+            f.G[5][q] = bp.z - f.h_b * (npyr - np.y);
+        }
+    }
+}
+
+// Rows per segment. A warp's walk is serial (each row waits for its loads, ~0.7 us), while the row and
+// a half that every segment repeats comes from L2: short segments win on every grid (2048^2: 97 us
+// at 4 rows, 101 at 8, 99 at 16, 102 at 64; 403 x 311: 10.3, 12.3, 22, 82; with the events' ~3 us). The
+// last segment takes the remainder (at least kSeg rows: the wall row needs the row beside it).
+constexpr int kSeg = 4;
+__host__ __device__ inline int field_segments(int nz) { return (nz + 1) / kSeg; }     // nz >= 4
+
+__device__ __forceinline__ void field_item(const FieldArgs& f, int item, float a0, float a1)
+{
+    const int nseg = field_segments(f.nz), col = item / nseg, s = item - col * nseg;
+    if (col * kCols >= f.nx) return;
+    field_rows(f, col * kCols, s * kSeg, s + 1 == nseg ? f.nz + 1 : (s + 1) * kSeg, a0, a1);
+}
+static int field_blocks(const FieldArgs& f)
+{
+    const int items = (f.nx + kCols - 1) / kCols * field_segments(f.nz), w = kFieldThreads / 32;
+    return (items + w - 1) / w;
+}
+
+__global__ void __launch_bounds__(kFieldThreads, 8) k_fields(const __grid_constant__ FieldArgs f)
+{
+    field_item(f, (int)(blockIdx.x * (kFieldThreads / 32) + threadIdx.x / 32), f.ant0, f.ant1);
+}
+
+// All slabs of a batch: blockIdx.x runs over every slab's blocks, slab s owning blocks rb[s] ..
+// rb[s + 1] - 1; every slab's arguments travel in the launch's parameter block. The antenna scalars
+// of this step were written by the previous one (or with the prepare kernel): the last block evaluates
+// the next step's into the other half of the array and advances the step counters.
+__global__ void __launch_bounds__(kFieldThreads, 8)
+    k_fields_batch(const __grid_constant__ FieldBatch P, const AntennaParams* ap, long long* step, float* ant_next)
+{
+    const int g = (int)blockIdx.x;
+    if (g == P.rb[P.n]) {
+        const int s = threadIdx.x;
+        if (s < P.n) {
+            const long long n = step[s] + 1;
+            step[s] = n;
+            antenna_scalars(ap[s], n, ant_next + 2 * s);
+        }
+        return;
+    }
+    int s = 0;
+    while (s + 1 < P.n && P.rb[s + 1] <= g) s++;
+    const FieldArgs& f = P.f[s];
+    field_item(f, (g - P.rb[s]) * (kFieldThreads / 32) + (int)threadIdx.x / 32, f.ant[0], f.ant[1]);
+}
+
+// antenna scalars of the step each slab is at
 __global__ void k_antenna_batch(const AntennaParams* p, const long long* step, float* ant, int nslab)
 {
     const int s = threadIdx.x;
     if (s < nslab) antenna_scalars(p[s], step[s], ant + 2 * s);
 }
 
-__global__ void k_step_done(long long* step, int nslab)
-{
-    const int s = threadIdx.x;
-    if (s < nslab) step[s] += 1;
-}
-
-__device__ __forceinline__ void half_B_node(const FieldArgs& f, int i, int k, int save)
-{
-    const int nx = f.nx, nz = f.nz;
-    const int ip = i + 1 == nx ? 0 : i + 1;
-    const size_t c = (size_t)k * nx + i;
-    const float *Ex = f.F[0], *Ey = f.F[1], *Ez = f.F[2];
-    float *Bx = f.F[3], *By = f.F[4], *Bz = f.F[5];
-    const float ey = Ey[c];
-    if (k < nz) {
-        const size_t u = c + nx;
-        Bx[c] += f.h_b * (Ey[u] - ey);
-        By[c] += f.h_b * ((Ez[(size_t)k * nx + ip] - Ez[c]) - (Ex[u] - Ex[c]));
-    }
-    Bz[c] -= f.h_b * (Ey[(size_t)k * nx + ip] - ey);
-    if (save) {
-        int slot = -1;
-        if (k == 0) slot = 0;
-        else if (k == 1) slot = 1;
-        else if (k == nz - 1) slot = 2;
-        else if (k == nz) slot = 3;
-        if (slot >= 0) {
-            f.save[slot * nx + i] = Ex[c];
-            f.save[(4 + slot) * nx + i] = ey;
-        }
-    }
-}
-
-// new Ex / Ey of an interior node (i, k) from its old value
-__device__ __forceinline__ float ex_new(const FieldArgs& f, int i, int k, float old)
-{
-    const size_t c = (size_t)k * f.nx + i;
-    float v = old - f.h_e * (f.F[4][c] - f.F[4][c - f.nx]) - f.cj * (float)(long long)f.J[0][c];
-    if (k == f.k_ant) v += f.antc[i] * f.ant[0] + f.ants[i] * f.ant[1];
-    return v;
-}
-__device__ __forceinline__ float ey_new(const FieldArgs& f, int i, int k, float old)
-{
-    const size_t c = (size_t)k * f.nx + i;
-    const int im = i == 0 ? f.nx - 1 : i - 1;
-    return old + f.h_e * ((f.F[3][c] - f.F[3][c - f.nx]) - (f.F[5][c] - f.F[5][(size_t)k * f.nx + im])) -
-           f.cjy * (float)(long long)f.J[1][c];
-}
-
-// E update of one node; returns, on the flux row, the node's (Ex By - Ey Bx) at the half step
-// (E the mean of old and new, B averaged over the half rows on either side), else 0
-__device__ __forceinline__ float E_node(const FieldArgs& f, int i, int k)
-{
-    const int nx = f.nx, nz = f.nz;
-    const size_t c = (size_t)k * nx + i;
-    float* Ex = f.F[0];
-    float* Ey = f.F[1];
-    float* Ez = f.F[2];
-    float s = 0.0f;
-    if (k > 0 && k < nz) {
-        const float ex0 = Ex[c], ey0 = Ey[c];
-        const float ex1 = ex_new(f, i, k, ex0), ey1 = ey_new(f, i, k, ey0);
-        Ex[c] = ex1;
-        Ey[c] = ey1;
-        if (k == f.k_flux)
-            s = 0.25f * ((ex0 + ex1) * (f.F[4][c - nx] + f.F[4][c]) - (ey0 + ey1) * (f.F[3][c - nx] + f.F[3][c]));
-    } else if (k == 0) {
-        const float x0 = f.save[0 * nx + i], x1 = f.save[1 * nx + i];
-        const float y0 = f.save[4 * nx + i], y1 = f.save[5 * nx + i];
-        Ex[c] = x1 + f.mur * (ex_new(f, i, 1, x1) - x0);
-        Ey[c] = y1 + f.mur * (ey_new(f, i, 1, y1) - y0);
-    } else {
-        const float x1 = f.save[2 * nx + i], x0 = f.save[3 * nx + i];
-        const float y1 = f.save[6 * nx + i], y0 = f.save[7 * nx + i];
-        Ex[c] = x1 + f.mur * (ex_new(f, i, nz - 1, x1) - x0);
-        Ey[c] = y1 + f.mur * (ey_new(f, i, nz - 1, y1) - y0);
-    }
-    if (k < nz) {
-        const int im = i == 0 ? nx - 1 : i - 1;
-        Ez[c] += f.h_e * (f.F[4][c] - f.F[4][(size_t)k * nx + im]) - f.cj * (float)(long long)f.J[2][c];
-    }
-    return s;
-}
-
-// the flux row's warp sums into the FP64 accumulator
-__device__ __forceinline__ void add_flux(const FieldArgs& f, int k, float s)
-{
-    if (k != f.k_flux) return;
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0 && s != 0.0f) atomicAdd(f.flux, (double)s);
-}
-
-__global__ void k_half_B(const FieldArgs f, int save)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < f.nx) half_B_node(f, i, blockIdx.y, save);
-}
-
-__global__ void k_E(const FieldArgs f)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const float s = i < f.nx ? E_node(f, i, blockIdx.y) : 0.0f;
-    add_flux(f, blockIdx.y, s);
-}
-
-// Batched field kernels: blockIdx.x runs over every slab's (row, 256-node segment) blocks, slab s
-// owning blocks rb[s] .. rb[s + 1] - 1. Every slab's arguments travel in the launch's parameter
-// block (a grid over the largest slab's rows for every slab, reading the arguments from global
-// memory, took 0.27 ms per step of the 16-slab sweep).
-__device__ __forceinline__ int batch_slab(const FieldBatch& P, int g)
-{
-    int s = 0;
-    while (s + 1 < P.n && P.rb[s + 1] <= g) s++;
-    return s;
-}
-
-__global__ void k_half_B_batch(const __grid_constant__ FieldBatch P, int save)
-{
-    const int s = batch_slab(P, (int)blockIdx.x);
-    const FieldArgs& f = P.f[s];
-    const int local = (int)blockIdx.x - P.rb[s], nxb = (f.nx + 255) >> 8;
-    const int k = local / nxb, i = (local - k * nxb) * 256 + (int)threadIdx.x;
-    if (i < f.nx) half_B_node(f, i, k, save);
-}
-
-__global__ void k_E_batch(const __grid_constant__ FieldBatch P)
-{
-    const int s = batch_slab(P, (int)blockIdx.x);
-    const FieldArgs& f = P.f[s];
-    const int local = (int)blockIdx.x - P.rb[s], nxb = (f.nx + 255) >> 8;
-    const int k = local / nxb, i = (local - k * nxb) * 256 + (int)threadIdx.x;   // k uniform over the block
-    const float v = i < f.nx ? E_node(f, i, k) : 0.0f;
-    add_flux(f, k, v);
-}
-
 // each slab's first block (rb[n] = the total)
 void field_row_blocks(FieldBatch& P)
 {
     P.rb[0] = 0;
-    for (int s = 0; s < P.n; s++) P.rb[s + 1] = P.rb[s] + (P.f[s].nz + 1) * ((P.f[s].nx + 255) / 256);
+    for (int s = 0; s < P.n; s++) P.rb[s + 1] = P.rb[s] + field_blocks(P.f[s]);
 }
 
 AntennaParams make_antenna_params(const Ctx& c)
@@ -190,6 +238,8 @@ AntennaParams make_antenna_params(const Ctx& c)
     return p;
 }
 
+// The arguments of the field update that follows the particle kernel: density rho[cur] and currents J
+// just deposited, fields F read and Fn written, Jn cleared for the next step.
 FieldArgs make_field_args(const Ctx& c)
 {
     FieldArgs f;
@@ -203,11 +253,15 @@ FieldArgs make_field_args(const Ctx& c)
     const double cdt = kC * c.dt;
     f.mur = (float)((cdt - c.cfg.dx) / (cdt + c.cfg.dx));
     for (int q = 0; q < 6; q++) f.F[q] = c.F[q];
+    for (int q = 0; q < 6; q++) f.G[q] = c.Fn[q];
     for (int q = 0; q < 3; q++) f.J[q] = c.J[q];
-    f.save = c.mur_save;
+    for (int q = 0; q < 3; q++) f.Z[q] = c.Jn[q];
+    f.rho = c.rho[c.cur];
+    f.rho_next = c.rho[1 - c.cur];
     f.antc = c.ant_c;
     f.ants = c.ant_s;
-    f.ant = c.ant;
+    f.ant = nullptr;
+    f.ant0 = f.ant1 = 0.0f;
     f.k_flux = c.k_ant - 1 >= 1 ? c.k_ant - 1 : -1;
     f.flux = c.red_out + 5;
     return f;
@@ -215,25 +269,29 @@ FieldArgs make_field_args(const Ctx& c)
 
 void launch_fields(Ctx& c, cudaStream_t st, int64_t step, int64_t* launches)
 {
-    const FieldArgs f = make_field_args(c);
-    k_antenna<<<1, 1, 0, st>>>(make_antenna_params(c), (long long)step, c.ant);
-    dim3 block(256);
-    dim3 grid((c.nx + 255) / 256, c.nz + 1);
-    k_half_B<<<grid, block, 0, st>>>(f, 1);
-    k_E<<<grid, block, 0, st>>>(f);
-    k_half_B<<<grid, block, 0, st>>>(f, 0);
-    if (launches) *launches += 4;
+    FieldArgs f = make_field_args(c);
+    float ant[2];
+    antenna_scalars(make_antenna_params(c), (long long)step, ant);
+    f.ant0 = ant[0];
+    f.ant1 = ant[1];
+    k_fields<<<field_blocks(f), kFieldThreads, 0, st>>>(f);
+    for (int q = 0; q < 6; q++) {
+        float* p = c.F[q];
+        c.F[q] = c.Fn[q];
+        c.Fn[q] = p;
+    }
+    if (launches) *launches += 1;
 }
 
-void launch_fields_batch(const FieldBatch& P, const AntennaParams* ap_dev, long long* step_dev, float* ant_dev,
+void launch_antenna_batch(const AntennaParams* ap_dev, const long long* step_dev, float* ant, int n, cudaStream_t st)
+{
+    k_antenna_batch<<<1, 64, 0, st>>>(ap_dev, step_dev, ant, n);
+}
+
+void launch_fields_batch(const FieldBatch& P, const AntennaParams* ap_dev, long long* step_dev, float* ant_next,
                          cudaStream_t st)
 {
-    k_antenna_batch<<<1, 32, 0, st>>>(ap_dev, step_dev, ant_dev, P.n);
-    const int blocks = P.rb[P.n];
-    k_half_B_batch<<<blocks, 256, 0, st>>>(P, 1);
-    k_E_batch<<<blocks, 256, 0, st>>>(P);
-    k_half_B_batch<<<blocks, 256, 0, st>>>(P, 0);
-    k_step_done<<<1, 32, 0, st>>>(step_dev, P.n);
+    k_fields_batch<<<P.rb[P.n] + 1, kFieldThreads, 0, st>>>(P, ap_dev, step_dev, ant_next);
 }
 
 }  // namespace gbpic

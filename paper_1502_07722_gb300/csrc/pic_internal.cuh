@@ -125,10 +125,13 @@ struct Ctx {
     Species sp[2];
     // grids
     float* F[6];
-    u64* J[3];
+    u64* J[3];            // currents of the last step
     u64* rho[2];
     int32_t cur;          // rho[cur] holds the node density at the current positions
-    float* mur_save;      // 8 * nx
+    float* Fn[6];         // 2D full mode: the fields the next update writes (swapped with F after it)
+    u64* Jn[3];           // 2D full mode: the currents the next step deposits into
+    int32_t prepared;     // Jn is clear and rho[1 - cur] equals rho[cur]
+    float* mur_save;      // 3D: 8 planes
     float* ant_c;         // nx: amplitude * cos(phase(x)) at x = i + 1/2
     float* ant_s;         // nx: amplitude * sin(phase(x))
     float* ant;           // 2: antenna scalars of the current step (written on the device)
@@ -160,7 +163,7 @@ struct AntennaParams {
     double dt, t_ant, tau_fwhm, omega, coef;
 };
 
-// Everything a field kernel needs for one simulation.
+// Everything the field kernel needs for one simulation.
 struct FieldArgs {
     int nx, nz, k_ant;
     float h_b;           // dt / (2 dx)      (half step of B)
@@ -168,12 +171,16 @@ struct FieldArgs {
     float cj;            // J2x, J2z -> dt J / eps0
     float cjy;           // J6y -> dt J_y / eps0
     float mur;           // (c dt - dx) / (c dt + dx)
-    float* F[6];
-    const u64* J[3];
-    float* save;         // 8 * nx: Ex(0) Ex(1) Ex(nz-1) Ex(nz) Ey(0) Ey(1) Ey(nz-1) Ey(nz) before the E step
+    float ant0, ant1;    // this step's antenna scalars (single simulation)
+    const float* F[6];   // read
+    float* G[6];         // written
+    const u64* J[3];     // this step's currents
+    u64* Z[3];           // cleared for the next step
+    const u64* rho;      // node density after this step's moves
+    u64* rho_next;       // starts as its copy
     const float* antc;   // nx: amplitude * cos(phase(x))
     const float* ants;   // nx: amplitude * sin(phase(x))
-    const float* ant;    // 2: this step's antenna scalars
+    const float* ant;    // 2: this step's antenna scalars (batch)
     int k_flux;          // node row below the antenna: Poynting flux of the injected energy
     double* flux;        // accumulates sum (Ex By - Ey Bx) over that row at the half step
 };
@@ -211,11 +218,12 @@ void launch_fields(Ctx& c, cudaStream_t st, int64_t step, int64_t* launches);
 constexpr int kMaxFieldSlabs = 48;
 struct FieldBatch {
     FieldArgs f[kMaxFieldSlabs];
-    int rb[kMaxFieldSlabs + 1];      // first (row, 256-node segment) block of each slab
+    int rb[kMaxFieldSlabs + 1];      // first block of each slab
     int n;
 };
-void launch_fields_batch(const FieldBatch& P, const AntennaParams* ap_dev, long long* step_dev, float* ant_dev,
+void launch_fields_batch(const FieldBatch& P, const AntennaParams* ap_dev, long long* step_dev, float* ant_next,
                          cudaStream_t st);
+void launch_antenna_batch(const AntennaParams* ap_dev, const long long* step_dev, float* ant, int n, cudaStream_t st);
 void field_row_blocks(FieldBatch& P);
 FieldArgs make_field_args(const Ctx& c);
 AntennaParams make_antenna_params(const Ctx& c);
