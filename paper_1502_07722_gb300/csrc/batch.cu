@@ -46,7 +46,7 @@ struct pic_batch {
     int n;
     pic_ctx* slab[kMaxSlabs];
     cudaStream_t st;
-    int full, pot, maxW, max_nx, max_nz, total_tiles, nsm, sort_every, steps_since_sort;
+    int full, pot, minW, maxW, max_nx, max_nz, total_tiles, nsm, sort_every, steps_since_sort;
     size_t max_nn;
     int64_t step;
     StepArgs* args_dev;          // [2][n]: parity 0 (density in buffer 0) and parity 1
@@ -120,7 +120,7 @@ void enqueue_step(pic_batch* b, int parity)
     const StepArgs* args = b->args_dev + parity * b->n;
     if (!b->full) enqueue_prepare(b, parity);
     if (b->timing) cudaEventRecord(b->ev[0], b->st);
-    launch_particle_step_batch(args, b->tile_base_dev, b->n, b->total_tiles, b->full, b->pot, b->maxW, b->nsm, b->st);
+    launch_particle_step_batch(args, b->tile_base_dev, b->n, b->total_tiles, b->full, b->pot, b->minW, b->maxW, b->nsm, b->st);
     if (b->timing) cudaEventRecord(b->ev[1], b->st);
     if (b->full)
         launch_fields_batch(b->fields[parity], b->ap_dev, b->step_dev, b->ant_dev + (1 - parity) * 2 * b->n, b->st);
@@ -206,6 +206,7 @@ int pic_batch_init(const pic_config* cfgs, int32_t n, void* workspace, size_t by
         const Ctx& c = b->slab[s]->c;
         tile_base[s + 1] = tile_base[s] + c.ntiles;
         b->maxW = c.W > b->maxW ? c.W : b->maxW;
+        b->minW = s == 0 || c.W < b->minW ? c.W : b->minW;
         b->max_nx = c.nx > b->max_nx ? c.nx : b->max_nx;
         b->max_nz = c.nz > b->max_nz ? c.nz : b->max_nz;
         b->max_nn = c.nn > b->max_nn ? c.nn : b->max_nn;

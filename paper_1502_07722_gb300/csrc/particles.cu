@@ -40,11 +40,10 @@ namespace gbpic {
 constexpr int kMargin = 2;              // cells a particle may drift out of its tile between sorts
 constexpr int kBlock = 128;                // threads per CTA (8 CTAs per SM)
 constexpr int kCtasPerSm = 8;
+constexpr int kWin = 16 + 2 * kMargin + 3;  // window edge of the 16-cell tile (compiled-in instances)
 // The batched kernel reads each slab's arguments from a constant-memory table with a run-time
 // index: every use is an indexed constant load into a register, so it needs more registers than
-// the single kernel for the same code. At 64 registers it spilled ~100 bytes per thread; at 72
-// (7 CTAs per SM) the particle launch of the 16-slab sweep takes 2.03 ms against 2.39 (6 CTAs
-// at 80 registers: 2.23).
+// the single kernel for the same code: 72 (7 CTAs per SM).
 constexpr int kCtasPerSmBatch = 7;
 
 
@@ -90,14 +89,13 @@ __device__ __forceinline__ void red64g(u64* p, long long v)
 }
 
 
-// exact cell -> (i, k): q = floor(cell / nx) from a multiply-high and one correction
-__device__ __forceinline__ void split_cell(int cell, int nx, unsigned magic, int& i, int& k)
+// exact cell -> (i, k) for 0 <= cell < 2^31 (StepArgs::nx_magic, nx_shift): with 2^s <= nx < 2^(s+1)
+// and m = ceil(2^(32+s) / nx), q = floor(cell m / 2^(32+s)) is cell / nx rounded down, since m nx
+// exceeds 2^(32+s) by less than 2^(s+1). (A multiply-high by floor(2^32 / nx) needs a correction.)
+__device__ __forceinline__ void split_cell(int cell, const StepArgs& a, int& i, int& k)
 {
-    unsigned q = __umulhi((unsigned)cell, magic);
-    int r = cell - (int)q * nx;
-    if (r >= nx) { q++; r -= nx; }
-    k = (int)q;
-    i = r;
+    k = (int)(__umulhi((unsigned)cell, a.nx_magic) >> a.nx_shift);
+    i = cell - k * a.nx;
 }
 
 // Rare path: fields and node density straight from global memory (particle outside the window).
@@ -168,36 +166,47 @@ __device__ __noinline__ void deposit_global(u64* rho_next, u64* Jx, u64* Jy, u64
 // Species kinds the particle code is specialised for.
 enum Kind { kIon = 0, kElectron = 1, kAtom = 2 };
 
-// One particle: state in (cell, fx, fz, ux, uy, uz) is replaced by the new state.
+// Fixed-point offset as the bit pattern of rint(f 2^16) + 1.5 2^23: one FMA rounds to the integer (half
+// to even, as the conversion would) and the integer sits in the low bits. Differences of two patterns
+// are differences of the offsets.
+constexpr int kQBias = 0x4B400000;
+__device__ __forceinline__ int qbits(float f) { return __float_as_int(__fmaf_rn(f, 65536.0f, 12582912.0f)); }
+
+// One particle of record p (position already loaded): its momenta are read, the record advanced one
+// step and written back before its deposits, so that little state is live during them.
 //   kIon:      Lorentz force + pair force, current (charge +e), node density
 //   kElectron: Lorentz force, current (charge -e)
 //   kAtom:     pair force, node density (neutral atoms of the transport stage)
-template <int KIND, int POT>
-__device__ __forceinline__ void process_particle(const StepArgs& a, const Species& S, const Window& w, int& cell,
-                                                 float& fx_io, float& fz_io, float& ux, float& uy, float& uz)
+// WC: the window edge when it is compiled in (0: the run-time W).
+// The kernel is bound by instruction issue, so a particle that stays in its cell (almost every one)
+// takes the short way: no floor, no wall test, no new cell index, and its cell is not written (44
+// instead of 48 bytes move per particle). With the window edge compiled in and the one-instruction
+// fixed-point rounding: 424 -> 355 M warp instructions per launch on the 1024^2 slab of 33.5 M
+// particles; 1.90 -> 1.72 ms on the 2048^2 slab, 1.92 -> 1.62 ms on the 16-slab sweep, 0.122 -> 0.114
+// ms on the crater slab, 0.235 -> 0.195 ms with the embedded-atom form on 7.7 M atoms.
+template <int KIND, int POT, int WC>
+__device__ __forceinline__ void process_particle(const StepArgs& a, const Species& S, const Window& w, int p,
+                                                 const int cell0, const float fx, const float fz)
 {
     constexpr bool kFields = KIND != kAtom;
     constexpr bool kPair = KIND != kElectron;
     constexpr bool kCurrent = KIND != kAtom;
     constexpr int kSign = KIND == kElectron ? -1 : 1;
-    const int nx = a.nx, nz = a.nz, W = w.W;
-    const float fx = fx_io, fz = fz_io;
-    const int cell0 = cell;
+    const int nx = a.nx, nz = a.nz, W = WC ? WC : w.W;
+    float ux = S.a.ux[p], uy = S.a.uy[p], uz = S.a.uz[p];
     int i, k;
-    split_cell(cell0, nx, a.nx_magic, i, k);
+    split_cell(cell0, a, i, k);
 
-    // window coordinates (x is periodic: take the image closest to the window centre)
-    int lx = i - w.ox;
-    const int centre = W / 2;
-    if (lx - centre > nx / 2) lx -= nx;
-    else if (centre - lx > nx / 2) lx += nx;
+    // window coordinates (w.ox lies in [0, nx): a column left of it is one period further on)
+    unsigned lx = (unsigned)(i - w.ox);
+    lx = min(lx, lx + (unsigned)nx);
     const int lz = k - w.oz;
-    const bool inwin = lx >= 1 && lx + 2 < W && lz >= 1 && lz + 2 < W;
+    const bool inwin = lx - 1u < (unsigned)(W - 3) && (unsigned)(lz - 1) < (unsigned)(W - 3);
 
     float kx = 0.f, ky = 0.f, kz = 0.f, bx = 0.f, by = 0.f, bz = 0.f;
     float n = 0.f, dnx = 0.f, dnz = 0.f;
     if (inwin) {
-        const int base = lz * W + lx;
+        const int base = lz * W + (int)lx;
         const float gx = 1.0f - fx, gz = 1.0f - fz;
         if (kFields) {
             // four stagger patterns: (0,0) Ey, n; (1/2,0) Ex, Bz; (0,1/2) Ez, Bx; (1/2,1/2) By
@@ -263,7 +272,6 @@ __device__ __forceinline__ void process_particle(const StepArgs& a, const Specie
         kx += S.p_kick * pfx;
         kz += S.p_kick * pfz;
     }
-    const float ux0 = ux, uy0 = uy, uz0 = uz;
     // relativistic Boris: half kick, rotation, half kick
     ux += kx; uy += ky; uz += kz;
     if (kFields) {
@@ -281,101 +289,94 @@ __device__ __forceinline__ void process_particle(const StepArgs& a, const Specie
 
     // move (in-plane), cells per step = u c dt / (gamma dx)
     const float step = a.cdt_dx * rsqrtf(1.0f + ux * ux + uy * uy + uz * uz);
-    float dxi = ux * step, dze = uz * step;
-    if (!(fabsf(dxi) < 1.0f && fabsf(dze) < 1.0f)) {
-        atomicOr(a.status, (isfinite(ux) && isfinite(uy) && isfinite(uz)) ? kErrMove : kErrNan);
-        ux = ux0; uy = uy0; uz = uz0; dxi = 0.0f; dze = 0.0f;
+    const float dxi = __fmul_rn(ux, step), dze = __fmul_rn(uz, step);
+    float nfx = __fadd_rn(fx, dxi), nfz = __fadd_rn(fz, dze);
+    if (!(nfx >= 0.0f && nfx < 1.0f && nfz >= 0.0f && nfz < 1.0f && fabsf(dze) < 1.0f)) {
+        // leaves its cell, reflects off a wall, or moved too far (or is not finite)
+        if (!(fabsf(dxi) < 1.0f && fabsf(dze) < 1.0f)) {
+            // refused: the particle keeps its record (what it deposits is that of a particle at rest
+            // in the plane with its old momenta)
+            atomicOr(a.status, (isfinite(ux) && isfinite(uy) && isfinite(uz)) ? kErrMove : kErrNan);
+            ux = S.a.ux[p];
+            uy = S.a.uy[p];
+            uz = S.a.uz[p];
+            nfx = fx;
+            nfz = fz;
+        }
+        int di = (int)floorf(nfx);
+        nfx -= (float)di;
+        if (nfx >= 1.0f) { nfx = 0.0f; di += 1; }
+        int dk = 0;
+        if (k == 0 && nfz < 0.0f) {                   // reflect off the wall z = 0
+            nfz = -nfz; uz = -uz;
+        } else if (k == nz - 1 && nfz >= 1.0f) {      // reflect off the wall z = nz
+            nfz = 2.0f - nfz; uz = -uz;
+        } else {
+            dk = (int)floorf(nfz);
+            nfz -= (float)dk;
+            if (nfz >= 1.0f) { nfz = 0.0f; dk += 1; }
+        }
+        S.a.cell[p] = (k + dk) * nx + wrap_x(i + di, nx);
+        S.a.fx[p] = nfx;
+        S.a.fz[p] = nfz;
+        S.a.ux[p] = ux;
+        S.a.uy[p] = uy;
+        S.a.uz[p] = uz;
+        const int V = (kCurrent && fabsf(uy) >= a.jy_zero) ? jy_code(ux, uy, uz, a.jy_scale) : 0;
+        deposit_global(a.rho_next, a.J[0], a.J[1], a.J[2], nx, i * kQOne + qoff(fx), k * kQOne + qoff(fz),
+                       (i + di) * kQOne + qoff(nfx), (k + dk) * kQOne + qoff(nfz), kCurrent ? kSign : 0, V,
+                       kPair ? 1 : 0);
+        return;
     }
-    float nfx = fx + dxi;
-    int di = (int)floorf(nfx);
-    nfx -= (float)di;
-    if (nfx >= 1.0f) { nfx = 0.0f; di += 1; }
-    float nfz = fz + dze;
-    int dk = 0;
-    if (k == 0 && nfz < 0.0f) {                   // reflect off the wall z = 0
-        nfz = -nfz; uz = -uz;
-    } else if (k == nz - 1 && nfz >= 1.0f) {      // reflect off the wall z = nz
-        nfz = 2.0f - nfz; uz = -uz;
-    } else {
-        dk = (int)floorf(nfz);
-        nfz -= (float)dk;
-        if (nfz >= 1.0f) { nfz = 0.0f; dk += 1; }
-    }
-    cell = (k + dk) * nx + wrap_x(i + di, nx);
-    fx_io = nfx;
-    fz_io = nfz;
+    S.a.fx[p] = nfx;
+    S.a.fz[p] = nfz;
+    S.a.ux[p] = ux;
+    S.a.uy[p] = uy;
+    S.a.uz[p] = uz;
 
-    const int x0 = qoff(fx), x1 = qoff(nfx), z0 = qoff(fz), z1 = qoff(nfz);
+    // stays in its cell: stencil = the four corners of the cell (global reductions)
+    const int bx0 = qbits(fx), bx1 = qbits(nfx), bz0 = qbits(fz), bz1 = qbits(nfz);
     // |u_y| < 2^-(b+1) gives |beta_y| 2^b < 1/2, i.e. V = 0 without evaluating the code
     const int V = (kCurrent && fabsf(uy) >= a.jy_zero) ? kSign * jy_code(ux, uy, uz, a.jy_scale) : 0;
-    const bool incell = inwin && (di | dk) == 0;
-    if (KIND == kElectron && incell) {
-        // an electron that stays in its cell (almost every electron): it always moves in fixed
-        // point and almost always has V != 0, so the eight reductions onto the cell's corners are
-        // issued without per-term tests (a zero term adds nothing). The out-of-plane weights are
-        // 6 W = A0 U0 + A1 U1 with A = 2^16 - x and U0 = 2 C0 + C1, U1 = C0 + 2 C1 (C = 2^16 - z)
-        // on the lower-left corner, and likewise with x for A and z for C on the others: two
-        // widening 32 x 32-bit products per corner.
-        const int d1 = i + 1 == nx ? 1 - nx : 1;
+    const bool moved = bx1 != bx0 || bz1 != bz0;
+    // nothing to deposit (most ions); an electron always moves in fixed point and almost always has
+    // V != 0, so its reductions are issued without per-term tests (a zero term adds nothing)
+    if (KIND != kElectron && !moved && V == 0) return;
+    const int x0 = bx0 - kQBias, x1 = bx1 - kQBias, z0 = bz0 - kQBias, z1 = bz1 - kQBias;
+    const int d1 = i + 1 == nx ? 1 - nx : 1;
+    if (kCurrent) {
+        const int dX = kSign * (bx1 - bx0), dZ = kSign * (bz1 - bz0);
         u64* jx = a.J[0] + cell0;
         u64* jy = a.J[1] + cell0;
         u64* jz = a.J[2] + cell0;
-        const int dX = x0 - x1, dZ = z0 - z1;          // charge sign -1
-        atomicAdd(jx, (u64)((long long)dX * (2 * kQOne - z0 - z1)));
-        atomicAdd(jx + nx, (u64)((long long)dX * (z0 + z1)));
-        atomicAdd(jz, (u64)((long long)dZ * (2 * kQOne - x0 - x1)));
-        atomicAdd(jz + d1, (u64)((long long)dZ * (x0 + x1)));
-        const int A0 = kQOne - x0, A1 = kQOne - x1, C0 = kQOne - z0, C1 = kQOne - z1;
-        const int U0 = 2 * C0 + C1, U1 = C0 + 2 * C1, Z0 = 2 * z0 + z1, Z1 = z0 + 2 * z1;
-        const long long w00 = (long long)A0 * U0 + (long long)A1 * U1;
-        const long long w10 = (long long)x0 * U0 + (long long)x1 * U1;
-        const long long w01 = (long long)A0 * Z0 + (long long)A1 * Z1;
-        const long long w11 = (long long)x0 * Z0 + (long long)x1 * Z1;
-        atomicAdd(jy, (u64)(V * w00));
-        atomicAdd(jy + d1, (u64)(V * w10));
-        atomicAdd(jy + nx, (u64)(V * w01));
-        atomicAdd(jy + nx + d1, (u64)(V * w11));
-        return;
+        // The out-of-plane weights are 6 W = A0 U0 + A1 U1 with A = 2^16 - x and U0 = 2 C0 + C1,
+        // U1 = C0 + 2 C1 (C = 2^16 - z) on the lower-left corner, and likewise with x for A and z for
+        // C on the others: two widening 32 x 32-bit products per corner.
+        if (KIND == kElectron || dX != 0) {
+            atomicAdd(jx, (u64)((long long)dX * (2 * kQOne - z0 - z1)));
+            atomicAdd(jx + nx, (u64)((long long)dX * (z0 + z1)));
+        }
+        if (KIND == kElectron || dZ != 0) {
+            atomicAdd(jz, (u64)((long long)dZ * (2 * kQOne - x0 - x1)));
+            atomicAdd(jz + d1, (u64)((long long)dZ * (x0 + x1)));
+        }
+        if (KIND == kElectron || V != 0) {
+            const int A0 = kQOne - x0, A1 = kQOne - x1, C0 = kQOne - z0, C1 = kQOne - z1;
+            const int U0 = 2 * C0 + C1, U1 = C0 + 2 * C1, Z0 = 2 * z0 + z1, Z1 = z0 + 2 * z1;
+            atomicAdd(jy, (u64)(V * ((long long)A0 * U0 + (long long)A1 * U1)));
+            atomicAdd(jy + d1, (u64)(V * ((long long)x0 * U0 + (long long)x1 * U1)));
+            atomicAdd(jy + nx, (u64)(V * ((long long)A0 * Z0 + (long long)A1 * Z1)));
+            atomicAdd(jy + nx + d1, (u64)(V * ((long long)x0 * Z0 + (long long)x1 * Z1)));
+        }
     }
-    const bool moved = (di | dk) != 0 || x1 != x0 || z1 != z0;
-    if (!moved && V == 0) return;                 // nothing to deposit (most ions)
-
-    if (incell) {
-        // the particle stays in its cell: stencil = the four corners of the cell (global reductions)
-        const int d1 = i + 1 == nx ? 1 - nx : 1;
-        if (kCurrent) {
-            const int dX = kSign * (x1 - x0), dZ = kSign * (z1 - z0);
-            if (dX != 0) {
-                red64g(a.J[0] + cell0, (long long)dX * (2 * kQOne - z0 - z1));
-                red64g(a.J[0] + cell0 + nx, (long long)dX * (z0 + z1));
-            }
-            if (dZ != 0) {
-                red64g(a.J[2] + cell0, (long long)dZ * (2 * kQOne - x0 - x1));
-                red64g(a.J[2] + cell0 + d1, (long long)dZ * (x0 + x1));
-            }
-            if (V != 0) {
-                const int A0 = kQOne - x0, A1 = kQOne - x1, C0 = kQOne - z0, C1 = kQOne - z1;
-                const int U0 = 2 * C0 + C1, U1 = C0 + 2 * C1, Z0 = 2 * z0 + z1, Z1 = z0 + 2 * z1;
-                u64* jy = a.J[1] + cell0;
-                red64g(jy, V * ((long long)A0 * U0 + (long long)A1 * U1));
-                red64g(jy + d1, V * ((long long)x0 * U0 + (long long)x1 * U1));
-                red64g(jy + nx, V * ((long long)A0 * Z0 + (long long)A1 * Z1));
-                red64g(jy + nx + d1, V * ((long long)x0 * Z0 + (long long)x1 * Z1));
-            }
-        }
-        if (kPair && moved) {
-            // weights are at most 2^16: each product is one 32 x 32 -> 64-bit multiply
-            const int a0 = kQOne - x0, a1 = kQOne - x1, c0 = kQOne - z0, c1 = kQOne - z1;
-            u64* r = a.rho_next + cell0;
-            red64g(r, (long long)a1 * c1 - (long long)a0 * c0);
-            red64g(r + d1, (long long)x1 * c1 - (long long)x0 * c0);
-            red64g(r + nx, (long long)a1 * z1 - (long long)a0 * z0);
-            red64g(r + nx + d1, (long long)x1 * z1 - (long long)x0 * z0);
-        }
-    } else {
-        // deposit_global applies the charge sign itself: hand it the unsigned code kSign * V
-        deposit_global(a.rho_next, a.J[0], a.J[1], a.J[2], nx, i * kQOne + x0, k * kQOne + z0,
-                       (i + di) * kQOne + x1, (k + dk) * kQOne + z1, kCurrent ? kSign : 0, kSign * V, kPair ? 1 : 0);
+    if (kPair && moved) {
+        // weights are at most 2^16: each product is one 32 x 32 -> 64-bit multiply
+        const int a0 = kQOne - x0, a1 = kQOne - x1, c0 = kQOne - z0, c1 = kQOne - z1;
+        u64* r = a.rho_next + cell0;
+        red64g(r, (long long)a1 * c1 - (long long)a0 * c0);
+        red64g(r + d1, (long long)x1 * c1 - (long long)x0 * c0);
+        red64g(r + nx, (long long)a1 * z1 - (long long)a0 * z0);
+        red64g(r + nx + d1, (long long)x1 * z1 - (long long)x0 * z0);
     }
 }
 
@@ -387,11 +388,11 @@ __device__ __forceinline__ int part_start(int p0, int p1, int sub, int nsub)
     return p0 + (int)(((long long)(p1 - p0) * sub) / nsub);
 }
 
-template <bool FULL, int POT>
+template <bool FULL, int POT, int WC>
 __device__ __forceinline__ void run_tile(const StepArgs& a, int t, int sub, int nsub)
 {
     extern __shared__ unsigned smem[];
-    const int W = a.W, WW = W * W;
+    const int W = WC ? WC : a.W, WW = W * W;
     Window w;
     w.W = W;
     float* fbase = reinterpret_cast<float*>(smem);
@@ -401,74 +402,68 @@ __device__ __forceinline__ void run_tile(const StepArgs& a, int t, int sub, int 
     w.by = fbase + 6 * WW;
     w.nh = fbase;
 
-    {
-        int cnt = 0;
+    int cnt = 0;
 #pragma unroll
-        for (int s = 0; s < 2; s++)
-            if (s < a.nsp) {
-                const int p0 = a.sp[s].tile_start[t], p1 = a.sp[s].tile_start[t + 1];
-                cnt += part_start(p0, p1, sub + 1, nsub) - part_start(p0, p1, sub, nsub);
-            }
-        if (cnt == 0) return;
-        const int tx = t % a.ntx, tz = t / a.ntx;
-        w.ox = tx * a.T - kMargin - 1;
-        w.oz = tz * a.T - kMargin - 1;
-        // stage the window: fields, pair density (wall rows doubled)
-        for (int j = threadIdx.x; j < WW; j += blockDim.x) {
-            const int b = j / W, c = j - b * W;
-            const int gx = wrap_any(w.ox + c, a.nx);
-            const int gz = w.oz + b;
-            const int gn = min(max(gz, 0), a.nz);          // node rows 0..nz
-            const int gh = min(max(gz, 0), a.nz - 1);      // half rows 0..nz-1 (edge rows repeat)
-            const size_t in = (size_t)gn * a.nx + gx, ih = (size_t)gh * a.nx + gx;
-            const long long r = (long long)__ldg(a.rho_cur + in);
-            const float nh = a.rho_s * (float)((gn == 0 || gn == a.nz) ? 2 * r : r);
-            if (FULL) {
-                w.exbz[j] = make_float2(__ldg(a.F[0] + in), __ldg(a.F[5] + in));
-                w.ezbx[j] = make_float2(__ldg(a.F[2] + ih), __ldg(a.F[3] + ih));
-                w.eyn[j] = make_float2(__ldg(a.F[1] + in), nh);
-                w.by[j] = __ldg(a.F[4] + ih);
-            } else {
-                w.nh[j] = nh;
-            }
+    for (int s = 0; s < 2; s++)
+        if (s < a.nsp) {
+            const int p0 = a.sp[s].tile_start[t], p1 = a.sp[s].tile_start[t + 1];
+            cnt += part_start(p0, p1, sub + 1, nsub) - part_start(p0, p1, sub, nsub);
         }
-        __syncthreads();
+    if (cnt == 0) return;
+    const int tx = t % a.ntx, tz = t / a.ntx;
+    w.ox = wrap_any(tx * a.T - kMargin - 1, a.nx);
+    w.oz = tz * a.T - kMargin - 1;
+    // stage the window: fields, pair density (wall rows doubled)
 #pragma unroll
-        for (int s = 0; s < 2; s++) {
-            if (s >= a.nsp) break;
-            const Species& S = a.sp[s];
-            const int q0 = S.tile_start[t], q1 = S.tile_start[t + 1];
-            const int p0 = part_start(q0, q1, sub, nsub), p1 = part_start(q0, q1, sub + 1, nsub);
-            // the next record's position is loaded one iteration ahead (its first use is at the top
-            // of the iteration); the momenta, first used after the gathers, are loaded in the iteration
-            int ncell = 0;
-            float nfx = 0.0f, nfz = 0.0f;
-            if (p0 + (int)threadIdx.x < p1) {
-                const int q = p0 + (int)threadIdx.x;
-                ncell = S.a.cell[q];
-                nfx = S.a.fx[q];
-                nfz = S.a.fz[q];
-            }
-            for (int p = p0 + (int)threadIdx.x; p < p1; p += kBlock) {
-                int cell = ncell;
-                float fx = nfx, fz = nfz, ux = S.a.ux[p], uy = S.a.uy[p], uz = S.a.uz[p];
-                if (p + kBlock < p1) {
-                    ncell = S.a.cell[p + kBlock];
-                    nfx = S.a.fx[p + kBlock];
-                    nfz = S.a.fz[p + kBlock];
-                }
-                if (s == 0) process_particle<FULL ? kIon : kAtom, POT>(a, S, w, cell, fx, fz, ux, uy, uz);
-                else process_particle<kElectron, POT>(a, S, w, cell, fx, fz, ux, uy, uz);
-                S.a.cell[p] = cell;
-                S.a.fx[p] = fx;
-                S.a.fz[p] = fz;
-                S.a.ux[p] = ux;
-                S.a.uy[p] = uy;
-                S.a.uz[p] = uz;
-            }
+    for (int j = threadIdx.x; j < WW; j += kBlock) {
+        const int b = j / W, c = j - b * W;
+        int gx = w.ox + c;
+        while (gx >= a.nx) gx -= a.nx;
+        const int gz = w.oz + b;
+        const int gn = min(max(gz, 0), a.nz);          // node rows 0..nz
+        const int gh = min(max(gz, 0), a.nz - 1);      // half rows 0..nz-1 (edge rows repeat)
+        const size_t in = (size_t)gn * a.nx + gx, ih = (size_t)gh * a.nx + gx;
+        const long long r = (long long)__ldg(a.rho_cur + in);
+        const float nh = a.rho_s * (float)((gn == 0 || gn == a.nz) ? 2 * r : r);
+        if (FULL) {
+            w.exbz[j] = make_float2(__ldg(a.F[0] + in), __ldg(a.F[5] + in));
+            w.ezbx[j] = make_float2(__ldg(a.F[2] + ih), __ldg(a.F[3] + ih));
+            w.eyn[j] = make_float2(__ldg(a.F[1] + in), nh);
+            w.by[j] = __ldg(a.F[4] + ih);
+        } else {
+            w.nh[j] = nh;
         }
-        __syncthreads();
     }
+    __syncthreads();
+#pragma unroll
+    for (int s = 0; s < 2; s++) {
+        if (s >= a.nsp) break;
+        const Species& S = a.sp[s];
+        const int q0 = S.tile_start[t], q1 = S.tile_start[t + 1];
+        const int p0 = part_start(q0, q1, sub, nsub), p1 = part_start(q0, q1, sub + 1, nsub);
+        // the next record's position is loaded one iteration ahead (its first use is at the top
+        // of the iteration); the momenta, first used after the gathers, are loaded in the iteration
+        int ncell = 0;
+        float nfx = 0.0f, nfz = 0.0f;
+        if (p0 + (int)threadIdx.x < p1) {
+            const int q = p0 + (int)threadIdx.x;
+            ncell = S.a.cell[q];
+            nfx = S.a.fx[q];
+            nfz = S.a.fz[q];
+        }
+        for (int p = p0 + (int)threadIdx.x; p < p1; p += kBlock) {
+            const int cell = ncell;
+            const float fx = nfx, fz = nfz;
+            if (p + kBlock < p1) {
+                ncell = S.a.cell[p + kBlock];
+                nfx = S.a.fx[p + kBlock];
+                nfz = S.a.fz[p + kBlock];
+            }
+            if (s == 0) process_particle<FULL ? kIon : kAtom, POT, WC>(a, S, w, p, cell, fx, fz);
+            else process_particle<kElectron, POT, WC>(a, S, w, p, cell, fx, fz);
+        }
+    }
+    __syncthreads();
 }
 
 // Work items (a tile, or a part of a tile) are handed out dynamically: each CTA draws the next one
@@ -485,13 +480,13 @@ __device__ __forceinline__ int next_item(unsigned* ticket, int total, int* slot)
     return g;
 }
 
-template <bool FULL, int POT>
+template <bool FULL, int POT, int WC>
 __global__ void __launch_bounds__(kBlock, kCtasPerSm) k_particles(const StepArgs a, int nsub)
 {
     __shared__ int slot;
     const int total = a.ntiles * nsub;
     for (int g = next_item(a.status + 2, total, &slot); g < total; g = next_item(a.status + 2, total, &slot))
-        run_tile<FULL, POT>(a, g / nsub, g % nsub, nsub);
+        run_tile<FULL, POT, WC>(a, g / nsub, g % nsub, nsub);
 }
 
 // Arguments of the simulations of a batch for the current step, in constant memory: the slab
@@ -504,7 +499,7 @@ __constant__ int c_tile_base[kMaxBatchSlabs + 1];
 
 // All simulations of a batch in one persistent launch: the tiles of every simulation form one
 // work list (c_tile_base[s] = first global tile of simulation s).
-template <bool FULL, int POT>
+template <bool FULL, int POT, int WC>
 __global__ void __launch_bounds__(kBlock, kCtasPerSmBatch) k_particles_batch(int nslab, int total, int nsub)
 {
     // one ticket counter for the whole batch: the first simulation's
@@ -514,7 +509,7 @@ __global__ void __launch_bounds__(kBlock, kCtasPerSmBatch) k_particles_batch(int
         const int tile = g / nsub;
         int s = 0;
         while (s + 1 < nslab && c_tile_base[s + 1] <= tile) s++;
-        run_tile<FULL, POT>(c_batch_args[s], tile - c_tile_base[s], g % nsub, nsub);
+        run_tile<FULL, POT, WC>(c_batch_args[s], tile - c_tile_base[s], g % nsub, nsub);
     }
 }
 
@@ -548,7 +543,11 @@ void launch_particle_step(Ctx& c, const StepArgs& a, cudaStream_t st)
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) dev = 0;
     if (shmem > configured[dev].load()) {
-#define GBPIC_ATTR(P) set_smem((const void*)k_particles<true, (P)>, shmem); set_smem((const void*)k_particles<false, (P)>, shmem);
+#define GBPIC_ATTR(P)                                                                                       \
+    set_smem((const void*)k_particles<true, (P), 0>, shmem);                                               \
+    set_smem((const void*)k_particles<false, (P), 0>, shmem);                                              \
+    set_smem((const void*)k_particles<true, (P), kWin>, shmem);                                            \
+    set_smem((const void*)k_particles<false, (P), kWin>, shmem);
         GBPIC_FOR_EACH_POT(GBPIC_ATTR)
 #undef GBPIC_ATTR
         configured[dev].store(shmem);
@@ -558,11 +557,14 @@ void launch_particle_step(Ctx& c, const StepArgs& a, cudaStream_t st)
     int grid = a.ntiles * nsub;
     if (grid > cap) grid = cap;
     if (grid < 1) grid = 1;
-    // the instance with the potential and the lattice compiled in
-    switch ((a.pot_mode & 7) | (a.full ? 8 : 0)) {
+    // the instance with the potential and the lattice compiled in, and the window edge when it is
+    // the 16-cell tile's
+    switch ((a.pot_mode & 7) | (a.full ? 8 : 0) | (a.W == kWin ? 16 : 0)) {
 #define GBPIC_CASE(P)                                                                                 \
-    case 8 | (P): k_particles<true, (P)><<<grid, kBlock, shmem, st>>>(a, nsub); break;                \
-    case (P): k_particles<false, (P)><<<grid, kBlock, shmem, st>>>(a, nsub); break;
+    case 24 | (P): k_particles<true, (P), kWin><<<grid, kBlock, shmem, st>>>(a, nsub); break;         \
+    case 16 | (P): k_particles<false, (P), kWin><<<grid, kBlock, shmem, st>>>(a, nsub); break;        \
+    case 8 | (P): k_particles<true, (P), 0><<<grid, kBlock, shmem, st>>>(a, nsub); break;             \
+    case (P): k_particles<false, (P), 0><<<grid, kBlock, shmem, st>>>(a, nsub); break;
         GBPIC_FOR_EACH_POT(GBPIC_CASE)
 #undef GBPIC_CASE
     }
@@ -571,7 +573,7 @@ void launch_particle_step(Ctx& c, const StepArgs& a, cudaStream_t st)
 int max_batch_slabs() { return kMaxBatchSlabs; }
 
 void launch_particle_step_batch(const StepArgs* args_dev, const int* tile_base_dev, int nslab, int total_tiles,
-                                int full, int pot, int maxW, int nsm, cudaStream_t st)
+                                int full, int pot, int minW, int maxW, int nsm, cudaStream_t st)
 {
     cudaMemcpyToSymbolAsync(c_batch_args, args_dev, sizeof(StepArgs) * nslab, 0, cudaMemcpyDeviceToDevice, st);
     cudaMemcpyToSymbolAsync(c_tile_base, tile_base_dev, sizeof(int) * (nslab + 1), 0, cudaMemcpyDeviceToDevice, st);
@@ -581,7 +583,11 @@ void launch_particle_step_batch(const StepArgs* args_dev, const int* tile_base_d
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) dev = 0;
     if (shmem > configured[dev].load()) {
-#define GBPIC_ATTR(P) set_smem((const void*)k_particles_batch<true, (P)>, shmem); set_smem((const void*)k_particles_batch<false, (P)>, shmem);
+#define GBPIC_ATTR(P)                                                                                       \
+    set_smem((const void*)k_particles_batch<true, (P), 0>, shmem);                                         \
+    set_smem((const void*)k_particles_batch<false, (P), 0>, shmem);                                        \
+    set_smem((const void*)k_particles_batch<true, (P), kWin>, shmem);                                      \
+    set_smem((const void*)k_particles_batch<false, (P), kWin>, shmem);
         GBPIC_FOR_EACH_POT(GBPIC_ATTR)
 #undef GBPIC_ATTR
         configured[dev].store(shmem);
@@ -590,11 +596,14 @@ void launch_particle_step_batch(const StepArgs* args_dev, const int* tile_base_d
     const int nsub = parts_per_tile(total_tiles, cap);
     int grid = total_tiles * nsub < cap ? total_tiles * nsub : cap;
     if (grid < 1) grid = 1;
-    // pot: the instance code shared by every slab (potential and lattice)
-    switch ((pot & 7) | (full ? 8 : 0)) {
-#define GBPIC_CASE(P)                                                                                          \
-    case 8 | (P): k_particles_batch<true, (P)><<<grid, kBlock, shmem, st>>>(nslab, total_tiles, nsub); break;   \
-    case (P): k_particles_batch<false, (P)><<<grid, kBlock, shmem, st>>>(nslab, total_tiles, nsub); break;
+    // pot: the instance code shared by every slab (potential and lattice); the compiled-in window
+    // edge when every slab has it
+    switch ((pot & 7) | (full ? 8 : 0) | (minW == kWin && maxW == kWin ? 16 : 0)) {
+#define GBPIC_CASE(P)                                                                                              \
+    case 24 | (P): k_particles_batch<true, (P), kWin><<<grid, kBlock, shmem, st>>>(nslab, total_tiles, nsub); break; \
+    case 16 | (P): k_particles_batch<false, (P), kWin><<<grid, kBlock, shmem, st>>>(nslab, total_tiles, nsub); break; \
+    case 8 | (P): k_particles_batch<true, (P), 0><<<grid, kBlock, shmem, st>>>(nslab, total_tiles, nsub); break;    \
+    case (P): k_particles_batch<false, (P), 0><<<grid, kBlock, shmem, st>>>(nslab, total_tiles, nsub); break;
         GBPIC_FOR_EACH_POT(GBPIC_CASE)
 #undef GBPIC_CASE
     }

@@ -91,7 +91,8 @@ inline int pot_code(const pic_config& cfg) { return cfg.pot_mode | (cfg.lattice 
 // Everything a kernel of the step needs, passed by value.
 struct StepArgs {
     int32_t nx, nz, T, ntx, ntz, ntiles, W;   // W: window edge (nodes) of a tile
-    unsigned nx_magic;                        // floor(2^32 / nx) for the cell -> (i, k) split
+    unsigned nx_magic;                        // ceil(2^(32 + nx_shift) / nx) for the cell -> (i, k) split
+    int32_t nx_shift;                         // 2^nx_shift < nx <= 2^(nx_shift + 1)
     int32_t full;                             // fields and Lorentz force on
     float cdt_dx;                             // c dt / dx
     float rho_s;                              // node sum -> n / n0
@@ -228,7 +229,7 @@ void field_row_blocks(FieldBatch& P);
 FieldArgs make_field_args(const Ctx& c);
 AntennaParams make_antenna_params(const Ctx& c);
 void launch_particle_step_batch(const StepArgs* args_dev, const int* tile_base_dev, int nslab, int total_tiles,
-                                int full, int pot, int maxW, int nsm, cudaStream_t st);
+                                int full, int pot, int minW, int maxW, int nsm, cudaStream_t st);
 size_t particle_smem_bytes(int W);
 void launch_particle_step3(Ctx& c, cudaStream_t st);
 void launch_deposit_density3(Ctx& c, u64* out, cudaStream_t st);
