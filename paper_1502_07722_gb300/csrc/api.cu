@@ -237,8 +237,7 @@ StepArgs make_step_args(Ctx& c)
     a.ntz = c.ntz;
     a.ntiles = c.ntiles;
     a.W = c.W;
-    while ((2 << a.nx_shift) < c.nx) a.nx_shift++;       // 2^shift < nx <= 2^(shift + 1), so the magic fits 32 bits
-    a.nx_magic = (unsigned)(((1ULL << (32 + a.nx_shift)) + (unsigned)c.nx - 1) / (unsigned)c.nx);
+    magic_div(c.nx, a.nx_magic, a.nx_shift);
     a.full = c.cfg.mode == PIC_MODE_FULL;
     a.cdt_dx = (float)(kC * c.dt / c.cfg.dx);
     a.rho_s = (float)c.rho_scale;

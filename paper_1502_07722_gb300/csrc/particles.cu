@@ -89,9 +89,7 @@ __device__ __forceinline__ void red64g(u64* p, long long v)
 }
 
 
-// exact cell -> (i, k) for 0 <= cell < 2^31 (StepArgs::nx_magic, nx_shift): with 2^s <= nx < 2^(s+1)
-// and m = ceil(2^(32+s) / nx), q = floor(cell m / 2^(32+s)) is cell / nx rounded down, since m nx
-// exceeds 2^(32+s) by less than 2^(s+1). (A multiply-high by floor(2^32 / nx) needs a correction.)
+// exact cell -> (i, k) (magic_div; a multiply-high by floor(2^32 / nx) needs a correction)
 __device__ __forceinline__ void split_cell(int cell, const StepArgs& a, int& i, int& k)
 {
     k = (int)(__umulhi((unsigned)cell, a.nx_magic) >> a.nx_shift);

@@ -40,20 +40,16 @@ __device__ __forceinline__ void hat3q(int d, int& s0, int& s1, int& s2)
 
 struct Geo3 {
     int nx, ny, nz;
-    unsigned mag_x, mag_y;     // floor(2^32 / nx), floor(2^32 / ny)
+    unsigned mag_x, mag_y;     // exact division by nx and ny: q = umulhi(v, mag) >> shift for v < 2^31
+    int sh_x, sh_y;            // 2^shift < n <= 2^(shift + 1), mag = ceil(2^(32 + shift) / n)
 };
 
 __device__ __forceinline__ void split3(int cell, const Geo3& g, int& i, int& j, int& k)
 {
-    unsigned q = __umulhi((unsigned)cell, g.mag_x);
-    int r = cell - (int)q * g.nx;
-    if (r >= g.nx) { q++; r -= g.nx; }
-    i = r;
-    unsigned q2 = __umulhi(q, g.mag_y);
-    int r2 = (int)q - (int)q2 * g.ny;
-    if (r2 >= g.ny) { q2++; r2 -= g.ny; }
-    j = r2;
-    k = (int)q2;
+    const int q = (int)(__umulhi((unsigned)cell, g.mag_x) >> g.sh_x);
+    i = cell - q * g.nx;
+    k = (int)(__umulhi((unsigned)q, g.mag_y) >> g.sh_y);
+    j = q - k * g.ny;
 }
 
 __device__ __forceinline__ size_t idx3(const Geo3& g, int i, int j, int k)
@@ -309,14 +305,12 @@ __device__ __noinline__ void gather_global3(const float* F0, const float* F1, co
 // without a zero test: a particle that moved along an axis almost never has a zero term, and a zero
 // adds nothing. Inlined: the currents' base pointers stay kernel parameters (against an
 // out-of-line call: 7.68 -> 7.44 ms per launch on the 384^2 x 256 slab).
-__device__ __forceinline__ void deposit3_cell(Geo3 g, u64* J0, u64* J1, u64* J2, u64* rho_next, int i, int j,
-                                                   int k, int x0, int y0, int z0, int x1, int y1, int z1, int jsign,
-                                                   int pair)
+// The offsets to the cell's other corners (x, y periodic) fit 32 bits: a grid has fewer than 2^31 nodes.
+__device__ __forceinline__ void deposit3_cell(Geo3 g, u64* J0, u64* J1, u64* J2, u64* rho_next, int base, int i,
+                                              int j, int x0, int y0, int z0, int x1, int y1, int z1, int jsign,
+                                              int pair)
 {
-    const int i1 = wrapn(i + 1, g.nx), j1 = wrapn(j + 1, g.ny);
-    // one base index and the offsets to the cell's other corners (x, y periodic)
-    const size_t base = idx3(g, i, j, k);
-    const ptrdiff_t ox = i1 - i, oy = (ptrdiff_t)(j1 - j) * g.nx, oz = (ptrdiff_t)g.nx * g.ny;
+    const int ox = i + 1 == g.nx ? 1 - g.nx : 1, oy = j + 1 == g.ny ? (1 - g.ny) * g.nx : g.nx, oz = g.nx * g.ny;
     const int ax0 = kQ3 - x0, ax1 = kQ3 - x1, ay0 = kQ3 - y0, ay1 = kQ3 - y1, az0 = kQ3 - z0, az1 = kQ3 - z1;
     if (jsign) {
         const int dX = jsign * (x1 - x0), dY = jsign * (y1 - y0), dZ = jsign * (z1 - z0);
@@ -359,11 +353,20 @@ __device__ __forceinline__ void deposit3_cell(Geo3 g, u64* J0, u64* J1, u64* J2,
     }
 }
 
+// Fixed-point offset as the bit pattern of rint(f 2^14) + 1.5 2^23: one FMA rounds to the integer (half
+// to even, as the conversion would); differences of two patterns are differences of the offsets.
+constexpr int kQ3Bias = 0x4B400000;
+__device__ __forceinline__ int qbits3(float f) { return __float_as_int(__fmaf_rn(f, 16384.0f, 12582912.0f)); }
+
 // Particle p of species S (position (cell, fx, fy, fz) loaded by the caller): its momenta are read,
 // the record advanced one step and written back before its deposits, so that little state is live
 // during them. PAIR is a run-time flag (the pair species): one instance of this code serves both
 // species, which keeps the kernel inside the instruction cache. WC is the window edge when it is
 // compiled in (0: the run-time a.W).
+// As in 2D, a particle that stays in its cell (almost every one) takes the short way: no floor, no
+// wall test, no new cell index, and its cell is not written (52 instead of 56 bytes move per particle):
+// 602 -> 526 warp instructions per 32 particles, 7.39 -> 7.01 ms per launch on the 384^2 x 256 slab, 2.89
+// -> 2.79 ms on the 144 M atoms of the 3D crater slab.
 template <bool FULL, int POT, int WC>
 __device__ __forceinline__ void process3(const Args3& a, const Species3& S, const Win3& w, const bool PAIR, int p,
                                          const int cell, const float fx, const float fy, const float fz)
@@ -372,20 +375,19 @@ __device__ __forceinline__ void process3(const Args3& a, const Species3& S, cons
     float ux = S.ux[p], uy = S.uy[p], uz = S.uz[p];
     int i, j, k;
     split3(cell, g, i, j, k);
-    // window coordinates (x, y periodic: the image closest to the window centre)
-    const int W = WC ? WC : w.W, cen = W / 2;
-    int lx = i - w.ox, ly = j - w.oy;
-    if (lx - cen > g.nx / 2) lx -= g.nx;
-    else if (cen - lx > g.nx / 2) lx += g.nx;
-    if (ly - cen > g.ny / 2) ly -= g.ny;
-    else if (cen - ly > g.ny / 2) ly += g.ny;
+    // window coordinates (w.ox, w.oy lie in [0, n): a node before them is one period further on)
+    const int W = WC ? WC : w.W;
+    unsigned lx = (unsigned)(i - w.ox), ly = (unsigned)(j - w.oy);
+    lx = min(lx, lx + (unsigned)g.nx);
+    ly = min(ly, ly + (unsigned)g.ny);
     const int lz = k - w.oz;
-    const bool inwin = W > 0 && lx >= 1 && lx + 2 < W && ly >= 1 && ly + 2 < W && lz >= 1 && lz + 2 < W;
+    const bool inwin = W > 0 && lx - 1u < (unsigned)(W - 3) && ly - 1u < (unsigned)(W - 3) &&
+                       (unsigned)(lz - 1) < (unsigned)(W - 3);
     float kx = 0.f, ky = 0.f, kz = 0.f, bx = 0.f, by = 0.f, bz = 0.f;
     float n = 0.f, gr[3] = {0.f, 0.f, 0.f};
     if (inwin) {
         const int Wk = WC ? WC : W;
-        const int base = (lz * Wk + ly) * Wk + lx;
+        const int base = (lz * Wk + (int)ly) * Wk + (int)lx;
         if (FULL) {
             float o[6];
             wfields3<WC>(w.f, W, base, fx, fy, fz, o);
@@ -414,7 +416,6 @@ __device__ __forceinline__ void process3(const Args3& a, const Species3& S, cons
             kz += S.p_kick * pf[2];
         }
     }
-    const float ux0 = ux, uy0 = uy, uz0 = uz;
     ux += kx; uy += ky; uz += kz;
     if (FULL) {
         const float ig = rsqrtf(1.0f + ux * ux + uy * uy + uz * uz);
@@ -429,29 +430,49 @@ __device__ __forceinline__ void process3(const Args3& a, const Species3& S, cons
     }
     ux += kx; uy += ky; uz += kz;
     const float ig = rsqrtf(1.0f + ux * ux + uy * uy + uz * uz);
-    float dxi = ux * a.cdt_dx * ig, dyi = uy * a.cdt_dx * ig, dze = uz * a.cdt_dx * ig;
-    if (!(fabsf(dxi) < 1.0f && fabsf(dyi) < 1.0f && fabsf(dze) < 1.0f)) {
-        atomicOr(a.status, (isfinite(ux) && isfinite(uy) && isfinite(uz)) ? kErrMove : kErrNan);
-        ux = ux0; uy = uy0; uz = uz0; dxi = dyi = dze = 0.0f;
+    const float dxi = __fmul_rn(__fmul_rn(ux, a.cdt_dx), ig), dyi = __fmul_rn(__fmul_rn(uy, a.cdt_dx), ig),
+                dze = __fmul_rn(__fmul_rn(uz, a.cdt_dx), ig);
+    float nfx = __fadd_rn(fx, dxi), nfy = __fadd_rn(fy, dyi), nfz = __fadd_rn(fz, dze);
+    if (!(nfx >= 0.0f && nfx < 1.0f && nfy >= 0.0f && nfy < 1.0f && nfz >= 0.0f && nfz < 1.0f && fabsf(dze) < 1.0f)) {
+        // leaves its cell, reflects off a wall, or moved too far (or is not finite)
+        if (!(fabsf(dxi) < 1.0f && fabsf(dyi) < 1.0f && fabsf(dze) < 1.0f)) {
+            // refused: the particle keeps its record
+            atomicOr(a.status, (isfinite(ux) && isfinite(uy) && isfinite(uz)) ? kErrMove : kErrNan);
+            ux = S.ux[p];
+            uy = S.uy[p];
+            uz = S.uz[p];
+            nfx = fx;
+            nfy = fy;
+            nfz = fz;
+        }
+        int di = (int)floorf(nfx);
+        nfx -= (float)di;
+        if (nfx >= 1.0f) { nfx = 0.0f; di += 1; }
+        int dj = (int)floorf(nfy);
+        nfy -= (float)dj;
+        if (nfy >= 1.0f) { nfy = 0.0f; dj += 1; }
+        int dk = 0;
+        if (k == 0 && nfz < 0.0f) {
+            nfz = -nfz; uz = -uz;
+        } else if (k == g.nz - 1 && nfz >= 1.0f) {
+            nfz = 2.0f - nfz; uz = -uz;
+        } else {
+            dk = (int)floorf(nfz);
+            nfz -= (float)dk;
+            if (nfz >= 1.0f) { nfz = 0.0f; dk += 1; }
+        }
+        S.cell[p] = (int)idx3(g, wrapn(i + di, g.nx), wrapn(j + dj, g.ny), k + dk);
+        S.fx[p] = nfx;
+        S.fy[p] = nfy;
+        S.fz[p] = nfz;
+        S.ux[p] = ux;
+        S.uy[p] = uy;
+        S.uz[p] = uz;
+        deposit3_general(g, a.J[0], a.J[1], a.J[2], a.rho_next, i * kQ3 + qoff3(fx), j * kQ3 + qoff3(fy),
+                         k * kQ3 + qoff3(fz), (i + di) * kQ3 + qoff3(nfx), (j + dj) * kQ3 + qoff3(nfy),
+                         (k + dk) * kQ3 + qoff3(nfz), S.jsign, PAIR ? 1 : 0);
+        return;
     }
-    float nfx = fx + dxi, nfy = fy + dyi, nfz = fz + dze;
-    int di = (int)floorf(nfx);
-    nfx -= (float)di;
-    if (nfx >= 1.0f) { nfx = 0.0f; di += 1; }
-    int dj = (int)floorf(nfy);
-    nfy -= (float)dj;
-    if (nfy >= 1.0f) { nfy = 0.0f; dj += 1; }
-    int dk = 0;
-    if (k == 0 && nfz < 0.0f) {
-        nfz = -nfz; uz = -uz;
-    } else if (k == g.nz - 1 && nfz >= 1.0f) {
-        nfz = 2.0f - nfz; uz = -uz;
-    } else {
-        dk = (int)floorf(nfz);
-        nfz -= (float)dk;
-        if (nfz >= 1.0f) { nfz = 0.0f; dk += 1; }
-    }
-    S.cell[p] = (int)idx3(g, wrapn(i + di, g.nx), wrapn(j + dj, g.ny), k + dk);
     S.fx[p] = nfx;
     S.fy[p] = nfy;
     S.fz[p] = nfz;
@@ -459,15 +480,10 @@ __device__ __forceinline__ void process3(const Args3& a, const Species3& S, cons
     S.uy[p] = uy;
     S.uz[p] = uz;
 
-    const int x0 = qoff3(fx), x1 = qoff3(nfx), y0 = qoff3(fy), y1 = qoff3(nfy), z0 = qoff3(fz), z1 = qoff3(nfz);
-    const bool moved = (di | dj | dk) != 0 || x1 != x0 || y1 != y0 || z1 != z0;
-    if (!moved) return;
-    if ((di | dj | dk) == 0) {
-        deposit3_cell(g, a.J[0], a.J[1], a.J[2], a.rho_next, i, j, k, x0, y0, z0, x1, y1, z1, S.jsign, PAIR ? 1 : 0);
-    } else {
-        deposit3_general(g, a.J[0], a.J[1], a.J[2], a.rho_next, i * kQ3 + x0, j * kQ3 + y0, k * kQ3 + z0,
-                         (i + di) * kQ3 + x1, (j + dj) * kQ3 + y1, (k + dk) * kQ3 + z1, S.jsign, PAIR ? 1 : 0);
-    }
+    const int x0 = qbits3(fx), x1 = qbits3(nfx), y0 = qbits3(fy), y1 = qbits3(nfy), z0 = qbits3(fz), z1 = qbits3(nfz);
+    if (x1 == x0 && y1 == y0 && z1 == z0) return;
+    deposit3_cell(g, a.J[0], a.J[1], a.J[2], a.rho_next, cell, i, j, x0 - kQ3Bias, y0 - kQ3Bias, z0 - kQ3Bias,
+                  x1 - kQ3Bias, y1 - kQ3Bias, z1 - kQ3Bias, S.jsign, PAIR ? 1 : 0);
 }
 
 template <bool FULL, int POT, int WC>
@@ -494,16 +510,16 @@ __global__ void __launch_bounds__(kBlock3, 3) k_particles3(const __grid_constant
         for (int s = 0; s < a.nsp; s++) cnt += a.sp[s].tile_start[t + 1] - a.sp[s].tile_start[t];
         if (cnt == 0) continue;
         const int tx = t % a.ntx, ty = (t / a.ntx) % a.nty, tz = t / (a.ntx * a.nty);
-        w.ox = tx * a.T - 1;
-        w.oy = ty * a.T - 1;
+        w.ox = wrapn(tx * a.T - 1, g.nx);
+        w.oy = wrapn(ty * a.T - 1, g.ny);
         w.oz = tz * a.T - 1;
         if (W > 0) {
             __syncthreads();                       // the previous tile is done with the window
-            for (int q = threadIdx.x; q < WWW; q += blockDim.x) {
+            for (int q = threadIdx.x; q < WWW; q += kBlock3) {
                 const int c = q / WW, r = q - c * WW, b = r / W, e = r - b * W;
-                int gx = (w.ox + e) % g.nx, gy = (w.oy + b) % g.ny;
-                gx = gx < 0 ? gx + g.nx : gx;
-                gy = gy < 0 ? gy + g.ny : gy;
+                int gx = w.ox + e, gy = w.oy + b;
+                while (gx >= g.nx) gx -= g.nx;
+                while (gy >= g.ny) gy -= g.ny;
                 const int gz = w.oz + c;
                 const int gn = min(max(gz, 0), g.nz), gh = min(max(gz, 0), g.nz - 1);
                 const size_t in = idx3(g, gx, gy, gn), ih = idx3(g, gx, gy, gh);
@@ -554,8 +570,8 @@ static Geo3 geo_of(const Ctx& c)
     g.nx = c.nx;
     g.ny = c.ny;
     g.nz = c.nz;
-    g.mag_x = (unsigned)(4294967296ULL / (unsigned long long)c.nx);
-    g.mag_y = (unsigned)(4294967296ULL / (unsigned long long)c.ny);
+    magic_div(c.nx, g.mag_x, g.sh_x);
+    magic_div(c.ny, g.mag_y, g.sh_y);
     return g;
 }
 

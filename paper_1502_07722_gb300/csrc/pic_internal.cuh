@@ -88,11 +88,21 @@ inline float pot_param(const pic_config& cfg) { return (float)(cfg.pot_mode == 2
 // in bits 0-1, the HCP lattice in bit 2 (kLatHcp).
 inline int pot_code(const pic_config& cfg) { return cfg.pot_mode | (cfg.lattice == PIC_LATTICE_HCP ? 4 : 0); }
 
+// Exact division of 0 <= v < 2^31 by n >= 2: q = umulhi(v, m) >> s with 2^s < n <= 2^(s + 1) and
+// m = ceil(2^(32 + s) / n) < 2^32; v m / 2^(32 + s) exceeds v / n by less than 1 / n because m n exceeds
+// 2^(32 + s) by less than 2^(s + 1).
+inline void magic_div(int n, unsigned& m, int& s)
+{
+    s = 0;
+    while ((2 << s) < n) s++;
+    m = (unsigned)(((1ULL << (32 + s)) + (unsigned)n - 1) / (unsigned)n);
+}
+
 // Everything a kernel of the step needs, passed by value.
 struct StepArgs {
     int32_t nx, nz, T, ntx, ntz, ntiles, W;   // W: window edge (nodes) of a tile
-    unsigned nx_magic;                        // ceil(2^(32 + nx_shift) / nx) for the cell -> (i, k) split
-    int32_t nx_shift;                         // 2^nx_shift < nx <= 2^(nx_shift + 1)
+    unsigned nx_magic;                        // magic_div of nx for the cell -> (i, k) split
+    int nx_shift;
     int32_t full;                             // fields and Lorentz force on
     float cdt_dx;                             // c dt / dx
     float rho_s;                              // node sum -> n / n0
