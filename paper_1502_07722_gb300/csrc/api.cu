@@ -33,7 +33,7 @@ struct Layout {
     int64_t count_limit;
     bool twin;
     size_t nn;
-    int64_t cap[2], n0[2];
+    int64_t cap[2], n0[2], items;
     size_t total;
 };
 
@@ -105,6 +105,9 @@ int derive_layout(const pic_config* cfg, Layout& L)
     t += 6 * align256(4 * L.nn) + 5 * align256(8 * L.nn);
     L.twin = L.dims == 2 && full;         // the field update's second set of field and current grids
     if (L.twin) t += 6 * align256(4 * L.nn) + 3 * align256(8 * L.nn);
+    L.items = L.dims == 2 ? work_item_cap(L.cap[0] + L.cap[1], L.ntiles) : 0;
+    if (L.items >= (1LL << 31)) return PIC_EINVAL;
+    t += align256(sizeof(WorkItem) * (size_t)L.items) + align256(4);
     const size_t plane = (size_t)L.nx * L.ny;
     t += (L.dims == 3 ? align256(4 * 8 * plane) : 0) + 2 * align256(4 * plane) + align256(8);
     t += 2 * align256(4 * ((size_t)L.nkeys + 1));
@@ -224,6 +227,12 @@ void swap_currents(Ctx& c)
         c.J[q] = c.Jn[q];
         c.Jn[q] = p;
     }
+}
+
+int64_t work_item_cap_of(const pic_config* cfg)
+{
+    Layout L;
+    return derive_layout(cfg, L) == PIC_OK ? L.items : 0;
 }
 
 StepArgs make_step_args(Ctx& c)
@@ -349,6 +358,9 @@ int pic_init(const pic_config* cfg, void* workspace, size_t workspace_bytes, voi
         for (int q = 0; q < 6; q++) c.Fn[q] = cv.take<float>(L.nn);
         for (int q = 0; q < 3; q++) c.Jn[q] = cv.take<u64>(L.nn);
     }
+    c.items = cv.take<WorkItem>((size_t)L.items);
+    c.items_cap = (int32_t)L.items;
+    c.nitems = cv.take<int32_t>(1);
     const size_t plane = (size_t)L.nx * L.ny;
     c.mur_save = d3 ? cv.take<float>(8 * plane) : nullptr;
     c.ant_c = cv.take<float>(plane);
@@ -856,6 +868,7 @@ int pic_checkpoint_restore(pic_ctx* h, const void* buf, int32_t on_host)
     int r = ckpt_copy(h, (char*)const_cast<void*>(buf), false, on_host != 0);
     if (r) return r;
     c.prepared = 0;
+    c.items_ok = 0;
     c.step = hd.step;
     c.steps_since_sort = hd.steps_since_sort;
     CK(cudaStreamSynchronize(c.stream));

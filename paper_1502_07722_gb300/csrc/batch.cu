@@ -46,7 +46,7 @@ struct pic_batch {
     int n;
     pic_ctx* slab[kMaxSlabs];
     cudaStream_t st;
-    int full, pot, minW, maxW, max_nx, max_nz, total_tiles, nsm, sort_every, steps_since_sort;
+    int full, pot, minW, maxW, max_nx, max_nz, nsm, sort_every, steps_since_sort;
     size_t max_nn;
     int64_t step;
     StepArgs* args_dev;          // [2][n]: parity 0 (density in buffer 0) and parity 1
@@ -54,7 +54,9 @@ struct pic_batch {
     AntennaParams* ap_dev;       // [n]
     long long* step_dev;         // [n]
     float* ant_dev;              // [2][n][2]: the antenna scalars of a step of each parity
-    int* tile_base_dev;          // [n + 1]
+    WorkItem* items;             // work items of every slab's tiles, rebuilt after a sort
+    int* nitems;
+    int items_cap;
     cudaGraphExec_t graph[2];
     int captured;
     int timing;
@@ -68,10 +70,18 @@ namespace {
 
 size_t a256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-size_t batch_tail_bytes(int n)
+int64_t batch_items_cap(const pic_config* cfgs, int n)
 {
-    return a256(sizeof(StepArgs) * 2 * n) + a256(sizeof(AntennaParams) * n) + a256(8 * (size_t)n) +
-           a256(16 * (size_t)n) + a256(4 * ((size_t)n + 1));
+    int64_t t = 0;
+    for (int s = 0; s < n; s++) t += work_item_cap_of(&cfgs[s]);
+    return t;
+}
+
+size_t batch_tail_bytes(const pic_config* cfgs, int n)
+{
+    return a256(sizeof(WorkItem) * (size_t)batch_items_cap(cfgs, n)) + a256(4) +
+           a256(sizeof(StepArgs) * 2 * n) + a256(sizeof(AntennaParams) * n) + a256(8 * (size_t)n) +
+           a256(16 * (size_t)n);
 }
 
 // The other parity of a slab's double-buffered grids (density; with fields also the fields and the
@@ -120,17 +130,37 @@ void enqueue_step(pic_batch* b, int parity)
     const StepArgs* args = b->args_dev + parity * b->n;
     if (!b->full) enqueue_prepare(b, parity);
     if (b->timing) cudaEventRecord(b->ev[0], b->st);
-    launch_particle_step_batch(args, b->tile_base_dev, b->n, b->total_tiles, b->full, b->pot, b->minW, b->maxW, b->nsm, b->st);
+    launch_particle_step_batch(args, b->n, b->items, b->nitems, b->full, b->pot, b->minW, b->maxW, b->nsm, b->st);
     if (b->timing) cudaEventRecord(b->ev[1], b->st);
     if (b->full)
         launch_fields_batch(b->fields[parity], b->ap_dev, b->step_dev, b->ant_dev + (1 - parity) * 2 * b->n, b->st);
     if (b->timing) cudaEventRecord(b->ev[2], b->st);
 }
 
+// One list of work items over every slab's tiles, after a sort or a slab's state was written.
+void build_items(pic_batch* b)
+{
+    bool ok = true;
+    int64_t n = 0;
+    for (int s = 0; s < b->n; s++) {
+        const Ctx& c = b->slab[s]->c;
+        ok &= c.items_ok != 0;
+        n += c.sp[0].n + (c.nsp > 1 ? c.sp[1].n : 0);
+    }
+    if (ok) return;
+    cudaMemsetAsync(b->nitems, 0, sizeof(int), b->st);
+    const int chunk = item_chunk(n, particle_slots(b->nsm, b->full, 1));
+    for (int s = 0; s < b->n; s++) {
+        launch_work_items(b->slab[s]->c, s, chunk, b->items, b->nitems, b->items_cap, b->st);
+        b->slab[s]->c.items_ok = 1;
+    }
+}
+
 // The fields' update prepares the step after it; the first step, and one after a slab's state was
 // written from outside (a checkpoint, new particles), is prepared here.
 void prepare(pic_batch* b)
 {
+    build_items(b);
     if (!b->full) return;
     bool ready = true;
     for (int s = 0; s < b->n; s++) ready &= b->slab[s]->c.prepared != 0;
@@ -173,7 +203,8 @@ int pic_batch_workspace_size(const pic_config* cfgs, int32_t n, size_t* bytes)
         if (r) return r;
         t += a256(b);
     }
-    *bytes = t + batch_tail_bytes(n);
+    if (batch_items_cap(cfgs, n) >= (1LL << 31)) return PIC_EINVAL;
+    *bytes = t + batch_tail_bytes(cfgs, n);
     return PIC_OK;
 }
 
@@ -191,7 +222,6 @@ int pic_batch_init(const pic_config* cfgs, int32_t n, void* workspace, size_t by
     b->n = n;
     b->st = (cudaStream_t)stream;
     char* p = (char*)workspace;
-    std::vector<int> tile_base(n + 1, 0);
     for (int s = 0; s < n; s++) {
         size_t sb = 0;
         pic_workspace_size(&cfgs[s], &sb);
@@ -204,7 +234,6 @@ int pic_batch_init(const pic_config* cfgs, int32_t n, void* workspace, size_t by
         b->slab[s]->c.in_batch = 1;
         p += a256(sb);
         const Ctx& c = b->slab[s]->c;
-        tile_base[s + 1] = tile_base[s] + c.ntiles;
         b->maxW = c.W > b->maxW ? c.W : b->maxW;
         b->minW = s == 0 || c.W < b->minW ? c.W : b->minW;
         b->max_nx = c.nx > b->max_nx ? c.nx : b->max_nx;
@@ -212,7 +241,6 @@ int pic_batch_init(const pic_config* cfgs, int32_t n, void* workspace, size_t by
         b->max_nn = c.nn > b->max_nn ? c.nn : b->max_nn;
         b->nsm = c.nsm;
     }
-    b->total_tiles = tile_base[n];
     b->full = cfgs[0].mode == PIC_MODE_FULL;
     b->pot = pot_code(cfgs[0]);   // kernel instance
     b->sort_every = cfgs[0].sort_every;
@@ -224,7 +252,10 @@ int pic_batch_init(const pic_config* cfgs, int32_t n, void* workspace, size_t by
     p += a256(8 * (size_t)n);
     b->ant_dev = reinterpret_cast<float*>(p);
     p += a256(16 * (size_t)n);
-    b->tile_base_dev = reinterpret_cast<int*>(p);
+    b->items = reinterpret_cast<WorkItem*>(p);
+    b->items_cap = (int)batch_items_cap(cfgs, n);
+    p += a256(sizeof(WorkItem) * (size_t)b->items_cap);
+    b->nitems = reinterpret_cast<int*>(p);
     std::vector<AntennaParams> ap(n);
     for (int s = 0; s < n; s++) {
         Ctx& c = b->slab[s]->c;
@@ -250,8 +281,6 @@ int pic_batch_init(const pic_config* cfgs, int32_t n, void* workspace, size_t by
     }
     bool ok = cudaMemcpyAsync(b->ap_dev, ap.data(), sizeof(AntennaParams) * n, cudaMemcpyHostToDevice, b->st) ==
                   cudaSuccess &&
-              cudaMemcpyAsync(b->tile_base_dev, tile_base.data(), 4 * (size_t)(n + 1), cudaMemcpyHostToDevice,
-                              b->st) == cudaSuccess &&
               cudaMemsetAsync(b->step_dev, 0, 8 * (size_t)n, b->st) == cudaSuccess;
     r = ok ? upload_args(b) : PIC_ECUDA;
     for (int q = 0; q < 6 && r == PIC_OK; q++)
@@ -304,6 +333,7 @@ int pic_batch_step(pic_batch* b, int32_t nsteps)
             }
             const int r = upload_args(b);      // the sort swapped the particle buffers
             if (r) return r;
+            build_items(b);
             b->steps_since_sort = 0;
         }
         const int parity = b->slab[0]->c.cur;

@@ -4,17 +4,16 @@
 // current deposition (Esirkepov, fixed point) -> node density at the new position.
 //
 // Work decomposition (GB300):
-//  * one CTA owns one tile of T x T cells at a time (particles are sorted into tiles);
+//  * one CTA takes one work item at a time: a tile of T x T cells (particles are sorted into tiles), or
+//    a part of a tile when tiles are few; the items are listed after each sort (k_work_items);
 //  * the CTA stages a window of (T + 2M + 3)^2 nodes in shared memory: the six field
 //    components and the pair density n / n0 in FP32, components of one Yee stagger side by side
 //    (one 64-bit load per corner fetches two of them);
-//  * thread t of the CTA (128 threads, 8 CTAs per SM) takes the tile's records t, t + 128, ...
-//    straight from global memory (coalesced loads and stores, no block barrier); the position of
-//    its next record is loaded one iteration ahead. The cell sort
-//    stores each block of 1024 of
-//    a tile's cell-ordered particles as a 32-row matrix, column by column, so the lanes of a warp
-//    hold particles 32 places apart in the cell order: neighbouring cells, whose deposits go to
-//    distinct nodes that share cache sectors;
+//  * thread t of the CTA (128 threads) takes the item's records t, t + 128, ... straight from global
+//    memory (coalesced loads and stores, no block barrier), in warps aligned to 32 records; the
+//    position of its next record is loaded one iteration ahead. The cell sort stores each block of a
+//    tile's cell-ordered particles as a 32-row matrix, column by column, so the lanes of a warp hold
+//    particles of neighbouring cells, whose deposits go to distinct nodes that share cache sectors;
 //  * deposits (current, node-density change) are exact 64-bit integer reductions straight into
 //    global memory: fire-and-forget on the SM, native in L2. Measured against exact sums in the
 //    shared-memory window (32-bit (lo, hi) pairs whose low-word atomic must return the old value
@@ -39,7 +38,11 @@ namespace gbpic {
 
 constexpr int kMargin = 2;              // cells a particle may drift out of its tile between sorts
 constexpr int kBlock = 128;                // threads per CTA (8 CTAs per SM)
-constexpr int kCtasPerSm = 8;
+// Resident CTAs: with fields 9 (56 registers; 8 at 64: 1.74 against 1.70 ms per launch on the 2048^2
+// slab), the transport stage 8 (9: 0.129 against 0.116 ms on the crater slab).
+constexpr int kCtasPerSm = 9;
+constexpr int kCtasPerSmAtoms = 8;
+constexpr int kMinChunk = 512;
 constexpr int kWin = 16 + 2 * kMargin + 3;  // window edge of the 16-cell tile (compiled-in instances)
 // The batched kernel reads each slab's arguments from a constant-memory table with a run-time
 // index: every use is an indexed constant load into a register, so it needs more registers than
@@ -378,16 +381,17 @@ __device__ __forceinline__ void process_particle(const StepArgs& a, const Specie
     }
 }
 
-// Part `sub` of `nsub` of one tile of one simulation: stage the tile's window, then advance that
-// part of each species' particles of the tile in storage order (tiles holding many particles are
-// split over several CTAs when the tiles are fewer than the CTA slots).
+// start of part `sub` of `nsub` of the records p0 .. p1 - 1; inner boundaries lie on multiples of 32
 __device__ __forceinline__ int part_start(int p0, int p1, int sub, int nsub)
 {
-    return p0 + (int)(((long long)(p1 - p0) * sub) / nsub);
+    const int p = p0 + (int)(((long long)(p1 - p0) * sub) / nsub);
+    return sub == 0 ? p0 : (sub == nsub ? p1 : max(p0, p & ~31));
 }
 
+// One work item: stage the tile's window, then advance the item's records of each species in storage
+// order.
 template <bool FULL, int POT, int WC>
-__device__ __forceinline__ void run_tile(const StepArgs& a, int t, int sub, int nsub)
+__device__ __forceinline__ void run_item(const StepArgs& a, const WorkItem& item)
 {
     extern __shared__ unsigned smem[];
     const int W = WC ? WC : a.W, WW = W * W;
@@ -400,15 +404,8 @@ __device__ __forceinline__ void run_tile(const StepArgs& a, int t, int sub, int 
     w.by = fbase + 6 * WW;
     w.nh = fbase;
 
-    int cnt = 0;
-#pragma unroll
-    for (int s = 0; s < 2; s++)
-        if (s < a.nsp) {
-            const int p0 = a.sp[s].tile_start[t], p1 = a.sp[s].tile_start[t + 1];
-            cnt += part_start(p0, p1, sub + 1, nsub) - part_start(p0, p1, sub, nsub);
-        }
-    if (cnt == 0) return;
-    const int tx = t % a.ntx, tz = t / a.ntx;
+    const int t = item.tile, tx = t % a.ntx, tz = t / a.ntx;
+    const int q0[2] = {item.p0[0], item.p0[1]}, q1[2] = {item.p1[0], item.p1[1]};
     w.ox = wrap_any(tx * a.T - kMargin - 1, a.nx);
     w.oz = tz * a.T - kMargin - 1;
     // stage the window: fields, pair density (wall rows doubled)
@@ -435,21 +432,23 @@ __device__ __forceinline__ void run_tile(const StepArgs& a, int t, int sub, int 
     __syncthreads();
 #pragma unroll
     for (int s = 0; s < 2; s++) {
-        if (s >= a.nsp) break;
+        if (s >= (FULL ? 2 : 1)) break;
         const Species& S = a.sp[s];
-        const int q0 = S.tile_start[t], q1 = S.tile_start[t + 1];
-        const int p0 = part_start(q0, q1, sub, nsub), p1 = part_start(q0, q1, sub + 1, nsub);
+        const int p0 = q0[s], p1 = q1[s];
         // the next record's position is loaded one iteration ahead (its first use is at the top
         // of the iteration); the momenta, first used after the gathers, are loaded in the iteration
+        // Warps take aligned groups of 32 records: every access of a warp is one full 128-byte line. After
+        // the first re-sort a tile starts anywhere: over steps 330-350 on the 2048^2 slab 1.919 -> 1.769 ms
+        // per launch, 1.538 -> 1.468 in the sweep (aligned tiles, before it: 1.674 -> 1.696, the test).
         int ncell = 0;
         float nfx = 0.0f, nfz = 0.0f;
-        if (p0 + (int)threadIdx.x < p1) {
-            const int q = p0 + (int)threadIdx.x;
-            ncell = S.a.cell[q];
-            nfx = S.a.fx[q];
-            nfz = S.a.fz[q];
+        const int first = (p0 & ~31) + (int)threadIdx.x;
+        if (first < p1) {
+            ncell = S.a.cell[first];
+            nfx = S.a.fx[first];
+            nfz = S.a.fz[first];
         }
-        for (int p = p0 + (int)threadIdx.x; p < p1; p += kBlock) {
+        for (int p = first; p < p1; p += kBlock) {
             const int cell = ncell;
             const float fx = nfx, fz = nfz;
             if (p + kBlock < p1) {
@@ -457,6 +456,7 @@ __device__ __forceinline__ void run_tile(const StepArgs& a, int t, int sub, int 
                 nfx = S.a.fx[p + kBlock];
                 nfz = S.a.fz[p + kBlock];
             }
+            if (p < p0) continue;
             if (s == 0) process_particle<FULL ? kIon : kAtom, POT, WC>(a, S, w, p, cell, fx, fz);
             else process_particle<kElectron, POT, WC>(a, S, w, p, cell, fx, fz);
         }
@@ -464,27 +464,40 @@ __device__ __forceinline__ void run_tile(const StepArgs& a, int t, int sub, int 
     __syncthreads();
 }
 
-// Work items (a tile, or a part of a tile) are handed out dynamically: each CTA draws the next one
-// from a ticket counter in the status words (measured against a static round robin: 2.034 ->
-// 1.899 ms per launch on the 2048^2 slab, whose occupied tiles do not divide evenly over the
-// CTAs). atomicInc wraps the counter to 0 after total + gridDim.x tickets, i.e. exactly when every
-// CTA has drawn its last (failing) ticket, so every launch finds it at 0.
-__device__ __forceinline__ int next_item(unsigned* ticket, int total, int* slot)
+// The CTA's work items: the first is its block index, the others come from a ticket counter in the
+// status words (dynamic assignment: the items take uneven times). atomicInc wraps the counter to 0
+// after n draws, i.e. exactly when every CTA has drawn its last (failing) ticket, so every launch finds
+// it at 0; with no more items than CTAs nothing is drawn.
+__device__ __forceinline__ int next_item(const WorkItem* __restrict__ items, int n, unsigned* ticket, int first,
+                                         WorkItem* buf, int* slot)
 {
-    if (threadIdx.x == 0) *slot = (int)atomicInc(ticket, (unsigned)(total + gridDim.x - 1));
+    if (threadIdx.x < 32) {
+        int g = first;
+        if (first < 0) {
+            g = n;
+            if (n > (int)gridDim.x) {
+                if (threadIdx.x == 0) g = (int)(atomicInc(ticket, (unsigned)(n - 1)) + gridDim.x);
+                g = __shfl_sync(0xffffffffu, g, 0);
+            }
+        }
+        if (g < n && threadIdx.x < sizeof(WorkItem) / 4)
+            reinterpret_cast<int*>(buf)[threadIdx.x] = reinterpret_cast<const int*>(items + g)[threadIdx.x];
+        if (threadIdx.x == 0) *slot = g;
+    }
     __syncthreads();
-    const int g = *slot;
-    __syncthreads();
-    return g;
+    return *slot;
 }
 
 template <bool FULL, int POT, int WC>
-__global__ void __launch_bounds__(kBlock, kCtasPerSm) k_particles(const StepArgs a, int nsub)
+__global__ void __launch_bounds__(kBlock, FULL ? kCtasPerSm : kCtasPerSmAtoms)
+    k_particles(const StepArgs a, const WorkItem* __restrict__ items, const int* __restrict__ nitems)
 {
+    __shared__ WorkItem item;
     __shared__ int slot;
-    const int total = a.ntiles * nsub;
-    for (int g = next_item(a.status + 2, total, &slot); g < total; g = next_item(a.status + 2, total, &slot))
-        run_tile<FULL, POT, WC>(a, g / nsub, g % nsub, nsub);
+    const int n = *nitems;
+    for (int g = next_item(items, n, a.status + 2, (int)blockIdx.x, &item, &slot); g < n;
+         g = next_item(items, n, a.status + 2, -1, &item, &slot))
+        run_item<FULL, POT, WC>(a, item);
 }
 
 // Arguments of the simulations of a batch for the current step, in constant memory: the slab
@@ -493,29 +506,101 @@ __global__ void __launch_bounds__(kBlock, kCtasPerSm) k_particles(const StepArgs
 // batched launch; two batches stepping at the same time on different streams would race on it.
 constexpr int kMaxBatchSlabs = 48;
 __constant__ StepArgs c_batch_args[kMaxBatchSlabs];
-__constant__ int c_tile_base[kMaxBatchSlabs + 1];
 
-// All simulations of a batch in one persistent launch: the tiles of every simulation form one
-// work list (c_tile_base[s] = first global tile of simulation s).
+// All simulations of a batch in one persistent launch over one list of work items.
 template <bool FULL, int POT, int WC>
-__global__ void __launch_bounds__(kBlock, kCtasPerSmBatch) k_particles_batch(int nslab, int total, int nsub)
+__global__ void __launch_bounds__(kBlock, kCtasPerSmBatch)
+    k_particles_batch(const WorkItem* __restrict__ items, const int* __restrict__ nitems)
 {
     // one ticket counter for the whole batch: the first simulation's
+    __shared__ WorkItem item;
     __shared__ int slot;
+    const int n = *nitems;
     unsigned* ticket = c_batch_args[0].status + 2;
-    for (int g = next_item(ticket, total * nsub, &slot); g < total * nsub; g = next_item(ticket, total * nsub, &slot)) {
-        const int tile = g / nsub;
-        int s = 0;
-        while (s + 1 < nslab && c_tile_base[s + 1] <= tile) s++;
-        run_tile<FULL, POT, WC>(c_batch_args[s], tile - c_tile_base[s], g % nsub, nsub);
-    }
+    for (int g = next_item(items, n, ticket, (int)blockIdx.x, &item, &slot); g < n;
+         g = next_item(items, n, ticket, -1, &item, &slot))
+        run_item<FULL, POT, WC>(c_batch_args[item.slab], item);
 }
 
-// parts per tile: about four work items per CTA slot (a slab often fills under half of the tiles)
-static int parts_per_tile(int ntiles, int slots)
+// Work items from the tiles' particle counts (rebuilt after a sort), appended to the list in tile order
+// (neighbouring tiles run at about the same time and share lines of the grids in L2: a scrambled order
+// took 1.735 instead of 1.695 ms on the 2048^2 slab). A tile of cnt particles is cut into
+// round(cnt / chunk) parts, at least one, each with its share of both species; tiles without particles
+// give none. One block: a scan over the tiles.
+constexpr int kItemThreads = 1024;
+__global__ void __launch_bounds__(kItemThreads) k_work_items(const int32_t* __restrict__ start0,
+                                                            const int32_t* __restrict__ start1, int ntiles, int slab,
+                                                            int chunk, WorkItem* items, int* nitems, int cap)
 {
-    int nsub = (4 * slots + ntiles - 1) / (ntiles > 0 ? ntiles : 1);
-    return nsub < 1 ? 1 : (nsub > 16 ? 16 : nsub);
+    __shared__ int sums[kItemThreads / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int base = *nitems;
+    for (int t0 = 0; t0 < ntiles; t0 += kItemThreads) {
+        const int t = t0 + (int)threadIdx.x;
+        int i0 = 0, ni = 0, e0 = 0, ne = 0, parts = 0;
+        if (t < ntiles) {
+            i0 = start0[t];
+            ni = start0[t + 1] - i0;
+            if (start1) {
+                e0 = start1[t];
+                ne = start1[t + 1] - e0;
+            }
+            if (ni + ne > 0) parts = max(1, (int)(((long long)ni + ne + chunk / 2) / chunk));
+        }
+        int scan = parts;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, scan, o);
+            if (lane >= o) scan += v;
+        }
+        if (lane == 31) sums[warp] = scan;
+        __syncthreads();
+        int before = 0, total = 0;
+        for (int q = 0; q < kItemThreads / 32; q++) {
+            if (q < warp) before += sums[q];
+            total += sums[q];
+        }
+        const int at = base + before + scan - parts;
+        if (at + parts <= cap)                 // always: the list is sized for every tile's parts
+            for (int q = 0; q < parts; q++) {
+                WorkItem w;
+                w.tile = t;
+                w.slab = slab;
+                w.p0[0] = part_start(i0, i0 + ni, q, parts);
+                w.p1[0] = part_start(i0, i0 + ni, q + 1, parts);
+                w.p0[1] = part_start(e0, e0 + ne, q, parts);
+                w.p1[1] = part_start(e0, e0 + ne, q + 1, parts);
+                w.pad[0] = w.pad[1] = 0;
+                items[at + q] = w;
+            }
+        base += total;
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) *nitems = base;
+}
+
+// Particles per work item: about four items per resident CTA, at least 512 particles (an item costs its
+// window's staging: 403 x 311 cells of 13 + 13 particles 0.041 ms per launch at 512, 0.048 at 300). With
+// fewer than 512 particles per CTA the launch is one chain of latencies and takes one round of the CTA's
+// threads per species (64^2 cells of 8 + 8: 14.1 us at 512, 12.6 at 256).
+int item_chunk(int64_t n, int slots)
+{
+    if (n < (int64_t)slots * kMinChunk) return 2 * kBlock;
+    const int64_t c = n / ((int64_t)slots * 4);
+    return (int)(c < kMinChunk ? kMinChunk : (c > (1 << 30) ? (1 << 30) : c));
+}
+
+// Entries of a list for n particles on ntiles tiles: round(cnt / chunk) or one per tile.
+int64_t work_item_cap(int64_t n, int64_t ntiles) { return n / (2 * kBlock) + 2 * ntiles; }
+
+void launch_work_items(const Ctx& c, int slab, int chunk, WorkItem* items, int* nitems, int cap, cudaStream_t st)
+{
+    k_work_items<<<1, kItemThreads, 0, st>>>(c.sp[0].tile_start, c.nsp > 1 ? c.sp[1].tile_start : nullptr, c.ntiles, slab,
+                                             chunk, items, nitems, cap);
+}
+
+int particle_slots(int nsm, int full, int batch)
+{
+    return nsm * (batch ? kCtasPerSmBatch : (full ? kCtasPerSm : kCtasPerSmAtoms));
 }
 
 size_t particle_smem_bytes(int W) { return sizeof(unsigned) * (size_t)7 * W * W; }
@@ -550,19 +635,21 @@ void launch_particle_step(Ctx& c, const StepArgs& a, cudaStream_t st)
 #undef GBPIC_ATTR
         configured[dev].store(shmem);
     }
-    const int cap = c.nsm * kCtasPerSm;
-    const int nsub = parts_per_tile(a.ntiles, cap);
-    int grid = a.ntiles * nsub;
-    if (grid > cap) grid = cap;
-    if (grid < 1) grid = 1;
+    const int grid = particle_slots(c.nsm, a.full, 0);
+    if (!c.items_ok) {
+        const int64_t n = c.sp[0].n + (c.nsp > 1 ? c.sp[1].n : 0);
+        cudaMemsetAsync(c.nitems, 0, sizeof(int), st);
+        launch_work_items(c, 0, item_chunk(n, grid), c.items, c.nitems, c.items_cap, st);
+        c.items_ok = 1;
+    }
     // the instance with the potential and the lattice compiled in, and the window edge when it is
     // the 16-cell tile's
     switch ((a.pot_mode & 7) | (a.full ? 8 : 0) | (a.W == kWin ? 16 : 0)) {
 #define GBPIC_CASE(P)                                                                                 \
-    case 24 | (P): k_particles<true, (P), kWin><<<grid, kBlock, shmem, st>>>(a, nsub); break;         \
-    case 16 | (P): k_particles<false, (P), kWin><<<grid, kBlock, shmem, st>>>(a, nsub); break;        \
-    case 8 | (P): k_particles<true, (P), 0><<<grid, kBlock, shmem, st>>>(a, nsub); break;             \
-    case (P): k_particles<false, (P), 0><<<grid, kBlock, shmem, st>>>(a, nsub); break;
+    case 24 | (P): k_particles<true, (P), kWin><<<grid, kBlock, shmem, st>>>(a, c.items, c.nitems); break;         \
+    case 16 | (P): k_particles<false, (P), kWin><<<grid, kBlock, shmem, st>>>(a, c.items, c.nitems); break;        \
+    case 8 | (P): k_particles<true, (P), 0><<<grid, kBlock, shmem, st>>>(a, c.items, c.nitems); break;             \
+    case (P): k_particles<false, (P), 0><<<grid, kBlock, shmem, st>>>(a, c.items, c.nitems); break;
         GBPIC_FOR_EACH_POT(GBPIC_CASE)
 #undef GBPIC_CASE
     }
@@ -570,11 +657,10 @@ void launch_particle_step(Ctx& c, const StepArgs& a, cudaStream_t st)
 
 int max_batch_slabs() { return kMaxBatchSlabs; }
 
-void launch_particle_step_batch(const StepArgs* args_dev, const int* tile_base_dev, int nslab, int total_tiles,
-                                int full, int pot, int minW, int maxW, int nsm, cudaStream_t st)
+void launch_particle_step_batch(const StepArgs* args_dev, int nslab, const WorkItem* items, const int* nitems, int full,
+                                int pot, int minW, int maxW, int nsm, cudaStream_t st)
 {
     cudaMemcpyToSymbolAsync(c_batch_args, args_dev, sizeof(StepArgs) * nslab, 0, cudaMemcpyDeviceToDevice, st);
-    cudaMemcpyToSymbolAsync(c_tile_base, tile_base_dev, sizeof(int) * (nslab + 1), 0, cudaMemcpyDeviceToDevice, st);
     const size_t shmem = particle_smem_bytes(maxW);
     // the attributes are per device: remember what each device has been given
     static std::atomic<size_t> configured[kMaxDevices];
@@ -590,18 +676,15 @@ void launch_particle_step_batch(const StepArgs* args_dev, const int* tile_base_d
 #undef GBPIC_ATTR
         configured[dev].store(shmem);
     }
-    const int cap = nsm * kCtasPerSmBatch;
-    const int nsub = parts_per_tile(total_tiles, cap);
-    int grid = total_tiles * nsub < cap ? total_tiles * nsub : cap;
-    if (grid < 1) grid = 1;
+    const int grid = particle_slots(nsm, full, 1);
     // pot: the instance code shared by every slab (potential and lattice); the compiled-in window
     // edge when every slab has it
     switch ((pot & 7) | (full ? 8 : 0) | (minW == kWin && maxW == kWin ? 16 : 0)) {
 #define GBPIC_CASE(P)                                                                                              \
-    case 24 | (P): k_particles_batch<true, (P), kWin><<<grid, kBlock, shmem, st>>>(nslab, total_tiles, nsub); break; \
-    case 16 | (P): k_particles_batch<false, (P), kWin><<<grid, kBlock, shmem, st>>>(nslab, total_tiles, nsub); break; \
-    case 8 | (P): k_particles_batch<true, (P), 0><<<grid, kBlock, shmem, st>>>(nslab, total_tiles, nsub); break;    \
-    case (P): k_particles_batch<false, (P), 0><<<grid, kBlock, shmem, st>>>(nslab, total_tiles, nsub); break;
+    case 24 | (P): k_particles_batch<true, (P), kWin><<<grid, kBlock, shmem, st>>>(items, nitems); break; \
+    case 16 | (P): k_particles_batch<false, (P), kWin><<<grid, kBlock, shmem, st>>>(items, nitems); break; \
+    case 8 | (P): k_particles_batch<true, (P), 0><<<grid, kBlock, shmem, st>>>(items, nitems); break;    \
+    case (P): k_particles_batch<false, (P), 0><<<grid, kBlock, shmem, st>>>(items, nitems); break;
         GBPIC_FOR_EACH_POT(GBPIC_CASE)
 #undef GBPIC_CASE
     }

@@ -121,6 +121,13 @@ struct StepArgs {
     float jy_zero;                            // 2^-(jy_bits + 1): |u_y| below it gives V = 0
 };
 
+// One unit of work of the 2D particle kernel: the records p0[s] .. p1[s] - 1 of species s, all of one tile.
+struct WorkItem {
+    int32_t tile, slab;      // slab: index in a batch
+    int32_t p0[2], p1[2];
+    int32_t pad[2];
+};
+
 struct Ctx {
     pic_config cfg;
     cudaStream_t stream;
@@ -142,6 +149,10 @@ struct Ctx {
     float* Fn[6];         // 2D full mode: the fields the next update writes (swapped with F after it)
     u64* Jn[3];           // 2D full mode: the currents the next step deposits into
     int32_t prepared;     // Jn is clear and rho[1 - cur] equals rho[cur]
+    WorkItem* items;      // 2D: work items of the particle kernel, from the tile offsets
+    int32_t* nitems;
+    int32_t items_cap;
+    int32_t items_ok;     // the list matches the tile offsets
     float* mur_save;      // 3D: 8 planes
     float* ant_c;         // nx: amplitude * cos(phase(x)) at x = i + 1/2
     float* ant_s;         // nx: amplitude * sin(phase(x))
@@ -238,8 +249,13 @@ void launch_antenna_batch(const AntennaParams* ap_dev, const long long* step_dev
 void field_row_blocks(FieldBatch& P);
 FieldArgs make_field_args(const Ctx& c);
 AntennaParams make_antenna_params(const Ctx& c);
-void launch_particle_step_batch(const StepArgs* args_dev, const int* tile_base_dev, int nslab, int total_tiles,
-                                int full, int pot, int minW, int maxW, int nsm, cudaStream_t st);
+void launch_particle_step_batch(const StepArgs* args_dev, int nslab, const WorkItem* items, const int* nitems, int full,
+                                int pot, int minW, int maxW, int nsm, cudaStream_t st);
+int64_t work_item_cap(int64_t n, int64_t ntiles);
+void launch_work_items(const Ctx& c, int slab, int chunk, WorkItem* items, int* nitems, int cap, cudaStream_t st);
+int particle_slots(int nsm, int full, int batch);
+int item_chunk(int64_t n, int slots);
+int64_t work_item_cap_of(const pic_config* cfg);     // 0 for an invalid configuration
 size_t particle_smem_bytes(int W);
 void launch_particle_step3(Ctx& c, cudaStream_t st);
 void launch_deposit_density3(Ctx& c, u64* out, cudaStream_t st);

@@ -337,6 +337,7 @@ void sort_species_impl(Ctx& c, int s, cudaStream_t st, int from_b, int64_t* laun
     k_scan_sums<<<1, kScanBlock, 0, st>>>(c.scan_tmp, nb);
     // the cursor reuses the count array (counts are consumed by the scan)
     k_scan_add<<<(c.nkeys + 255) / 256, 256, 0, st>>>(c.keys_off, c.scan_tmp, c.nkeys, c.keys_count, (int32_t)S.n);
+    c.items_ok = 0;
     k_tile_starts<<<(c.ntiles + 1 + 255) / 256, 256, 0, st>>>(c.keys_off, c.ntiles, TT, S.tile_start);
     if (S.n > 0) k_scatter<<<(int)g, 256, 0, st>>>(src, dst, S.n, kg, c.keys_count, S.tile_start);
     k_count_check<<<1, 32, 0, st>>>(c.status, c.count_limit);
