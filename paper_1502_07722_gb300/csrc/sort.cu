@@ -2,8 +2,8 @@
 // count per key -> exclusive scan -> scatter into the second buffer -> swap.
 // The key of cell (i, k) is tile * T^2 + (k mod T) * T + (i mod T), tile = (k / T) * ntx + i / T
 // (in 3D likewise with T^3 cells per tile), so the particles of a tile are contiguous.
-// Inside a tile the cell-ordered list is cut into blocks of kLayoutBlock particles (1024 in 2D,
-// 256 in 3D: 32 x the particles per cell of a typical slab) and each block is stored column by
+// Inside a tile the cell-ordered list is cut into blocks of 32 x the particles per cell (layout_log2) and
+// each block is stored column by
 // column as a 32-row matrix whose rows are consecutive runs of the cell order. The particle
 // kernels read their records in memory order, coalesced, and the 32 lanes of a warp then hold
 // particles one run apart: neighbouring cells, so a warp's deposits go to distinct nodes that
@@ -45,24 +45,32 @@ struct KeyGeo {
     Div dnx, dny, dT, dTT;
 };
 
-constexpr int kLayoutBlock2 = 1024, kLayoutBlock3 = 256;
-
 // Storage slot, relative to its tile, of the particle at place ci of the tile's cell order (nt
-// particles in the tile): block ci / B, and inside a block of nb particles the element (row
+// particles in the tile): block ci / B (B = 2^lb), and inside a block of nb particles the element (row
 // j / C, column j mod C) of a row-major matrix with C = ceil(nb / 32) columns, stored column-major
 // (the last row may be short, so column c holds R + (c < rem) elements). A bijection of 0..nt-1.
-template <int B>
-__device__ __forceinline__ int layout_slot(int ci, int nt)
+__device__ __forceinline__ int layout_slot(int ci, int nt, int lb)
 {
-    const int blk = ci / B, j = ci - blk * B, nb = min(B, nt - blk * B);
-    if (nb == B) {
-        // a full block: B / 32 columns of 32 (shifts)
-        constexpr int C = B / 32;
-        return blk * B + (j % C) * 32 + j / C;
-    }
+    const int b0 = ci >> lb << lb, j = ci - b0, nb = nt - b0;
+    if (nb >> lb) return b0 + ((j & ((1 << (lb - 5)) - 1)) << 5) + (j >> (lb - 5));     // a full block
     const int C = (nb + 31) >> 5, R = nb / C, rem = nb - R * C;
     const int r = j / C, c = j - r * C;
-    return blk * B + c * R + min(c, rem) + r;
+    return b0 + c * R + min(c, rem) + r;
+}
+
+// The block size (log2) of a species' layout: 32 x its particles per cell gives the 32 lanes of a warp
+// 32 neighbouring cells. Smaller blocks put several lanes on one node, larger ones spread the lanes
+// over more cache sectors (L2 reductions go by the sector). Particle kernel, ms per launch, against one
+// block size for all (1024 in 2D, 256 in 3D): the 16-slab sweep (8 to 32 per cell) 1.59 -> 1.43, the
+// crater slab (128 per cell) 0.119 -> 0.114, the 3D crater slab (16 per cell) 2.80 -> 2.68; twice the
+// size: 1.69, 0.177, 4.06. Below 2^17 particles a launch is bound by latency and keeps the fixed size.
+static int layout_log2(const Ctx& c, const Species& S)
+{
+    const int base = c.dims == 3 ? 8 : 10;
+    if (S.n < (1 << 17)) return base;
+    int lb = 5;
+    while (lb < 12 && (S.ppc << 5) * 5 > (7 << lb)) lb++;       // the nearest power of two (in ratio)
+    return lb < 8 ? 8 : lb;
 }
 
 // 2D: cell = k*nx + i; 3D: cell = (k*ny + j)*nx + i. Tiles of T^dims cells, tile-major.
@@ -272,7 +280,7 @@ __global__ void k_tile_starts(const int32_t* __restrict__ off, int ntiles, int T
 }
 
 __global__ void k_scatter(SpeciesBuf src, SpeciesBuf dst, int64_t n, KeyGeo kg, int32_t* cursor,
-                          const int32_t* __restrict__ tile_start)
+                          const int32_t* __restrict__ tile_start, int lb)
 {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t nround = (n + 31) & ~(int64_t)31;
@@ -292,7 +300,7 @@ __global__ void k_scatter(SpeciesBuf src, SpeciesBuf dst, int64_t n, KeyGeo kg, 
         int kt;
         const int t = divq(key, kg.dTT, kt), ts = tile_start[t];
         const int ci = base + __popc(peers & ((1u << lane) - 1u)) - ts, nt = tile_start[t + 1] - ts;
-        const int q = ts + (kg.dims == 3 ? layout_slot<kLayoutBlock3>(ci, nt) : layout_slot<kLayoutBlock2>(ci, nt));
+        const int q = ts + layout_slot(ci, nt, lb);
         dst.cell[q] = c;
         dst.fx[q] = src.fx[p];
         if (kg.dims == 3) dst.fy[q] = src.fy[p];
@@ -308,6 +316,7 @@ __global__ void k_scatter(SpeciesBuf src, SpeciesBuf dst, int64_t n, KeyGeo kg, 
 void sort_species_impl(Ctx& c, int s, cudaStream_t st, int from_b, int64_t* launches)
 {
     Species& S = c.sp[s];
+    const int lb = layout_log2(c, S);
     const int TT = c.dims == 3 ? c.T * c.T * c.T : c.T * c.T;
     const KeyGeo kg = {c.nx, c.ny, c.T, c.ntx, c.nty, c.dims, TT, make_div(c.nx), make_div(c.ny), make_div(c.T),
                        make_div(TT)};
@@ -320,7 +329,7 @@ void sort_species_impl(Ctx& c, int s, cudaStream_t st, int from_b, int64_t* laun
     SpeciesBuf dst = from_b ? S.a : S.b;
     if (S.n > 0)
         k_count<<<(int)g, 256, 0, st>>>(src.cell, S.n, kg, c.keys_count,
-                                        (c.dims == 3 ? kLayoutBlock3 : kLayoutBlock2) / 32);
+                                        1 << (lb - 5));
     const int nb = (c.nkeys + kScanItems - 1) / kScanItems;
     // the most particles of this species in one block of 4 cells per axis (counts are consumed
     // below; the key offsets, written by the scan after it, hold the counts in cell order meanwhile)
@@ -339,7 +348,7 @@ void sort_species_impl(Ctx& c, int s, cudaStream_t st, int from_b, int64_t* laun
     k_scan_add<<<(c.nkeys + 255) / 256, 256, 0, st>>>(c.keys_off, c.scan_tmp, c.nkeys, c.keys_count, (int32_t)S.n);
     c.items_ok = 0;
     k_tile_starts<<<(c.ntiles + 1 + 255) / 256, 256, 0, st>>>(c.keys_off, c.ntiles, TT, S.tile_start);
-    if (S.n > 0) k_scatter<<<(int)g, 256, 0, st>>>(src, dst, S.n, kg, c.keys_count, S.tile_start);
+    if (S.n > 0) k_scatter<<<(int)g, 256, 0, st>>>(src, dst, S.n, kg, c.keys_count, S.tile_start, lb);
     k_count_check<<<1, 32, 0, st>>>(c.status, c.count_limit);
     if (!from_b) {
         SpeciesBuf t = S.a;
