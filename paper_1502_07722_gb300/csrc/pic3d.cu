@@ -27,6 +27,7 @@ namespace gbpic {
 constexpr int kQ3Bits = 14;
 constexpr int kQ3 = 1 << kQ3Bits;
 constexpr int kBlock3 = 256;
+constexpr int kCtas3 = 3, kCtas3Atoms = 4;
 
 __device__ __forceinline__ int wrapn(int i, int n) { return i < 0 ? i + n : (i >= n ? i - n : i); }
 __device__ __forceinline__ int qoff3(float f) { return __float2int_rn(f * 16384.0f); }
@@ -204,8 +205,8 @@ __device__ __noinline__ void deposit3_general(Geo3 g, u64* J0, u64* J1, u64* J2,
 // doubled) on W^3 nodes from (ox, oy, oz); x and y wrap, z rows outside 0..nz repeat the edge row
 // (the same values the global gathers clamp to).
 struct Win3 {
-    const float* f;         // component q (Ex, Ey, Ez, Bx, By, Bz) at f + q W^3, density at f + 6 W^3
-    int ox, oy, oz, W, WWW;
+    const float* f;         // fields and density, laid out as Lay3 says
+    int ox, oy, oz, W;
 };
 
 // Window gathers. Every component of a particle reads the corners of one cell of the window: the
@@ -214,6 +215,31 @@ struct Win3 {
 // weight f -+ 1/2). One base index serves all seven components; with the window edge WC known
 // at compile time the corner and component offsets are immediates.
 constexpr int kWin3 = 13;               // window edge of the 10-cell tile (compiled-in instances)
+
+// The window's layout in shared memory. The run-time window is seven dense W^3 arrays, x fastest. The
+// compiled-in one stores three components side by side in each x row, 42 floats from row to row (42 = 10
+// mod 32) and 576 from plane to plane (0 mod 32): the 32 lanes of a warp sit in 32 consecutive cells of
+// the tile's cell order (rows of 10), so lane l reads bank l + const at every corner, and the lanes that a
+// half-node axis sends one node down meet either the same word or a free bank. (Dense rows of 13 gave
+// two wavefronts per load.) The density stays dense behind them.
+template <int WC>
+struct Lay3 {
+    int W;
+    __device__ __forceinline__ int sy() const { return WC ? 42 : W; }
+    __device__ __forceinline__ int sz() const { return WC ? 576 : W * W; }
+    // component q (Ex, Ey, Ez, Bx, By, Bz)
+    __device__ __forceinline__ int comp(int q) const { return WC ? (q / 3) * (576 * WC) + (q % 3) * 14 : q * W * W * W; }
+    template <bool FULL>
+    __device__ __forceinline__ int density() const
+    {
+        return !FULL ? 0 : (WC ? 2 * 576 * WC : 6 * W * W * W);
+    }
+};
+static size_t window3_floats(int W, int full)
+{
+    const size_t n = (size_t)W * W * W;
+    return !full ? n : (W == kWin3 ? 2 * 576 * (size_t)kWin3 + n : 7 * n);
+}
 
 struct Axis3 {
     float g, w;       // weights of the lower and upper node (1 - w, w)
@@ -233,22 +259,23 @@ __device__ __forceinline__ float trilerp3(const float* p, int sy, int sz, Axis3 
 }
 
 // E and B at the particle from the window (out: Ex, Ey, Ez, Bx, By, Bz); base = index of the
-// particle's cell in the window
+// particle's cell in the fields' layout
 template <int WC>
 __device__ __forceinline__ void wfields3(const float* f, int Wr, int base, float fx, float fy, float fz, float* out)
 {
-    const int W = WC ? WC : Wr, WW = W * W, WWW = WW * W;
+    const Lay3<WC> L{Wr};
+    const int W = L.sy(), WW = L.sz();
     const bool ux = fx >= 0.5f, uy = fy >= 0.5f, uz = fz >= 0.5f;
     const int ox = ux ? 0 : -1, oy = uy ? 0 : -W, oz = uz ? 0 : -WW;
     const Axis3 X{1.0f - fx, fx}, Y{1.0f - fy, fy}, Z{1.0f - fz, fz};
     const float hx = ux ? fx - 0.5f : fx + 0.5f, hy = uy ? fy - 0.5f : fy + 0.5f, hz = uz ? fz - 0.5f : fz + 0.5f;
     const Axis3 HX{1.0f - hx, hx}, HY{1.0f - hy, hy}, HZ{1.0f - hz, hz};
-    out[0] = trilerp3(f + base + ox, W, WW, HX, Y, Z);                       // Ex (i+1/2, j, k)
-    out[1] = trilerp3(f + WWW + base + oy, W, WW, X, HY, Z);                 // Ey (i, j+1/2, k)
-    out[2] = trilerp3(f + 2 * WWW + base + oz, W, WW, X, Y, HZ);             // Ez (i, j, k+1/2)
-    out[3] = trilerp3(f + 3 * WWW + base + oy + oz, W, WW, X, HY, HZ);       // Bx (i, j+1/2, k+1/2)
-    out[4] = trilerp3(f + 4 * WWW + base + ox + oz, W, WW, HX, Y, HZ);       // By (i+1/2, j, k+1/2)
-    out[5] = trilerp3(f + 5 * WWW + base + ox + oy, W, WW, HX, HY, Z);       // Bz (i+1/2, j+1/2, k)
+    out[0] = trilerp3(f + L.comp(0) + base + ox, W, WW, HX, Y, Z);                       // Ex (i+1/2, j, k)
+    out[1] = trilerp3(f + L.comp(1) + base + oy, W, WW, X, HY, Z);                 // Ey (i, j+1/2, k)
+    out[2] = trilerp3(f + L.comp(2) + base + oz, W, WW, X, Y, HZ);             // Ez (i, j, k+1/2)
+    out[3] = trilerp3(f + L.comp(3) + base + oy + oz, W, WW, X, HY, HZ);       // Bx (i, j+1/2, k+1/2)
+    out[4] = trilerp3(f + L.comp(4) + base + ox + oz, W, WW, HX, Y, HZ);       // By (i+1/2, j, k+1/2)
+    out[5] = trilerp3(f + L.comp(5) + base + ox + oy, W, WW, HX, HY, Z);       // Bz (i+1/2, j+1/2, k)
 }
 
 // trilinear density and exact gradient from the window (the arithmetic of density3)
@@ -386,15 +413,15 @@ __device__ __forceinline__ void process3(const Args3& a, const Species3& S, cons
     float kx = 0.f, ky = 0.f, kz = 0.f, bx = 0.f, by = 0.f, bz = 0.f;
     float n = 0.f, gr[3] = {0.f, 0.f, 0.f};
     if (inwin) {
-        const int Wk = WC ? WC : W;
-        const int base = (lz * Wk + (int)ly) * Wk + (int)lx;
+        const Lay3<WC> L{W};
         if (FULL) {
             float o[6];
-            wfields3<WC>(w.f, W, base, fx, fy, fz, o);
+            wfields3<WC>(w.f, W, lz * L.sz() + (int)ly * L.sy() + (int)lx, fx, fy, fz, o);
             kx = S.e_kick * o[0]; ky = S.e_kick * o[1]; kz = S.e_kick * o[2];
             bx = o[3]; by = o[4]; bz = o[5];
         }
-        if (PAIR) wdensity3<WC>(w.f + 6 * (WC ? WC * WC * WC : w.WWW), W, base, fx, fy, fz, n, gr);
+        if (PAIR)
+            wdensity3<WC>(w.f + L.template density<FULL>(), W, (lz * W + (int)ly) * W + (int)lx, fx, fy, fz, n, gr);
     } else {
         float o[10];
         gather_global3(a.F[0], a.F[1], a.F[2], a.F[3], a.F[4], a.F[5], a.rho_cur, g, a.rho_s, FULL ? 1 : 0,
@@ -487,7 +514,7 @@ __device__ __forceinline__ void process3(const Args3& a, const Species3& S, cons
 }
 
 template <bool FULL, int POT, int WC>
-__global__ void __launch_bounds__(kBlock3, 3) k_particles3(const __grid_constant__ Args3 a)
+__global__ void __launch_bounds__(kBlock3, FULL ? kCtas3 : kCtas3Atoms) k_particles3(const __grid_constant__ Args3 a)
 {
     extern __shared__ unsigned smem3[];
     const int W = WC ? WC : a.W, WW = W * W, WWW = WW * W;
@@ -495,7 +522,7 @@ __global__ void __launch_bounds__(kBlock3, 3) k_particles3(const __grid_constant
     w.W = W;
     float* wf = reinterpret_cast<float*>(smem3);
     w.f = wf;
-    w.WWW = WWW;
+    const Lay3<WC> L{W};
     const Geo3& g = a.g;
     // tiles are handed out dynamically from the ticket counter in the status words (atomicInc wraps
     // it back to 0 once every CTA has drawn its last, failing, ticket)
@@ -524,15 +551,16 @@ __global__ void __launch_bounds__(kBlock3, 3) k_particles3(const __grid_constant
                 const int gn = min(max(gz, 0), g.nz), gh = min(max(gz, 0), g.nz - 1);
                 const size_t in = idx3(g, gx, gy, gn), ih = idx3(g, gx, gy, gh);
                 if (FULL) {
-                    wf[q] = __ldg(a.F[0] + in);
-                    wf[WWW + q] = __ldg(a.F[1] + in);
-                    wf[2 * WWW + q] = __ldg(a.F[2] + ih);
-                    wf[3 * WWW + q] = __ldg(a.F[3] + ih);
-                    wf[4 * WWW + q] = __ldg(a.F[4] + ih);
-                    wf[5 * WWW + q] = __ldg(a.F[5] + in);
+                    float* d = wf + c * L.sz() + b * L.sy() + e;
+                    d[L.comp(0)] = __ldg(a.F[0] + in);
+                    d[L.comp(1)] = __ldg(a.F[1] + in);
+                    d[L.comp(2)] = __ldg(a.F[2] + ih);
+                    d[L.comp(3)] = __ldg(a.F[3] + ih);
+                    d[L.comp(4)] = __ldg(a.F[4] + ih);
+                    d[L.comp(5)] = __ldg(a.F[5] + in);
                 }
                 const long long r0 = (long long)__ldg(a.rho_cur + in);
-                wf[6 * WWW + q] = a.rho_s * (float)((gn == 0 || gn == g.nz) ? 2 * r0 : r0);
+                wf[L.template density<FULL>() + q] = a.rho_s * (float)((gn == 0 || gn == g.nz) ? 2 * r0 : r0);
             }
             __syncthreads();
         }
@@ -613,7 +641,7 @@ void launch_particle_step3(Ctx& c, cudaStream_t st)
     // still fit on one SM
     const int W = c.T + 3;
     a.W = (size_t)7 * W * W * W * 4 <= 72 * 1024 ? W : 0;
-    const size_t shmem = sizeof(unsigned) * ((size_t)7 * a.W * a.W * a.W);
+    const size_t shmem = sizeof(float) * window3_floats(a.W, a.full);
     // the attributes are per device: remember what each device has been given
     static std::atomic<size_t> configured[kMaxDevices];
     int dev = 0;
@@ -630,7 +658,8 @@ void launch_particle_step3(Ctx& c, cudaStream_t st)
 #undef GBPIC_ATTR
         configured[dev].store(shmem);
     }
-    int grid = c.ntiles < c.nsm * 3 ? c.ntiles : c.nsm * 3;
+    const int slots = c.nsm * (a.full ? kCtas3 : kCtas3Atoms);
+    int grid = c.ntiles < slots ? c.ntiles : slots;
     if (grid < 1) grid = 1;
     // the instance with the potential and the lattice compiled in, and the window edge when it is
     // the 10-cell tile's
