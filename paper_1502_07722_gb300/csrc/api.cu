@@ -12,7 +12,6 @@
 namespace gbpic {
 int tile_window(int T);
 int energy_blocks(const Ctx& c);
-void swap_currents(Ctx& c);
 void sort_species_impl(Ctx& c, int s, cudaStream_t st, int from_b, int64_t* launches);
 }  // namespace gbpic
 
@@ -103,13 +102,13 @@ int derive_layout(const pic_config* cfg, Layout& L)
     const int arrays = L.dims == 3 ? 7 : 6;
     for (int s = 0; s < 2; s++) t += 2 * arrays * align256(4 * (size_t)L.cap[s]) + align256(4 * (size_t)(L.ntiles + 1));
     t += 6 * align256(4 * L.nn) + 5 * align256(8 * L.nn);
-    L.twin = L.dims == 2 && full;         // the field update's second set of field and current grids
+    L.twin = full;         // the field update's second set of field and current grids
     if (L.twin) t += 6 * align256(4 * L.nn) + 3 * align256(8 * L.nn);
     L.items = L.dims == 2 ? work_item_cap(L.cap[0] + L.cap[1], L.ntiles) : 0;
     if (L.items >= (1LL << 31)) return PIC_EINVAL;
     t += align256(sizeof(WorkItem) * (size_t)L.items) + align256(4);
     const size_t plane = (size_t)L.nx * L.ny;
-    t += (L.dims == 3 ? align256(4 * 8 * plane) : 0) + 2 * align256(4 * plane) + align256(8);
+    t += 2 * align256(4 * plane);
     t += 2 * align256(4 * ((size_t)L.nkeys + 1));
     t += align256(4 * (((size_t)L.nkeys + 2047) / 2048 + 1));
     t += align256(8 * 5 * (size_t)kMaxEnergyBlocks) + align256(8 * 8) + align256(32);
@@ -197,8 +196,8 @@ int redeposit(Ctx& c)
 }
 
 // The currents a step deposits into start clear (the transport stage has none) and the next node
-// density from the current one (the particle kernel adds the changes). In 2D the field update of
-// the step before has done both.
+// density from the current one (the particle kernel adds the changes). The field update of the step
+// before has done both.
 int prepare_step(Ctx& c)
 {
     const bool twin = c.Jn[0] != nullptr;
@@ -233,6 +232,15 @@ int64_t work_item_cap_of(const pic_config* cfg)
 {
     Layout L;
     return derive_layout(cfg, L) == PIC_OK ? L.items : 0;
+}
+
+void swap_fields(Ctx& c)
+{
+    for (int q = 0; q < 6; q++) {
+        float* p = c.F[q];
+        c.F[q] = c.Fn[q];
+        c.Fn[q] = p;
+    }
 }
 
 StepArgs make_step_args(Ctx& c)
@@ -362,10 +370,8 @@ int pic_init(const pic_config* cfg, void* workspace, size_t workspace_bytes, voi
     c.items_cap = (int32_t)L.items;
     c.nitems = cv.take<int32_t>(1);
     const size_t plane = (size_t)L.nx * L.ny;
-    c.mur_save = d3 ? cv.take<float>(8 * plane) : nullptr;
     c.ant_c = cv.take<float>(plane);
     c.ant_s = cv.take<float>(plane);
-    c.ant = cv.take<float>(2);
     c.keys_count = cv.take<int32_t>((size_t)L.nkeys + 1);
     c.keys_off = cv.take<int32_t>((size_t)L.nkeys + 1);
     c.scan_tmp = cv.take<int32_t>(((size_t)L.nkeys + 2047) / 2048 + 1);
@@ -434,7 +440,6 @@ int pic_init(const pic_config* cfg, void* workspace, size_t workspace_bytes, voi
     for (int q = 0; q < 6; q++) ok &= cudaMemsetAsync(c.F[q], 0, 4 * L.nn, c.stream) == cudaSuccess;
     for (int q = 0; q < 3; q++) ok &= cudaMemsetAsync(c.J[q], 0, 8 * L.nn, c.stream) == cudaSuccess;
     for (int q = 0; q < 2; q++) ok &= cudaMemsetAsync(c.rho[q], 0, 8 * L.nn, c.stream) == cudaSuccess;
-    if (d3) ok &= cudaMemsetAsync(c.mur_save, 0, 4 * 8 * plane, c.stream) == cudaSuccess;
     ok &= cudaMemsetAsync(c.red_out, 0, 8 * sizeof(double), c.stream) == cudaSuccess;   // incl. the injected-energy sum
     ok &= cudaMemsetAsync(c.status, 0, 32, c.stream) == cudaSuccess;
     if (!ok) {
@@ -499,7 +504,7 @@ int pic_step(pic_ctx* h, int32_t nsteps)
             c.nlaunch[3] += c.nlaunch[1] - before;
         }
         CK(cudaGetLastError());
-        // the 2D field update has prepared the next step
+        // the field update has prepared the next step
         c.prepared = c.Jn[0] != nullptr;
         c.step++;
         c.steps_since_sort++;

@@ -17,7 +17,6 @@
 namespace gbpic {
 void sort_species_impl(Ctx& c, int s, cudaStream_t st, int from_b, int64_t* launches);
 int max_batch_slabs();
-void swap_currents(Ctx& c);
 
 constexpr int kMaxSlabs = 48;    // the constant-memory argument table of the batched particle kernel
 static_assert(kMaxSlabs <= kMaxFieldSlabs, "every slab's field arguments fit the batched field kernels' parameters");
@@ -91,11 +90,7 @@ void flip_parity(Ctx& c)
     c.cur = 1 - c.cur;
     if (!c.Jn[0]) return;
     swap_currents(c);
-    for (int q = 0; q < 6; q++) {
-        float* f = c.F[q];
-        c.F[q] = c.Fn[q];
-        c.Fn[q] = f;
-    }
+    swap_fields(c);
 }
 
 // Arguments of a step that starts at parity p: the particle kernel deposits into the cleared

@@ -12,8 +12,6 @@
 // What bounds it: memory traffic on the large grids, the launch on the small ones. Against three
 // in-place passes (B half, E, B half) with a copy/clear kernel and a one-thread antenna kernel, a
 // node moves 112 bytes instead of 172 and a step has two launches instead of six.
-#include <cmath>
-
 #include "pic_internal.cuh"
 
 namespace gbpic {
@@ -23,25 +21,6 @@ namespace gbpic {
 // z neighbours from the row before, and no barrier or shared memory is needed. The next row's loads
 // are issued one row ahead.
 constexpr int kCols = 29, kFieldThreads = 128;
-
-// Antenna amplitude of one step (FP64):
-//   E_x += 2 (c dt / dx) E0 env(t) amp(x) sin(w (t - t_ant) + phi(x))
-// split as ant[0] * amp cos(phi) + ant[1] * amp sin(phi) with ant = A (sin, cos)(w (t - t_ant)).
-// A single simulation evaluates it on the host with the launch's arguments (one thread of the GPU
-// took 5.3 us for it); a batch, whose steps are replayed from a graph, on the device.
-__host__ __device__ inline void antenna_scalars(const AntennaParams& p, long long step, float* ant)
-{
-    float s = 0.0f, c = 0.0f;
-    if (p.on) {
-        const double tau = ((double)step + 0.5) * p.dt - p.t_ant;
-        const double env = exp(-2.0 * 0.6931471805599453 * tau * tau / (p.tau_fwhm * p.tau_fwhm));
-        const double a = p.coef * env;
-        s = (float)(a * sin(p.omega * tau));
-        c = (float)(a * cos(p.omega * tau));
-    }
-    ant[0] = s;
-    ant[1] = c;
-}
 
 __device__ __forceinline__ int wrap_col(int i, int nx)
 {
@@ -275,11 +254,7 @@ void launch_fields(Ctx& c, cudaStream_t st, int64_t step, int64_t* launches)
     f.ant0 = ant[0];
     f.ant1 = ant[1];
     k_fields<<<field_blocks(f), kFieldThreads, 0, st>>>(f);
-    for (int q = 0; q < 6; q++) {
-        float* p = c.F[q];
-        c.F[q] = c.Fn[q];
-        c.Fn[q] = p;
-    }
+    swap_fields(c);
     if (launches) *launches += 1;
 }
 

@@ -751,120 +751,157 @@ struct Field3 {
     Geo3 g;
     int k_ant;
     float h_b, h_e, cj, mur;
-    float* F[6];
-    const u64* J[3];
-    float* save;          // 8 planes of nx*ny: Ex(0) Ex(1) Ex(nz-1) Ex(nz) Ey(0) Ey(1) Ey(nz-1) Ey(nz)
+    float ant0, ant1;     // this step's antenna scalars
+    const float* F[6];    // read
+    float* G[6];          // written
+    const u64* J[3];      // this step's currents
+    u64* Z[3];            // cleared for the next step
+    const u64* rho;       // node density after this step's moves
+    u64* rho_next;        // starts as its copy
     const float* antc;    // nx*ny
     const float* ants;
-    const float* ant;
     int k_flux;           // node plane below the antenna (Poynting flux of the injected energy)
     double* flux;
 };
 
-__global__ void k_half_B3(const Field3 f, int save)
+// The whole update as one out-of-place kernel, as in 2D (fields.cu): B half step, E step with current,
+// antenna and Mur planes, B half step, the clear of the next step's currents and the start of its density.
+// A block walks up a segment of planes with a patch of kRows3 + 3 rows (one per warp) of 32 columns:
+// x neighbours come by shuffle, y neighbours through shared memory, z neighbours from the plane before
+// in registers. The patch recomputes one row and column below and two above what it writes (13 x 29).
+// It is bound by memory traffic: 112 bytes per node and step instead of 172 in three in-place passes and
+// a copy/clear kernel. 384^2 x 256 cells: 0.92 ms against 1.06 plus 0.3 of the copy (segments of 8 planes
+// 0.97, 32 planes 0.91; 192^2 x 128: 0.130, 0.137, 0.153); one block per SM 1.44.
+constexpr int kCols3 = 29, kRows3 = 13, kWarps3 = kRows3 + 3, kSeg3 = 16;
+
+struct F3 {
+    float x, y, z;
+};
+
+__global__ void __launch_bounds__(32 * kWarps3, 2) k_fields3(const __grid_constant__ Field3 f)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y, k = blockIdx.z;
+    __shared__ float sex[kWarps3][32], sez[kWarps3][32], sbx[kWarps3][32], sbz[kWarps3][32], snx[kWarps3][32],
+        snz[kWarps3][32];
     const Geo3& g = f.g;
-    if (i >= g.nx) return;
-    const int ip = i + 1 == g.nx ? 0 : i + 1, jp = j + 1 == g.ny ? 0 : j + 1;
-    const size_t c = idx3(g, i, j, k);
-    const float *Ex = f.F[0], *Ey = f.F[1], *Ez = f.F[2];
-    float *Bx = f.F[3], *By = f.F[4], *Bz = f.F[5];
-    const float ex = Ex[c], ey = Ey[c];
-    if (k < g.nz) {
-        const float ez = Ez[c];
-        const size_t up = c + (size_t)g.nx * g.ny;
-        Bx[c] += f.h_b * ((Ey[up] - ey) - (Ez[idx3(g, i, jp, k)] - ez));
-        By[c] += f.h_b * ((Ez[idx3(g, ip, j, k)] - ez) - (Ex[up] - ex));
+    const int nz = g.nz, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int i = (int)blockIdx.x * kCols3 + lane - 1, j = (int)blockIdx.y * kRows3 + w - 1;
+    int gi = i < 0 ? i + g.nx : i, gj = j < 0 ? j + g.ny : j;
+    while (gi >= g.nx) gi -= g.nx;
+    while (gj >= g.ny) gj -= g.ny;
+    const bool own = lane >= 1 && lane <= kCols3 && i < g.nx && w >= 1 && w <= kRows3 && j < g.ny;
+    const int wm = w > 0 ? w - 1 : 0, wp = w + 1 < kWarps3 ? w + 1 : w;     // the patch's outer rows are not written
+    // planes k0 .. k1 - 1; the last segment takes the remainder
+    const int k0 = (int)blockIdx.z * kSeg3, k1 = blockIdx.z + 1 == gridDim.z ? nz + 1 : k0 + kSeg3;
+    const size_t plane = (size_t)g.nx * g.ny;
+    const size_t col = (size_t)gj * g.nx + gi;
+    const float antc = f.antc[col], ants = f.ants[col];
+    const int r0 = k0 > 0 ? k0 - 1 : 0;
+    size_t c = (size_t)r0 * plane + col;
+    F3 e = {__ldg(f.F[0] + c), __ldg(f.F[1] + c), __ldg(f.F[2] + c)};                     // old E of plane r
+    F3 en = {__ldg(f.F[0] + c + plane), __ldg(f.F[1] + c + plane), __ldg(f.F[2] + c + plane)};   // and r + 1
+    F3 b = {__ldg(f.F[3] + c), __ldg(f.F[4] + c), __ldg(f.F[5] + c)};
+    u64 jx = __ldg(f.J[0] + c), jy = __ldg(f.J[1] + c), jz = __ldg(f.J[2] + c);
+    F3 ep = {0, 0, 0}, bp = {0, 0, 0}, np = {0, 0, 0};       // plane r - 1: old E, half-step B, new E
+    sex[w][lane] = e.x;
+    sez[w][lane] = e.z;
+    __syncthreads();
+    for (int r = r0; r <= k1 && r <= nz; r++, c += plane) {
+        // one plane ahead
+        F3 e2 = {0, 0, 0}, b2 = {0, 0, 0};
+        u64 jx2 = 0, jy2 = 0, jz2 = 0;
+        if (r < k1 && r + 1 <= nz) {
+            const size_t u = c + plane;
+            b2 = F3{__ldg(f.F[3] + u), __ldg(f.F[4] + u), __ldg(f.F[5] + u)};
+            jx2 = __ldg(f.J[0] + u);
+            jy2 = __ldg(f.J[1] + u);
+            jz2 = __ldg(f.J[2] + u);
+            if (r + 2 <= nz) e2 = F3{__ldg(f.F[0] + u + plane), __ldg(f.F[1] + u + plane), __ldg(f.F[2] + u + plane)};
+        }
+        // B(r) to the half step (Bx, By have nz planes)
+        const float exj = sex[wp][lane], ezj = sez[wp][lane];
+        const float eyi = __shfl_down_sync(0xffffffffu, e.y, 1), ezi = __shfl_down_sync(0xffffffffu, e.z, 1);
+        if (r < nz) {
+            b.x += f.h_b * ((en.y - e.y) - (ezj - e.z));
+            b.y += f.h_b * ((ezi - e.z) - (en.x - e.x));
+        }
+        b.z += f.h_b * ((exj - e.x) - (eyi - e.y));
+        sbx[w][lane] = b.x;
+        sbz[w][lane] = b.z;
+        __syncthreads();
+        // E(r) to the new step
+        const float bxj = sbx[wm][lane], bzj = sbz[wm][lane];
+        const float byi = __shfl_up_sync(0xffffffffu, b.y, 1), bzi = __shfl_up_sync(0xffffffffu, b.z, 1);
+        F3 n = e;
+        if (r > 0 && r < nz) {
+            float v = e.x + f.h_e * ((b.z - bzj) - (b.y - bp.y)) - f.cj * (float)(long long)jx;
+            if (r == f.k_ant) v += antc * f.ant0 + ants * f.ant1;
+            n.x = v;
+            n.y = e.y + f.h_e * ((b.x - bp.x) - (b.z - bzi)) - f.cj * (float)(long long)jy;
+        }
+        if (r < nz) n.z += f.h_e * ((b.y - byi) - (b.x - bxj)) - f.cj * (float)(long long)jz;
+        if (r == 1) {                      // Mur: the wall planes from the new plane beside them
+            np.x = e.x + f.mur * (n.x - ep.x);
+            np.y = e.y + f.mur * (n.y - ep.y);
+        } else if (r == nz) {
+            n.x = ep.x + f.mur * (np.x - e.x);
+            n.y = ep.y + f.mur * (np.y - e.y);
+        }
+        if (r == f.k_flux && r >= k0 && r < k1) {             // uniform over the block
+            // (Ex By - Ey Bx) at the half step
+            float s = own ? 0.25f * ((e.x + n.x) * (bp.y + b.y) - (e.y + n.y) * (bp.x + b.x)) : 0.0f;
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (lane == 0 && s != 0.0f) atomicAdd(f.flux, (double)s);
+        }
+        // the new E of plane r - 1 for the rows below, the old E of plane r + 1 for the next turn
+        snx[w][lane] = np.x;
+        snz[w][lane] = np.z;
+        sex[w][lane] = en.x;
+        sez[w][lane] = en.z;
+        __syncthreads();
+        // finish plane r - 1
+        const float npyi = __shfl_down_sync(0xffffffffu, np.y, 1), npzi = __shfl_down_sync(0xffffffffu, np.z, 1);
+        if (r > k0 && own) {
+            const size_t q = c - plane;
+            const float npxj = snx[wp][lane], npzj = snz[wp][lane];
+            f.G[0][q] = np.x;
+            f.G[1][q] = np.y;
+            f.G[2][q] = np.z;
+            f.G[3][q] = bp.x + f.h_b * ((n.y - np.y) - (npzj - np.z));
+            f.G[4][q] = bp.y + f.h_b * ((npzi - np.z) - (n.x - np.x));
+            f.G[5][q] = bp.z + f.h_b * ((npxj - np.x) - (npyi - np.y));
+        }
+        // the next step's currents and node density
+        if (r >= k0 && r < k1 && own) {
+            f.Z[0][c] = 0;
+            f.Z[1][c] = 0;
+            f.Z[2][c] = 0;
+            f.rho_next[c] = f.rho[c];
+        }
+        ep = e;
+        bp = b;
+        np = n;
+        e = en;
+        en = e2;
+        b = b2;
+        jx = jx2;
+        jy = jy2;
+        jz = jz2;
     }
-    Bz[c] += f.h_b * ((Ex[idx3(g, i, jp, k)] - ex) - (Ey[idx3(g, ip, j, k)] - ey));
-    if (save) {
-        int slot = -1;
-        if (k == 0) slot = 0;
-        else if (k == 1) slot = 1;
-        else if (k == g.nz - 1) slot = 2;
-        else if (k == g.nz) slot = 3;
-        if (slot >= 0) {
-            const size_t plane = (size_t)g.nx * g.ny, q = (size_t)j * g.nx + i;
-            f.save[slot * plane + q] = ex;
-            f.save[(4 + slot) * plane + q] = ey;
+    if (k1 == nz + 1) {                    // the wall plane nz: only its Bz is updated
+        __syncthreads();                   // the rows below have read plane nz - 1
+        snx[w][lane] = np.x;
+        __syncthreads();
+        const float npyi = __shfl_down_sync(0xffffffffu, np.y, 1);
+        if (own) {
+            const size_t q = (size_t)nz * plane + col;
+            f.G[0][q] = np.x;
+            f.G[1][q] = np.y;
+            f.G[2][q] = np.z;
+            f.G[3][q] = bp.x;
+            f.G[4][q] = bp.y;
+            f.G[5][q] = bp.z + f.h_b * ((snx[wp][lane] - np.x) - (npyi - np.y));
         }
     }
-}
-
-__device__ __forceinline__ float ex3_new(const Field3& f, int i, int j, int k, float old)
-{
-    const Geo3& g = f.g;
-    const size_t c = idx3(g, i, j, k);
-    const int jm = j == 0 ? g.ny - 1 : j - 1;
-    float v = old + f.h_e * ((f.F[5][c] - f.F[5][idx3(g, i, jm, k)]) - (f.F[4][c] - f.F[4][idx3(g, i, j, k - 1)])) -
-              f.cj * (float)(long long)f.J[0][c];
-    if (k == f.k_ant) {
-        const size_t q = (size_t)j * g.nx + i;
-        v += f.antc[q] * f.ant[0] + f.ants[q] * f.ant[1];
-    }
-    return v;
-}
-__device__ __forceinline__ float ey3_new(const Field3& f, int i, int j, int k, float old)
-{
-    const Geo3& g = f.g;
-    const size_t c = idx3(g, i, j, k);
-    const int im = i == 0 ? g.nx - 1 : i - 1;
-    return old + f.h_e * ((f.F[3][c] - f.F[3][idx3(g, i, j, k - 1)]) - (f.F[5][c] - f.F[5][idx3(g, im, j, k)])) -
-           f.cj * (float)(long long)f.J[1][c];
-}
-
-__global__ void k_E3(const Field3 f)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y, k = blockIdx.z;
-    const Geo3& g = f.g;
-    float s = 0.0f;            // on the flux plane: this node's (Ex By - Ey Bx) at the half step
-    if (i < g.nx) {
-        const size_t c = idx3(g, i, j, k), plane = (size_t)g.nx * g.ny, q = (size_t)j * g.nx + i;
-        float* Ex = f.F[0];
-        float* Ey = f.F[1];
-        if (k > 0 && k < g.nz) {
-            const float ex0 = Ex[c], ey0 = Ey[c];
-            const float ex1 = ex3_new(f, i, j, k, ex0), ey1 = ey3_new(f, i, j, k, ey0);
-            Ex[c] = ex1;
-            Ey[c] = ey1;
-            if (k == f.k_flux)
-                s = 0.25f * ((ex0 + ex1) * (f.F[4][c - plane] + f.F[4][c]) -
-                             (ey0 + ey1) * (f.F[3][c - plane] + f.F[3][c]));
-        } else if (k == 0) {
-            const float x0 = f.save[q], x1 = f.save[plane + q], y0 = f.save[4 * plane + q], y1 = f.save[5 * plane + q];
-            Ex[c] = x1 + f.mur * (ex3_new(f, i, j, 1, x1) - x0);
-            Ey[c] = y1 + f.mur * (ey3_new(f, i, j, 1, y1) - y0);
-        } else {
-            const float x1 = f.save[2 * plane + q], x0 = f.save[3 * plane + q], y1 = f.save[6 * plane + q],
-                        y0 = f.save[7 * plane + q];
-            Ex[c] = x1 + f.mur * (ex3_new(f, i, j, g.nz - 1, x1) - x0);
-            Ey[c] = y1 + f.mur * (ey3_new(f, i, j, g.nz - 1, y1) - y0);
-        }
-        if (k < g.nz) {
-            const int im = i == 0 ? g.nx - 1 : i - 1, jm = j == 0 ? g.ny - 1 : j - 1;
-            f.F[2][c] += f.h_e * ((f.F[4][c] - f.F[4][idx3(g, im, j, k)]) - (f.F[3][c] - f.F[3][idx3(g, i, jm, k)])) -
-                         f.cj * (float)(long long)f.J[2][c];
-        }
-    }
-    if (k == f.k_flux) {                                  // uniform over the block
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if ((threadIdx.x & 31) == 0 && s != 0.0f) atomicAdd(f.flux, (double)s);
-    }
-}
-
-__global__ void k_antenna3(AntennaParams p, long long step, float* ant)
-{
-    float s = 0.0f, c = 0.0f;
-    if (p.on) {
-        const double tau = ((double)step + 0.5) * p.dt - p.t_ant;
-        const double env = exp(-2.0 * 0.6931471805599453 * tau * tau / (p.tau_fwhm * p.tau_fwhm));
-        const double a = p.coef * env;
-        s = (float)(a * sin(p.omega * tau));
-        c = (float)(a * cos(p.omega * tau));
-    }
-    ant[0] = s;
-    ant[1] = c;
 }
 
 void launch_fields3(Ctx& c, cudaStream_t st, int64_t step, int64_t* launches)
@@ -877,20 +914,25 @@ void launch_fields3(Ctx& c, cudaStream_t st, int64_t step, int64_t* launches)
     f.cj = (float)(kQe * c.w / (6.0 * 4398046511104.0 * c.cfg.dx * c.cfg.dx * kEps0));
     const double cdt = kC * c.dt;
     f.mur = (float)((cdt - c.cfg.dx) / (cdt + c.cfg.dx));
+    float ant[2];
+    antenna_scalars(make_antenna_params(c), (long long)step, ant);
+    f.ant0 = ant[0];
+    f.ant1 = ant[1];
     for (int q = 0; q < 6; q++) f.F[q] = c.F[q];
+    for (int q = 0; q < 6; q++) f.G[q] = c.Fn[q];
     for (int q = 0; q < 3; q++) f.J[q] = c.J[q];
-    f.save = c.mur_save;
+    for (int q = 0; q < 3; q++) f.Z[q] = c.Jn[q];
+    f.rho = c.rho[c.cur];
+    f.rho_next = c.rho[1 - c.cur];
     f.antc = c.ant_c;
     f.ants = c.ant_s;
-    f.ant = c.ant;
     f.k_flux = c.k_ant - 1 >= 1 ? c.k_ant - 1 : -1;
     f.flux = c.red_out + 5;
-    k_antenna3<<<1, 1, 0, st>>>(make_antenna_params(c), (long long)step, c.ant);
-    dim3 block(256), grid((c.nx + 255) / 256, c.ny, c.nz + 1);
-    k_half_B3<<<grid, block, 0, st>>>(f, 1);
-    k_E3<<<grid, block, 0, st>>>(f);
-    k_half_B3<<<grid, block, 0, st>>>(f, 0);
-    if (launches) *launches += 4;
+    const int seg = (c.nz + 1) / kSeg3;
+    const dim3 grid((c.nx + kCols3 - 1) / kCols3, (c.ny + kRows3 - 1) / kRows3, seg > 1 ? seg : 1);
+    k_fields3<<<grid, 32 * kWarps3, 0, st>>>(f);
+    swap_fields(c);
+    if (launches) *launches += 1;
 }
 
 // ---- energies ------------------------------------------------------------------------------

@@ -1,6 +1,7 @@
 // Internal types and launch declarations of the GB300 PIC library (not part of the C ABI).
 #pragma once
 
+#include <cmath>
 #include <cstddef>
 #include <cstdint>
 #include <vector>
@@ -146,17 +147,15 @@ struct Ctx {
     u64* J[3];            // currents of the last step
     u64* rho[2];
     int32_t cur;          // rho[cur] holds the node density at the current positions
-    float* Fn[6];         // 2D full mode: the fields the next update writes (swapped with F after it)
-    u64* Jn[3];           // 2D full mode: the currents the next step deposits into
+    float* Fn[6];         // full mode: the fields the next update writes (swapped with F after it)
+    u64* Jn[3];           // full mode: the currents the next step deposits into
     int32_t prepared;     // Jn is clear and rho[1 - cur] equals rho[cur]
     WorkItem* items;      // 2D: work items of the particle kernel, from the tile offsets
     int32_t* nitems;
     int32_t items_cap;
     int32_t items_ok;     // the list matches the tile offsets
-    float* mur_save;      // 3D: 8 planes
     float* ant_c;         // nx: amplitude * cos(phase(x)) at x = i + 1/2
     float* ant_s;         // nx: amplitude * sin(phase(x))
-    float* ant;           // 2: antenna scalars of the current step (written on the device)
     // scratch
     int32_t* keys_count;  // nkeys + 1
     int32_t* keys_off;    // nkeys + 1
@@ -185,7 +184,26 @@ struct AntennaParams {
     double dt, t_ant, tau_fwhm, omega, coef;
 };
 
-// Everything the field kernel needs for one simulation.
+// Antenna amplitude of one step (FP64):
+//   E_x += 2 (c dt / dx) E0 env(t) amp(x) sin(w (t - t_ant) + phi(x))
+// split as ant[0] * amp cos(phi) + ant[1] * amp sin(phi) with ant = A (sin, cos)(w (t - t_ant)).
+// A single simulation evaluates it on the host with the launch's arguments (one thread of the GPU
+// took 5.3 us for it); a batch, whose steps are replayed from a graph, on the device.
+__host__ __device__ inline void antenna_scalars(const AntennaParams& p, long long step, float* ant)
+{
+    float s = 0.0f, c = 0.0f;
+    if (p.on) {
+        const double tau = ((double)step + 0.5) * p.dt - p.t_ant;
+        const double env = exp(-2.0 * 0.6931471805599453 * tau * tau / (p.tau_fwhm * p.tau_fwhm));
+        const double a = p.coef * env;
+        s = (float)(a * sin(p.omega * tau));
+        c = (float)(a * cos(p.omega * tau));
+    }
+    ant[0] = s;
+    ant[1] = c;
+}
+
+// Everything the 2D field kernel needs for one simulation.
 struct FieldArgs {
     int nx, nz, k_ant;
     float h_b;           // dt / (2 dx)      (half step of B)
@@ -208,6 +226,9 @@ struct FieldArgs {
 };
 
 // kernels launched from the host side of the library (defined in the .cu files)
+// the two sets of current and field grids (full mode) change places
+void swap_currents(Ctx& c);
+void swap_fields(Ctx& c);
 void launch_init_particles(Ctx& c, int s, cudaStream_t st);
 void launch_sort_species(Ctx& c, int s, cudaStream_t st, int64_t* launches);
 // Fixed-point range: the J_y code resolution for a 2D full-mode slab of n particles per cell (both
