@@ -532,20 +532,15 @@ __global__ void __launch_bounds__(kItemThreads) k_work_items(const int32_t* __re
                                                             const int32_t* __restrict__ start1, int ntiles, int slab,
                                                             int chunk, WorkItem* items, int* nitems, int cap)
 {
-    __shared__ int sums[kItemThreads / 32];
+    __shared__ int sums[kItemThreads / 32], first[kItemThreads];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int base = *nitems;
     for (int t0 = 0; t0 < ntiles; t0 += kItemThreads) {
         const int t = t0 + (int)threadIdx.x;
-        int i0 = 0, ni = 0, e0 = 0, ne = 0, parts = 0;
+        int parts = 0;
         if (t < ntiles) {
-            i0 = start0[t];
-            ni = start0[t + 1] - i0;
-            if (start1) {
-                e0 = start1[t];
-                ne = start1[t + 1] - e0;
-            }
-            if (ni + ne > 0) parts = max(1, (int)(((long long)ni + ne + chunk / 2) / chunk));
+            const long long cnt = (long long)(start0[t + 1] - start0[t]) + (start1 ? start1[t + 1] - start1[t] : 0);
+            if (cnt > 0) parts = max(1, (int)((cnt + chunk / 2) / chunk));
         }
         int scan = parts;
         for (int o = 1; o < 32; o <<= 1) {
@@ -559,19 +554,27 @@ __global__ void __launch_bounds__(kItemThreads) k_work_items(const int32_t* __re
             if (q < warp) before += sums[q];
             total += sums[q];
         }
-        const int at = base + before + scan - parts;
-        if (at + parts <= cap)                 // always: the list is sized for every tile's parts
-            for (int q = 0; q < parts; q++) {
-                WorkItem w;
-                w.tile = t;
-                w.slab = slab;
-                w.p0[0] = part_start(i0, i0 + ni, q, parts);
-                w.p1[0] = part_start(i0, i0 + ni, q + 1, parts);
-                w.p0[1] = part_start(e0, e0 + ne, q, parts);
-                w.p1[1] = part_start(e0, e0 + ne, q + 1, parts);
-                w.pad[0] = w.pad[1] = 0;
-                items[at + q] = w;
+        // the items of these tiles, one per thread: its tile is the last one that starts at or before it
+        first[threadIdx.x] = before + scan - parts;
+        __syncthreads();
+        for (int q = threadIdx.x; q < total && base + q < cap; q += kItemThreads) {     // always below cap
+            int lo = 0, hi = kItemThreads - 1;
+            while (lo < hi) {
+                const int mid = (lo + hi + 1) >> 1;
+                if (first[mid] <= q) lo = mid;
+                else hi = mid - 1;
             }
+            const int u = t0 + lo, sub = q - first[lo], n = (lo + 1 < kItemThreads ? first[lo + 1] : total) - first[lo];
+            WorkItem w;
+            w.tile = u;
+            w.slab = slab;
+            w.p0[0] = part_start(start0[u], start0[u + 1], sub, n);
+            w.p1[0] = part_start(start0[u], start0[u + 1], sub + 1, n);
+            w.p0[1] = start1 ? part_start(start1[u], start1[u + 1], sub, n) : 0;
+            w.p1[1] = start1 ? part_start(start1[u], start1[u + 1], sub + 1, n) : 0;
+            w.pad[0] = w.pad[1] = 0;
+            items[base + q] = w;
+        }
         base += total;
         __syncthreads();
     }

@@ -231,6 +231,11 @@ void swap_currents(Ctx& c);
 void swap_fields(Ctx& c);
 void launch_init_particles(Ctx& c, int s, cudaStream_t st);
 void launch_sort_species(Ctx& c, int s, cudaStream_t st, int64_t* launches);
+// Kernels that sum runs of particles of one cell: columns of the storage layout a lane walks, and the
+// grid of 256-thread blocks for chunks of 32 x that many records.
+int run_columns(const Ctx& c, const Species& S);
+constexpr int kRunBatch = 4;      // records of a lane whose loads are in flight together
+int run_grid(const Ctx& c, int64_t n, int cols);
 // Fixed-point range: the J_y code resolution for a 2D full-mode slab of n particles per cell (both
 // species) and the particle count per block of 4^dims cells up to which every int64 node sum is
 // proven exact.

@@ -92,23 +92,32 @@ __device__ __forceinline__ int cell_key(int cell, const KeyGeo& g)
 // a lane that walks its warp's chunk of B slots with stride 32 meets consecutive particles of the
 // cell order (between sorts they have barely moved) and issues one atomic per run of equal keys
 // instead of one per particle (any order stays correct; only the runs get shorter).
-__global__ void k_count(const int32_t* __restrict__ cell, int64_t n, KeyGeo kg, int32_t* count, int cols)
+constexpr int kCountBatch = 8;      // loads in flight per lane
+__global__ void __launch_bounds__(256) k_count(const int32_t* __restrict__ cell, int64_t n, KeyGeo kg, int32_t* count, int cols)
 {
     const int lane = threadIdx.x & 31;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarp = ((int64_t)gridDim.x * blockDim.x) >> 5, chunk = 32 * (int64_t)cols;
     for (int64_t base = warp * chunk; base < n; base += nwarp * chunk) {
         int key = -1, run = 0;
-        for (int c = 0; c < cols; c++) {
-            const int64_t p = base + 32 * (int64_t)c + lane;
-            if (p >= n) break;
-            const int k = cell_key(cell[p], kg);
-            if (k != key) {
-                if (run) atomicAdd(count + key, run);
-                key = k;
-                run = 0;
+        for (int c0 = 0; c0 < cols; c0 += kCountBatch) {
+            int ce[kCountBatch];
+#pragma unroll
+            for (int q = 0; q < kCountBatch; q++) {
+                const int64_t p = base + 32 * (int64_t)(c0 + q) + lane;
+                ce[q] = c0 + q < cols && p < n ? cell[p] : -1;
             }
-            run++;
+#pragma unroll
+            for (int q = 0; q < kCountBatch; q++) {
+                if (ce[q] < 0) continue;
+                const int k = cell_key(ce[q], kg);
+                if (k != key) {
+                    if (run) atomicAdd(count + key, run);
+                    key = k;
+                    run = 0;
+                }
+                run++;
+            }
         }
         if (run) atomicAdd(count + key, run);
     }
@@ -176,15 +185,40 @@ __global__ void k_scan_sums(int32_t* bsum, int nb)
     }
 }
 
-__global__ void k_scan_add(int32_t* out, const int32_t* __restrict__ bsum, int n, int32_t* cursor, int32_t total)
+// Adds the block totals' prefix (sums: already scanned by k_scan_sums; otherwise each block sums the
+// totals before its own), writes the cursors and the tiles' first particles, and checks the fixed-point
+// range: every int64 node sum is exact while the particles that can reach one node (both species: bounded
+// by the sum of the two species' largest block counts from their last sorts) stay within the limit the
+// context was set up for; beyond it the sticky overflow bit is raised.
+__global__ void __launch_bounds__(256) k_scan_add(int32_t* out, const int32_t* __restrict__ bsum, int scanned, int n,
+                                                  int32_t* cursor, int32_t total, int TT, int32_t* tile_start,
+                                                  unsigned* status, long long limit)
 {
+    __shared__ int32_t sh[8];
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    const int sb = (int)(blockIdx.x * blockDim.x) / kScanItems;        // the same for the whole block
+    int32_t before = 0;
+    if (scanned) {
+        before = bsum[sb];
+    } else {
+        for (int q = threadIdx.x; q < sb; q += blockDim.x) before += bsum[q];
+        for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
+        if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = before;
+        __syncthreads();
+        before = 0;
+        for (int w = 0; w < 8; w++) before += sh[w];
+    }
     if (j < n) {
-        const int32_t v = out[j] + bsum[j / kScanItems];
+        const int32_t v = out[j] + before;
         out[j] = v;
         cursor[j] = v;
+        if (j % TT == 0) tile_start[j / TT] = v;
     }
-    if (j == 0) out[n] = total;
+    if (j == 0) {
+        out[n] = total;
+        tile_start[n / TT] = total;
+        if ((long long)status[4] + (long long)status[5] > limit) atomicOr(status, kErrOverflow);
+    }
 }
 
 // Key of cell (i, j, k) (j = 0 in 2D), as cell_key computes it from the cell index.
@@ -206,8 +240,9 @@ __device__ __forceinline__ int key_of(int i, int j, int k, const KeyGeo& g)
 // shared-memory copy of the patch with its halo, keeps the last three rows' sums in registers and
 // closes the block of base row k - 3 at row k. One atomicMax per warp into *out. (The direct
 // form, 4^dims key lookups per cell, took 1.9 ms per species on the 384^2 x 256 slab.)
-__global__ void k_counts_to_cells(const int32_t* __restrict__ count, KeyGeo kg, int nz, int32_t* out)
+__global__ void k_counts_to_cells(const int32_t* __restrict__ count, KeyGeo kg, int nz, int32_t* out, unsigned* largest)
 {
+    if (blockIdx.x == 0 && threadIdx.x == 0) *largest = 0;          // k_block_max takes the maximum into it
     const int64_t ncell = (int64_t)kg.nx * kg.ny * nz;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < ncell; c += stride) {
@@ -218,7 +253,10 @@ __global__ void k_counts_to_cells(const int32_t* __restrict__ count, KeyGeo kg, 
     }
 }
 
-constexpr int kMaxRows = 64;      // rows of cells per CTA of k_block_max
+// Rows of cells per CTA of k_block_max: a walk is serial (two barriers and a load per row), and each
+// segment reads three rows more than it closes (64 rows: 57 us on 64^2 cells and 79 on 192^2 x 128; 16
+// rows: 17 and 40).
+constexpr int kMaxRows = 16;
 
 template <int TX, int TY, int KY>
 __global__ void __launch_bounds__(TX * TY) k_block_max(const int32_t* __restrict__ cc, int nx, int ny, int nz,
@@ -264,21 +302,6 @@ static int64_t ncell_blocks(const Ctx& c)
     return (ncell + 255) / 256 > 0 ? (ncell + 255) / 256 : 1;
 }
 
-// Fixed-point range: every int64 node sum is exact while the particles that can reach one node
-// (both species: bounded by the sum of the two species' largest block counts from their last
-// sorts) stay within the limit the context was set up for; beyond it the sticky overflow bit is
-// raised.
-__global__ void k_count_check(unsigned* status, long long limit)
-{
-    if (threadIdx.x == 0 && (long long)status[4] + (long long)status[5] > limit) atomicOr(status, kErrOverflow);
-}
-
-__global__ void k_tile_starts(const int32_t* __restrict__ off, int ntiles, int TT, int32_t* tile_start)
-{
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t <= ntiles) tile_start[t] = off[(size_t)t * TT];
-}
-
 __global__ void k_scatter(SpeciesBuf src, SpeciesBuf dst, int64_t n, KeyGeo kg, int32_t* cursor,
                           const int32_t* __restrict__ tile_start, int lb)
 {
@@ -311,6 +334,21 @@ __global__ void k_scatter(SpeciesBuf src, SpeciesBuf dst, int64_t n, KeyGeo kg, 
     }
 }
 
+// A chunk is a layout block (32 x cols records), or the part of one that leaves every SM about 16 warps
+// when particles are few (a walk is serial: 22 us for 16384 particles in 16 chunks).
+int run_columns(const Ctx& c, const Species& S)
+{
+    int cols = 1 << (layout_log2(c, S) - 5);
+    while (cols > 1 && S.n / (32 * cols) < (int64_t)c.nsm * 16) cols >>= 1;
+    return cols;
+}
+
+int run_grid(const Ctx& c, int64_t n, int cols)
+{
+    const int64_t chunks = (n + 32 * (int64_t)cols - 1) / (32 * (int64_t)cols), g = (chunks + 7) / 8;
+    return (int)(g < 1 ? 1 : (g > (int64_t)c.nsm * 16 ? (int64_t)c.nsm * 16 : g));
+}
+
 // Sort species s: its particles are read from `b` when from_b != 0 (fresh data), else from `a`;
 // the sorted result always ends in `a`.
 void sort_species_impl(Ctx& c, int s, cudaStream_t st, int from_b, int64_t* launches)
@@ -324,17 +362,15 @@ void sort_species_impl(Ctx& c, int s, cudaStream_t st, int from_b, int64_t* laun
     if (g > (int64_t)c.nsm * 16) g = (int64_t)c.nsm * 16;
     if (g < 1) g = 1;
     cudaMemsetAsync(c.keys_count, 0, sizeof(int32_t) * (size_t)(c.nkeys + 1), st);
-    cudaMemsetAsync(c.status + 4 + s, 0, sizeof(unsigned), st);
     SpeciesBuf src = from_b ? S.b : S.a;
     SpeciesBuf dst = from_b ? S.a : S.b;
     if (S.n > 0)
-        k_count<<<(int)g, 256, 0, st>>>(src.cell, S.n, kg, c.keys_count,
-                                        1 << (lb - 5));
+        k_count<<<run_grid(c, S.n, run_columns(c, S)), 256, 0, st>>>(src.cell, S.n, kg, c.keys_count, run_columns(c, S));
     const int nb = (c.nkeys + kScanItems - 1) / kScanItems;
     // the most particles of this species in one block of 4 cells per axis (counts are consumed
     // below; the key offsets, written by the scan after it, hold the counts in cell order meanwhile)
     k_counts_to_cells<<<(int)(ncell_blocks(c) < (int64_t)c.nsm * 16 ? ncell_blocks(c) : (int64_t)c.nsm * 16), 256, 0,
-                        st>>>(c.keys_count, kg, c.nz, c.keys_off);
+                        st>>>(c.keys_count, kg, c.nz, c.keys_off, c.status + 4 + s);
     const unsigned zs = (unsigned)((c.nz + kMaxRows - 1) / kMaxRows);
     if (c.dims == 3)
         k_block_max<32, 8, 4><<<dim3((unsigned)((c.nx + 31) / 32), (unsigned)((c.ny + 7) / 8), zs), 256, 0, st>>>(
@@ -343,19 +379,20 @@ void sort_species_impl(Ctx& c, int s, cudaStream_t st, int from_b, int64_t* laun
         k_block_max<256, 1, 1><<<dim3((unsigned)((c.nx + 255) / 256), 1u, zs), 256, 0, st>>>(c.keys_off, c.nx, 1, c.nz,
                                                                                            c.status + 4 + s);
     k_scan_block<<<nb, kScanBlock, 0, st>>>(c.keys_count, c.keys_off, c.scan_tmp, c.nkeys);
-    k_scan_sums<<<1, kScanBlock, 0, st>>>(c.scan_tmp, nb);
+    // few block totals: every block of k_scan_add sums those before its own
+    const int scanned = nb > kScanBlock;
+    if (scanned) k_scan_sums<<<1, kScanBlock, 0, st>>>(c.scan_tmp, nb);
     // the cursor reuses the count array (counts are consumed by the scan)
-    k_scan_add<<<(c.nkeys + 255) / 256, 256, 0, st>>>(c.keys_off, c.scan_tmp, c.nkeys, c.keys_count, (int32_t)S.n);
     c.items_ok = 0;
-    k_tile_starts<<<(c.ntiles + 1 + 255) / 256, 256, 0, st>>>(c.keys_off, c.ntiles, TT, S.tile_start);
+    k_scan_add<<<(c.nkeys + 255) / 256, 256, 0, st>>>(c.keys_off, c.scan_tmp, scanned, c.nkeys, c.keys_count, (int32_t)S.n,
+                                                     TT, S.tile_start, c.status, c.count_limit);
     if (S.n > 0) k_scatter<<<(int)g, 256, 0, st>>>(src, dst, S.n, kg, c.keys_count, S.tile_start, lb);
-    k_count_check<<<1, 32, 0, st>>>(c.status, c.count_limit);
     if (!from_b) {
         SpeciesBuf t = S.a;
         S.a = S.b;
         S.b = t;
     }
-    if (launches) *launches += 7 + (S.n > 0 ? 2 : 0);
+    if (launches) *launches += 4 + scanned + (S.n > 0 ? 2 : 0);
 }
 
 void launch_sort_species(Ctx& c, int s, cudaStream_t st, int64_t* launches)
