@@ -10,16 +10,29 @@
 
 namespace gbpic {
 
-__global__ void k_crater_profile(const u64* __restrict__ rho0, const u64* __restrict__ rho, int64_t ncol,
-                                 int rows, double depth_scale, double* __restrict__ out)
+// 32 columns per block (a warp reads 32 neighbouring nodes of a row); the block's warps take every 16th
+// row and their integer sums meet in shared memory. One thread per column, walking all rows, was one chain
+// of dependent loads: 139 us for 1024 columns of 513 rows, 12 us now.
+constexpr int kProfileWarps = 16;
+__global__ void __launch_bounds__(32 * kProfileWarps)
+    k_crater_profile(const u64* __restrict__ rho0, const u64* __restrict__ rho, int64_t ncol, int rows, double depth_scale,
+                     double* __restrict__ out)
 {
-    for (int64_t col = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; col < ncol;
-         col += (int64_t)gridDim.x * blockDim.x) {
-        long long s = 0;
-        for (int k = 0; k < rows; k++) {
+    __shared__ long long sh[kProfileWarps][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t col = blockIdx.x * (int64_t)32 + lane;
+    long long s = 0;
+    if (col < ncol) {
+#pragma unroll 4
+        for (int k = w; k < rows; k += kProfileWarps) {
             const size_t q = (size_t)k * (size_t)ncol + (size_t)col;
             s += (long long)(__ldg(rho0 + q) - __ldg(rho + q));
         }
+    }
+    sh[w][lane] = s;
+    __syncthreads();
+    if (w == 0 && col < ncol) {
+        for (int q = 1; q < kProfileWarps; q++) s += sh[q][lane];
         out[col] = (double)s * depth_scale;
     }
 }
@@ -28,9 +41,8 @@ void launch_crater_profile(Ctx& c, const u64* rho0, double depth_scale, double* 
 {
     const int64_t ncol = (int64_t)c.nx * c.ny;
     const int rows = c.cfg.slab_k + 1 < c.nz + 1 ? c.cfg.slab_k + 1 : c.nz + 1;
-    int64_t g = (ncol + 255) / 256;
-    if (g > (int64_t)c.nsm * 8) g = (int64_t)c.nsm * 8;
-    k_crater_profile<<<(int)g, 256, 0, st>>>(rho0, c.rho[c.cur], ncol, rows, depth_scale, out);
+    k_crater_profile<<<(unsigned)((ncol + 31) / 32), 32 * kProfileWarps, 0, st>>>(rho0, c.rho[c.cur], ncol, rows,
+                                                                                  depth_scale, out);
 }
 
 }  // namespace gbpic

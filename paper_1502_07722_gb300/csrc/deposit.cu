@@ -5,20 +5,58 @@
 
 namespace gbpic {
 
-__global__ void k_deposit_density(const int32_t* __restrict__ cell, const float* __restrict__ fx,
-                                  const float* __restrict__ fz, int64_t n, int nx, int nz, u64* out)
+// A warp takes chunks of 32 x cols records; lane l walks records l, l + 32, ... of its chunk. The sort
+// stores a block of the cell order as a 32-row matrix column by column, so these are consecutive
+// particles of the cell order (between sorts they have barely moved): the lane sums a run of particles of one
+// cell in registers and issues the four corner reductions once per run (any order stays exact; only
+// the runs get shorter). One set of reductions per particle was bound by them: 128 us for 16.8 M ions on
+// 1024^2 cells, 36 us now.
+__global__ void __launch_bounds__(256) k_deposit_density(const int32_t* __restrict__ cell, const float* __restrict__ fx,
+                                                         const float* __restrict__ fz, int64_t n, int nx, unsigned magic,
+                                                         int shift, int cols, u64* out)
 {
-    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x) {
-        const int c = cell[p];
-        const int k = c / nx, i = c - k * nx;
-        const int qx = qoff(fx[p]), qz = qoff(fz[p]);
-        const int i1 = i + 1 == nx ? 0 : i + 1;
-        const long long sx0 = kQOne - qx, sx1 = qx, sz0 = kQOne - qz, sz1 = qz;
-        const size_t r0 = (size_t)k * nx, r1 = r0 + nx;
-        if (sx0 * sz0) atomicAdd(out + r0 + i, (u64)(sx0 * sz0));
-        if (sx1 * sz0) atomicAdd(out + r0 + i1, (u64)(sx1 * sz0));
-        if (sx0 * sz1) atomicAdd(out + r1 + i, (u64)(sx0 * sz1));
-        if (sx1 * sz1) atomicAdd(out + r1 + i1, (u64)(sx1 * sz1));
+    const int lane = threadIdx.x & 31;
+    const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5, nwarp = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int64_t chunk = 32 * (int64_t)cols;
+    for (int64_t base = warp * chunk; base < n; base += nwarp * chunk) {
+        int at = -1;
+        u64 s00 = 0, s10 = 0, s01 = 0, s11 = 0;
+        auto flush = [&]() {
+            const int k = (int)(__umulhi((unsigned)at, magic) >> shift), i = at - k * nx;
+            u64* r = out + at;
+            const int d1 = i + 1 == nx ? 1 - nx : 1;
+            if (s00) atomicAdd(r, s00);
+            if (s10) atomicAdd(r + d1, s10);
+            if (s01) atomicAdd(r + nx, s01);
+            if (s11) atomicAdd(r + nx + d1, s11);
+            s00 = s10 = s01 = s11 = 0;
+        };
+        for (int q0 = 0; q0 < cols; q0 += kRunBatch) {
+            int c[kRunBatch];
+            float ox[kRunBatch], oz[kRunBatch];
+#pragma unroll
+            for (int q = 0; q < kRunBatch; q++) {
+                const int64_t p = base + 32 * (int64_t)(q0 + q) + lane;
+                const bool in = q0 + q < cols && p < n;
+                c[q] = in ? cell[p] : -1;
+                ox[q] = in ? fx[p] : 0.0f;
+                oz[q] = in ? fz[p] : 0.0f;
+            }
+#pragma unroll
+            for (int q = 0; q < kRunBatch; q++) {
+                if (c[q] < 0) continue;
+                if (c[q] != at) {
+                    if (at >= 0) flush();
+                    at = c[q];
+                }
+                const unsigned x = (unsigned)qoff(ox[q]), z = (unsigned)qoff(oz[q]), ax = kQOne - x, az = kQOne - z;
+                s00 += (u64)ax * az;
+                s10 += (u64)x * az;
+                s01 += (u64)ax * z;
+                s11 += (u64)x * z;
+            }
+        }
+        if (at >= 0) flush();
     }
 }
 
@@ -92,7 +130,12 @@ void launch_deposit_density(Ctx& c, u64* out, cudaStream_t st)
     cudaMemsetAsync(out, 0, sizeof(u64) * c.nn, st);
     const Species& S = c.sp[0];
     if (S.n == 0) return;
-    k_deposit_density<<<grid_for(c, S.n), 256, 0, st>>>(S.a.cell, S.a.fx, S.a.fz, S.n, c.nx, c.nz, out);
+    unsigned magic;
+    int shift;
+    magic_div(c.nx, magic, shift);
+    const int cols = run_columns(c, S);
+    k_deposit_density<<<run_grid(c, S.n, cols), 256, 0, st>>>(S.a.cell, S.a.fx, S.a.fz, S.n, c.nx, magic, shift, cols,
+                                                              out);
 }
 
 void launch_validate(Ctx& c, const SpeciesBuf& b, int64_t n, unsigned* bad, cudaStream_t st)

@@ -7,23 +7,25 @@
 namespace gbpic {
 
 constexpr int kEBlock = 256;
+constexpr int kBatch = 4;   // particles of a thread whose loads are in flight together
 constexpr int kSlots = 5;   // 0 KE ions, 1 KE electrons, 2 field E, 3 field B, 4 pair
 
+// a fixed-shape tree: lanes of a warp, then the warps (the result in every thread)
 __device__ __forceinline__ double block_sum(double v, double* sh)
 {
-    sh[threadIdx.x] = v;
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
     __syncthreads();
-    for (int s = kEBlock / 2; s > 0; s >>= 1) {
-        if ((int)threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
-        __syncthreads();
-    }
-    const double r = sh[0];
+    double r = sh[0];
+    for (int w = 1; w < kEBlock / 32; w++) r += sh[w];
     __syncthreads();
     return r;
 }
 
 struct EnergyArgs {
     int nx, nz, nsp;
+    unsigned nx_magic;
+    int nx_shift;
     SpeciesBuf sp[2];
     int64_t n[2];
     const float* F[6];
@@ -34,30 +36,53 @@ struct EnergyArgs {
     double* partials;   // gridDim.x * kSlots
 };
 
+// LJ: Eq. (3) on the cubic lattice compiled in (the run-time potential code costs the other forms' branches).
+template <bool LJ>
 __global__ void __launch_bounds__(kEBlock) k_energy(const EnergyArgs a)
 {
-    __shared__ double sh[kEBlock];
+    __shared__ double sh[kEBlock / 32];
     const int64_t tid = blockIdx.x * (int64_t)kEBlock + threadIdx.x;
     const int64_t stride = (int64_t)gridDim.x * kEBlock;
-    double ke[2] = {0.0, 0.0}, pe = 0.0, fe = 0.0, fb = 0.0;
+    Sum2 ke[2], pe;
+    double fe = 0.0, fb = 0.0;
 #pragma unroll
     for (int s = 0; s < 2; s++) {
         if (s >= a.nsp) break;
         const SpeciesBuf& S = a.sp[s];
-        for (int64_t p = tid; p < a.n[s]; p += stride) {
-            const float ux = S.ux[p], uy = S.uy[p], uz = S.uz[p];
-            const float u2 = ux * ux + uy * uy + uz * uz;
-            ke[s] += (double)(u2 / (sqrtf(1.0f + u2) + 1.0f));
+        for (int64_t p0 = tid; p0 < a.n[s]; p0 += kBatch * stride) {
+            float ux[kBatch], uy[kBatch], uz[kBatch], fx[kBatch], fz[kBatch];
+            int cell[kBatch];
+#pragma unroll
+            for (int q = 0; q < kBatch; q++) {
+                const int64_t p = p0 + q * stride;
+                const bool in = p < a.n[s];
+                cell[q] = in ? S.cell[p] : -1;
+                ux[q] = in ? S.ux[p] : 0.0f;
+                uy[q] = in ? S.uy[p] : 0.0f;
+                uz[q] = in ? S.uz[p] : 0.0f;
+                if (s == 0) {
+                    fx[q] = in ? S.fx[p] : 0.0f;
+                    fz[q] = in ? S.fz[p] : 0.0f;
+                }
+            }
+            float n[kBatch], dnx[kBatch], dnz[kBatch];
             if (s == 0) {
-                const int c = S.cell[p];
-                const int k = c / a.nx, i = c - k * a.nx;
-                float n, dnx, dnz;
-                gather_density(a.rho, a.nx, a.nz, a.rho_s, i, k, S.fx[p], S.fz[p], n, dnx, dnz);
-                if (n > 0.0f) {
-                    const float cr = fast_cbrt(n);
-                    const float inv43 = fast_rcp(n * cr);
-                    float e = pair_energy_xz(cr, inv43, dnx, dnz, a.h_coef, a.pot_mode, a.c_att, a.s_rep, a.eam);
-                    pe += (double)e;
+#pragma unroll
+                for (int q = 0; q < kBatch; q++) {
+                    const int c = cell[q] < 0 ? 0 : cell[q];
+                    const int k = (int)(__umulhi((unsigned)c, a.nx_magic) >> a.nx_shift), i = c - k * a.nx;
+                    gather_density(a.rho, a.nx, a.nz, a.rho_s, i, k, fx[q], fz[q], n[q], dnx[q], dnz[q]);
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < kBatch; q++) {
+                if (cell[q] < 0) continue;
+                const float u2 = ux[q] * ux[q] + uy[q] * uy[q] + uz[q] * uz[q];
+                ke[s].add(u2 / (sqrtf(1.0f + u2) + 1.0f));
+                if (s == 0 && n[q] > 0.0f) {
+                    const float cr = fast_cbrt(n[q]);
+                    const float inv43 = fast_rcp(n[q] * cr);
+                    pe.add(pair_energy_xz(cr, inv43, dnx[q], dnz[q], a.h_coef, LJ ? 0 : a.pot_mode, a.c_att, a.s_rep, a.eam));
                 }
             }
         }
@@ -75,8 +100,8 @@ __global__ void __launch_bounds__(kEBlock) k_energy(const EnergyArgs a)
             fb += bx * bx + by * by;
         }
     }
-    const double r0 = block_sum(ke[0], sh), r1 = block_sum(ke[1], sh), r2 = block_sum(fe, sh),
-                 r3 = block_sum(fb, sh), r4 = block_sum(pe, sh);
+    const double r0 = block_sum(ke[0].value(), sh), r1 = block_sum(ke[1].value(), sh), r2 = block_sum(fe, sh),
+                 r3 = block_sum(fb, sh), r4 = block_sum(pe.value(), sh);
     if (threadIdx.x == 0) {
         double* o = a.partials + (size_t)blockIdx.x * kSlots;
         o[0] = r0; o[1] = r1; o[2] = r2; o[3] = r3; o[4] = r4;
@@ -85,7 +110,7 @@ __global__ void __launch_bounds__(kEBlock) k_energy(const EnergyArgs a)
 
 __global__ void k_energy_final(const double* __restrict__ partials, int nb, double* out)
 {
-    __shared__ double sh[kEBlock];
+    __shared__ double sh[kEBlock / 32];
     for (int s = 0; s < kSlots; s++) {
         double v = 0.0;
         // fixed assignment of blocks to threads, then a fixed-shape tree
@@ -95,6 +120,14 @@ __global__ void k_energy_final(const double* __restrict__ partials, int nb, doub
     }
 }
 
+// Sums of FP32 terms by two-sum and the FP64 conversions kept off the common way: 482 -> 277 us for the
+// 33.5 M particles and 1 M nodes of the 1024^2 slab (8 FP64-pipe instructions per particle were its bound).
+static void run_energy(const EnergyArgs& a, int nb, cudaStream_t st)
+{
+    if (a.pot_mode == 0) k_energy<true><<<nb, kEBlock, 0, st>>>(a);
+    else k_energy<false><<<nb, kEBlock, 0, st>>>(a);
+}
+
 int energy_blocks(const Ctx& c) { return c.nsm * 4; }
 
 void launch_energy(Ctx& c, cudaStream_t st, double* host_out5)
@@ -102,6 +135,7 @@ void launch_energy(Ctx& c, cudaStream_t st, double* host_out5)
     EnergyArgs a;
     a.nx = c.nx;
     a.nz = c.nz;
+    magic_div(c.nx, a.nx_magic, a.nx_shift);
     a.nsp = c.nsp;
     for (int s = 0; s < 2; s++) {
         a.sp[s] = c.sp[s].a;
@@ -117,7 +151,7 @@ void launch_energy(Ctx& c, cudaStream_t st, double* host_out5)
     a.eam = eam_params(c.cfg);
     a.partials = c.partials;
     const int nb = energy_blocks(c);
-    k_energy<<<nb, kEBlock, 0, st>>>(a);
+    run_energy(a, nb, st);
     k_energy_final<<<1, kEBlock, 0, st>>>(c.partials, nb, c.red_out);
     double raw[kSlots];
     cudaMemcpyAsync(raw, c.red_out, sizeof(raw), cudaMemcpyDeviceToHost, st);
@@ -153,7 +187,7 @@ static __device__ __align__(256) double g_noalloc_scratch[kStaticBlocks * kSlots
 __global__ void k_energy_final_scaled(const double* __restrict__ partials, int nb, double s0, double s1, double s2,
                                       double s3, double s4, double* out)
 {
-    __shared__ double sh[kEBlock];
+    __shared__ double sh[kEBlock / 32];
     const double scale[kSlots] = {s0, s1, s2, s3, s4};
     for (int s = 0; s < kSlots; s++) {
         double v = 0.0;
@@ -233,6 +267,7 @@ extern "C" int pic_energy_noalloc(const pic_config* cfg, const pic_state_view* i
     EnergyArgs a;
     a.nx = cfg->nx;
     a.nz = cfg->nz;
+    magic_div(cfg->nx, a.nx_magic, a.nx_shift);
     a.nsp = nsp;
     for (int s = 0; s < 2; s++) {
         const bool on = s < nsp;
@@ -256,7 +291,7 @@ extern "C" int pic_energy_noalloc(const pic_config* cfg, const pic_state_view* i
     const cudaStream_t st = (cudaStream_t)stream;
     const double vol = cfg->dx * cfg->dx;
     const double mu0 = 1.0 / (kEps0 * kC * kC);
-    k_energy<<<nb, kEBlock, 0, st>>>(a);
+    run_energy(a, nb, st);
     k_energy_final_scaled<<<1, kEBlock, 0, st>>>(scratch, nb, w * mi * kC * kC, nsp > 1 ? w * kMe * kC * kC : 0.0,
                                                   0.5 * kEps0 * vol, 0.5 / mu0 * vol, 0.5 * D * w, dev_out5);
     return cudaGetLastError() == cudaSuccess ? PIC_OK : PIC_ECUDA;

@@ -107,7 +107,7 @@ __device__ __forceinline__ void density3(const u64* __restrict__ rho, const Geo3
             for (int a = 0; a < 2; a++) {
                 long long r = (long long)__ldg(rho + idx3(g, a ? i1 : i, b ? j1 : j, k + c));
                 if (k + c == 0 || k + c == g.nz) r *= 2;
-                v[c * 4 + b * 2 + a] = rho_s * (float)r;
+                v[c * 4 + b * 2 + a] = rho_s * i64_f32(r);
             }
     const float gx = 1.0f - fx, gy = 1.0f - fy, gz = 1.0f - fz;
     // along x: differences of the x-pairs weighted in y and z
@@ -681,19 +681,61 @@ void launch_particle_step3(Ctx& c, cudaStream_t st)
 
 // ---- stand-alone node density and pair force ------------------------------------------------
 
-__global__ void k_deposit_density3(const int32_t* __restrict__ cell, const float* __restrict__ fx,
-                                   const float* __restrict__ fy, const float* __restrict__ fz, int64_t n, Geo3 g,
-                                   u64* out)
+// as k_deposit_density (deposit.cu): a lane walks runs of particles of one cell and issues the eight corner
+// reductions once per run
+__global__ void __launch_bounds__(256) k_deposit_density3(const int32_t* __restrict__ cell, const float* __restrict__ fx,
+                                                          const float* __restrict__ fy, const float* __restrict__ fz,
+                                                          int64_t n, Geo3 g, int cols, u64* out)
 {
-    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x) {
-        int i, j, k;
-        split3(cell[p], g, i, j, k);
-        const long long x = qoff3(fx[p]), y = qoff3(fy[p]), z = qoff3(fz[p]);
-        const long long sx[2] = {kQ3 - x, x}, sy[2] = {kQ3 - y, y}, sz[2] = {kQ3 - z, z};
-        const int i1 = wrapn(i + 1, g.nx), j1 = wrapn(j + 1, g.ny);
-        for (int c = 0; c < 2; c++)
-            for (int b = 0; b < 2; b++)
-                for (int q = 0; q < 2; q++) red64(out + idx3(g, q ? i1 : i, b ? j1 : j, k + c), sx[q] * sy[b] * sz[c]);
+    const int lane = threadIdx.x & 31;
+    const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5, nwarp = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int64_t chunk = 32 * (int64_t)cols;
+    for (int64_t base = warp * chunk; base < n; base += nwarp * chunk) {
+        int at = -1;
+        u64 s[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+        auto flush = [&]() {
+            int i, j, k;
+            split3(at, g, i, j, k);
+            const int i1 = wrapn(i + 1, g.nx), j1 = wrapn(j + 1, g.ny);
+#pragma unroll
+            for (int c = 0; c < 8; c++) {
+                if (s[c]) atomicAdd(out + idx3(g, c & 1 ? i1 : i, c & 2 ? j1 : j, k + (c >> 2)), s[c]);
+                s[c] = 0;
+            }
+        };
+        for (int q0 = 0; q0 < cols; q0 += kRunBatch) {
+            int c[kRunBatch];
+            float ox[kRunBatch], oy[kRunBatch], oz[kRunBatch];
+#pragma unroll
+            for (int q = 0; q < kRunBatch; q++) {
+                const int64_t p = base + 32 * (int64_t)(q0 + q) + lane;
+                const bool in = q0 + q < cols && p < n;
+                c[q] = in ? cell[p] : -1;
+                ox[q] = in ? fx[p] : 0.0f;
+                oy[q] = in ? fy[p] : 0.0f;
+                oz[q] = in ? fz[p] : 0.0f;
+            }
+#pragma unroll
+            for (int q = 0; q < kRunBatch; q++) {
+                if (c[q] < 0) continue;
+                if (c[q] != at) {
+                    if (at >= 0) flush();
+                    at = c[q];
+                }
+                const unsigned x = (unsigned)qoff3(ox[q]), y = (unsigned)qoff3(oy[q]), z = (unsigned)qoff3(oz[q]);
+                const unsigned ax = kQ3 - x, ay = kQ3 - y, az = kQ3 - z;
+                const unsigned w00 = ax * ay, w10 = x * ay, w01 = ax * y, w11 = x * y;       // at most 2^28
+                s[0] += (u64)w00 * az;
+                s[1] += (u64)w10 * az;
+                s[2] += (u64)w01 * az;
+                s[3] += (u64)w11 * az;
+                s[4] += (u64)w00 * z;
+                s[5] += (u64)w10 * z;
+                s[6] += (u64)w01 * z;
+                s[7] += (u64)w11 * z;
+            }
+        }
+        if (at >= 0) flush();
     }
 }
 
@@ -732,7 +774,9 @@ void launch_deposit_density3(Ctx& c, u64* out, cudaStream_t st)
     cudaMemsetAsync(out, 0, sizeof(u64) * c.nn, st);
     const Species& S = c.sp[0];
     if (S.n == 0) return;
-    k_deposit_density3<<<grid3(c, S.n), 256, 0, st>>>(S.a.cell, S.a.fx, S.a.fy, S.a.fz, S.n, geo_of(c), out);
+    const int cols = run_columns(c, S);
+    k_deposit_density3<<<run_grid(c, S.n, cols), 256, 0, st>>>(S.a.cell, S.a.fx, S.a.fy, S.a.fz, S.n, geo_of(c), cols,
+                                                               out);
 }
 
 void launch_pair_force3(Ctx& c, float* out, cudaStream_t st)
@@ -937,32 +981,68 @@ void launch_fields3(Ctx& c, cudaStream_t st, int64_t step, int64_t* launches)
 
 // ---- energies ------------------------------------------------------------------------------
 
+// a fixed-shape tree over 256 threads: lanes of a warp, then the warps
+__device__ __forceinline__ double block_sum3(double v, double* sh)
+{
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+    __syncthreads();
+    double r = sh[0];
+    for (int w = 1; w < 8; w++) r += sh[w];
+    __syncthreads();
+    return r;
+}
+
 __global__ void __launch_bounds__(256) k_energy3(const Species3 s0, const Species3 s1, int64_t n0, int64_t n1, int nsp, Geo3 g,
                                                  const float* F0, const float* F1, const float* F2, const float* F3,
                                                  const float* F4, const float* F5, const u64* rho, float rho_s,
                                                  float h_coef, int pot_mode, float c_att, float s_rep, EamP eam,
                                                  double* partials)
 {
-    __shared__ double sh[256];
+    __shared__ double sh[8];
     const int64_t tid = blockIdx.x * (int64_t)256 + threadIdx.x, stride = (int64_t)gridDim.x * 256;
-    double ke[2] = {0.0, 0.0}, pe = 0.0, fe = 0.0, fb = 0.0;
+    Sum2 ke[2], pe;
+    double fe = 0.0, fb = 0.0;
     for (int s = 0; s < nsp; s++) {
         const Species3& S = s == 0 ? s0 : s1;
         const int64_t ns = s == 0 ? n0 : n1;
-        for (int64_t p = tid; p < ns; p += stride) {
-            const float ux = S.ux[p], uy = S.uy[p], uz = S.uz[p];
-            const float u2 = ux * ux + uy * uy + uz * uz;
-            ke[s] += (double)(u2 / (sqrtf(1.0f + u2) + 1.0f));
+        for (int64_t p0 = tid; p0 < ns; p0 += 2 * stride) {
+            // two particles' loads in flight together
+            float ux[2], uy[2], uz[2], fx[2], fy[2], fz[2];
+            int cell[2];
+#pragma unroll
+            for (int q = 0; q < 2; q++) {
+                const int64_t p = p0 + q * stride;
+                const bool in = p < ns;
+                cell[q] = in ? S.cell[p] : -1;
+                ux[q] = in ? S.ux[p] : 0.0f;
+                uy[q] = in ? S.uy[p] : 0.0f;
+                uz[q] = in ? S.uz[p] : 0.0f;
+                if (s == 0) {
+                    fx[q] = in ? S.fx[p] : 0.0f;
+                    fy[q] = in ? S.fy[p] : 0.0f;
+                    fz[q] = in ? S.fz[p] : 0.0f;
+                }
+            }
+            float dens[2], gr[2][3];
             if (s == 0) {
-                int i, j, k;
-                split3(S.cell[p], g, i, j, k);
-                float dens, gr[3];
-                density3(rho, g, rho_s, i, j, k, S.fx[p], S.fy[p], S.fz[p], dens, gr);
-                if (dens > 0.0f) {
-                    const float cr = fast_cbrt(dens), inv43 = fast_rcp(dens * cr);
-                    float e = 0.0f;
-                    e += pair_energy3(cr, inv43, gr, h_coef, pot_mode, c_att, s_rep, eam);
-                    pe += (double)e;
+#pragma unroll
+                for (int q = 0; q < 2; q++) {
+                    int i, j, k;
+                    split3(cell[q] < 0 ? 0 : cell[q], g, i, j, k);
+                    density3(rho, g, rho_s, i, j, k, fx[q], fy[q], fz[q], dens[q], gr[q]);
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < 2; q++) {
+                if (cell[q] < 0) continue;
+                const float u2 = ux[q] * ux[q] + uy[q] * uy[q] + uz[q] * uz[q];
+                const float t = u2 / (sqrtf(1.0f + u2) + 1.0f);
+                if (s == 0) ke[0].add(t);
+                else ke[1].add(t);
+                if (s == 0 && dens[q] > 0.0f) {
+                    const float cr = fast_cbrt(dens[q]), inv43 = fast_rcp(dens[q] * cr);
+                    pe.add(pair_energy3(cr, inv43, gr[q], h_coef, pot_mode, c_att, s_rep, eam));
                 }
             }
         }
@@ -980,33 +1060,22 @@ __global__ void __launch_bounds__(256) k_energy3(const Species3 s0, const Specie
             fb += bx * bx + by * by;
         }
     }
-    double vals[5] = {ke[0], ke[1], fe, fb, pe};
+    const double vals[5] = {ke[0].value(), ke[1].value(), fe, fb, pe.value()};
+#pragma unroll
     for (int q = 0; q < 5; q++) {
-        sh[threadIdx.x] = vals[q];
-        __syncthreads();
-        for (int w = 128; w > 0; w >>= 1) {
-            if ((int)threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) partials[(size_t)blockIdx.x * 5 + q] = sh[0];
-        __syncthreads();
+        const double r = block_sum3(vals[q], sh);
+        if (threadIdx.x == 0) partials[(size_t)blockIdx.x * 5 + q] = r;
     }
 }
 
 __global__ void k_energy3_final(const double* __restrict__ partials, int nb, double* out)
 {
-    __shared__ double sh[256];
+    __shared__ double sh[8];
     for (int q = 0; q < 5; q++) {
         double v = 0.0;
         for (int b = threadIdx.x; b < nb; b += 256) v += partials[(size_t)b * 5 + q];
-        sh[threadIdx.x] = v;
-        __syncthreads();
-        for (int w = 128; w > 0; w >>= 1) {
-            if ((int)threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) out[q] = sh[0];
-        __syncthreads();
+        const double r = block_sum3(v, sh);
+        if (threadIdx.x == 0) out[q] = r;
     }
 }
 

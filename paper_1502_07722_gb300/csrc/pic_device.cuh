@@ -8,6 +8,37 @@ namespace gbpic {
 
 __device__ __forceinline__ int wrap_x(int i, int nx) { return i < 0 ? i + nx : (i >= nx ? i - nx : i); }
 
+// Correctly rounded int64 -> FP32. The conversion instruction runs on the FP64 pipe (2 lanes per SM and
+// clock); below 2^48 both halves of a split at 24 bits are exact in FP32 and one FMA rounds their sum,
+// which is the same result. (The rare ways here are calls: written inline the compiler executes them
+// for every value, predicated, and they occupy the FP64 pipe all the same.)
+static __device__ __noinline__ float i64_f32_wide(long long v) { return (float)v; }
+__device__ __forceinline__ float i64_f32(long long v)
+{
+    if ((u64)(v + (1LL << 48)) >> 49) return i64_f32_wide(v);
+    return __fmaf_rn((float)(int)(v >> 24), 16777216.0f, (float)((int)v & 0xffffff));
+}
+
+// Sum of FP32 terms with its rounding errors carried along (Knuth's two-sum): about 48 bits. The FP64
+// adds and conversions it replaces in the energy reductions were those kernels' bound. Terms so large
+// that an FP32 sum could overflow (or infinite, or NaN) are added in FP64.
+static __device__ __noinline__ double add_wide(double s, float x) { return s + (double)x; }
+struct Sum2 {
+    float s = 0.0f, c = 0.0f;
+    double big = 0.0;
+    __device__ __forceinline__ void add(float x)
+    {
+        if (!(fabsf(x) < 1e30f)) {
+            big = add_wide(big, x);
+            return;
+        }
+        const float t = __fadd_rn(s, x), b = __fsub_rn(t, s);
+        c = __fadd_rn(c, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(x, b)));
+        s = t;
+    }
+    __device__ __forceinline__ double value() const { return ((double)s + (double)c) + big; }
+};
+
 // Pair-species node sum with the wall rows doubled (mirror image of the slab behind a wall).
 __device__ __forceinline__ long long rho_node(const u64* __restrict__ rho, int nx, int nz, int i, int k)
 {
@@ -27,10 +58,10 @@ __device__ __forceinline__ void gather_density(const u64* __restrict__ rho, int 
     long long r00 = rho_node(rho, nx, nz, i, k), r10 = rho_node(rho, nx, nz, i1, k);
     long long r01 = rho_node(rho, nx, nz, i, k + 1), r11 = rho_node(rho, nx, nz, i1, k + 1);
     float gx = 1.0f - fx, gz = 1.0f - fz;
-    float a00 = (float)r00, a10 = (float)r10, a01 = (float)r01, a11 = (float)r11;
+    float a00 = i64_f32(r00), a10 = i64_f32(r10), a01 = i64_f32(r01), a11 = i64_f32(r11);
     n = rho_s * (gz * (gx * a00 + fx * a10) + fz * (gx * a01 + fx * a11));
-    dnx = rho_s * (gz * (float)(r10 - r00) + fz * (float)(r11 - r01));
-    dnz = rho_s * (gx * (float)(r01 - r00) + fx * (float)(r11 - r10));
+    dnx = rho_s * (gz * i64_f32(r10 - r00) + fz * i64_f32(r11 - r01));
+    dnz = rho_s * (gx * i64_f32(r01 - r00) + fx * i64_f32(r11 - r10));
 }
 
 // Lennard-Jones derivative U'(r) (units D/r0) from inv = r0 / r.

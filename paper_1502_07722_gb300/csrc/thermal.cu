@@ -2,7 +2,7 @@
 // the laser-interaction run leaves once electrons and lattice have equilibrated).
 //  * Lattice temperature per cell of one species: T = m c^2 / (3 k_B) sum |u - mean u|^2 / (N - 1)
 //    over the N particles of the cell (the thermal spread about the cell's mean flow); cells with
-//    fewer than two particles get 0. Per-cell sums in FP64 (atomics), then one thread per cell.
+//    fewer than two particles get 0. Per-cell sums (FP64 atomics), then one thread per cell.
 //  * Re-tempering to a map: momenta drawn at the uniform temperature T_from become the same draws
 //    at the temperature of their cell, u -> u sqrt(T_cell / T_from).
 //  * Regridding a cell map between stages of different cells: a conservative (volume-weighted)
@@ -11,19 +11,129 @@
 
 namespace gbpic {
 
-__global__ void k_cell_moments(const int32_t* __restrict__ cell, const float* __restrict__ ux,
-                               const float* __restrict__ uy, const float* __restrict__ uz, int64_t n, int64_t ncell,
-                               double* __restrict__ acc)
-{
-    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t q = cell[p];
-        const double a = ux[p], b = uy[p], c = uz[p];
-        atomicAdd(acc + q, 1.0);
-        atomicAdd(acc + ncell + q, a);
-        atomicAdd(acc + 2 * ncell + q, b);
-        atomicAdd(acc + 3 * ncell + q, c);
-        atomicAdd(acc + 4 * ncell + q, a * a + b * b + c * c);
+// Exact enough to replace FP64: a sum of FP32 terms as three FP32 numbers, every rounding error carried to
+// the next (Knuth's two-sum), about 70 bits.
+struct Sum3 {
+    float s0, s1, s2;
+    __device__ __forceinline__ void zero() { s0 = s1 = s2 = 0.0f; }
+    __device__ __forceinline__ static float two_sum(float& s, float x)
+    {
+        const float t = __fadd_rn(s, x), b = __fsub_rn(t, s);
+        const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(x, b));
+        s = t;
+        return e;
     }
+    __device__ __forceinline__ void add_low(float x) { s2 = __fadd_rn(s2, two_sum(s1, x)); }
+    __device__ __forceinline__ void add(float x) { add_low(two_sum(s0, x)); }
+    __device__ __forceinline__ void add_square(float x)       // x^2 = p + e exactly
+    {
+        const float p = __fmul_rn(x, x);
+        add(p);
+        add_low(__fmaf_rn(x, x, -p));
+    }
+    __device__ __forceinline__ double value() const { return ((double)s2 + (double)s1) + (double)s0; }
+};
+
+// momenta whose squares leave FP32's range (or that are not finite)
+static __device__ __noinline__ void add_wide_moments(double* acc, int64_t ncell, int at, float a, float b, float c)
+{
+    const double da = a, db = b, dc = c;
+    atomicAdd(acc + at, 1.0);
+    atomicAdd(acc + ncell + at, da);
+    atomicAdd(acc + 2 * ncell + at, db);
+    atomicAdd(acc + 3 * ncell + at, dc);
+    atomicAdd(acc + 4 * ncell + at, da * da + db * db + dc * dc);
+}
+
+// Number, sums of u and of u^2 of each cell's particles. Lanes walk runs of particles of one cell
+// (run_columns) and sum them in registers as three FP32 numbers: GB300's FP64 rate is 1/64 of its FP32
+// rate, and the conversions and products of one FP64 reduction per particle took 189 us for 16.8 M
+// particles on 1024^2 cells, 85 to 131 us now. A run that ends goes to the warp's queue; the queue is
+// converted to FP64 and reduced into the cells 32 runs at a time (lanes end their runs at different turns,
+// and an FP64 instruction costs the same for one lane as for 32).
+constexpr int kMomWarps = 4, kMomWords = 14;
+__global__ void __launch_bounds__(32 * kMomWarps)
+    k_cell_moments(const int32_t* __restrict__ cell, const float* __restrict__ ux, const float* __restrict__ uy,
+                   const float* __restrict__ uz, int64_t n, int64_t ncell, int cols, double* __restrict__ acc)
+{
+    __shared__ int queue_all[kMomWarps][kMomWords][64];      // at most 31 left over + 32 new per warp
+    int(*queue)[64] = queue_all[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31;
+    const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5, nwarp = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int64_t chunk = 32 * (int64_t)cols;
+    int at = -1, num = 0, nq = 0;
+    Sum3 v[4];            // u and u^2
+    auto drain = [&](int count) {
+        __syncwarp();
+        nq -= count;
+        if (lane < count) {
+            const int e = nq + lane, c = queue[0][e];
+            atomicAdd(acc + c, (double)queue[1][e]);
+#pragma unroll
+            for (int d = 0; d < 4; d++) {
+                const Sum3 t = {__int_as_float(queue[2 + 3 * d][e]), __int_as_float(queue[3 + 3 * d][e]),
+                                __int_as_float(queue[4 + 3 * d][e])};
+                atomicAdd(acc + (d + 1) * ncell + c, t.value());
+            }
+        }
+        __syncwarp();
+    };
+    // queues the run of every lane with `end` set (all lanes of the warp call it)
+    auto close = [&](bool end) {
+        const unsigned m = __ballot_sync(0xffffffffu, end);
+        if (m == 0) return;
+        if (end) {
+            const int e = nq + __popc(m & ((1u << lane) - 1u));
+            queue[0][e] = at;
+            queue[1][e] = num;
+#pragma unroll
+            for (int d = 0; d < 4; d++) {
+                queue[2 + 3 * d][e] = __float_as_int(v[d].s0);
+                queue[3 + 3 * d][e] = __float_as_int(v[d].s1);
+                queue[4 + 3 * d][e] = __float_as_int(v[d].s2);
+                v[d].zero();
+            }
+            num = 0;
+        }
+        nq += __popc(m);
+        if (nq >= 32) drain(32);
+    };
+    for (int d = 0; d < 4; d++) v[d].zero();
+    for (int64_t base = warp * chunk; base < n; base += nwarp * chunk) {
+        for (int q0 = 0; q0 < cols; q0 += kRunBatch) {
+            int k[kRunBatch];
+            float va[kRunBatch], vb[kRunBatch], vc[kRunBatch];
+#pragma unroll
+            for (int q = 0; q < kRunBatch; q++) {
+                const int64_t p = base + 32 * (int64_t)(q0 + q) + lane;
+                const bool in = q0 + q < cols && p < n;
+                k[q] = in ? cell[p] : -1;
+                va[q] = in ? ux[p] : 0.0f;
+                vb[q] = in ? uy[p] : 0.0f;
+                vc[q] = in ? uz[p] : 0.0f;
+            }
+#pragma unroll
+            for (int q = 0; q < kRunBatch; q++) {
+                close(k[q] >= 0 && k[q] != at && num > 0);
+                if (k[q] < 0) continue;
+                at = k[q];
+                const float a = va[q], b = vb[q], c = vc[q];
+                if (!(fabsf(a) + fabsf(b) + fabsf(c) < 1e15f)) {
+                    add_wide_moments(acc, ncell, at, a, b, c);
+                    continue;
+                }
+                num++;
+                v[0].add(a);
+                v[1].add(b);
+                v[2].add(c);
+                v[3].add_square(a);
+                v[3].add_square(b);
+                v[3].add_square(c);
+            }
+        }
+        close(num > 0);
+    }
+    if (nq > 0) drain(nq);
 }
 
 __global__ void k_cell_temperature(const double* __restrict__ acc, int64_t ncell, double mc2_3k, double* __restrict__ T)
@@ -34,8 +144,8 @@ __global__ void k_cell_temperature(const double* __restrict__ acc, int64_t ncell
             T[q] = 0.0;
             continue;
         }
-        const double mx = acc[ncell + q] / n, my = acc[2 * ncell + q] / n, mz = acc[3 * ncell + q] / n;
-        T[q] = mc2_3k * (acc[4 * ncell + q] - n * (mx * mx + my * my + mz * mz)) / (n - 1.0);
+        const double sx = acc[ncell + q], sy = acc[2 * ncell + q], sz = acc[3 * ncell + q];
+        T[q] = mc2_3k * (acc[4 * ncell + q] - (sx * sx + sy * sy + sz * sz) / n) / (n - 1.0);
     }
 }
 
@@ -62,7 +172,9 @@ void launch_cell_temperature(Ctx& c, int s, double* work, double* T, cudaStream_
     const Species& S = c.sp[s];
     const int64_t ncell = (int64_t)c.nx * c.ny * c.nz;
     cudaMemsetAsync(work, 0, sizeof(double) * 5 * (size_t)ncell, st);
-    if (S.n > 0) k_cell_moments<<<grid_of(c, S.n), 256, 0, st>>>(S.a.cell, S.a.ux, S.a.uy, S.a.uz, S.n, ncell, work);
+    const int cols = run_columns(c, S);
+    if (S.n > 0)
+        k_cell_moments<<<2 * run_grid(c, S.n, cols), 32 * kMomWarps, 0, st>>>(S.a.cell, S.a.ux, S.a.uy, S.a.uz, S.n, ncell, cols, work);
     k_cell_temperature<<<grid_of(c, ncell), 256, 0, st>>>(work, ncell, S.mass * kC * kC / (3.0 * kKb), T);
 }
 
