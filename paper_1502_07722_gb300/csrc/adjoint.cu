@@ -122,12 +122,12 @@ __device__ __forceinline__ DensAt dens_at(const u64* rho, float rho_s, int nx, i
 // transpose of the pair force given the adjoints of (Fx, Fz): position adjoints (added to lx, lz),
 // node adjoints (FP64 atomics), and the D, r0 derivative terms (gFF += lF . F, gR += dL/dr0 part)
 __device__ __forceinline__ void pair_T(const DensAt& d, const PairD& px, const PairD& pz, float lFx, float lFz,
-                                       float inv_r0, int nx, float* lam_nodes, float& lx, float& lz, double& gFF,
-                                       double& gR)
+                                       float inv_r0, int nx, float* lam_nodes, float& lx, float& lz, Sum2& gFF,
+                                       Sum2& gR)
 {
-    gFF += (double)(lFx * px.F + lFz * pz.F);
-    gR += (double)(lFx * (px.dr0 + 3.0f * inv_r0 * (px.dn * d.n + px.dq * d.qx)) +
-                   lFz * (pz.dr0 + 3.0f * inv_r0 * (pz.dn * d.n + pz.dq * d.qz)));
+    gFF.add(lFx * px.F + lFz * pz.F);
+    gR.add(lFx * (px.dr0 + 3.0f * inv_r0 * (px.dn * d.n + px.dq * d.qx)) +
+           lFz * (pz.dr0 + 3.0f * inv_r0 * (pz.dn * d.n + pz.dq * d.qz)));
     const float ln = lFx * px.dn + lFz * pz.dn, lqx = lFx * px.dq, lqz = lFz * pz.dq;
     lx += ln * d.qx + lqz * d.gxz;
     lz += ln * d.qz + lqx * d.gxz;
@@ -187,7 +187,7 @@ struct AdjArgs {
 __global__ void __launch_bounds__(256) k_adjoint_a(const AdjArgs a)
 {
     __shared__ double sh[256];
-    double gFF = 0.0, gR = 0.0;
+    Sum2 gFF, gR;
     const float r0_dx = (float)(a.r0 / a.dx), fu = (float)(a.D / a.r0), inv_r0 = (float)(1.0 / a.r0);
     const float rho_s = (float)a.rho_s, kick = (float)a.kick, cs0 = (float)a.cs0;
     for (int64_t ch = blockIdx.x; ch * 256 < a.n; ch += gridDim.x) {
@@ -220,7 +220,7 @@ __global__ void __launch_bounds__(256) k_adjoint_a(const AdjArgs a)
         a.lam_u[3 * p + 1] = luy;
         a.lam_u[3 * p + 2] = luz;
     }
-    const double sD = block_sum_d(gFF, sh), sR = block_sum_d(gR, sh);
+    const double sD = block_sum_d(gFF.value(), sh), sR = block_sum_d(gR.value(), sh);
     if (threadIdx.x == 0) {
         atomicAdd(a.grads, sD / a.D);
         atomicAdd(a.grads + 1, sR);
@@ -458,6 +458,8 @@ __global__ void __launch_bounds__(256) k_adj_feT(const MaxAdjArgs a)
     }
 }
 
+constexpr int kAdjCtas = 3;
+
 struct FullAdjArgs {
     int nx, nz;
     unsigned nx_magic;
@@ -470,11 +472,10 @@ struct FullAdjArgs {
     float r0_dx, fu, inv_r0;  // r0 / dx, D / r0, 1 / r0
     float eps, fk, tq, cs0;   // q dt / (2 m c), dt / (2 m c), q dt / (2 m), c dt / dx
     float sg;                 // charge sign of the current
-    int pair;
     float cx, cy;             // scaled current per unit Esirkepov sum: x/z and y
     float* lam_pos;
     float* lam_u;
-    float* lF;                // 6 float grids: the particles' scatter onto the field nodes
+    float* lF;                // the particles' scatter onto the field nodes: (Ex, Bz), (Ez, Bx) pairs, Ey, By
     const float* lj;          // 3 grids
     float* lam_nodes;
     double* grads;
@@ -488,41 +489,107 @@ __device__ __forceinline__ float hat_c(float d)
 }
 __device__ __forceinline__ float dhat_c(float d) { return fabsf(d) < 1.0f ? (d > 0.0f ? -1.0f : 1.0f) : 0.0f; }
 
-// staggered bilinear gather of a Yee component at (i + sx, k + sz) for a particle at cell (ci, ck),
-// offsets (fx, fz); with lv != 0 also its transpose (node adjoints, position adjoints)
-__device__ __forceinline__ float gather_stag(const FullAdjArgs& a, int f, int ci, int ck, float fx, float fz, float sx,
-                                             float sz, float lv, float& lx, float& lz)
+// The stencil of a staggered Yee component at (i + sx, k + sz) for a particle at cell (ci, ck), offsets
+// (fx, fz): node offsets from the component's grid and weights.
+struct Stag {
+    int r0, dx, dz;        // first node (row k, column i), to the next column, to the next row
+    float xs, zs;          // weights of the upper column and row
+    bool clamped;          // a half row beyond the grid takes the edge row: no z derivative
+};
+__device__ __forceinline__ Stag stag_at(int nx, int nz, int ci, int ck, float fx, float fz, float sx, float sz)
 {
-    const int nx = a.nx, nz = a.nz;
-    float xs = fx - sx, fzz = fz - sz;
+    Stag t;
+    t.xs = fx - sx;
+    t.zs = fz - sz;
     int i = ci, k = ck;
-    if (xs < 0.0f) { xs += 1.0f; i -= 1; }
-    if (fzz < 0.0f) { fzz += 1.0f; k -= 1; }
+    if (t.xs < 0.0f) { t.xs += 1.0f; i -= 1; }
+    if (t.zs < 0.0f) { t.zs += 1.0f; k -= 1; }
     const int rows = sz > 0.0f ? nz : nz + 1;      // half-row components have nz rows
-    bool clamped = false;
-    if (k < 0) { k = 0; fzz = 0.0f; clamped = true; }
-    else if (k > rows - 1 || (k == rows - 1 && fzz > 0.0f)) { k = rows - 1; fzz = 0.0f; clamped = true; }
-    if (k >= rows - 1) { k = rows - 2; fzz = 1.0f; }
+    t.clamped = false;
+    if (k < 0) { k = 0; t.zs = 0.0f; t.clamped = true; }
+    else if (k > rows - 1 || (k == rows - 1 && t.zs > 0.0f)) { k = rows - 1; t.zs = 0.0f; t.clamped = true; }
+    if (k >= rows - 1) { k = rows - 2; t.zs = 1.0f; }
     const int i0 = i < 0 ? i + nx : i;
-    const int i1 = i0 + 1 == nx ? 0 : i0 + 1;
-    const float* A = a.F[f];
-    const size_t r0 = (size_t)k * nx, r1 = r0 + nx;
-    const float a00 = A[r0 + i0], a10 = A[r0 + i1], a01 = A[r1 + i0], a11 = A[r1 + i1];
-    if (lv != 0.0f) {
-        float* L = a.lF + (size_t)f * (nz + 1) * nx;
-        atomicAdd(L + r0 + i0, lv * (1 - xs) * (1 - fzz));
-        atomicAdd(L + r0 + i1, lv * xs * (1 - fzz));
-        atomicAdd(L + r1 + i0, lv * (1 - xs) * fzz);
-        atomicAdd(L + r1 + i1, lv * xs * fzz);
-        lx += lv * ((1 - fzz) * (a10 - a00) + fzz * (a11 - a01));
-        if (!clamped) lz += lv * ((1 - xs) * (a01 - a00) + xs * (a11 - a10));
-    }
-    return (1 - xs) * (1 - fzz) * a00 + xs * (1 - fzz) * a10 + (1 - xs) * fzz * a01 + xs * fzz * a11;
+    t.r0 = k * nx + i0;
+    t.dx = i0 + 1 == nx ? 1 - nx : 1;
+    t.dz = nx;
+    return t;
+}
+
+// A component's value at the particle and its derivatives along x and z (0 along z where clamped), kept
+// from the forward gather for its transpose: the corners are not loaded a second time.
+struct Gathered {
+    float v, gx, gz;
+};
+__device__ __forceinline__ Gathered gather_at(const float* __restrict__ A, const Stag& t)
+{
+    const float* p = A + t.r0;
+    const float a00 = __ldg(p), a10 = __ldg(p + t.dx), a01 = __ldg(p + t.dz), a11 = __ldg(p + t.dz + t.dx);
+    const float xs = t.xs, zs = t.zs;
+    Gathered g;
+    g.v = (1 - xs) * (1 - zs) * a00 + xs * (1 - zs) * a10 + (1 - xs) * zs * a01 + xs * zs * a11;
+    g.gx = (1 - zs) * (a10 - a00) + zs * (a11 - a01);
+    g.gz = t.clamped ? 0.0f : (1 - xs) * (a01 - a00) + xs * (a11 - a10);
+    return g;
+}
+
+// transpose onto the nodes: one component, or the two that share a stagger side by side in the scatter
+// grids (one 8-byte reduction per corner)
+__device__ __forceinline__ void scatter_at(float* L, const Stag& t, float lv)
+{
+    float* p = L + t.r0;
+    const float xs = t.xs, zs = t.zs;
+    atomicAdd(p, lv * (1 - xs) * (1 - zs));
+    atomicAdd(p + t.dx, lv * xs * (1 - zs));
+    atomicAdd(p + t.dz, lv * (1 - xs) * zs);
+    atomicAdd(p + t.dz + t.dx, lv * xs * zs);
+}
+__device__ __forceinline__ void scatter_at(float2* L, const Stag& t, float la, float lb)
+{
+    float2* p = L + t.r0;
+    const float xs = t.xs, zs = t.zs;
+    const float w00 = (1 - xs) * (1 - zs), w10 = xs * (1 - zs), w01 = (1 - xs) * zs, w11 = xs * zs;
+    atomicAdd(p, make_float2(la * w00, lb * w00));
+    atomicAdd(p + t.dx, make_float2(la * w10, lb * w10));
+    atomicAdd(p + t.dz, make_float2(la * w01, lb * w01));
+    atomicAdd(p + t.dz + t.dx, make_float2(la * w11, lb * w11));
+}
+
+// transpose of the continuous current of a particle that stays inside its cell: only the cell's two x
+// edges, four corners and two z edges carry it,
+//   Lx(b) cx (x1 - x0) (S0z + S1z)_b,  Lz(a) cx (z1 - z0) (S0x + S1x)_a,  Ly(a, b) cy by W_ab,
+// with S_0 = 1 - s, S_1 = s and W = 2 S0xS0z + S1xS0z + S0xS1z + 2 S1xS1z (8 node adjoints instead of the
+// 27 of the general stencil). Adds d/d(x0, z0, x1, z1, by) into g.
+__device__ __forceinline__ void cur_T_cell(const FullAdjArgs& a, int ci, int ck, float x0, float z0, float x1, float z1,
+                                           float by, float g[5])
+{
+    const size_t nn = (size_t)(a.nz + 1) * a.nx;
+    const int dx = ci + 1 == a.nx ? 1 - a.nx : 1, dz = a.nx;
+    const float* L = a.lj + (size_t)ck * a.nx + ci;
+    const float lx0 = __ldg(L), lx1 = __ldg(L + dz);
+    const float *Ly = L + nn, *Lz = Ly + nn;
+    const float y00 = __ldg(Ly), y10 = __ldg(Ly + dx), y01 = __ldg(Ly + dz), y11 = __ldg(Ly + dz + dx);
+    const float lz0 = __ldg(Lz), lz1 = __ldg(Lz + dx);
+    const float cx = a.sg * a.cx, cy = a.sg * a.cy, mx = x1 - x0, mz = z1 - z0;
+    const float X0 = 1 - x0, X1 = 1 - x1, Z0 = 1 - z0, Z1 = 1 - z1;
+    // x edges and z edges
+    const float ax = cx * (lx0 * (Z0 + Z1) + lx1 * (z0 + z1)), bx = cx * mx * (lx1 - lx0);
+    const float az = cx * (lz0 * (X0 + X1) + lz1 * (x0 + x1)), bz = cx * mz * (lz1 - lz0);
+    // corners: (2 S0 + S1, S0 + 2 S1) of the lower and upper node
+    const float Pz0 = 2 * Z0 + Z1, Pz1 = 2 * z0 + z1, Qz0 = Z0 + 2 * Z1, Qz1 = z0 + 2 * z1;
+    const float Px0 = 2 * X0 + X1, Px1 = 2 * x0 + x1, Qx0 = X0 + 2 * X1, Qx1 = x0 + 2 * x1;
+    const float cb = cy * by;
+    g[0] += bz - ax + cb * ((y10 - y00) * Pz0 + (y11 - y01) * Pz1);
+    g[2] += bz + ax + cb * ((y10 - y00) * Qz0 + (y11 - y01) * Qz1);
+    g[1] += bx - az + cb * ((y01 - y00) * Px0 + (y11 - y10) * Px1);
+    g[3] += bx + az + cb * ((y01 - y00) * Qx0 + (y11 - y10) * Qx1);
+    g[4] += cy * (y00 * (X0 * Pz0 + X1 * Qz0) + y10 * (x0 * Pz0 + x1 * Qz0) + y01 * (X0 * Pz1 + X1 * Qz1) +
+                  y11 * (x0 * Pz1 + x1 * Qz1));
 }
 
 // transpose of the continuous Esirkepov current of one particle moving (x0, z0) -> (x1, z1) in
 // coordinates local to its start cell (ci, ck): adds d/d(x0, z0, x1, z1, by) of sum lj * j into g
-__device__ void cur_T(const FullAdjArgs& a, int ci, int ck, float x0, float z0, float x1, float z1, float by,
+static __device__ __noinline__ void cur_T(const FullAdjArgs& a, int ci, int ck, float x0, float z0, float x1, float z1, float by,
                       float g[5])
 {
     const int nx = a.nx, nz = a.nz;
@@ -592,51 +659,17 @@ __device__ void cur_T(const FullAdjArgs& a, int ci, int ck, float x0, float z0, 
     g[4] += gby;
 }
 
-// two fields with the same stagger pattern through one stencil (index, clamping, weights)
-__device__ __forceinline__ void gather_stag2(const FullAdjArgs& a, int fA, int fB, int ci, int ck, float fx, float fz,
-                                             float sx, float sz, float lvA, float lvB, float& lx, float& lz,
-                                             float& vA, float& vB)
-{
-    const int nx = a.nx, nz = a.nz;
-    float xs = fx - sx, fzz = fz - sz;
-    int i = ci, k = ck;
-    if (xs < 0.0f) { xs += 1.0f; i -= 1; }
-    if (fzz < 0.0f) { fzz += 1.0f; k -= 1; }
-    const int rows = sz > 0.0f ? nz : nz + 1;
-    bool clamped = false;
-    if (k < 0) { k = 0; fzz = 0.0f; clamped = true; }
-    else if (k > rows - 1 || (k == rows - 1 && fzz > 0.0f)) { k = rows - 1; fzz = 0.0f; clamped = true; }
-    if (k >= rows - 1) { k = rows - 2; fzz = 1.0f; }
-    const int i0 = i < 0 ? i + nx : i;
-    const int i1 = i0 + 1 == nx ? 0 : i0 + 1;
-    const size_t r0 = (size_t)k * nx, r1 = r0 + nx;
-    const float w00 = (1 - xs) * (1 - fzz), w10 = xs * (1 - fzz), w01 = (1 - xs) * fzz, w11 = xs * fzz;
-    const size_t nn = (size_t)(nz + 1) * nx;
-#pragma unroll
-    for (int h = 0; h < 2; h++) {
-        const int f = h ? fB : fA;
-        const float lv = h ? lvB : lvA;
-        const float* A = a.F[f];
-        const float a00 = A[r0 + i0], a10 = A[r0 + i1], a01 = A[r1 + i0], a11 = A[r1 + i1];
-        if (lv != 0.0f) {
-            float* L = a.lF + (size_t)f * nn;
-            atomicAdd(L + r0 + i0, lv * w00);
-            atomicAdd(L + r0 + i1, lv * w10);
-            atomicAdd(L + r1 + i0, lv * w01);
-            atomicAdd(L + r1 + i1, lv * w11);
-            lx += lv * ((1 - fzz) * (a10 - a00) + fzz * (a11 - a01));
-            if (!clamped) lz += lv * ((1 - xs) * (a01 - a00) + xs * (a11 - a10));
-        }
-        const float v = w00 * a00 + w10 * a10 + w01 * a01 + w11 * a11;
-        if (h) vB = v; else vA = v;
-    }
-}
-
-
-__global__ void __launch_bounds__(256, 2) k_adjoint_full(const FullAdjArgs a)
+// ION: the pair force, positive charge; else the electrons. (One kernel for both with run-time flags carried
+// the pair force's registers through the electrons.)
+template <bool ION>
+__global__ void __launch_bounds__(256, kAdjCtas) k_adjoint_full(const FullAdjArgs a)
 {
     __shared__ double sh[256];
-    double gFF = 0.0, gR = 0.0;
+    Sum2 gFF, gR;
+    const size_t nn = (size_t)(a.nz + 1) * a.nx;
+    float2* LExBz = reinterpret_cast<float2*>(a.lF);
+    float2* LEzBx = LExBz + nn;
+    float *LEy = a.lF + 4 * nn, *LBy = LEy + nn;
     for (int64_t ch = blockIdx.x; ch * 256 < a.n; ch += gridDim.x) {
         const int64_t p = spread_index(ch);
         if (p >= a.n) continue;
@@ -644,14 +677,20 @@ __global__ void __launch_bounds__(256, 2) k_adjoint_full(const FullAdjArgs a)
         split2(a.cell[p], a.nx, a.nx_magic, ci, ck);
         const float fx = a.fx[p], fz = a.fz[p];
         // ---- forward recompute (FP32, positions local to the cell) ----
-        float E[3], B[3], dummy = 0.0f;
-        gather_stag2(a, 0, 5, ci, ck, fx, fz, 0.5f, 0.0f, 0.0f, 0.0f, dummy, dummy, E[0], B[2]);
-        gather_stag2(a, 2, 3, ci, ck, fx, fz, 0.0f, 0.5f, 0.0f, 0.0f, dummy, dummy, E[2], B[0]);
-        E[1] = gather_stag(a, 1, ci, ck, fx, fz, 0.0f, 0.0f, 0.0f, dummy, dummy);
-        B[1] = gather_stag(a, 4, ci, ck, fx, fz, 0.5f, 0.5f, 0.0f, dummy, dummy);
+        float E[3], B[3];
+        const Stag sx_ = stag_at(a.nx, a.nz, ci, ck, fx, fz, 0.5f, 0.0f), sz_ = stag_at(a.nx, a.nz, ci, ck, fx, fz, 0.0f, 0.5f);
+        const Stag s0_ = stag_at(a.nx, a.nz, ci, ck, fx, fz, 0.0f, 0.0f), sxz = stag_at(a.nx, a.nz, ci, ck, fx, fz, 0.5f, 0.5f);
+        const Gathered gEx = gather_at(a.F[0], sx_), gBz = gather_at(a.F[5], sx_), gEz = gather_at(a.F[2], sz_),
+                       gBx = gather_at(a.F[3], sz_), gEy = gather_at(a.F[1], s0_), gBy = gather_at(a.F[4], sxz);
+        E[0] = gEx.v;
+        E[1] = gEy.v;
+        E[2] = gEz.v;
+        B[0] = gBx.v;
+        B[1] = gBy.v;
+        B[2] = gBz.v;
         DensAt d = {};
         PairD px = {0.0f, 0.0f, 0.0f, 0.0f}, pz = px;
-        if (a.pair) {
+        if (ION) {
             d = dens_at(a.rho, a.rho_s, a.nx, a.nz, ci, ck, fx, fz);
             px = pair_axis_d(d.n, d.qx, a.r0_dx, a.fu, a.inv_r0);
             pz = pair_axis_d(d.n, d.qz, a.r0_dx, a.fu, a.inv_r0);
@@ -686,9 +725,13 @@ __global__ void __launch_bounds__(256, 2) k_adjoint_full(const FullAdjArgs a)
         float lx1 = a.lam_pos[2 * p], lz1 = a.lam_pos[2 * p + 1];
         float luf[3] = {a.lam_u[3 * p], a.lam_u[3 * p + 1], a.lam_u[3 * p + 2]};
         float lx0 = 0.0f, lz0 = 0.0f;
-        if (a.sg != 0.0f) {
+        {
             float g5[5] = {0, 0, 0, 0, 0};
-            cur_T(a, ci, ck, fx, fz, xl, z1, by, g5);
+            // strictly inside one cell (on an edge the general stencil picks its one-sided derivative)
+            if (fx > 0.0f && xl > 0.0f && xl < 1.0f && fz > 0.0f && fz < 1.0f && z1 > 0.0f && z1 < 1.0f)
+                cur_T_cell(a, ci, ck, fx, fz, xl, z1, by, g5);
+            else
+                cur_T(a, ci, ck, fx, fz, xl, z1, by, g5);
             lx0 += g5[0]; lz0 += g5[1]; lx1 += g5[2]; lz1 += g5[3];
             const float ig = 1.0f / g, ig3 = ig * ig * ig;
             luf[0] -= g5[4] * uf[1] * uf[0] * ig3;
@@ -737,18 +780,20 @@ __global__ void __launch_bounds__(256, 2) k_adjoint_full(const FullAdjArgs a)
         a.lam_u[3 * p + 2] = lum[2];
         // field gathers
         {
-            float t0, t1;
-            gather_stag2(a, 0, 5, ci, ck, fx, fz, 0.5f, 0.0f, a.eps * la[0], lB[2], lx0, lz0, t0, t1);
-            gather_stag2(a, 2, 3, ci, ck, fx, fz, 0.0f, 0.5f, a.eps * la[2], lB[0], lx0, lz0, t0, t1);
-            gather_stag(a, 1, ci, ck, fx, fz, 0.0f, 0.0f, a.eps * la[1], lx0, lz0);
-            gather_stag(a, 4, ci, ck, fx, fz, 0.5f, 0.5f, lB[1], lx0, lz0);
+            const float vx = a.eps * la[0], vy = a.eps * la[1], vz = a.eps * la[2];
+            lx0 += vx * gEx.gx + vy * gEy.gx + vz * gEz.gx + lB[0] * gBx.gx + lB[1] * gBy.gx + lB[2] * gBz.gx;
+            lz0 += vx * gEx.gz + vy * gEy.gz + vz * gEz.gz + lB[0] * gBx.gz + lB[1] * gBy.gz + lB[2] * gBz.gz;
+            scatter_at(LExBz, sx_, vx, lB[2]);
+            scatter_at(LEzBx, sz_, vz, lB[0]);
+            scatter_at(LEy, s0_, vy);
+            scatter_at(LBy, sxz, lB[1]);
         }
-        if (a.pair) pair_T(d, px, pz, a.fk * la[0], a.fk * la[2], a.inv_r0, a.nx, a.lam_nodes, lx0, lz0, gFF, gR);
+        if (ION) pair_T(d, px, pz, a.fk * la[0], a.fk * la[2], a.inv_r0, a.nx, a.lam_nodes, lx0, lz0, gFF, gR);
         a.lam_pos[2 * p] = lx0;
         a.lam_pos[2 * p + 1] = lz0;
     }
-    if (a.pair) {
-        const double sD = block_sum_d(gFF, sh), sR = block_sum_d(gR, sh);
+    if (ION) {
+        const double sD = block_sum_d(gFF.value(), sh), sR = block_sum_d(gR.value(), sh);
         if (threadIdx.x == 0) {
             atomicAdd(a.grads, sD * a.inv_D);
             atomicAdd(a.grads + 1, sR);
@@ -770,11 +815,21 @@ __global__ void k_adjoint_seed_u(int64_t n, const float* ux, const float* uy, co
     }
 }
 
-// the particles' FP32 scatter added into the FP64 field adjoints
-__global__ void k_fold_scatter(double* __restrict__ lF, const float* __restrict__ scatter, int64_t n)
+// the particles' FP32 scatter (grids (Ex, Bz) and (Ez, Bx) in pairs, Ey, By) added into the FP64 field adjoints
+__global__ void k_fold_scatter(double* __restrict__ lF, const float* __restrict__ scatter, int64_t nn)
 {
-    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x)
-        lF[q] += (double)scatter[q];
+    const float2* exbz = reinterpret_cast<const float2*>(scatter);
+    const float2* ezbx = exbz + nn;
+    const float *ey = scatter + 4 * nn, *by = ey + nn;
+    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < nn; q += (int64_t)gridDim.x * blockDim.x) {
+        const float2 a = exbz[q], b = ezbx[q];
+        lF[q] += (double)a.x;
+        lF[nn + q] += (double)ey[q];
+        lF[2 * nn + q] += (double)b.x;
+        lF[3 * nn + q] += (double)b.y;
+        lF[4 * nn + q] += (double)by[q];
+        lF[5 * nn + q] += (double)a.y;
+    }
 }
 
 static FullAdjArgs make_full_adj(Ctx& c, int s, float* const* lam_pos, float* const* lam_u, float* lam_nodes,
@@ -804,7 +859,6 @@ static FullAdjArgs make_full_adj(Ctx& c, int s, float* const* lam_pos, float* co
     a.tq = (float)(q * c.dt / (2.0 * S.mass));
     a.cs0 = (float)(kC * c.dt / c.cfg.dx);
     a.sg = (float)S.jsign;
-    a.pair = S.pair;
     a.cx = (float)(kQe * c.w / (2.0 * c.cfg.dx * kEps0));
     a.cy = (float)(kQe * c.w * kC * c.dt / (6.0 * c.cfg.dx * c.cfg.dx * kEps0));
     a.lam_pos = lam_pos[s];
@@ -862,10 +916,13 @@ void launch_adjoint_step_full(Ctx& c, float* const* lam_pos, float* const* lam_u
     float* scatter = reinterpret_cast<float*>(lF + 6 * nn);        // six float grids
     cudaMemsetAsync(scatter, 0, sizeof(float) * 6 * nn, st);
     for (int s = 0; s < c.nsp; s++) {
+        const Species& S = c.sp[s];
         FullAdjArgs a = make_full_adj(c, s, lam_pos, lam_u, lam_nodes, scatter, lj, grads);
-        if (a.n > 0) k_adjoint_full<<<agrid(c, a.n), 256, 0, st>>>(a);
+        if (a.n == 0) continue;
+        if (S.pair) k_adjoint_full<true><<<agrid(c, a.n), 256, 0, st>>>(a);
+        else k_adjoint_full<false><<<agrid(c, a.n), 256, 0, st>>>(a);
     }
-    k_fold_scatter<<<agrid(c, (int64_t)(6 * nn)), 256, 0, st>>>(lF, scatter, (int64_t)(6 * nn));
+    k_fold_scatter<<<agrid(c, (int64_t)nn), 256, 0, st>>>(lF, scatter, (int64_t)nn);
     if (c.sp[0].pair) {
         AdjArgs b = make_adj(c, 0, lam_pos[0], lam_u[0], lam_nodes, grads);
         k_adjoint_b<<<agrid(c, b.n), 256, 0, st>>>(b);
