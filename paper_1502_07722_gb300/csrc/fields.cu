@@ -146,20 +146,24 @@ __device__ __forceinline__ void field_rows(const FieldArgs& f, int i0, int k0, i
 
 // Rows per segment. A warp's walk is serial (each row waits for its loads, ~0.7 us), while the row and
 // a half that every segment repeats comes from L2: short segments win on every grid (2048^2: 97 us
-// at 4 rows, 101 at 8, 99 at 16, 102 at 64; 403 x 311: 10.3, 12.3, 22, 82; with the events' ~3 us). The
-// last segment takes the remainder (at least kSeg rows: the wall row needs the row beside it).
-constexpr int kSeg = 4;
-__host__ __device__ inline int field_segments(int nz) { return (nz + 1) / kSeg; }     // nz >= 4
+// at 4 rows, 101 at 8, 99 at 16, 102 at 64; 403 x 311: 10.3, 12.3, 22, 82; with the events' ~3 us), and two
+// rows where the grid gives under four warps per SM (64^2: 21.4 -> 19.4 us per step). The last segment takes the remainder (at
+// least seg rows: the wall row needs the row beside it).
+static int field_segment(const Ctx& c)
+{
+    return (int64_t)((c.nx + kCols - 1) / kCols) * ((c.nz + 1) / 4) < 4 * (int64_t)c.nsm ? 2 : 4;
+}
+__host__ __device__ inline int field_segments(int nz, int seg) { return (nz + 1) / seg; }     // nz >= 4
 
 __device__ __forceinline__ void field_item(const FieldArgs& f, int item, float a0, float a1)
 {
-    const int nseg = field_segments(f.nz), col = item / nseg, s = item - col * nseg;
+    const int nseg = field_segments(f.nz, f.seg), col = item / nseg, s = item - col * nseg;
     if (col * kCols >= f.nx) return;
-    field_rows(f, col * kCols, s * kSeg, s + 1 == nseg ? f.nz + 1 : (s + 1) * kSeg, a0, a1);
+    field_rows(f, col * kCols, s * f.seg, s + 1 == nseg ? f.nz + 1 : (s + 1) * f.seg, a0, a1);
 }
 static int field_blocks(const FieldArgs& f)
 {
-    const int items = (f.nx + kCols - 1) / kCols * field_segments(f.nz), w = kFieldThreads / 32;
+    const int items = (f.nx + kCols - 1) / kCols * field_segments(f.nz, f.seg), w = kFieldThreads / 32;
     return (items + w - 1) / w;
 }
 
@@ -225,6 +229,7 @@ FieldArgs make_field_args(const Ctx& c)
     f.nx = c.nx;
     f.nz = c.nz;
     f.k_ant = c.k_ant;
+    f.seg = field_segment(c);
     f.h_b = (float)(0.5 * c.dt / c.cfg.dx);
     f.h_e = (float)(kC * kC * c.dt / c.cfg.dx);
     f.cj = (float)(kQe * c.w / (8589934592.0 * c.cfg.dx * kEps0));

@@ -28,6 +28,12 @@ constexpr int kQ3Bits = 14;
 constexpr int kQ3 = 1 << kQ3Bits;
 constexpr int kBlock3 = 256;
 constexpr int kCtas3 = 3, kCtas3Atoms = 4;
+// Parts per tile (a power of two up to 16) until there are kFill3 items per resident CTA: a grid of few
+// tiles left most of the chip idle. Every item stages its tile's window, seven arrays with fields and the
+// density alone without. ms per launch, whole tiles -> parts: 37 x 27 x 32 cells of 16 + 16 particles 0.176 ->
+// 0.041, 90 x 80 x 60 of 8 + 8 0.205 -> 0.118 (at 2 per CTA 0.126), 88 x 246 x 28 of 9 atoms 0.143 -> 0.083
+// (at 2 per CTA 0.087).
+constexpr int kMaxLog2Sub3 = 4, kFill3 = 1, kFill3Atoms = 4;
 
 __device__ __forceinline__ int wrapn(int i, int n) { return i < 0 ? i + n : (i >= n ? i - n : i); }
 __device__ __forceinline__ int qoff3(float f) { return __float2int_rn(f * 16384.0f); }
@@ -132,6 +138,7 @@ struct Species3 {
 struct Args3 {
     Geo3 g;
     int ntiles, nsp, full, pot_mode;
+    int log2sub;            // parts per tile
     int T, ntx, nty, W;     // tile edge, tiles along x and y, staged window edge (0: no window)
     float cdt_dx, rho_s, h_coef, c_att, s_rep;
     EamP eam;
@@ -513,6 +520,14 @@ __device__ __forceinline__ void process3(const Args3& a, const Species3& S, cons
                   x1 - kQ3Bias, y1 - kQ3Bias, z1 - kQ3Bias, S.jsign, PAIR ? 1 : 0);
 }
 
+// start of part `sub` of 2^log2sub of the records q0 .. q1 - 1; inner boundaries lie on multiples of 32
+__device__ __forceinline__ int part3(int q0, int q1, int sub, int log2sub)
+{
+    if (sub == 0) return q0;
+    if (sub >> log2sub) return q1;
+    return max(q0, (q0 + (int)((u64)(unsigned)(q1 - q0) * (unsigned)sub >> log2sub)) & ~31);
+}
+
 template <bool FULL, int POT, int WC>
 __global__ void __launch_bounds__(kBlock3, FULL ? kCtas3 : kCtas3Atoms) k_particles3(const __grid_constant__ Args3 a)
 {
@@ -528,9 +543,9 @@ __global__ void __launch_bounds__(kBlock3, FULL ? kCtas3 : kCtas3Atoms) k_partic
     // it back to 0 once every CTA has drawn its last, failing, ticket)
     __shared__ int slot;
     for (;;) {
-        if (threadIdx.x == 0) slot = (int)atomicInc(a.status + 2, (unsigned)(a.ntiles + gridDim.x - 1));
+        if (threadIdx.x == 0) slot = (int)atomicInc(a.status + 2, (unsigned)((a.ntiles << a.log2sub) + gridDim.x - 1));
         __syncthreads();
-        const int t = slot;
+        const int t = slot >> a.log2sub, sub = slot & ((1 << a.log2sub) - 1);
         __syncthreads();
         if (t >= a.ntiles) break;
         int cnt = 0;
@@ -568,7 +583,8 @@ __global__ void __launch_bounds__(kBlock3, FULL ? kCtas3 : kCtas3Atoms) k_partic
         for (int s = 0; s < 2; s++) {
             if (s >= a.nsp) break;
             const Species3& S = a.sp[s];
-            const int p0 = S.tile_start[t], p1 = S.tile_start[t + 1];
+            const int p0 = part3(S.tile_start[t], S.tile_start[t + 1], sub, a.log2sub),
+                      p1 = part3(S.tile_start[t], S.tile_start[t + 1], sub + 1, a.log2sub);
             // consecutive threads take consecutive records (coalesced); the cell sort's block
             // layout gives a warp's lanes neighbouring cells
             // the next record's position is loaded one iteration ahead (its first use is at the top
@@ -659,7 +675,10 @@ void launch_particle_step3(Ctx& c, cudaStream_t st)
         configured[dev].store(shmem);
     }
     const int slots = c.nsm * (a.full ? kCtas3 : kCtas3Atoms);
-    int grid = c.ntiles < slots ? c.ntiles : slots;
+    a.log2sub = 0;
+    while (a.log2sub < kMaxLog2Sub3 && ((int64_t)c.ntiles << a.log2sub) < (int64_t)slots * (a.full ? kFill3 : kFill3Atoms)) a.log2sub++;
+    const int64_t items = (int64_t)c.ntiles << a.log2sub;
+    int grid = items < slots ? (int)items : slots;
     if (grid < 1) grid = 1;
     // the instance with the potential and the lattice compiled in, and the window edge when it is
     // the 10-cell tile's
@@ -794,6 +813,7 @@ void launch_pair_force3(Ctx& c, float* out, cudaStream_t st)
 struct Field3 {
     Geo3 g;
     int k_ant;
+    int seg;              // planes per block
     float h_b, h_e, cj, mur;
     float ant0, ant1;     // this step's antenna scalars
     const float* F[6];    // read
@@ -816,7 +836,7 @@ struct Field3 {
 // It is bound by memory traffic: 112 bytes per node and step instead of 172 in three in-place passes and
 // a copy/clear kernel. 384^2 x 256 cells: 0.92 ms against 1.06 plus 0.3 of the copy (segments of 8 planes
 // 0.97, 32 planes 0.91; 192^2 x 128: 0.130, 0.137, 0.153); one block per SM 1.44.
-constexpr int kCols3 = 29, kRows3 = 13, kWarps3 = kRows3 + 3, kSeg3 = 16;
+constexpr int kCols3 = 29, kRows3 = 13, kWarps3 = kRows3 + 3;
 
 struct F3 {
     float x, y, z;
@@ -835,7 +855,7 @@ __global__ void __launch_bounds__(32 * kWarps3, 2) k_fields3(const __grid_consta
     const bool own = lane >= 1 && lane <= kCols3 && i < g.nx && w >= 1 && w <= kRows3 && j < g.ny;
     const int wm = w > 0 ? w - 1 : 0, wp = w + 1 < kWarps3 ? w + 1 : w;     // the patch's outer rows are not written
     // planes k0 .. k1 - 1; the last segment takes the remainder
-    const int k0 = (int)blockIdx.z * kSeg3, k1 = blockIdx.z + 1 == gridDim.z ? nz + 1 : k0 + kSeg3;
+    const int k0 = (int)blockIdx.z * f.seg, k1 = blockIdx.z + 1 == gridDim.z ? nz + 1 : k0 + f.seg;
     const size_t plane = (size_t)g.nx * g.ny;
     const size_t col = (size_t)gj * g.nx + gi;
     const float antc = f.antc[col], ants = f.ants[col];
@@ -972,8 +992,12 @@ void launch_fields3(Ctx& c, cudaStream_t st, int64_t step, int64_t* launches)
     f.ants = c.ant_s;
     f.k_flux = c.k_ant - 1 >= 1 ? c.k_ant - 1 : -1;
     f.flux = c.red_out + 5;
-    const int seg = (c.nz + 1) / kSeg3;
-    const dim3 grid((c.nx + kCols3 - 1) / kCols3, (c.ny + kRows3 - 1) / kRows3, seg > 1 ? seg : 1);
+    // 16 planes per block (every segment repeats about two), fewer where that leaves under four blocks per SM
+    // (90 x 80 x 60 cells: 56 us at 16 planes, 29 at 4; 37 x 27 x 32: 29, 15, 11 at 2); the last segment takes the remainder, at least `seg` planes
+    dim3 grid((c.nx + kCols3 - 1) / kCols3, (c.ny + kRows3 - 1) / kRows3);
+    f.seg = 16;
+    while (f.seg > 2 && (int64_t)grid.x * grid.y * ((c.nz + 1) / f.seg) < 4 * (int64_t)c.nsm) f.seg >>= 1;
+    grid.z = (c.nz + 1) / f.seg > 1 ? (c.nz + 1) / f.seg : 1;
     k_fields3<<<grid, 32 * kWarps3, 0, st>>>(f);
     swap_fields(c);
     if (launches) *launches += 1;

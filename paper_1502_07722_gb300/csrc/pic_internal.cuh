@@ -206,6 +206,7 @@ __host__ __device__ inline void antenna_scalars(const AntennaParams& p, long lon
 // Everything the 2D field kernel needs for one simulation.
 struct FieldArgs {
     int nx, nz, k_ant;
+    int seg;             // rows of a warp's segment
     float h_b;           // dt / (2 dx)      (half step of B)
     float h_e;           // c^2 dt / dx      (full step of E)
     float cj;            // J2x, J2z -> dt J / eps0
