@@ -44,10 +44,11 @@ constexpr int kCtasPerSm = 9;
 constexpr int kCtasPerSmAtoms = 8;
 constexpr int kMinChunk = 512;
 constexpr int kWin = 16 + 2 * kMargin + 3;  // window edge of the 16-cell tile (compiled-in instances)
-// The batched kernel reads each slab's arguments from a constant-memory table with a run-time
-// index: every use is an indexed constant load into a register, so it needs more registers than
-// the single kernel for the same code: 72 (7 CTAs per SM).
-constexpr int kCtasPerSmBatch = 7;
+// The batched kernel reads each slab's arguments from a constant-memory table with a run-time index:
+// every use is an indexed constant load into a register, so it needs more registers than the single
+// kernel for the same code: 8 CTAs (64 registers) on the 16-slab sweep 1.37 ms per launch, 7 CTAs (72) 1.42,
+// 9 CTAs (56) 1.73.
+constexpr int kCtasPerSmBatch = 8;
 
 
 __device__ __forceinline__ int wrap_any(int i, int nx)
