@@ -412,7 +412,10 @@ PIC_API int pic_checkpoint_restore(pic_ctx* ctx, const void* buf, int32_t on_hos
  *   derivative of the density unit in the functional (add it to grads[1]).
  * pic_adjoint_step: with the context at the state of step t (restore it from a checkpoint), map the
  *   adjoints of step t+1 to step t in place and add this step's parameter derivatives to grads.
- * Both return PIC_ESTATE outside 2D, sort_every = 0 and pot_mode 0. */
+ * pic_adjoint_step_at: the same, the state of step t read in place from a device checkpoint that this
+ *   context saved with its present particle counts (the context itself need not be at step t and is left
+ *   as it is; dev_ckpt is 256-byte aligned as for pic_checkpoint_save). Asynchronous on the stream.
+ * All return PIC_ESTATE outside 2D, sort_every = 0 and pot_mode 0. */
 typedef struct {
     float* lam_pos[2];
     float* lam_u[2];
@@ -426,6 +429,7 @@ PIC_API int pic_node_functional(pic_ctx* ctx, const double* dev_weights, double*
 PIC_API int pic_adjoint_seed(pic_ctx* ctx, double kin, const double* dev_weights, const pic_adjoint_buffers* bufs,
                              double* host_dLdr0);
 PIC_API int pic_adjoint_step(pic_ctx* ctx, const pic_adjoint_buffers* bufs);
+PIC_API int pic_adjoint_step_at(pic_ctx* ctx, const void* dev_ckpt, const pic_adjoint_buffers* bufs);
 
 /* Static text for a return code. */
 PIC_API const char* pic_strerror(int code);

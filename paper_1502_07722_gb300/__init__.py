@@ -115,6 +115,7 @@ _SIGNATURES = {
     "pic_adjoint_seed": (ctypes.c_int, [_VP, ctypes.c_double, _VP, ctypes.POINTER(pic_adjoint_buffers),
                                         ctypes.POINTER(ctypes.c_double)]),
     "pic_adjoint_step": (ctypes.c_int, [_VP, ctypes.POINTER(pic_adjoint_buffers)]),
+    "pic_adjoint_step_at": (ctypes.c_int, [_VP, _VP, ctypes.POINTER(pic_adjoint_buffers)]),
 }
 
 _lib = None
@@ -362,6 +363,10 @@ def pic_adjoint_seed(h, kin, dev_weights_ptr, bufs) -> float:
 
 def pic_adjoint_step(h, bufs):
     _check(load_library().pic_adjoint_step(h, ctypes.byref(bufs)), "pic_adjoint_step")
+
+
+def pic_adjoint_step_at(h, ckpt_ptr, bufs):
+    _check(load_library().pic_adjoint_step_at(h, ckpt_ptr, ctypes.byref(bufs)), "pic_adjoint_step_at")
 
 
 # ---- convenience wrapper: torch owns the workspace and the stream -----------------------------

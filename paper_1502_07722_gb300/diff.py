@@ -22,7 +22,8 @@ from __future__ import annotations
 import torch
 
 from . import (PIC_MODE_FULL, Simulation, pic_adjoint_buffers, pic_adjoint_seed, pic_adjoint_step,
-               pic_checkpoint_restore, pic_checkpoint_save, pic_checkpoint_size, pic_node_functional)
+               pic_adjoint_step_at, pic_checkpoint_restore, pic_checkpoint_save, pic_checkpoint_size,
+               pic_node_functional)
 
 QE = 1.602176634e-19
 
@@ -101,18 +102,21 @@ class DiffRun:
         """(dL/dD (1/J), dL/dr0 (1/m), dL/dI0 (m^2/W)); leaves the context at the initial state."""
         bufs, grads = self._buffers(w.numel())
         g_r0 = pic_adjoint_seed(self.sim.h, kin, w.data_ptr(), bufs)
-        seg_states = [self._buf() for _ in range(min(self.every, self.nsteps))]
+        # states 1 .. m - 2 of a segment are saved; state 0 is its checkpoint, the last one the context's own
+        seg_states = [self._buf() for _ in range(max(0, min(self.every, self.nsteps) - 2))]
         for si in range(len(self.checkpoints) - 1, -1, -1):
             t0 = si * self.every
             m = min(self.every, self.nsteps - t0)
             pic_checkpoint_restore(self.sim.h, self.checkpoints[si].data_ptr())
-            for j in range(m):
-                pic_checkpoint_save(self.sim.h, seg_states[j].data_ptr())
+            for j in range(1, m):
+                self.sim.step(1)
                 if j + 1 < m:
-                    self.sim.step(1)
-            for j in range(m - 1, -1, -1):
-                pic_checkpoint_restore(self.sim.h, seg_states[j].data_ptr())
-                pic_adjoint_step(self.sim.h, bufs)
+                    pic_checkpoint_save(self.sim.h, seg_states[j - 1].data_ptr())
+            pic_adjoint_step(self.sim.h, bufs)
+            for j in range(m - 2, -1, -1):
+                pic_adjoint_step_at(self.sim.h, (seg_states[j - 1] if j else self.checkpoints[si]).data_ptr(), bufs)
+        if self.checkpoints:
+            pic_checkpoint_restore(self.sim.h, self.checkpoints[0].data_ptr())
         torch.cuda.current_stream().synchronize()
         gD, gR, gI = grads.tolist()
         self._keep = []
