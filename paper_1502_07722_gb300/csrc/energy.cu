@@ -71,7 +71,7 @@ __global__ void __launch_bounds__(kEBlock) k_energy(const EnergyArgs a)
                 for (int q = 0; q < kBatch; q++) {
                     const int c = cell[q] < 0 ? 0 : cell[q];
                     const int k = (int)(__umulhi((unsigned)c, a.nx_magic) >> a.nx_shift), i = c - k * a.nx;
-                    gather_density(a.rho, a.nx, a.nz, a.rho_s, i, k, fx[q], fz[q], n[q], dnx[q], dnz[q]);
+                    gather_density<true>(a.rho, a.nx, a.nz, a.rho_s, i, k, fx[q], fz[q], n[q], dnx[q], dnz[q]);
                 }
             }
 #pragma unroll

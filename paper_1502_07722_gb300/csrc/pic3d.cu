@@ -100,6 +100,7 @@ __device__ __forceinline__ float gather3(const float* __restrict__ A, const Geo3
 }
 
 // trilinear node density (units n0) and its exact gradient (units n0 per cell); wall rows doubled
+template <bool NARROW = false>   // as gather_density
 __device__ __forceinline__ void density3(const u64* __restrict__ rho, const Geo3& g, float rho_s, int i, int j, int k,
                                          float fx, float fy, float fz, float& n, float* grad)
 {
@@ -113,7 +114,7 @@ __device__ __forceinline__ void density3(const u64* __restrict__ rho, const Geo3
             for (int a = 0; a < 2; a++) {
                 long long r = (long long)__ldg(rho + idx3(g, a ? i1 : i, b ? j1 : j, k + c));
                 if (k + c == 0 || k + c == g.nz) r *= 2;
-                v[c * 4 + b * 2 + a] = rho_s * i64_f32(r);
+                v[c * 4 + b * 2 + a] = rho_s * (NARROW ? i64_f32(r) : (float)r);
             }
     const float gx = 1.0f - fx, gy = 1.0f - fy, gz = 1.0f - fz;
     // along x: differences of the x-pairs weighted in y and z
@@ -1054,7 +1055,7 @@ __global__ void __launch_bounds__(256) k_energy3(const Species3 s0, const Specie
                 for (int q = 0; q < 2; q++) {
                     int i, j, k;
                     split3(cell[q] < 0 ? 0 : cell[q], g, i, j, k);
-                    density3(rho, g, rho_s, i, j, k, fx[q], fy[q], fz[q], dens[q], gr[q]);
+                    density3<true>(rho, g, rho_s, i, j, k, fx[q], fy[q], fz[q], dens[q], gr[q]);
                 }
             }
 #pragma unroll

@@ -50,6 +50,9 @@ __device__ __forceinline__ long long rho_node(const u64* __restrict__ rho, int n
 // offsets (fx, fz): bilinear density; the gradient is the edge difference of the node density
 // interpolated along the other axis, i.e. the exact gradient of the bilinear density.
 // Differences are taken in integers before the single rounding to FP32.
+// NARROW: by i64_f32, for the energy sums. The conversions are the same, but the compiler then fuses other
+// products of the sums below: the force of a probe would differ in its last bits.
+template <bool NARROW = false>
 __device__ __forceinline__ void gather_density(const u64* __restrict__ rho, int nx, int nz, float rho_s,
                                                int i, int k, float fx, float fz,
                                                float& n, float& dnx, float& dnz)
@@ -57,11 +60,12 @@ __device__ __forceinline__ void gather_density(const u64* __restrict__ rho, int 
     int i1 = wrap_x(i + 1, nx);
     long long r00 = rho_node(rho, nx, nz, i, k), r10 = rho_node(rho, nx, nz, i1, k);
     long long r01 = rho_node(rho, nx, nz, i, k + 1), r11 = rho_node(rho, nx, nz, i1, k + 1);
+    auto num = [](long long v) { return NARROW ? i64_f32(v) : (float)v; };
     float gx = 1.0f - fx, gz = 1.0f - fz;
-    float a00 = i64_f32(r00), a10 = i64_f32(r10), a01 = i64_f32(r01), a11 = i64_f32(r11);
+    float a00 = num(r00), a10 = num(r10), a01 = num(r01), a11 = num(r11);
     n = rho_s * (gz * (gx * a00 + fx * a10) + fz * (gx * a01 + fx * a11));
-    dnx = rho_s * (gz * i64_f32(r10 - r00) + fz * i64_f32(r11 - r01));
-    dnz = rho_s * (gx * i64_f32(r01 - r00) + fx * i64_f32(r11 - r10));
+    dnx = rho_s * (gz * num(r10 - r00) + fz * num(r11 - r01));
+    dnz = rho_s * (gx * num(r01 - r00) + fx * num(r11 - r10));
 }
 
 // Lennard-Jones derivative U'(r) (units D/r0) from inv = r0 / r.
