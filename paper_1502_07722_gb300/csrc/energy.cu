@@ -10,16 +10,11 @@ constexpr int kEBlock = 256;
 constexpr int kBatch = 4;   // particles of a thread whose loads are in flight together
 constexpr int kSlots = 5;   // 0 KE ions, 1 KE electrons, 2 field E, 3 field B, 4 pair
 
-// a fixed-shape tree: lanes of a warp, then the warps (the result in every thread)
-__device__ __forceinline__ double block_sum(double v, double* sh)
+// lanes of a warp, a fixed-shape tree (the result in lane 0)
+__device__ __forceinline__ double warp_sum(double v)
 {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
-    __syncthreads();
-    double r = sh[0];
-    for (int w = 1; w < kEBlock / 32; w++) r += sh[w];
-    __syncthreads();
-    return r;
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    return v;
 }
 
 struct EnergyArgs {
@@ -40,7 +35,7 @@ struct EnergyArgs {
 template <bool LJ>
 __global__ void __launch_bounds__(kEBlock) k_energy(const EnergyArgs a)
 {
-    __shared__ double sh[kEBlock / 32];
+    __shared__ double sh[kSlots][kEBlock];
     const int64_t tid = blockIdx.x * (int64_t)kEBlock + threadIdx.x;
     const int64_t stride = (int64_t)gridDim.x * kEBlock;
     Sum2 ke[2], pe;
@@ -100,32 +95,51 @@ __global__ void __launch_bounds__(kEBlock) k_energy(const EnergyArgs a)
             fb += bx * bx + by * by;
         }
     }
-    const double r0 = block_sum(ke[0].value(), sh), r1 = block_sum(ke[1].value(), sh), r2 = block_sum(fe, sh),
-                 r3 = block_sum(fb, sh), r4 = block_sum(pe.value(), sh);
-    if (threadIdx.x == 0) {
-        double* o = a.partials + (size_t)blockIdx.x * kSlots;
-        o[0] = r0; o[1] = r1; o[2] = r2; o[3] = r3; o[4] = r4;
+    // Warp s adds up slot s. (A shuffle tree in every warp for every slot took 60 FP64 instructions per warp, about
+    // 15 us whatever the size on 2 FP64 lanes per SM; this takes 13 per slot and block.)
+    sh[0][threadIdx.x] = ke[0].value();
+    sh[1][threadIdx.x] = ke[1].value();
+    sh[2][threadIdx.x] = fe;
+    sh[3][threadIdx.x] = fb;
+    sh[4][threadIdx.x] = pe.value();
+    __syncthreads();
+    const int s = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (s < kSlots) {
+        double v = sh[s][lane];
+        for (int w = 1; w < kEBlock / 32; w++) v += sh[s][lane + 32 * w];
+        v = warp_sum(v);
+        if (lane == 0) a.partials[(size_t)blockIdx.x * kSlots + s] = v;
     }
 }
 
-__global__ void k_energy_final(const double* __restrict__ partials, int nb, double* out)
+// one warp per slot, blocks assigned to lanes in a fixed way
+__device__ __forceinline__ double sum_slot(const double* __restrict__ partials, int nb, int s, int lane)
 {
-    __shared__ double sh[kEBlock / 32];
-    for (int s = 0; s < kSlots; s++) {
-        double v = 0.0;
-        // fixed assignment of blocks to threads, then a fixed-shape tree
-        for (int b = threadIdx.x; b < nb; b += kEBlock) v += partials[(size_t)b * kSlots + s];
-        const double r = block_sum(v, sh);
-        if (threadIdx.x == 0) out[s] = r;
-    }
+    double v = 0.0;
+    for (int b = lane; b < nb; b += 32) v += partials[(size_t)b * kSlots + s];
+    return warp_sum(v);
+}
+
+__global__ void __launch_bounds__(32 * kSlots) k_energy_final(const double* __restrict__ partials, int nb, double* out)
+{
+    const int s = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const double r = sum_slot(partials, nb, s, lane);
+    if (lane == 0) out[s] = r;
 }
 
 // Sums of FP32 terms by two-sum and the FP64 conversions kept off the common way: 482 -> 277 us for the
 // 33.5 M particles and 1 M nodes of the 1024^2 slab (8 FP64-pipe instructions per particle were its bound).
-static void run_energy(const EnergyArgs& a, int nb, cudaStream_t st)
+// Small states take as many blocks as give every thread a particle or a node: each block costs its share of
+// FP64 adds at the end (64^2 cells, 16384 ions: 23.1 us with every block and shuffle trees, 7.2 now; the final sum
+// 8.4 -> 2.3). Returns the blocks taken, at most `most`.
+static int run_energy(const EnergyArgs& a, int most, cudaStream_t st)
 {
+    const int64_t nn = (int64_t)(a.nz + 1) * a.nx, n = a.n[0] > a.n[1] ? a.n[0] : a.n[1];
+    const int64_t want = ((n > nn ? n : nn) + kEBlock - 1) / kEBlock;
+    const int nb = want < most ? (int)want : most;
     if (a.pot_mode == 0) k_energy<true><<<nb, kEBlock, 0, st>>>(a);
     else k_energy<false><<<nb, kEBlock, 0, st>>>(a);
+    return nb;
 }
 
 int energy_blocks(const Ctx& c) { return c.nsm * 4; }
@@ -150,9 +164,8 @@ void launch_energy(Ctx& c, cudaStream_t st, double* host_out5)
     a.pot_mode = pot_code(c.cfg);
     a.eam = eam_params(c.cfg);
     a.partials = c.partials;
-    const int nb = energy_blocks(c);
-    run_energy(a, nb, st);
-    k_energy_final<<<1, kEBlock, 0, st>>>(c.partials, nb, c.red_out);
+    const int nb = run_energy(a, energy_blocks(c), st);
+    k_energy_final<<<1, 32 * kSlots, 0, st>>>(c.partials, nb, c.red_out);
     double raw[kSlots];
     cudaMemcpyAsync(raw, c.red_out, sizeof(raw), cudaMemcpyDeviceToHost, st);
     cudaStreamSynchronize(st);
@@ -184,17 +197,13 @@ static __device__ __align__(256) double g_noalloc_scratch[kStaticBlocks * kSlots
 
 // Final pass of the workspace-free variant: adds the block partials in block order (the same
 // fixed-shape tree as k_energy_final) and writes the five energies in J per metre of y.
-__global__ void k_energy_final_scaled(const double* __restrict__ partials, int nb, double s0, double s1, double s2,
-                                      double s3, double s4, double* out)
+__global__ void __launch_bounds__(32 * kSlots)
+    k_energy_final_scaled(const double* __restrict__ partials, int nb, double s0, double s1, double s2, double s3,
+                          double s4, double* out)
 {
-    __shared__ double sh[kEBlock / 32];
-    const double scale[kSlots] = {s0, s1, s2, s3, s4};
-    for (int s = 0; s < kSlots; s++) {
-        double v = 0.0;
-        for (int b = threadIdx.x; b < nb; b += kEBlock) v += partials[(size_t)b * kSlots + s];
-        const double r = block_sum(v, sh);
-        if (threadIdx.x == 0) out[s] = r * scale[s];
-    }
+    const int s = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const double r = sum_slot(partials, nb, s, lane);
+    if (lane == 0) out[s] = r * (s == 0 ? s0 : s == 1 ? s1 : s == 2 ? s2 : s == 3 ? s3 : s4);
 }
 
 }  // namespace gbpic
@@ -255,7 +264,7 @@ extern "C" int pic_energy_noalloc(const pic_config* cfg, const pic_state_view* i
     int dev = 0, nsm = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return PIC_ECUDA;
-    const int nb = nsm * 4 < kStaticBlocks ? nsm * 4 : kStaticBlocks;
+    const int most = nsm * 4 < kStaticBlocks ? nsm * 4 : kStaticBlocks;
 
     // derived constants, as pic_init derives them
     const double w = cfg->n_atoms * cfg->dx * cfg->dx / (double)cfg->ppc_ion;
@@ -291,8 +300,8 @@ extern "C" int pic_energy_noalloc(const pic_config* cfg, const pic_state_view* i
     const cudaStream_t st = (cudaStream_t)stream;
     const double vol = cfg->dx * cfg->dx;
     const double mu0 = 1.0 / (kEps0 * kC * kC);
-    run_energy(a, nb, st);
-    k_energy_final_scaled<<<1, kEBlock, 0, st>>>(scratch, nb, w * mi * kC * kC, nsp > 1 ? w * kMe * kC * kC : 0.0,
+    const int nb = run_energy(a, most, st);
+    k_energy_final_scaled<<<1, 32 * kSlots, 0, st>>>(scratch, nb, w * mi * kC * kC, nsp > 1 ? w * kMe * kC * kC : 0.0,
                                                   0.5 * kEps0 * vol, 0.5 / mu0 * vol, 0.5 * D * w, dev_out5);
     return cudaGetLastError() == cudaSuccess ? PIC_OK : PIC_ECUDA;
 }

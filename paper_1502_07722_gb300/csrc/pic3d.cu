@@ -1006,16 +1006,11 @@ void launch_fields3(Ctx& c, cudaStream_t st, int64_t step, int64_t* launches)
 
 // ---- energies ------------------------------------------------------------------------------
 
-// a fixed-shape tree over 256 threads: lanes of a warp, then the warps
-__device__ __forceinline__ double block_sum3(double v, double* sh)
+// lanes of a warp, a fixed-shape tree (the result in lane 0)
+__device__ __forceinline__ double warp_sum3(double v)
 {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
-    __syncthreads();
-    double r = sh[0];
-    for (int w = 1; w < 8; w++) r += sh[w];
-    __syncthreads();
-    return r;
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    return v;
 }
 
 __global__ void __launch_bounds__(256) k_energy3(const Species3 s0, const Species3 s1, int64_t n0, int64_t n1, int nsp, Geo3 g,
@@ -1024,7 +1019,7 @@ __global__ void __launch_bounds__(256) k_energy3(const Species3 s0, const Specie
                                                  float h_coef, int pot_mode, float c_att, float s_rep, EamP eam,
                                                  double* partials)
 {
-    __shared__ double sh[8];
+    __shared__ double sh[5][256];
     const int64_t tid = blockIdx.x * (int64_t)256 + threadIdx.x, stride = (int64_t)gridDim.x * 256;
     Sum2 ke[2], pe;
     double fe = 0.0, fb = 0.0;
@@ -1085,23 +1080,30 @@ __global__ void __launch_bounds__(256) k_energy3(const Species3 s0, const Specie
             fb += bx * bx + by * by;
         }
     }
-    const double vals[5] = {ke[0].value(), ke[1].value(), fe, fb, pe.value()};
-#pragma unroll
-    for (int q = 0; q < 5; q++) {
-        const double r = block_sum3(vals[q], sh);
-        if (threadIdx.x == 0) partials[(size_t)blockIdx.x * 5 + q] = r;
+    // warp q adds up slot q (13 FP64 instructions per slot and block)
+    sh[0][threadIdx.x] = ke[0].value();
+    sh[1][threadIdx.x] = ke[1].value();
+    sh[2][threadIdx.x] = fe;
+    sh[3][threadIdx.x] = fb;
+    sh[4][threadIdx.x] = pe.value();
+    __syncthreads();
+    const int q = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (q < 5) {
+        double v = sh[q][lane];
+        for (int w = 1; w < 8; w++) v += sh[q][lane + 32 * w];
+        v = warp_sum3(v);
+        if (lane == 0) partials[(size_t)blockIdx.x * 5 + q] = v;
     }
 }
 
-__global__ void k_energy3_final(const double* __restrict__ partials, int nb, double* out)
+// one warp per slot, blocks assigned to lanes in a fixed way
+__global__ void __launch_bounds__(160) k_energy3_final(const double* __restrict__ partials, int nb, double* out)
 {
-    __shared__ double sh[8];
-    for (int q = 0; q < 5; q++) {
-        double v = 0.0;
-        for (int b = threadIdx.x; b < nb; b += 256) v += partials[(size_t)b * 5 + q];
-        const double r = block_sum3(v, sh);
-        if (threadIdx.x == 0) out[q] = r;
-    }
+    const int q = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double v = 0.0;
+    for (int b = lane; b < nb; b += 32) v += partials[(size_t)b * 5 + q];
+    v = warp_sum3(v);
+    if (lane == 0) out[q] = v;
 }
 
 void launch_energy3(Ctx& c, cudaStream_t st, double* host_out5)
@@ -1113,12 +1115,15 @@ void launch_energy3(Ctx& c, cudaStream_t st, double* host_out5)
         sp[s].cell = S.a.cell; sp[s].fx = S.a.fx; sp[s].fy = S.a.fy; sp[s].fz = S.a.fz;
         sp[s].ux = S.a.ux; sp[s].uy = S.a.uy; sp[s].uz = S.a.uz;
     }
-    const int nb = c.nsm * 4;
-    k_energy3<<<nb, 256, 0, st>>>(sp[0], sp[1], c.sp[0].n, c.nsp > 1 ? c.sp[1].n : 0, c.nsp, geo_of(c), c.F[0], c.F[1],
+    // small states take as many blocks as give every thread a particle or a node
+    const int64_t n1 = c.nsp > 1 ? c.sp[1].n : 0, n = c.sp[0].n > n1 ? c.sp[0].n : n1;
+    const int64_t want = ((n > (int64_t)c.nn ? n : (int64_t)c.nn) + 255) / 256;
+    const int nb = want < c.nsm * 4 ? (int)want : c.nsm * 4;
+    k_energy3<<<nb, 256, 0, st>>>(sp[0], sp[1], c.sp[0].n, n1, c.nsp, geo_of(c), c.F[0], c.F[1],
                                   c.F[2], c.F[3], c.F[4], c.F[5], c.rho[c.cur], (float)c.rho_scale,
                                   (float)(c.r0 / (6.0 * c.cfg.dx)), pot_code(c.cfg), pot_param(c.cfg),
                                   (float)c.cfg.s_rep, eam_params(c.cfg), c.partials);
-    k_energy3_final<<<1, 256, 0, st>>>(c.partials, nb, c.red_out);
+    k_energy3_final<<<1, 160, 0, st>>>(c.partials, nb, c.red_out);
     double raw[5];
     cudaMemcpyAsync(raw, c.red_out, sizeof(raw), cudaMemcpyDeviceToHost, st);
     cudaStreamSynchronize(st);
