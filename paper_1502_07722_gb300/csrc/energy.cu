@@ -51,11 +51,11 @@ __global__ void __launch_bounds__(kEBlock) k_energy(const EnergyArgs a)
             for (int q = 0; q < kBatch; q++) {
                 const int64_t p = p0 + q * stride;
                 const bool in = p < a.n[s];
-                cell[q] = in ? S.cell[p] : -1;
                 ux[q] = in ? S.ux[p] : 0.0f;
                 uy[q] = in ? S.uy[p] : 0.0f;
                 uz[q] = in ? S.uz[p] : 0.0f;
-                if (s == 0) {
+                if (s == 0) {            // the kinetic energy of the electrons needs no cell
+                    cell[q] = in ? S.cell[p] : 0;
                     fx[q] = in ? S.fx[p] : 0.0f;
                     fz[q] = in ? S.fz[p] : 0.0f;
                 }
@@ -64,14 +64,13 @@ __global__ void __launch_bounds__(kEBlock) k_energy(const EnergyArgs a)
             if (s == 0) {
 #pragma unroll
                 for (int q = 0; q < kBatch; q++) {
-                    const int c = cell[q] < 0 ? 0 : cell[q];
-                    const int k = (int)(__umulhi((unsigned)c, a.nx_magic) >> a.nx_shift), i = c - k * a.nx;
+                    const int c = cell[q], k = (int)(__umulhi((unsigned)c, a.nx_magic) >> a.nx_shift), i = c - k * a.nx;
                     gather_density<true>(a.rho, a.nx, a.nz, a.rho_s, i, k, fx[q], fz[q], n[q], dnx[q], dnz[q]);
                 }
             }
 #pragma unroll
             for (int q = 0; q < kBatch; q++) {
-                if (cell[q] < 0) continue;
+                if (p0 + q * stride >= a.n[s]) continue;
                 const float u2 = ux[q] * ux[q] + uy[q] * uy[q] + uz[q] * uz[q];
                 ke[s].add(u2 / (sqrtf(1.0f + u2) + 1.0f));
                 if (s == 0 && n[q] > 0.0f) {

@@ -1034,11 +1034,11 @@ __global__ void __launch_bounds__(256) k_energy3(const Species3 s0, const Specie
             for (int q = 0; q < 2; q++) {
                 const int64_t p = p0 + q * stride;
                 const bool in = p < ns;
-                cell[q] = in ? S.cell[p] : -1;
                 ux[q] = in ? S.ux[p] : 0.0f;
                 uy[q] = in ? S.uy[p] : 0.0f;
                 uz[q] = in ? S.uz[p] : 0.0f;
                 if (s == 0) {
+                    cell[q] = in ? S.cell[p] : 0;
                     fx[q] = in ? S.fx[p] : 0.0f;
                     fy[q] = in ? S.fy[p] : 0.0f;
                     fz[q] = in ? S.fz[p] : 0.0f;
@@ -1049,13 +1049,13 @@ __global__ void __launch_bounds__(256) k_energy3(const Species3 s0, const Specie
 #pragma unroll
                 for (int q = 0; q < 2; q++) {
                     int i, j, k;
-                    split3(cell[q] < 0 ? 0 : cell[q], g, i, j, k);
+                    split3(cell[q], g, i, j, k);
                     density3<true>(rho, g, rho_s, i, j, k, fx[q], fy[q], fz[q], dens[q], gr[q]);
                 }
             }
 #pragma unroll
             for (int q = 0; q < 2; q++) {
-                if (cell[q] < 0) continue;
+                if (p0 + q * stride >= ns) continue;
                 const float u2 = ux[q] * ux[q] + uy[q] * uy[q] + uz[q] * uz[q];
                 const float t = u2 / (sqrtf(1.0f + u2) + 1.0f);
                 if (s == 0) ke[0].add(t);
