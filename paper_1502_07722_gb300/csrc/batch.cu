@@ -45,9 +45,8 @@ struct pic_batch {
     int n;
     pic_ctx* slab[kMaxSlabs];
     cudaStream_t st;
-    int full, pot, minW, maxW, max_nx, max_nz, nsm, sort_every, steps_since_sort;
+    int full, pot, minW, maxW, nsm, sort_every;
     size_t max_nn;
-    int64_t step;
     StepArgs* args_dev;          // [2][n]: parity 0 (density in buffer 0) and parity 1
     FieldBatch fields[2];        // every slab's field arguments per parity (host copy, passed by value)
     AntennaParams* ap_dev;       // [n]
@@ -152,18 +151,35 @@ void build_items(pic_batch* b)
 }
 
 // The fields' update prepares the step after it; the first step, and one after a slab's state was
-// written from outside (a checkpoint, new particles), is prepared here.
-void prepare(pic_batch* b)
+// written from outside (a checkpoint, new particles), is prepared here. A restored slab is at its
+// checkpoint's step, so the counters of the laser pulse are taken from the slabs.
+int prepare(pic_batch* b)
 {
     build_items(b);
-    if (!b->full) return;
+    if (!b->full) return PIC_OK;
     bool ready = true;
-    for (int s = 0; s < b->n; s++) ready &= b->slab[s]->c.prepared != 0;
-    if (ready) return;
+    long long step[kMaxSlabs];
+    for (int s = 0; s < b->n; s++) {
+        ready &= b->slab[s]->c.prepared != 0;
+        step[s] = (long long)b->slab[s]->c.step;
+    }
+    if (ready) return PIC_OK;
+    // a pageable source: the call returns once the counters have been staged
+    if (cudaMemcpyAsync(b->step_dev, step, 8 * (size_t)b->n, cudaMemcpyHostToDevice, b->st) != cudaSuccess)
+        return PIC_ECUDA;
     const int parity = b->slab[0]->c.cur;
     enqueue_prepare(b, parity);
     launch_antenna_batch(b->ap_dev, b->step_dev, b->ant_dev + parity * 2 * b->n, b->n, b->st);
     b->nlaunch[3] += 2;
+    return PIC_OK;
+}
+
+// Steps since the last sort of the slab sorted longest ago (a restored slab brings its own count).
+int steps_since_sort(const pic_batch* b)
+{
+    int n = 0;
+    for (int s = 0; s < b->n; s++) n = b->slab[s]->c.steps_since_sort > n ? b->slab[s]->c.steps_since_sort : n;
+    return n;
 }
 
 int capture(pic_batch* b)
@@ -231,8 +247,6 @@ int pic_batch_init(const pic_config* cfgs, int32_t n, void* workspace, size_t by
         const Ctx& c = b->slab[s]->c;
         b->maxW = c.W > b->maxW ? c.W : b->maxW;
         b->minW = s == 0 || c.W < b->minW ? c.W : b->minW;
-        b->max_nx = c.nx > b->max_nx ? c.nx : b->max_nx;
-        b->max_nz = c.nz > b->max_nz ? c.nz : b->max_nz;
         b->max_nn = c.nn > b->max_nn ? c.nn : b->max_nn;
         b->nsm = c.nsm;
     }
@@ -274,9 +288,8 @@ int pic_batch_init(const pic_config* cfgs, int32_t n, void* workspace, size_t by
         b->fields[par].n = n;
         if (b->full) field_row_blocks(b->fields[par]);
     }
-    bool ok = cudaMemcpyAsync(b->ap_dev, ap.data(), sizeof(AntennaParams) * n, cudaMemcpyHostToDevice, b->st) ==
-                  cudaSuccess &&
-              cudaMemsetAsync(b->step_dev, 0, 8 * (size_t)n, b->st) == cudaSuccess;
+    const bool ok = cudaMemcpyAsync(b->ap_dev, ap.data(), sizeof(AntennaParams) * n, cudaMemcpyHostToDevice, b->st) ==
+                    cudaSuccess;
     r = ok ? upload_args(b) : PIC_ECUDA;
     for (int q = 0; q < 6 && r == PIC_OK; q++)
         if (cudaEventCreate(&b->ev[q]) != cudaSuccess) r = PIC_ECUDA;
@@ -311,13 +324,17 @@ int pic_batch_step(pic_batch* b, int32_t nsteps)
 {
     if (!b || nsteps < 0) return PIC_EINVAL;
     if (b->sticky) return b->sticky;
-    if (nsteps > 0) prepare(b);
+    if (nsteps > 0) {
+        const int r = prepare(b);
+        if (r) return r;
+    }
     for (int it = 0; it < nsteps; it++) {
-        if (b->sort_every > 0 && b->steps_since_sort >= b->sort_every) {
+        if (b->sort_every > 0 && steps_since_sort(b) >= b->sort_every) {
             if (b->timing) cudaEventRecord(b->ev[3], b->st);
             for (int s = 0; s < b->n; s++) {
                 Ctx& c = b->slab[s]->c;
                 for (int sp = 0; sp < c.nsp; sp++) sort_species_impl(c, sp, b->st, 0, &b->nlaunch[2]);
+                c.steps_since_sort = 0;
             }
             if (b->timing) {
                 cudaEventRecord(b->ev[4], b->st);
@@ -329,7 +346,6 @@ int pic_batch_step(pic_batch* b, int32_t nsteps)
             const int r = upload_args(b);      // the sort swapped the particle buffers
             if (r) return r;
             build_items(b);
-            b->steps_since_sort = 0;
         }
         const int parity = b->slab[0]->c.cur;
         if (b->timing) {
@@ -357,9 +373,8 @@ int pic_batch_step(pic_batch* b, int32_t nsteps)
             flip_parity(c);
             c.prepared = c.Jn[0] != nullptr;
             c.step++;
+            c.steps_since_sort++;
         }
-        b->step++;
-        b->steps_since_sort++;
     }
     if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(b->st) != cudaSuccess) return PIC_ECUDA;
     for (int s = 0; s < b->n; s++) {
