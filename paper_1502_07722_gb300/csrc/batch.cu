@@ -134,14 +134,11 @@ void enqueue_step(pic_batch* b, int parity)
 // One list of work items over every slab's tiles, after a sort or a slab's state was written.
 void build_items(pic_batch* b)
 {
-    bool ok = true;
     int64_t n = 0;
     for (int s = 0; s < b->n; s++) {
         const Ctx& c = b->slab[s]->c;
-        ok &= c.items_ok != 0;
         n += c.sp[0].n + (c.nsp > 1 ? c.sp[1].n : 0);
     }
-    if (ok) return;
     cudaMemsetAsync(b->nitems, 0, sizeof(int), b->st);
     const int chunk = item_chunk(n, particle_slots(b->nsm, b->full, 1));
     for (int s = 0; s < b->n; s++) {
@@ -151,19 +148,25 @@ void build_items(pic_batch* b)
 }
 
 // The fields' update prepares the step after it; the first step, and one after a slab's state was
-// written from outside (a checkpoint, new particles), is prepared here. A restored slab is at its
-// checkpoint's step, so the counters of the laser pulse are taken from the slabs.
+// written from outside (a checkpoint, new particles), is prepared here. A slab sorted on its own has
+// changed its two particle buffers over, and a restored one is at its checkpoint's step: the arguments
+// and the counters of the laser pulse are taken from the slabs.
 int prepare(pic_batch* b)
 {
-    build_items(b);
-    if (!b->full) return PIC_OK;
-    bool ready = true;
+    bool ready = true, listed = true;
     long long step[kMaxSlabs];
     for (int s = 0; s < b->n; s++) {
-        ready &= b->slab[s]->c.prepared != 0;
-        step[s] = (long long)b->slab[s]->c.step;
+        const Ctx& c = b->slab[s]->c;
+        listed &= c.items_ok != 0;
+        ready &= c.prepared != 0;
+        step[s] = (long long)c.step;
     }
-    if (ready) return PIC_OK;
+    if (!listed) {
+        const int r = upload_args(b);
+        if (r) return r;
+        build_items(b);
+    }
+    if (!b->full || ready) return PIC_OK;
     // a pageable source: the call returns once the counters have been staged
     if (cudaMemcpyAsync(b->step_dev, step, 8 * (size_t)b->n, cudaMemcpyHostToDevice, b->st) != cudaSuccess)
         return PIC_ECUDA;
@@ -290,7 +293,7 @@ int pic_batch_init(const pic_config* cfgs, int32_t n, void* workspace, size_t by
     }
     const bool ok = cudaMemcpyAsync(b->ap_dev, ap.data(), sizeof(AntennaParams) * n, cudaMemcpyHostToDevice, b->st) ==
                     cudaSuccess;
-    r = ok ? upload_args(b) : PIC_ECUDA;
+    r = ok && cudaStreamSynchronize(b->st) == cudaSuccess ? PIC_OK : PIC_ECUDA;
     for (int q = 0; q < 6 && r == PIC_OK; q++)
         if (cudaEventCreate(&b->ev[q]) != cudaSuccess) r = PIC_ECUDA;
     if (r) {

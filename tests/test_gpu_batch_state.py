@@ -36,3 +36,20 @@ def test_restored_slab_is_at_its_own_step(gb, sort_every):  # noqa: F811
         _same_grids(batch.slabs[i], single)
         single.close()
     batch.close()
+
+
+def test_slab_sorted_on_its_own(gb):  # noqa: F811
+    """The sort leaves the slab's particles in its second buffers; the batch moves those, and its own sorts (every 5
+    steps) go on from them."""
+    ws = small_sweep()
+    batch = gb.Batch(ws, sort_every=5)
+    batch.step(4)
+    batch.slabs[1].sort()
+    batch.step(7)
+    for i in range(3):
+        fresh, _ = batch.slabs[i].deposit_density()
+        assert fresh.equal(batch.slabs[i].get_density())
+        single = _single(gb, ws[i], 11, sort_every=5)
+        _same_grids(batch.slabs[i], single)
+        single.close()
+    batch.close()
