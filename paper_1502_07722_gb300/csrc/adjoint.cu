@@ -122,8 +122,8 @@ __device__ __forceinline__ DensAt dens_at(const u64* rho, float rho_s, int nx, i
 // transpose of the pair force given the adjoints of (Fx, Fz): position adjoints (added to lx, lz),
 // node adjoints (FP64 atomics), and the D, r0 derivative terms (gFF += lF . F, gR += dL/dr0 part)
 __device__ __forceinline__ void pair_T(const DensAt& d, const PairD& px, const PairD& pz, float lFx, float lFz,
-                                       float inv_r0, int nx, float* lam_nodes, float& lx, float& lz, Sum2& gFF,
-                                       Sum2& gR)
+                                       float inv_r0, int nx, float* lam_nodes, float& lx, float& lz, LongSum& gFF,
+                                       LongSum& gR)
 {
     gFF.add(lFx * px.F + lFz * pz.F);
     gR.add(lFx * (px.dr0 + 3.0f * inv_r0 * (px.dn * d.n + px.dq * d.qx)) +
@@ -187,7 +187,8 @@ struct AdjArgs {
 __global__ void __launch_bounds__(256) k_adjoint_a(const AdjArgs a)
 {
     __shared__ double sh[256];
-    Sum2 gFF, gR;
+    LongSum gFF, gR;
+    int terms = 0;
     const float r0_dx = (float)(a.r0 / a.dx), fu = (float)(a.D / a.r0), inv_r0 = (float)(1.0 / a.r0);
     const float rho_s = (float)a.rho_s, kick = (float)a.kick, cs0 = (float)a.cs0;
     for (int64_t ch = blockIdx.x; ch * 256 < a.n; ch += gridDim.x) {
@@ -219,6 +220,11 @@ __global__ void __launch_bounds__(256) k_adjoint_a(const AdjArgs a)
         a.lam_u[3 * p] = lux;
         a.lam_u[3 * p + 1] = luy;
         a.lam_u[3 * p + 2] = luz;
+        if (++terms == kFold) {
+            terms = 0;
+            gFF.fold();
+            gR.fold();
+        }
     }
     const double sD = block_sum_d(gFF.value(), sh), sR = block_sum_d(gR.value(), sh);
     if (threadIdx.x == 0) {
@@ -667,7 +673,8 @@ template <bool ION>
 __global__ void __launch_bounds__(256, kAdjCtas) k_adjoint_full(const FullAdjArgs a)
 {
     __shared__ double sh[256];
-    Sum2 gFF, gR;
+    LongSum gFF, gR;
+    int terms = 0;
     const size_t nn = (size_t)(a.nz + 1) * a.nx;
     float2* LExBz = reinterpret_cast<float2*>(a.lF);
     float2* LEzBx = LExBz + nn;
@@ -793,7 +800,14 @@ __global__ void __launch_bounds__(256, kAdjCtas) k_adjoint_full(const FullAdjArg
             scatter_at(LEy, s0_, vy);
             scatter_at(LBy, sxz, lB[1]);
         }
-        if (ION) pair_T(d, px, pz, a.fk * la[0], a.fk * la[2], a.inv_r0, a.nx, a.lam_nodes, lx0, lz0, gFF, gR);
+        if (ION) {
+            pair_T(d, px, pz, a.fk * la[0], a.fk * la[2], a.inv_r0, a.nx, a.lam_nodes, lx0, lz0, gFF, gR);
+            if (++terms == kFold) {
+                terms = 0;
+                gFF.fold();
+                gR.fold();
+            }
+        }
         a.lam_pos[2 * p] = lx0;
         a.lam_pos[2 * p + 1] = lz0;
     }

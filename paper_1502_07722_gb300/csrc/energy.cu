@@ -38,12 +38,13 @@ __global__ void __launch_bounds__(kEBlock) k_energy(const EnergyArgs a)
     __shared__ double sh[kSlots][kEBlock];
     const int64_t tid = blockIdx.x * (int64_t)kEBlock + threadIdx.x;
     const int64_t stride = (int64_t)gridDim.x * kEBlock;
-    Sum2 ke[2], pe;
+    LongSum ke[2], pe;
     double fe = 0.0, fb = 0.0;
 #pragma unroll
     for (int s = 0; s < 2; s++) {
         if (s >= a.nsp) break;
         const SpeciesBuf& S = a.sp[s];
+        int terms = 0;
         for (int64_t p0 = tid; p0 < a.n[s]; p0 += kBatch * stride) {
             float ux[kBatch], uy[kBatch], uz[kBatch], fx[kBatch], fz[kBatch];
             int cell[kBatch];
@@ -78,6 +79,11 @@ __global__ void __launch_bounds__(kEBlock) k_energy(const EnergyArgs a)
                     const float inv43 = fast_rcp(n[q] * cr);
                     pe.add(pair_energy_xz(cr, inv43, dnx[q], dnz[q], a.h_coef, LJ ? 0 : a.pot_mode, a.c_att, a.s_rep, a.eam));
                 }
+            }
+            if ((terms += kBatch) == kFold) {
+                terms = 0;
+                ke[s].fold();
+                if (s == 0) pe.fold();
             }
         }
     }

@@ -1021,11 +1021,12 @@ __global__ void __launch_bounds__(256) k_energy3(const Species3 s0, const Specie
 {
     __shared__ double sh[5][256];
     const int64_t tid = blockIdx.x * (int64_t)256 + threadIdx.x, stride = (int64_t)gridDim.x * 256;
-    Sum2 ke[2], pe;
+    LongSum ke[2], pe;
     double fe = 0.0, fb = 0.0;
     for (int s = 0; s < nsp; s++) {
         const Species3& S = s == 0 ? s0 : s1;
         const int64_t ns = s == 0 ? n0 : n1;
+        int terms = 0;
         for (int64_t p0 = tid; p0 < ns; p0 += 2 * stride) {
             // two particles' loads in flight together
             float ux[2], uy[2], uz[2], fx[2], fy[2], fz[2];
@@ -1064,6 +1065,12 @@ __global__ void __launch_bounds__(256) k_energy3(const Species3 s0, const Specie
                     const float cr = fast_cbrt(dens[q]), inv43 = fast_rcp(dens[q] * cr);
                     pe.add(pair_energy3(cr, inv43, gr[q], h_coef, pot_mode, c_att, s_rep, eam));
                 }
+            }
+            if ((terms += 2) == kFold) {
+                terms = 0;
+                if (s == 0) ke[0].fold();
+                else ke[1].fold();
+                if (s == 0) pe.fold();
             }
         }
     }

@@ -8,33 +8,11 @@
 //  * Regridding a cell map between stages of different cells: a conservative (volume-weighted)
 //    remap on grids placed on each other by the slab's surface and the laser axis.
 #include "pic_internal.cuh"
+#include "pic_device.cuh"
 
 namespace gbpic {
 
-// Exact enough to replace FP64: a sum of FP32 terms as three FP32 numbers, every rounding error carried to
-// the next (Knuth's two-sum), about 70 bits.
-struct Sum3 {
-    float s0, s1, s2;
-    __device__ __forceinline__ void zero() { s0 = s1 = s2 = 0.0f; }
-    __device__ __forceinline__ static float two_sum(float& s, float x)
-    {
-        const float t = __fadd_rn(s, x), b = __fsub_rn(t, s);
-        const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(x, b));
-        s = t;
-        return e;
-    }
-    __device__ __forceinline__ void add_low(float x) { s2 = __fadd_rn(s2, two_sum(s1, x)); }
-    __device__ __forceinline__ void add(float x) { add_low(two_sum(s0, x)); }
-    __device__ __forceinline__ void add_square(float x)       // x^2 = p + e exactly
-    {
-        const float p = __fmul_rn(x, x);
-        add(p);
-        add_low(__fmaf_rn(x, x, -p));
-    }
-    __device__ __forceinline__ double value() const { return ((double)s2 + (double)s1) + (double)s0; }
-};
-
-// momenta whose squares leave FP32's range (or that are not finite)
+// momenta whose squares, or the rounding errors of these, leave FP32's range (or that are not finite)
 static __device__ __noinline__ void add_wide_moments(double* acc, int64_t ncell, int at, float a, float b, float c)
 {
     const double da = a, db = b, dc = c;
