@@ -96,7 +96,8 @@ __global__ void __launch_bounds__(32 * kMomWarps)
                 if (k[q] < 0) continue;
                 at = k[q];
                 const float a = va[q], b = vb[q], c = vc[q];
-                if (!(fabsf(a) + fabsf(b) + fabsf(c) < 1e15f)) {
+                const float size = fabsf(a) + fabsf(b) + fabsf(c);       // a particle at rest has nothing to round
+                if (!(size < 1e15f) || (size < 0x1p-40f && size > 0.0f)) {
                     add_wide_moments(acc, ncell, at, a, b, c);
                     continue;
                 }
