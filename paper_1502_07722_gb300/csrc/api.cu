@@ -108,7 +108,7 @@ int derive_layout(const pic_config* cfg, Layout& L)
     if (L.items >= (1LL << 31)) return PIC_EINVAL;
     t += align256(sizeof(WorkItem) * (size_t)L.items) + align256(4);
     const size_t plane = (size_t)L.nx * L.ny;
-    t += 2 * align256(4 * plane);
+    t += 2 * align256(4 * plane) + align256(16);
     t += 2 * align256(4 * ((size_t)L.nkeys + 1));
     t += align256(4 * (((size_t)L.nkeys + 2047) / 2048 + 1));
     t += align256(8 * 5 * (size_t)kMaxEnergyBlocks) + align256(8 * 8) + align256(32);
@@ -196,8 +196,8 @@ int redeposit(Ctx& c)
 }
 
 // The currents a step deposits into start clear (the transport stage has none) and the next node
-// density from the current one (the particle kernel adds the changes). The field update of the step
-// before has done both.
+// density from the current one (the particle kernel adds the changes); with fields the antenna scalars of
+// the step are evaluated. The field update of the step before has done all of it.
 int prepare_step(Ctx& c)
 {
     const bool twin = c.Jn[0] != nullptr;
@@ -208,6 +208,10 @@ int prepare_step(Ctx& c)
         if (c.cfg.mode == PIC_MODE_FULL)
             for (int q = 0; q < 3; q++) prep[n++] = CopySeg{nullptr, J[q], 8 * c.nn};
         c.nlaunch[3] += launch_copy_segments(c, prep, n, c.stream);
+        if (c.cfg.mode == PIC_MODE_FULL) {
+            launch_antenna(c, c.stream, c.step);
+            c.nlaunch[3]++;
+        }
         CK(cudaGetLastError());
     }
     if (twin) swap_currents(c);
@@ -372,6 +376,7 @@ int pic_init(const pic_config* cfg, void* workspace, size_t workspace_bytes, voi
     const size_t plane = (size_t)L.nx * L.ny;
     c.ant_c = cv.take<float>(plane);
     c.ant_s = cv.take<float>(plane);
+    c.ant = cv.take<float>(4);
     c.keys_count = cv.take<int32_t>((size_t)L.nkeys + 1);
     c.keys_off = cv.take<int32_t>((size_t)L.nkeys + 1);
     c.scan_tmp = cv.take<int32_t>(((size_t)L.nkeys + 2047) / 2048 + 1);

@@ -12,6 +12,7 @@
 // What bounds it: memory traffic on the large grids, the launch on the small ones. Against three
 // in-place passes (B half, E, B half) with a copy/clear kernel and a one-thread antenna kernel, a
 // node moves 112 bytes instead of 172 and a step has two launches instead of six.
+#include "pic_device.cuh"
 #include "pic_internal.cuh"
 
 namespace gbpic {
@@ -167,9 +168,16 @@ static int field_blocks(const FieldArgs& f)
     return (items + w - 1) / w;
 }
 
-__global__ void __launch_bounds__(kFieldThreads, 8) k_fields(const __grid_constant__ FieldArgs f)
+// The first block evaluates the antenna scalars of the next step (it starts first: on the smallest grids the other
+// blocks take as long).
+__global__ void __launch_bounds__(kFieldThreads, 8)
+    k_fields(const __grid_constant__ FieldArgs f, const __grid_constant__ AntennaParams ap, long long next, float* ant_next)
 {
-    field_item(f, (int)(blockIdx.x * (kFieldThreads / 32) + threadIdx.x / 32), f.ant0, f.ant1);
+    if (blockIdx.x == 0) {
+        if (threadIdx.x == 0) antenna_scalars(ap, next, ant_next);
+        return;
+    }
+    field_item(f, (int)((blockIdx.x - 1) * (kFieldThreads / 32) + threadIdx.x / 32), f.ant[0], f.ant[1]);
 }
 
 // All slabs of a batch: blockIdx.x runs over every slab's blocks, slab s owning blocks rb[s] ..
@@ -195,7 +203,11 @@ __global__ void __launch_bounds__(kFieldThreads, 8)
     field_item(f, (g - P.rb[s]) * (kFieldThreads / 32) + (int)threadIdx.x / 32, f.ant[0], f.ant[1]);
 }
 
-// antenna scalars of the step each slab is at
+// antenna scalars of the step a simulation, or each slab of a batch, is at
+__global__ void k_antenna(const __grid_constant__ AntennaParams p, long long step, float* ant)
+{
+    antenna_scalars(p, step, ant);
+}
 __global__ void k_antenna_batch(const AntennaParams* p, const long long* step, float* ant, int nslab)
 {
     const int s = threadIdx.x;
@@ -244,8 +256,7 @@ FieldArgs make_field_args(const Ctx& c)
     f.rho_next = c.rho[1 - c.cur];
     f.antc = c.ant_c;
     f.ants = c.ant_s;
-    f.ant = nullptr;
-    f.ant0 = f.ant1 = 0.0f;
+    f.ant = c.ant + 2 * (c.step & 1);
     f.k_flux = c.k_ant - 1 >= 1 ? c.k_ant - 1 : -1;
     f.flux = c.red_out + 5;
     return f;
@@ -253,14 +264,16 @@ FieldArgs make_field_args(const Ctx& c)
 
 void launch_fields(Ctx& c, cudaStream_t st, int64_t step, int64_t* launches)
 {
-    FieldArgs f = make_field_args(c);
-    float ant[2];
-    antenna_scalars(make_antenna_params(c), (long long)step, ant);
-    f.ant0 = ant[0];
-    f.ant1 = ant[1];
-    k_fields<<<field_blocks(f), kFieldThreads, 0, st>>>(f);
+    const FieldArgs f = make_field_args(c);
+    k_fields<<<1 + field_blocks(f), kFieldThreads, 0, st>>>(f, make_antenna_params(c), (long long)step + 1,
+                                                            c.ant + 2 * ((step + 1) & 1));
     swap_fields(c);
     if (launches) *launches += 1;
+}
+
+void launch_antenna(const Ctx& c, cudaStream_t st, int64_t step)
+{
+    k_antenna<<<1, 1, 0, st>>>(make_antenna_params(c), (long long)step, c.ant + 2 * (step & 1));
 }
 
 void launch_antenna_batch(const AntennaParams* ap_dev, const long long* step_dev, float* ant, int n, cudaStream_t st)

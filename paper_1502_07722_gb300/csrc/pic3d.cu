@@ -816,7 +816,10 @@ struct Field3 {
     int k_ant;
     int seg;              // planes per block
     float h_b, h_e, cj, mur;
-    float ant0, ant1;     // this step's antenna scalars
+    const float* ant;     // 2: this step's antenna scalars
+    AntennaParams ap;     // for the next step's, into ant_next
+    long long next;
+    float* ant_next;
     const float* F[6];    // read
     float* G[6];          // written
     const u64* J[3];      // this step's currents
@@ -859,7 +862,7 @@ __global__ void __launch_bounds__(32 * kWarps3, 2) k_fields3(const __grid_consta
     const int k0 = (int)blockIdx.z * f.seg, k1 = blockIdx.z + 1 == gridDim.z ? nz + 1 : k0 + f.seg;
     const size_t plane = (size_t)g.nx * g.ny;
     const size_t col = (size_t)gj * g.nx + gi;
-    const float antc = f.antc[col], ants = f.ants[col];
+    const float antc = f.antc[col], ants = f.ants[col], ant0 = f.ant[0], ant1 = f.ant[1];
     const int r0 = k0 > 0 ? k0 - 1 : 0;
     size_t c = (size_t)r0 * plane + col;
     F3 e = {__ldg(f.F[0] + c), __ldg(f.F[1] + c), __ldg(f.F[2] + c)};                     // old E of plane r
@@ -899,7 +902,7 @@ __global__ void __launch_bounds__(32 * kWarps3, 2) k_fields3(const __grid_consta
         F3 n = e;
         if (r > 0 && r < nz) {
             float v = e.x + f.h_e * ((b.z - bzj) - (b.y - bp.y)) - f.cj * (float)(long long)jx;
-            if (r == f.k_ant) v += antc * f.ant0 + ants * f.ant1;
+            if (r == f.k_ant) v += antc * ant0 + ants * ant1;
             n.x = v;
             n.y = e.y + f.h_e * ((b.x - bp.x) - (b.z - bzi)) - f.cj * (float)(long long)jy;
         }
@@ -967,6 +970,8 @@ __global__ void __launch_bounds__(32 * kWarps3, 2) k_fields3(const __grid_consta
             f.G[5][q] = bp.z + f.h_b * ((snx[wp][lane] - np.x) - (npyi - np.y));
         }
     }
+    // the first block, done first, evaluates the next step's antenna scalars
+    if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0) antenna_scalars(f.ap, f.next, f.ant_next);
 }
 
 void launch_fields3(Ctx& c, cudaStream_t st, int64_t step, int64_t* launches)
@@ -979,10 +984,10 @@ void launch_fields3(Ctx& c, cudaStream_t st, int64_t step, int64_t* launches)
     f.cj = (float)(kQe * c.w / (6.0 * 4398046511104.0 * c.cfg.dx * c.cfg.dx * kEps0));
     const double cdt = kC * c.dt;
     f.mur = (float)((cdt - c.cfg.dx) / (cdt + c.cfg.dx));
-    float ant[2];
-    antenna_scalars(make_antenna_params(c), (long long)step, ant);
-    f.ant0 = ant[0];
-    f.ant1 = ant[1];
+    f.ant = c.ant + 2 * (step & 1);
+    f.ap = make_antenna_params(c);
+    f.next = (long long)step + 1;
+    f.ant_next = c.ant + 2 * ((step + 1) & 1);
     for (int q = 0; q < 6; q++) f.F[q] = c.F[q];
     for (int q = 0; q < 6; q++) f.G[q] = c.Fn[q];
     for (int q = 0; q < 3; q++) f.J[q] = c.J[q];

@@ -67,6 +67,27 @@ struct LongSum {
     __device__ __forceinline__ double value() const { return s + t.value(); }
 };
 
+// Antenna amplitude of one step (FP64):
+//   E_x += 2 (c dt / dx) E0 env(t) amp(x) sin(w (t - t_ant) + phi(x))
+// split as ant[0] * amp cos(phi) + ant[1] * amp sin(phi) with ant = A (sin, cos)(w (t - t_ant)).
+// Evaluated on the device alone, and not inlined: the single runs of one machine and another, and the slabs of a
+// batch, then round the same FP64 values (a host's mathematics library differs from the device's in the
+// last bit, which one step in 2^32 shows after the rounding to FP32). The field update of a step evaluates the next step's
+// beside its own work (a launch of one thread took 5.3 us).
+static __device__ __noinline__ void antenna_scalars(const AntennaParams& p, long long step, float* ant)
+{
+    float s = 0.0f, c = 0.0f;
+    if (p.on) {
+        const double tau = ((double)step + 0.5) * p.dt - p.t_ant;
+        const double env = exp(-2.0 * 0.6931471805599453 * tau * tau / (p.tau_fwhm * p.tau_fwhm));
+        const double a = p.coef * env;
+        s = (float)(a * sin(p.omega * tau));
+        c = (float)(a * cos(p.omega * tau));
+    }
+    ant[0] = s;
+    ant[1] = c;
+}
+
 // Pair-species node sum with the wall rows doubled (mirror image of the slab behind a wall).
 __device__ __forceinline__ long long rho_node(const u64* __restrict__ rho, int nx, int nz, int i, int k)
 {

@@ -156,6 +156,7 @@ struct Ctx {
     int32_t items_ok;     // the list matches the tile offsets
     float* ant_c;         // nx: amplitude * cos(phase(x)) at x = i + 1/2
     float* ant_s;         // nx: amplitude * sin(phase(x))
+    float* ant;           // 2 x 2: antenna scalars of the even and the odd steps (written on the device)
     // scratch
     int32_t* keys_count;  // nkeys + 1
     int32_t* keys_off;    // nkeys + 1
@@ -184,25 +185,6 @@ struct AntennaParams {
     double dt, t_ant, tau_fwhm, omega, coef;
 };
 
-// Antenna amplitude of one step (FP64):
-//   E_x += 2 (c dt / dx) E0 env(t) amp(x) sin(w (t - t_ant) + phi(x))
-// split as ant[0] * amp cos(phi) + ant[1] * amp sin(phi) with ant = A (sin, cos)(w (t - t_ant)).
-// A single simulation evaluates it on the host with the launch's arguments (one thread of the GPU
-// took 5.3 us for it); a batch, whose steps are replayed from a graph, on the device.
-__host__ __device__ inline void antenna_scalars(const AntennaParams& p, long long step, float* ant)
-{
-    float s = 0.0f, c = 0.0f;
-    if (p.on) {
-        const double tau = ((double)step + 0.5) * p.dt - p.t_ant;
-        const double env = exp(-2.0 * 0.6931471805599453 * tau * tau / (p.tau_fwhm * p.tau_fwhm));
-        const double a = p.coef * env;
-        s = (float)(a * sin(p.omega * tau));
-        c = (float)(a * cos(p.omega * tau));
-    }
-    ant[0] = s;
-    ant[1] = c;
-}
-
 // Everything the 2D field kernel needs for one simulation.
 struct FieldArgs {
     int nx, nz, k_ant;
@@ -212,7 +194,6 @@ struct FieldArgs {
     float cj;            // J2x, J2z -> dt J / eps0
     float cjy;           // J6y -> dt J_y / eps0
     float mur;           // (c dt - dx) / (c dt + dx)
-    float ant0, ant1;    // this step's antenna scalars (single simulation)
     const float* F[6];   // read
     float* G[6];         // written
     const u64* J[3];     // this step's currents
@@ -221,7 +202,7 @@ struct FieldArgs {
     u64* rho_next;       // starts as its copy
     const float* antc;   // nx: amplitude * cos(phase(x))
     const float* ants;   // nx: amplitude * sin(phase(x))
-    const float* ant;    // 2: this step's antenna scalars (batch)
+    const float* ant;    // 2: this step's antenna scalars
     int k_flux;          // node row below the antenna: Poynting flux of the injected energy
     double* flux;        // accumulates sum (Ex By - Ey Bx) over that row at the half step
 };
@@ -272,6 +253,7 @@ struct FieldBatch {
 };
 void launch_fields_batch(const FieldBatch& P, const AntennaParams* ap_dev, long long* step_dev, float* ant_next,
                          cudaStream_t st);
+void launch_antenna(const Ctx& c, cudaStream_t st, int64_t step);
 void launch_antenna_batch(const AntennaParams* ap_dev, const long long* step_dev, float* ant, int n, cudaStream_t st);
 void field_row_blocks(FieldBatch& P);
 FieldArgs make_field_args(const Ctx& c);
