@@ -100,7 +100,6 @@ __device__ __forceinline__ float gather3(const float* __restrict__ A, const Geo3
 }
 
 // trilinear node density (units n0) and its exact gradient (units n0 per cell); wall rows doubled
-template <bool NARROW = false>   // as gather_density
 __device__ __forceinline__ void density3(const u64* __restrict__ rho, const Geo3& g, float rho_s, int i, int j, int k,
                                          float fx, float fy, float fz, float& n, float* grad)
 {
@@ -114,7 +113,7 @@ __device__ __forceinline__ void density3(const u64* __restrict__ rho, const Geo3
             for (int a = 0; a < 2; a++) {
                 long long r = (long long)__ldg(rho + idx3(g, a ? i1 : i, b ? j1 : j, k + c));
                 if (k + c == 0 || k + c == g.nz) r *= 2;
-                v[c * 4 + b * 2 + a] = rho_s * (NARROW ? i64_f32(r) : (float)r);
+                v[c * 4 + b * 2 + a] = rho_s * (float)r;
             }
     const float gx = 1.0f - fx, gy = 1.0f - fy, gz = 1.0f - fz;
     // along x: differences of the x-pairs weighted in y and z
@@ -1018,7 +1017,10 @@ __device__ __forceinline__ double warp_sum3(double v)
     return v;
 }
 
-__global__ void __launch_bounds__(256) k_energy3(const Species3 s0, const Species3 s1, int64_t n0, int64_t n1, int nsp, Geo3 g,
+// Four blocks per SM, all that are launched, so that they run at once: without the bound the kernel takes 76 registers
+// and three fit (37.7 M particles 694 us with one particle at a time and FP64 sums, 1048 with three blocks and the density
+// conversions by i64_f32, 659 with four, 535 with plain conversions).
+__global__ void __launch_bounds__(256, 4) k_energy3(const Species3 s0, const Species3 s1, int64_t n0, int64_t n1, int nsp, Geo3 g,
                                                  const float* F0, const float* F1, const float* F2, const float* F3,
                                                  const float* F4, const float* F5, const u64* rho, float rho_s,
                                                  float h_coef, int pot_mode, float c_att, float s_rep, EamP eam,
@@ -1056,7 +1058,7 @@ __global__ void __launch_bounds__(256) k_energy3(const Species3 s0, const Specie
                 for (int q = 0; q < 2; q++) {
                     int i, j, k;
                     split3(cell[q], g, i, j, k);
-                    density3<true>(rho, g, rho_s, i, j, k, fx[q], fy[q], fz[q], dens[q], gr[q]);
+                    density3(rho, g, rho_s, i, j, k, fx[q], fy[q], fz[q], dens[q], gr[q]);
                 }
             }
 #pragma unroll
