@@ -67,7 +67,7 @@ struct Window {
     float2* eyn;
     float* by;
     float* nh;
-    int ox, oz, W;
+    int ox1, oz, W;           // grid column of the window's second column, grid row of its first row
 };
 
 // bilinear sum of the corners (c00, c10, c01, c11) of a stagger pair, both components at once
@@ -199,16 +199,18 @@ __device__ __forceinline__ void process_particle(const StepArgs& a, const Specie
     int i, k;
     split_cell(cell0, a, i, k);
 
-    // window coordinates (w.ox lies in [0, nx): a column left of it is one period further on)
-    unsigned lx = (unsigned)(i - w.ox);
-    lx = min(lx, lx + (unsigned)nx);
+    // window coordinates (w.ox1 lies in [0, nx): a column left of it is one period further on). A particle is
+    // inside from the window's second column on, so the period is taken there: on a grid narrower than the window
+    // its first column is the same as a later one.
+    unsigned lx1 = (unsigned)(i - w.ox1);
+    lx1 = min(lx1, lx1 + (unsigned)nx);
     const int lz = k - w.oz;
-    const bool inwin = lx - 1u < (unsigned)(W - 3) && (unsigned)(lz - 1) < (unsigned)(W - 3);
+    const bool inwin = lx1 < (unsigned)(W - 3) && (unsigned)(lz - 1) < (unsigned)(W - 3);
 
     float kx = 0.f, ky = 0.f, kz = 0.f, bx = 0.f, by = 0.f, bz = 0.f;
     float n = 0.f, dnx = 0.f, dnz = 0.f;
     if (inwin) {
-        const int base = lz * W + (int)lx;
+        const int base = lz * W + (int)lx1 + 1;
         const float gx = 1.0f - fx, gz = 1.0f - fz;
         if (kFields) {
             // four stagger patterns: (0,0) Ey, n; (1/2,0) Ex, Bz; (0,1/2) Ez, Bx; (1/2,1/2) By
@@ -407,13 +409,14 @@ __device__ __forceinline__ void run_item(const StepArgs& a, const WorkItem& item
 
     const int t = item.tile, tx = t % a.ntx, tz = t / a.ntx;
     const int q0[2] = {item.p0[0], item.p0[1]}, q1[2] = {item.p1[0], item.p1[1]};
-    w.ox = wrap_any(tx * a.T - kMargin - 1, a.nx);
+    const int ox = wrap_any(tx * a.T - kMargin - 1, a.nx);
+    w.ox1 = ox + 1 == a.nx ? 0 : ox + 1;
     w.oz = tz * a.T - kMargin - 1;
     // stage the window: fields, pair density (wall rows doubled)
 #pragma unroll
     for (int j = threadIdx.x; j < WW; j += kBlock) {
         const int b = j / W, c = j - b * W;
-        int gx = w.ox + c;
+        int gx = ox + c;
         while (gx >= a.nx) gx -= a.nx;
         const int gz = w.oz + b;
         const int gn = min(max(gz, 0), a.nz);          // node rows 0..nz

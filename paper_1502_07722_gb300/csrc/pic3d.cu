@@ -213,7 +213,7 @@ __device__ __noinline__ void deposit3_general(Geo3 g, u64* J0, u64* J1, u64* J2,
 // (the same values the global gathers clamp to).
 struct Win3 {
     const float* f;         // fields and density, laid out as Lay3 says
-    int ox, oy, oz, W;
+    int ox1, oy1, oz, W;    // grid column and row of the window's second ones, grid plane of its first
 };
 
 // Window gathers. Every component of a particle reads the corners of one cell of the window: the
@@ -409,26 +409,27 @@ __device__ __forceinline__ void process3(const Args3& a, const Species3& S, cons
     float ux = S.ux[p], uy = S.uy[p], uz = S.uz[p];
     int i, j, k;
     split3(cell, g, i, j, k);
-    // window coordinates (w.ox, w.oy lie in [0, n): a node before them is one period further on)
+    // window coordinates from its second column and row on, as in 2D (w.ox1, w.oy1 lie in [0, n): a node before
+    // them is one period further on)
     const int W = WC ? WC : w.W;
-    unsigned lx = (unsigned)(i - w.ox), ly = (unsigned)(j - w.oy);
-    lx = min(lx, lx + (unsigned)g.nx);
-    ly = min(ly, ly + (unsigned)g.ny);
+    unsigned lx1 = (unsigned)(i - w.ox1), ly1 = (unsigned)(j - w.oy1);
+    lx1 = min(lx1, lx1 + (unsigned)g.nx);
+    ly1 = min(ly1, ly1 + (unsigned)g.ny);
     const int lz = k - w.oz;
-    const bool inwin = W > 0 && lx - 1u < (unsigned)(W - 3) && ly - 1u < (unsigned)(W - 3) &&
-                       (unsigned)(lz - 1) < (unsigned)(W - 3);
+    const bool inwin = W > 0 && lx1 < (unsigned)(W - 3) && ly1 < (unsigned)(W - 3) && (unsigned)(lz - 1) < (unsigned)(W - 3);
     float kx = 0.f, ky = 0.f, kz = 0.f, bx = 0.f, by = 0.f, bz = 0.f;
     float n = 0.f, gr[3] = {0.f, 0.f, 0.f};
     if (inwin) {
         const Lay3<WC> L{W};
         if (FULL) {
             float o[6];
-            wfields3<WC>(w.f, W, lz * L.sz() + (int)ly * L.sy() + (int)lx, fx, fy, fz, o);
+            wfields3<WC>(w.f, W, lz * L.sz() + ((int)ly1 + 1) * L.sy() + (int)lx1 + 1, fx, fy, fz, o);
             kx = S.e_kick * o[0]; ky = S.e_kick * o[1]; kz = S.e_kick * o[2];
             bx = o[3]; by = o[4]; bz = o[5];
         }
         if (PAIR)
-            wdensity3<WC>(w.f + L.template density<FULL>(), W, (lz * W + (int)ly) * W + (int)lx, fx, fy, fz, n, gr);
+            wdensity3<WC>(w.f + L.template density<FULL>(), W, (lz * W + (int)ly1 + 1) * W + (int)lx1 + 1, fx, fy, fz, n,
+                          gr);
     } else {
         float o[10];
         gather_global3(a.F[0], a.F[1], a.F[2], a.F[3], a.F[4], a.F[5], a.rho_cur, g, a.rho_s, FULL ? 1 : 0,
@@ -552,14 +553,15 @@ __global__ void __launch_bounds__(kBlock3, FULL ? kCtas3 : kCtas3Atoms) k_partic
         for (int s = 0; s < a.nsp; s++) cnt += a.sp[s].tile_start[t + 1] - a.sp[s].tile_start[t];
         if (cnt == 0) continue;
         const int tx = t % a.ntx, ty = (t / a.ntx) % a.nty, tz = t / (a.ntx * a.nty);
-        w.ox = wrapn(tx * a.T - 1, g.nx);
-        w.oy = wrapn(ty * a.T - 1, g.ny);
+        const int ox = wrapn(tx * a.T - 1, g.nx), oy = wrapn(ty * a.T - 1, g.ny);
+        w.ox1 = tx * a.T;
+        w.oy1 = ty * a.T;
         w.oz = tz * a.T - 1;
         if (W > 0) {
             __syncthreads();                       // the previous tile is done with the window
             for (int q = threadIdx.x; q < WWW; q += kBlock3) {
                 const int c = q / WW, r = q - c * WW, b = r / W, e = r - b * W;
-                int gx = w.ox + e, gy = w.oy + b;
+                int gx = ox + e, gy = oy + b;
                 while (gx >= g.nx) gx -= g.nx;
                 while (gy >= g.ny) gy -= g.ny;
                 const int gz = w.oz + c;
