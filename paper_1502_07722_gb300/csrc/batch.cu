@@ -140,7 +140,7 @@ void build_items(pic_batch* b)
         n += c.sp[0].n + (c.nsp > 1 ? c.sp[1].n : 0);
     }
     cudaMemsetAsync(b->nitems, 0, sizeof(int), b->st);
-    const int chunk = item_chunk(n, particle_slots(b->nsm, b->full, 1));
+    const int chunk = item_chunk(n, particle_slots(b->nsm, b->full, 1, b->maxW));
     for (int s = 0; s < b->n; s++) {
         launch_work_items(b->slab[s]->c, s, chunk, b->items, b->nitems, b->items_cap, b->st);
         b->slab[s]->c.items_ok = 1;

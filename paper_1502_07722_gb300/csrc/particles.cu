@@ -585,7 +585,8 @@ __global__ void __launch_bounds__(kItemThreads) k_work_items(const int32_t* __re
     if (threadIdx.x == 0) *nitems = base;
 }
 
-// Particles per work item: about four items per resident CTA, at least 512 particles (an item costs its
+// Particles per work item: about four items per resident CTA (counted as if nine fitted, tiles of 64 cells had items of a
+// ninth of the size and staged nine times as much: 0.73 -> 1.25 ms a step for 8.4 M particles), at least 512 particles (an item costs its
 // window's staging: 403 x 311 cells of 13 + 13 particles 0.041 ms per launch at 512, 0.048 at 300). With
 // fewer than 512 particles per CTA the launch is one chain of latencies and takes one round of the CTA's
 // threads per species (64^2 cells of 8 + 8: 14.1 us at 512, 12.6 at 256).
@@ -605,12 +606,17 @@ void launch_work_items(const Ctx& c, int slab, int chunk, WorkItem* items, int* 
                                              chunk, items, nitems, cap);
 }
 
-int particle_slots(int nsm, int full, int batch)
+size_t particle_smem_bytes(int W) { return sizeof(unsigned) * (size_t)7 * W * W; }
+
+// Resident CTAs of the particle kernel: the registers' limit, or that of the windows in an SM's shared memory (228
+// KB, 1 KB of it per CTA the system's) for tiles above 22 cells.
+int particle_slots(int nsm, int full, int batch, int W)
 {
-    return nsm * (batch ? kCtasPerSmBatch : (full ? kCtasPerSm : kCtasPerSmAtoms));
+    const int regs = batch ? kCtasPerSmBatch : (full ? kCtasPerSm : kCtasPerSmAtoms);
+    const int smem = (int)(228 * 1024 / (particle_smem_bytes(W) + 1024 + sizeof(WorkItem) + sizeof(int)));
+    return nsm * (smem < 1 ? 1 : (smem < regs ? smem : regs));
 }
 
-size_t particle_smem_bytes(int W) { return sizeof(unsigned) * (size_t)7 * W * W; }
 
 // The kernel instances: Eq. (3), the altered potential and the Morse form, on the cubic and the
 // HCP lattice, and the embedded-atom form on the cubic lattice (potential code in bits 0-1,
@@ -642,7 +648,7 @@ void launch_particle_step(Ctx& c, const StepArgs& a, cudaStream_t st)
 #undef GBPIC_ATTR
         configured[dev].store(shmem);
     }
-    const int grid = particle_slots(c.nsm, a.full, 0);
+    const int grid = particle_slots(c.nsm, a.full, 0, a.W);
     if (!c.items_ok) {
         const int64_t n = c.sp[0].n + (c.nsp > 1 ? c.sp[1].n : 0);
         cudaMemsetAsync(c.nitems, 0, sizeof(int), st);
@@ -683,7 +689,7 @@ void launch_particle_step_batch(const StepArgs* args_dev, int nslab, const WorkI
 #undef GBPIC_ATTR
         configured[dev].store(shmem);
     }
-    const int grid = particle_slots(nsm, full, 1);
+    const int grid = particle_slots(nsm, full, 1, maxW);
     // pot: the instance code shared by every slab (potential and lattice); the compiled-in window
     // edge when every slab has it
     switch ((pot & 7) | (full ? 8 : 0) | (minW == kWin && maxW == kWin ? 16 : 0)) {

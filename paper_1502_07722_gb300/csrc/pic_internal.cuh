@@ -262,7 +262,7 @@ void launch_particle_step_batch(const StepArgs* args_dev, int nslab, const WorkI
                                 int pot, int minW, int maxW, int nsm, cudaStream_t st);
 int64_t work_item_cap(int64_t n, int64_t ntiles);
 void launch_work_items(const Ctx& c, int slab, int chunk, WorkItem* items, int* nitems, int cap, cudaStream_t st);
-int particle_slots(int nsm, int full, int batch);
+int particle_slots(int nsm, int full, int batch, int W);
 int item_chunk(int64_t n, int slots);
 int64_t work_item_cap_of(const pic_config* cfg);     // 0 for an invalid configuration
 size_t particle_smem_bytes(int W);
