@@ -115,6 +115,33 @@ __global__ void __launch_bounds__(32 * kMomWarps)
     if (nq > 0) drain(nq);
 }
 
+// One FP64 reduction per particle and sum.
+__global__ void k_cell_moments_direct(const int32_t* __restrict__ cell, const float* __restrict__ ux,
+                                      const float* __restrict__ uy, const float* __restrict__ uz, int64_t n, int64_t ncell,
+                                      double* __restrict__ acc)
+{
+    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t q = cell[p];
+        const double a = ux[p], b = uy[p], c = uz[p];
+        atomicAdd(acc + q, 1.0);
+        atomicAdd(acc + ncell + q, a);
+        atomicAdd(acc + 2 * ncell + q, b);
+        atomicAdd(acc + 3 * ncell + q, c);
+        atomicAdd(acc + 4 * ncell + q, a * a + b * b + c * c);
+    }
+}
+
+// Which of the two: the walk pays for its serial loads, queue and conversions with long runs and many of them. Whole
+// call, us, walk / direct after 43 steps: 0.5 M particles at 8 per cell 28 / 23 (2D) and 31 / 23 (3D), at 64 per cell
+// 27 / 23 and 28 / 25; 1 M at 16 per cell 31 / 27 and 37 / 29; 2 M at 32 per cell 39 / 40 and 45 / 45; 8 M at 8
+// per cell 140 / 158 and 179 / 162, at 32 per cell 87 / 119 and 111 / 124; 24 M at 32 per cell 196 / 324 and 240 / 322.
+// Lone particles have no runs (24 M: 1490 / 1243 in 2D), and below 12 per cell the rows of the layout have 8 records, which cut
+// the runs of a count that does not divide 8 (24 M at 9 per cell: 489 / 435 and 518 / 435).
+static bool direct_moments(const Ctx& c, const Species& S)
+{
+    return S.n < (c.dims == 3 ? 3 << 19 : 1 << 20) || S.ppc < 2 || (S.ppc < 12 && 8 % S.ppc != 0);
+}
+
 __global__ void k_cell_temperature(const double* __restrict__ acc, int64_t ncell, double mc2_3k, double* __restrict__ T)
 {
     for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < ncell; q += (int64_t)gridDim.x * blockDim.x) {
@@ -151,9 +178,13 @@ void launch_cell_temperature(Ctx& c, int s, double* work, double* T, cudaStream_
     const Species& S = c.sp[s];
     const int64_t ncell = (int64_t)c.nx * c.ny * c.nz;
     cudaMemsetAsync(work, 0, sizeof(double) * 5 * (size_t)ncell, st);
-    const int cols = run_columns(c, S);
-    if (S.n > 0)
-        k_cell_moments<<<2 * run_grid(c, S.n, cols), 32 * kMomWarps, 0, st>>>(S.a.cell, S.a.ux, S.a.uy, S.a.uz, S.n, ncell, cols, work);
+    if (S.n > 0 && direct_moments(c, S)) {
+        k_cell_moments_direct<<<grid_of(c, S.n), 256, 0, st>>>(S.a.cell, S.a.ux, S.a.uy, S.a.uz, S.n, ncell, work);
+    } else if (S.n > 0) {
+        const int cols = run_columns(c, S);
+        k_cell_moments<<<2 * run_grid(c, S.n, cols), 32 * kMomWarps, 0, st>>>(S.a.cell, S.a.ux, S.a.uy, S.a.uz, S.n, ncell,
+                                                                              cols, work);
+    }
     k_cell_temperature<<<grid_of(c, ncell), 256, 0, st>>>(work, ncell, S.mass * kC * kC / (3.0 * kKb), T);
 }
 
