@@ -32,8 +32,10 @@ constexpr int kCtas3 = 3, kCtas3Atoms = 4;
 // tiles left most of the chip idle. Every item stages its tile's window, seven arrays with fields and the
 // density alone without. ms per launch, whole tiles -> parts: 37 x 27 x 32 cells of 16 + 16 particles 0.176 ->
 // 0.041, 90 x 80 x 60 of 8 + 8 0.205 -> 0.118 (at 2 per CTA 0.126), 88 x 246 x 28 of 9 atoms 0.143 -> 0.083
-// (at 2 per CTA 0.087).
-constexpr int kMaxLog2Sub3 = 4, kFill3 = 1, kFill3Atoms = 4;
+// (at 2 per CTA 0.087). Past one item per CTA a part keeps at least kMinPart3
+// particles on average, a round of the CTA's threads (96 x 64 x 64 cells of 1 atom 43 -> 41 us a step; a bound on the
+// first parts too took 25 instead of 21 us on 24^3 cells of 4 atoms).
+constexpr int kMaxLog2Sub3 = 4, kFill3 = 1, kFill3Atoms = 4, kMinPart3 = 256;
 
 __device__ __forceinline__ int wrapn(int i, int n) { return i < 0 ? i + n : (i >= n ? i - n : i); }
 __device__ __forceinline__ int qoff3(float f) { return __float2int_rn(f * 16384.0f); }
@@ -559,6 +561,10 @@ __global__ void __launch_bounds__(kBlock3, FULL ? kCtas3 : kCtas3Atoms) k_partic
         w.oz = tz * a.T - 1;
         if (W > 0) {
             __syncthreads();                       // the previous tile is done with the window
+            // (the density alone: three nodes' loads in flight, as 64 registers would leave one; a step of 0.2 M atoms at one
+            // per cell 40.9 -> 37.5 us)
+            constexpr int kStage = FULL ? 1 : 3;
+#pragma unroll kStage
             for (int q = threadIdx.x; q < WWW; q += kBlock3) {
                 const int c = q / WW, r = q - c * WW, b = r / W, e = r - b * W;
                 int gx = ox + e, gy = oy + b;
@@ -677,8 +683,12 @@ void launch_particle_step3(Ctx& c, cudaStream_t st)
         configured[dev].store(shmem);
     }
     const int slots = c.nsm * (a.full ? kCtas3 : kCtas3Atoms);
-    a.log2sub = 0;
-    while (a.log2sub < kMaxLog2Sub3 && ((int64_t)c.ntiles << a.log2sub) < (int64_t)slots * (a.full ? kFill3 : kFill3Atoms)) a.log2sub++;
+    const int64_t n = c.sp[0].n + (c.nsp > 1 ? c.sp[1].n : 0);
+    for (a.log2sub = 0; a.log2sub < kMaxLog2Sub3; a.log2sub++) {
+        const int64_t items = (int64_t)c.ntiles << a.log2sub;
+        if (items >= (int64_t)slots * (a.full ? kFill3 : kFill3Atoms)) break;
+        if (items >= slots && n >> (a.log2sub + 1) < (int64_t)kMinPart3 * c.ntiles) break;
+    }
     const int64_t items = (int64_t)c.ntiles << a.log2sub;
     int grid = items < slots ? (int)items : slots;
     if (grid < 1) grid = 1;
