@@ -826,6 +826,7 @@ struct Field3 {
     Geo3 g;
     int k_ant;
     int seg;              // planes per block
+    int bx, by, bz;       // blocks along x, y and z
     float h_b, h_e, cj, mur;
     const float* ant;     // 2: this step's antenna scalars
     AntennaParams ap;     // for the next step's, into ant_next
@@ -862,15 +863,21 @@ __global__ void __launch_bounds__(32 * kWarps3, 2) k_fields3(const __grid_consta
     __shared__ float sex[kWarps3][32], sez[kWarps3][32], sbx[kWarps3][32], sbz[kWarps3][32], snx[kWarps3][32],
         snz[kWarps3][32];
     const Geo3& g = f.g;
+    // the first block evaluates the next step's antenna scalars
+    if (blockIdx.x == 0) {
+        if (threadIdx.x == 0) antenna_scalars(f.ap, f.next, f.ant_next);
+        return;
+    }
     const int nz = g.nz, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int i = (int)blockIdx.x * kCols3 + lane - 1, j = (int)blockIdx.y * kRows3 + w - 1;
+    const int blk = (int)blockIdx.x - 1, bxy = blk / f.bx, bz = bxy / f.by;
+    const int i = (blk - bxy * f.bx) * kCols3 + lane - 1, j = (bxy - bz * f.by) * kRows3 + w - 1;
     int gi = i < 0 ? i + g.nx : i, gj = j < 0 ? j + g.ny : j;
     while (gi >= g.nx) gi -= g.nx;
     while (gj >= g.ny) gj -= g.ny;
     const bool own = lane >= 1 && lane <= kCols3 && i < g.nx && w >= 1 && w <= kRows3 && j < g.ny;
     const int wm = w > 0 ? w - 1 : 0, wp = w + 1 < kWarps3 ? w + 1 : w;     // the patch's outer rows are not written
     // planes k0 .. k1 - 1; the last segment takes the remainder
-    const int k0 = (int)blockIdx.z * f.seg, k1 = blockIdx.z + 1 == gridDim.z ? nz + 1 : k0 + f.seg;
+    const int k0 = bz * f.seg, k1 = bz + 1 == f.bz ? nz + 1 : k0 + f.seg;
     const size_t plane = (size_t)g.nx * g.ny;
     const size_t col = (size_t)gj * g.nx + gi;
     const float antc = f.antc[col], ants = f.ants[col], ant0 = f.ant[0], ant1 = f.ant[1];
@@ -981,8 +988,6 @@ __global__ void __launch_bounds__(32 * kWarps3, 2) k_fields3(const __grid_consta
             f.G[5][q] = bp.z + f.h_b * ((snx[wp][lane] - np.x) - (npyi - np.y));
         }
     }
-    // the first block, done first, evaluates the next step's antenna scalars
-    if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0) antenna_scalars(f.ap, f.next, f.ant_next);
 }
 
 void launch_fields3(Ctx& c, cudaStream_t st, int64_t step, int64_t* launches)
@@ -1011,11 +1016,12 @@ void launch_fields3(Ctx& c, cudaStream_t st, int64_t step, int64_t* launches)
     f.flux = c.red_out + 5;
     // 16 planes per block (every segment repeats about two), fewer where that leaves under four blocks per SM
     // (90 x 80 x 60 cells: 56 us at 16 planes, 29 at 4; 37 x 27 x 32: 29, 15, 11 at 2); the last segment takes the remainder, at least `seg` planes
-    dim3 grid((c.nx + kCols3 - 1) / kCols3, (c.ny + kRows3 - 1) / kRows3);
+    f.bx = (c.nx + kCols3 - 1) / kCols3;
+    f.by = (c.ny + kRows3 - 1) / kRows3;
     f.seg = 16;
-    while (f.seg > 2 && (int64_t)grid.x * grid.y * ((c.nz + 1) / f.seg) < 4 * (int64_t)c.nsm) f.seg >>= 1;
-    grid.z = (c.nz + 1) / f.seg > 1 ? (c.nz + 1) / f.seg : 1;
-    k_fields3<<<grid, 32 * kWarps3, 0, st>>>(f);
+    while (f.seg > 2 && (int64_t)f.bx * f.by * ((c.nz + 1) / f.seg) < 4 * (int64_t)c.nsm) f.seg >>= 1;
+    f.bz = (c.nz + 1) / f.seg > 1 ? (c.nz + 1) / f.seg : 1;
+    k_fields3<<<1 + f.bx * f.by * f.bz, 32 * kWarps3, 0, st>>>(f);
     swap_fields(c);
     if (launches) *launches += 1;
 }
