@@ -414,7 +414,8 @@ PIC_API int pic_checkpoint_restore(pic_ctx* ctx, const void* buf, int32_t on_hos
  *   adjoints of step t+1 to step t in place and add this step's parameter derivatives to grads.
  * pic_adjoint_step_at: the same, the state of step t read in place from a device checkpoint that this
  *   context saved with its present particle counts (the context itself need not be at step t and is left
- *   as it is; dev_ckpt is 256-byte aligned as for pic_checkpoint_save). Asynchronous on the stream.
+ *   as it is; dev_ckpt is 256-byte aligned as for pic_checkpoint_save). The checkpoint's header is read back
+ *   first: PIC_EINVAL for a buffer that holds no checkpoint, or one of other species or particle counts.
  * All return PIC_ESTATE outside 2D, sort_every = 0 and pot_mode 0. */
 typedef struct {
     float* lam_pos[2];

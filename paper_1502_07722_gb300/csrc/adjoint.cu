@@ -387,7 +387,6 @@ struct MaxAdjArgs {
     const float *antc, *ants;  // antenna tables (amplitude * cos / sin of the phase)
     AntennaParams ap;          // coef = 2 c dt / dx (per unit E0)
     long long step;
-    const long long* step_dev; // where a checkpoint holds the step (NULL: `step`)
     double dE0_dI0;
     double* grads;             // grads[2] += dL/dI0
 };
@@ -453,8 +452,7 @@ __global__ void __launch_bounds__(256) k_adj_feT(const MaxAdjArgs a)
         a.lj[nn + c] = (float)-ly;
         a.lj[2 * nn + c] = k < nz ? (float)-lez : 0.0f;
         if (k == a.k_ant && a.ap.on) {
-            const long long step = a.step_dev ? *a.step_dev : a.step;
-            const double tau = ((double)step + 0.5) * a.ap.dt - a.ap.t_ant;
+            const double tau = ((double)a.step + 0.5) * a.ap.dt - a.ap.t_ant;
             const double env = exp(-2.0 * 0.6931471805599453 * tau * tau / (a.ap.tau_fwhm * a.ap.tau_fwhm));
             const double s = a.ap.coef * env * sin(a.ap.omega * tau), co = a.ap.coef * env * cos(a.ap.omega * tau);
             g = lx * ((double)a.antc[i] * s + (double)a.ants[i] * co) * a.dE0_dI0;
@@ -906,7 +904,7 @@ void launch_adjoint_seed_full(Ctx& c, double kin, const double* w_nodes, float* 
 }
 
 void launch_adjoint_step_full(Ctx& c, float* const* lam_pos, float* const* lam_u, float* lam_nodes, double* lF,
-                              float* lj, double* grads, const long long* step_dev, cudaStream_t st)
+                              float* lj, double* grads, cudaStream_t st)
 {
     const size_t nn = c.nn;
     MaxAdjArgs m;
@@ -924,7 +922,6 @@ void launch_adjoint_step_full(Ctx& c, float* const* lam_pos, float* const* lam_u
     m.ap = make_antenna_params(c);
     m.ap.coef = 2.0 * (kC * c.dt / c.cfg.dx);            // per unit E0
     m.step = (long long)c.step;
-    m.step_dev = step_dev;
     m.dE0_dI0 = c.cfg.I0 > 0 ? c.E0 / (2.0 * c.cfg.I0) : 0.0;
     m.grads = grads;
     const dim3 block(256), grid((c.nx + 255) / 256, c.nz + 1);

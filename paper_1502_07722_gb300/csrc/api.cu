@@ -938,8 +938,7 @@ int pic_adjoint_step(pic_ctx* h, const pic_adjoint_buffers* b)
     int r = adjoint_ok(c, b);
     if (r) return r;
     if (c.cfg.mode == PIC_MODE_FULL)
-        launch_adjoint_step_full(c, b->lam_pos, b->lam_u, b->lam_nodes, b->lam_F, b->lam_j, b->grads, nullptr,
-                                 c.stream);
+        launch_adjoint_step_full(c, b->lam_pos, b->lam_u, b->lam_nodes, b->lam_F, b->lam_j, b->grads, c.stream);
     else
         launch_adjoint_step(c, b->lam_pos[0], b->lam_u[0], b->lam_nodes, b->grads, c.stream);
     CK(cudaGetLastError());
@@ -948,13 +947,21 @@ int pic_adjoint_step(pic_ctx* h, const pic_adjoint_buffers* b)
 
 // The reverse step reads the state where the checkpoint holds it: a copy of the context whose particle,
 // field and density pointers lie in the buffer. (Restoring each state first moved it once more, 191 MB
-// and 54 us on the differentiable slab, with two host synchronisations.)
+// and 54 us on the differentiable slab.) A buffer without this context's header, or with other particle counts,
+// is refused as pic_checkpoint_restore would: its cells would index outside the grids.
 int pic_adjoint_step_at(pic_ctx* h, const void* ckpt, const pic_adjoint_buffers* b)
 {
     if (!h || !b || !ckpt || ((uintptr_t)ckpt & 255)) return PIC_EINVAL;
     int r = adjoint_ok(h->c, b);
     if (r) return r;
     Ctx c = h->c;
+    CkptHeader hd;
+    CK(cudaMemcpyAsync(&hd, ckpt, sizeof(hd), cudaMemcpyDeviceToHost, c.stream));
+    CK(cudaStreamSynchronize(c.stream));
+    if (hd.magic != kCkptMagic || hd.nsp != c.nsp) return PIC_EINVAL;
+    for (int s = 0; s < c.nsp; s++)
+        if (hd.n[s] != c.sp[s].n) return PIC_EINVAL;
+    c.step = hd.step;
     char* buf = (char*)const_cast<void*>(ckpt);
     size_t osp[2], otl[2], of, orho, oj;
     ckpt_layout(c, osp, otl, &of, &orho, &oj);
@@ -967,9 +974,8 @@ int pic_adjoint_step_at(pic_ctx* h, const void* ckpt, const pic_adjoint_buffers*
     }
     for (int q = 0; q < 6; q++) c.F[q] = (float*)(buf + of + q * align256(4 * c.nn));
     c.rho[c.cur] = (u64*)(buf + orho);
-    const long long* step = (const long long*)(buf + offsetof(CkptHeader, step));
     if (c.cfg.mode == PIC_MODE_FULL)
-        launch_adjoint_step_full(c, b->lam_pos, b->lam_u, b->lam_nodes, b->lam_F, b->lam_j, b->grads, step, c.stream);
+        launch_adjoint_step_full(c, b->lam_pos, b->lam_u, b->lam_nodes, b->lam_F, b->lam_j, b->grads, c.stream);
     else
         launch_adjoint_step(c, b->lam_pos[0], b->lam_u[0], b->lam_nodes, b->grads, c.stream);
     CK(cudaGetLastError());

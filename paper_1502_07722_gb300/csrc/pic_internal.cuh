@@ -279,7 +279,7 @@ void launch_node_functional(Ctx& c, const double* w_nodes, double* dev_out, cuda
 void launch_adjoint_seed_full(Ctx& c, double kin, const double* w_nodes, float* const* lam_pos, float* const* lam_u,
                               float* lam_nodes, double* lF, float* lj, double* r0_out, cudaStream_t st);
 void launch_adjoint_step_full(Ctx& c, float* const* lam_pos, float* const* lam_u, float* lam_nodes, double* lF,
-                              float* lj, double* grads, const long long* step_dev, cudaStream_t st);
+                              float* lj, double* grads, cudaStream_t st);
 int tile_window(int T);
 void launch_energy(Ctx& c, cudaStream_t st, double* host_out5);
 StepArgs make_step_args(Ctx& c);
