@@ -38,7 +38,8 @@ struct Layout {
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-int derive_layout(const pic_config* cfg, Layout& L)
+// twin: with a second set of grids in full mode, if the whole stays within kTwinBytes
+int derive_layout(const pic_config* cfg, Layout& L, bool twin)
 {
     if (!cfg) return PIC_EINVAL;
     L.dims = cfg->dims == 0 ? 2 : cfg->dims;
@@ -102,8 +103,6 @@ int derive_layout(const pic_config* cfg, Layout& L)
     const int arrays = L.dims == 3 ? 7 : 6;
     for (int s = 0; s < 2; s++) t += 2 * arrays * align256(4 * (size_t)L.cap[s]) + align256(4 * (size_t)(L.ntiles + 1));
     t += 6 * align256(4 * L.nn) + 5 * align256(8 * L.nn);
-    L.twin = full;         // the field update's second set of field and current grids
-    if (L.twin) t += 6 * align256(4 * L.nn) + 3 * align256(8 * L.nn);
     L.items = L.dims == 2 ? work_item_cap(L.cap[0] + L.cap[1], L.ntiles) : 0;
     if (L.items >= (1LL << 31)) return PIC_EINVAL;
     t += align256(sizeof(WorkItem) * (size_t)L.items) + align256(4);
@@ -112,6 +111,13 @@ int derive_layout(const pic_config* cfg, Layout& L)
     t += 2 * align256(4 * ((size_t)L.nkeys + 1));
     t += align256(4 * (((size_t)L.nkeys + 2047) / 2048 + 1));
     t += align256(8 * 5 * (size_t)kMaxEnergyBlocks) + align256(8 * 8) + align256(32);
+    // The field update writes a second set of field and current grids (48 bytes per node on 64). A state that would take
+    // more than kTwinBytes with it keeps one: what filled the GPU before there was a second set still fits, at the
+    // field update's old speed.
+    const size_t second = 6 * align256(4 * L.nn) + 3 * align256(8 * L.nn);
+    L.twin = full && twin && t + second <= kTwinBytes;
+    if (L.twin) t += second;
+    else if (full) t += align256(4 * 8 * plane);
     L.total = t;
     return PIC_OK;
 }
@@ -235,7 +241,7 @@ void swap_currents(Ctx& c)
 int64_t work_item_cap_of(const pic_config* cfg)
 {
     Layout L;
-    return derive_layout(cfg, L) == PIC_OK ? L.items : 0;
+    return derive_layout(cfg, L, false) == PIC_OK ? L.items : 0;
 }
 
 void swap_fields(Ctx& c)
@@ -279,28 +285,23 @@ StepArgs make_step_args(Ctx& c)
     return a;
 }
 
-}  // namespace gbpic
-
-extern "C" {
-
-size_t pic_config_bytes(void) { return sizeof(pic_config); }
-
-int pic_workspace_size(const pic_config* cfg, size_t* bytes)
+int workspace_bytes(const pic_config* cfg, bool* twin, size_t* bytes)
 {
     if (!bytes) return PIC_EINVAL;
     Layout L;
-    int r = derive_layout(cfg, L);
+    int r = derive_layout(cfg, L, *twin);
     if (r) return r;
+    *twin = L.twin;
     *bytes = L.total;
     return PIC_OK;
 }
 
-int pic_init(const pic_config* cfg, void* workspace, size_t workspace_bytes, void* stream, pic_ctx** out)
+int init_context(const pic_config* cfg, void* workspace, size_t workspace_bytes, void* stream, pic_ctx** out, bool twin)
 {
     if (!out) return PIC_EINVAL;
     *out = nullptr;
     Layout L;
-    int r = derive_layout(cfg, L);
+    int r = derive_layout(cfg, L, twin);
     if (r) return r;
     if (!workspace || ((uintptr_t)workspace & 255)) return PIC_EINVAL;
     if (workspace_bytes < L.total) return PIC_ENOMEM;
@@ -369,6 +370,8 @@ int pic_init(const pic_config* cfg, void* workspace, size_t workspace_bytes, voi
     if (L.twin) {
         for (int q = 0; q < 6; q++) c.Fn[q] = cv.take<float>(L.nn);
         for (int q = 0; q < 3; q++) c.Jn[q] = cv.take<u64>(L.nn);
+    } else if (c.cfg.mode == PIC_MODE_FULL) {
+        c.mur_save = cv.take<float>(8 * (size_t)L.nx * L.ny);
     }
     c.items = cv.take<WorkItem>((size_t)L.items);
     c.items_cap = (int32_t)L.items;
@@ -467,6 +470,23 @@ int pic_init(const pic_config* cfg, void* workspace, size_t workspace_bytes, voi
     }
     *out = h;
     return PIC_OK;
+}
+
+}  // namespace gbpic
+
+extern "C" {
+
+size_t pic_config_bytes(void) { return sizeof(pic_config); }
+
+int pic_workspace_size(const pic_config* cfg, size_t* bytes)
+{
+    bool twin = true;
+    return workspace_bytes(cfg, &twin, bytes);
+}
+
+int pic_init(const pic_config* cfg, void* workspace, size_t bytes, void* stream, pic_ctx** out)
+{
+    return init_context(cfg, workspace, bytes, stream, out, true);
 }
 
 void pic_free(pic_ctx* h)

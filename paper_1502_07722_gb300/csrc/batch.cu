@@ -4,7 +4,7 @@
 //   k_particles_batch    one persistent launch over the tiles of every slab
 //   k_fields_batch       the field update of every slab, which also prepares the next step (clears
 //                        its currents, starts its node density, evaluates its antenna scalars)
-// (the transport stage has k_prepare_batch in front instead) and is recorded once as a CUDA graph
+// (the transport stage, and slabs with one set of grids, have k_prepare_batch in front instead) and is recorded once as a CUDA graph
 // per parity of the double-buffered grids, then replayed. The per-slab arguments live in device memory (copied into a constant-memory table in
 // front of the particle kernel), so a cell sort (host-driven, every
 // sort_every steps) only refreshes them; the graphs stay valid.
@@ -45,7 +45,7 @@ struct pic_batch {
     int n;
     pic_ctx* slab[kMaxSlabs];
     cudaStream_t st;
-    int full, pot, minW, maxW, nsm, sort_every;
+    int full, twin, pot, minW, maxW, nsm, sort_every;     // twin: two sets of grids (full mode)
     size_t max_nn;
     StepArgs* args_dev;          // [2][n]: parity 0 (density in buffer 0) and parity 1
     FieldBatch fields[2];        // every slab's field arguments per parity (host copy, passed by value)
@@ -122,14 +122,24 @@ void enqueue_prepare(pic_batch* b, int parity)
 void enqueue_step(pic_batch* b, int parity)
 {
     const StepArgs* args = b->args_dev + parity * b->n;
-    if (!b->full) enqueue_prepare(b, parity);
+    if (!b->twin) enqueue_prepare(b, parity);
+    if (b->full && !b->twin)
+        launch_antenna_batch(b->ap_dev, b->step_dev, b->ant_dev + parity * 2 * b->n, b->n, b->st);
     if (b->timing) cudaEventRecord(b->ev[0], b->st);
     launch_particle_step_batch(args, b->n, b->items, b->nitems, b->full, b->pot, b->minW, b->maxW, b->nsm, b->st);
     if (b->timing) cudaEventRecord(b->ev[1], b->st);
-    if (b->full)
+    if (b->twin) {
         launch_fields_batch(b->fields[parity], b->ap_dev, b->step_dev, b->ant_dev + (1 - parity) * 2 * b->n, b->st);
+    } else if (b->full) {
+        for (int s = 0; s < b->n; s++) launch_fields_one_set(b->fields[parity].f[s], b->st);
+        launch_step_done(b->step_dev, b->n, b->st);
+    }
     if (b->timing) cudaEventRecord(b->ev[2], b->st);
 }
+
+// Kernels of a step: particles and fields, or prepare and particles (transport), or with one set of grids those, the
+// antenna's, three per slab and the counters'.
+int launches(const pic_batch* b) { return b->full && !b->twin ? 4 + 3 * b->n : 2; }
 
 // One list of work items over every slab's tiles, after a sort or a slab's state was written.
 void build_items(pic_batch* b)
@@ -170,6 +180,7 @@ int prepare(pic_batch* b)
     // a pageable source: the call returns once the counters have been staged
     if (cudaMemcpyAsync(b->step_dev, step, 8 * (size_t)b->n, cudaMemcpyHostToDevice, b->st) != cudaSuccess)
         return PIC_ECUDA;
+    if (!b->twin) return PIC_OK;             // every step prepares itself
     const int parity = b->slab[0]->c.cur;
     enqueue_prepare(b, parity);
     launch_antenna_batch(b->ap_dev, b->step_dev, b->ant_dev + parity * 2 * b->n, b->n, b->st);
@@ -202,24 +213,41 @@ int capture(pic_batch* b)
 
 }  // namespace
 
+// Bytes of the batch; *twin: the slabs have two sets of grids, which all of them have or none (kTwinBytes for all).
+static int batch_bytes(const pic_config* cfgs, int n, bool* twin, size_t* bytes)
+{
+    size_t t = 0;
+    bool all = true;
+    for (int s = 0; s < n; s++) {
+        size_t b = 0;
+        bool two = *twin;
+        const int r = workspace_bytes(&cfgs[s], &two, &b);
+        if (r) return r;
+        all &= two;
+        t += a256(b);
+    }
+    if (*twin && cfgs[0].mode == PIC_MODE_FULL && (!all || t > kTwinBytes)) {
+        *twin = false;
+        return batch_bytes(cfgs, n, twin, bytes);
+    }
+    *twin = all;
+    *bytes = t + batch_tail_bytes(cfgs, n);
+    return PIC_OK;
+}
+
 extern "C" {
 
 int pic_batch_workspace_size(const pic_config* cfgs, int32_t n, size_t* bytes)
 {
     if (!cfgs || !bytes || n < 1 || n > kMaxSlabs) return PIC_EINVAL;
-    size_t t = 0;
     for (int s = 0; s < n; s++) {
         if (cfgs[s].mode != cfgs[0].mode || (cfgs[s].dims != 0 && cfgs[s].dims != 2)) return PIC_EINVAL;
         if (cfgs[s].pot_mode != cfgs[0].pot_mode || cfgs[s].lattice != cfgs[0].lattice)
             return PIC_EINVAL;   // one kernel instance
-        size_t b = 0;
-        const int r = pic_workspace_size(&cfgs[s], &b);
-        if (r) return r;
-        t += a256(b);
     }
     if (batch_items_cap(cfgs, n) >= (1LL << 31)) return PIC_EINVAL;
-    *bytes = t + batch_tail_bytes(cfgs, n);
-    return PIC_OK;
+    bool twin = true;
+    return batch_bytes(cfgs, n, &twin, bytes);
 }
 
 int pic_batch_init(const pic_config* cfgs, int32_t n, void* workspace, size_t bytes, void* stream, pic_batch** out)
@@ -236,10 +264,14 @@ int pic_batch_init(const pic_config* cfgs, int32_t n, void* workspace, size_t by
     b->n = n;
     b->st = (cudaStream_t)stream;
     char* p = (char*)workspace;
+    bool twin = true;
+    batch_bytes(cfgs, n, &twin, &need);
+    b->twin = twin;
     for (int s = 0; s < n; s++) {
         size_t sb = 0;
-        pic_workspace_size(&cfgs[s], &sb);
-        r = pic_init(&cfgs[s], p, sb, stream, &b->slab[s]);
+        bool two = twin;
+        workspace_bytes(&cfgs[s], &two, &sb);
+        r = init_context(&cfgs[s], p, sb, stream, &b->slab[s], twin);
         if (r) {
             for (int q = 0; q < s; q++) pic_free(b->slab[q]);
             delete b;
@@ -272,24 +304,24 @@ int pic_batch_init(const pic_config* cfgs, int32_t n, void* workspace, size_t by
     for (int s = 0; s < n; s++) {
         Ctx& c = b->slab[s]->c;
         ap[s] = make_antenna_params(c);
-        if (!c.Jn[0]) continue;
+        if (!b->full) continue;
         for (int k = 0; k < 2; k++) {
             // the update of a step of this parity follows its moves: the density and the currents
             // are the other buffers, the fields not yet
             const int par = c.cur;
             c.cur = 1 - c.cur;
-            swap_currents(c);
+            if (twin) swap_currents(c);
             FieldArgs& f = b->fields[par].f[s];
             f = make_field_args(c);
             f.ant = b->ant_dev + par * 2 * n + 2 * s;
             c.cur = par;
-            swap_currents(c);
+            if (twin) swap_currents(c);
             flip_parity(c);
         }
     }
     for (int par = 0; par < 2; par++) {
         b->fields[par].n = n;
-        if (b->full) field_row_blocks(b->fields[par]);
+        if (b->twin) field_row_blocks(b->fields[par]);
     }
     const bool ok = cudaMemcpyAsync(b->ap_dev, ap.data(), sizeof(AntennaParams) * n, cudaMemcpyHostToDevice, b->st) ==
                     cudaSuccess;
@@ -361,15 +393,15 @@ int pic_batch_step(pic_batch* b, int32_t nsteps)
             b->ms[0] += m0;
             b->ms[1] += m1;
             b->nlaunch[0] += 1;
-            b->nlaunch[1] += b->full ? 1 : 0;
-            b->nlaunch[3] += 2;
+            b->nlaunch[1] += b->twin ? 1 : (b->full ? 3 * b->n : 0);
+            b->nlaunch[3] += launches(b);
         } else {
             if (!b->captured) {
                 const int r = capture(b);
                 if (r) return r;
             }
             if (cudaGraphLaunch(b->graph[parity], b->st) != cudaSuccess) return PIC_ECUDA;
-            b->nlaunch[3] += 2;
+            b->nlaunch[3] += launches(b);
         }
         for (int s = 0; s < b->n; s++) {
             Ctx& c = b->slab[s]->c;

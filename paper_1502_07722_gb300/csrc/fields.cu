@@ -214,6 +214,91 @@ __global__ void k_antenna_batch(const AntennaParams* p, const long long* step, f
     if (s < nslab) antenna_scalars(p[s], step[s], ant + 2 * s);
 }
 
+// ---- one set of grids ---------------------------------------------------------------------
+// States that leave no room for the second set (kTwinBytes) take the update in place, in three passes over the nodes: B
+// half, E with the current and the antenna, B half. The first one keeps the tangential E of the rows beside the walls for
+// the absorbing condition. 172 bytes per node with the copy and clear in front, and the same bits.
+__global__ void k_half_B(const __grid_constant__ FieldArgs f, int save)
+{
+    const int nx = f.nx, nz = f.nz, i = blockIdx.x * blockDim.x + threadIdx.x, k = blockIdx.y;
+    if (i >= nx) return;
+    const int ip = i + 1 == nx ? 1 - nx : 1;
+    const size_t c = (size_t)k * nx + i;
+    const float *Ex = f.G[0], *Ey = f.G[1], *Ez = f.G[2];
+    const float ey = Ey[c];
+    if (k < nz) {
+        const size_t u = c + nx;
+        f.G[3][c] += f.h_b * (Ey[u] - ey);
+        f.G[4][c] += f.h_b * ((Ez[c + ip] - Ez[c]) - (Ex[u] - Ex[c]));
+    }
+    f.G[5][c] -= f.h_b * (Ey[c + ip] - ey);
+    const int slot = k == 0 ? 0 : k == 1 ? 1 : k == nz - 1 ? 2 : k == nz ? 3 : -1;
+    if (save && slot >= 0) {
+        f.save[slot * nx + i] = Ex[c];
+        f.save[(4 + slot) * nx + i] = ey;
+    }
+}
+
+// new Ex / Ey of an interior node from its old value
+__device__ __forceinline__ float ex_new(const FieldArgs& f, size_t c, int i, int k, float old)
+{
+    float v = old - f.h_e * (f.G[4][c] - f.G[4][c - f.nx]) - f.cj * (float)(long long)f.J[0][c];
+    if (k == f.k_ant) v += f.antc[i] * f.ant[0] + f.ants[i] * f.ant[1];
+    return v;
+}
+__device__ __forceinline__ float ey_new(const FieldArgs& f, size_t c, int i, float old)
+{
+    const int im = i == 0 ? f.nx - 1 : -1;
+    return old + f.h_e * ((f.G[3][c] - f.G[3][c - f.nx]) - (f.G[5][c] - f.G[5][c + im])) - f.cjy * (float)(long long)f.J[1][c];
+}
+
+__global__ void k_E(const __grid_constant__ FieldArgs f)
+{
+    const int nx = f.nx, nz = f.nz, i = blockIdx.x * blockDim.x + threadIdx.x, k = blockIdx.y;
+    float s = 0.0f;              // on the flux row: (Ex By - Ey Bx) at the half step
+    if (i < nx) {
+        const size_t c = (size_t)k * nx + i;
+        if (k > 0 && k < nz) {
+            const float ex0 = f.G[0][c], ey0 = f.G[1][c];
+            const float ex1 = ex_new(f, c, i, k, ex0), ey1 = ey_new(f, c, i, ey0);
+            f.G[0][c] = ex1;
+            f.G[1][c] = ey1;
+            if (k == f.k_flux)
+                s = 0.25f * ((ex0 + ex1) * (f.G[4][c - nx] + f.G[4][c]) - (ey0 + ey1) * (f.G[3][c - nx] + f.G[3][c]));
+        } else {
+            // a wall row (Mur): its old value, and the row beside it before and after this step
+            const int w = k == 0 ? 0 : 3, b = k == 0 ? 1 : 2, kb = k == 0 ? 1 : nz - 1;
+            const size_t cb = (size_t)kb * nx + i;
+            const float x0 = f.save[w * nx + i], x1 = f.save[b * nx + i];
+            const float y0 = f.save[(4 + w) * nx + i], y1 = f.save[(4 + b) * nx + i];
+            f.G[0][c] = x1 + f.mur * (ex_new(f, cb, i, kb, x1) - x0);
+            f.G[1][c] = y1 + f.mur * (ey_new(f, cb, i, y1) - y0);
+        }
+        if (k < nz) {
+            const int im = i == 0 ? nx - 1 : -1;
+            f.G[2][c] += f.h_e * (f.G[4][c] - f.G[4][c + im]) - f.cj * (float)(long long)f.J[2][c];
+        }
+    }
+    if (k != f.k_flux) return;
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0 && s != 0.0f) atomicAdd(f.flux, (double)s);
+}
+
+void launch_fields_one_set(const FieldArgs& f, cudaStream_t st)
+{
+    const dim3 block(256), grid((f.nx + 255) / 256, f.nz + 1);
+    k_half_B<<<grid, block, 0, st>>>(f, 1);
+    k_E<<<grid, block, 0, st>>>(f);
+    k_half_B<<<grid, block, 0, st>>>(f, 0);
+}
+
+__global__ void k_step_done(long long* step, int n)
+{
+    if ((int)threadIdx.x < n) step[threadIdx.x]++;
+}
+
+void launch_step_done(long long* step_dev, int n, cudaStream_t st) { k_step_done<<<1, 64, 0, st>>>(step_dev, n); }
+
 // each slab's first block (rb[n] = the total)
 void field_row_blocks(FieldBatch& P)
 {
@@ -249,7 +334,8 @@ FieldArgs make_field_args(const Ctx& c)
     const double cdt = kC * c.dt;
     f.mur = (float)((cdt - c.cfg.dx) / (cdt + c.cfg.dx));
     for (int q = 0; q < 6; q++) f.F[q] = c.F[q];
-    for (int q = 0; q < 6; q++) f.G[q] = c.Fn[q];
+    for (int q = 0; q < 6; q++) f.G[q] = c.Fn[q] ? c.Fn[q] : c.F[q];
+    f.save = c.mur_save;
     for (int q = 0; q < 3; q++) f.J[q] = c.J[q];
     for (int q = 0; q < 3; q++) f.Z[q] = c.Jn[q];
     f.rho = c.rho[c.cur];
@@ -265,6 +351,11 @@ FieldArgs make_field_args(const Ctx& c)
 void launch_fields(Ctx& c, cudaStream_t st, int64_t step, int64_t* launches)
 {
     const FieldArgs f = make_field_args(c);
+    if (!c.Fn[0]) {
+        launch_fields_one_set(f, st);
+        if (launches) *launches += 3;
+        return;
+    }
     k_fields<<<1 + field_blocks(f), kFieldThreads, 0, st>>>(f, make_antenna_params(c), (long long)step + 1,
                                                             c.ant + 2 * ((step + 1) & 1));
     swap_fields(c);

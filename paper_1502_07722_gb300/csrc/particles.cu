@@ -597,8 +597,8 @@ int item_chunk(int64_t n, int slots)
     return (int)(c < kMinChunk ? kMinChunk : (c > (1 << 30) ? (1 << 30) : c));
 }
 
-// Entries of a list for n particles on ntiles tiles: round(cnt / chunk) or one per tile.
-int64_t work_item_cap(int64_t n, int64_t ntiles) { return n / (2 * kBlock) + 2 * ntiles; }
+// Entries of a list for n particles on ntiles tiles: a tile with particles has at most cnt / chunk + 1.
+int64_t work_item_cap(int64_t n, int64_t ntiles) { return n / (2 * kBlock) + ntiles; }
 
 void launch_work_items(const Ctx& c, int slab, int chunk, WorkItem* items, int* nitems, int cap, cudaStream_t st)
 {

@@ -833,7 +833,8 @@ struct Field3 {
     long long next;
     float* ant_next;
     const float* F[6];    // read
-    float* G[6];          // written
+    float* G[6];          // written (the same grids with one set)
+    float* save;          // one set: 8 planes of nx ny
     const u64* J[3];      // this step's currents
     u64* Z[3];            // cleared for the next step
     const u64* rho;       // node density after this step's moves
@@ -990,6 +991,84 @@ __global__ void __launch_bounds__(32 * kWarps3, 2) k_fields3(const __grid_consta
     }
 }
 
+// ---- one set of grids: in place, in three passes, as in 2D ----------------------------------
+__global__ void k_half_B3(const __grid_constant__ Field3 f, int save)
+{
+    const Geo3& g = f.g;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y, k = blockIdx.z;
+    if (i >= g.nx) return;
+    const int ip = i + 1 == g.nx ? 0 : i + 1, jp = j + 1 == g.ny ? 0 : j + 1;
+    const size_t c = idx3(g, i, j, k), plane = (size_t)g.nx * g.ny;
+    const float *Ex = f.G[0], *Ey = f.G[1], *Ez = f.G[2];
+    const float ex = Ex[c], ey = Ey[c];
+    if (k < g.nz) {
+        const float ez = Ez[c];
+        f.G[3][c] += f.h_b * ((Ey[c + plane] - ey) - (Ez[idx3(g, i, jp, k)] - ez));
+        f.G[4][c] += f.h_b * ((Ez[idx3(g, ip, j, k)] - ez) - (Ex[c + plane] - ex));
+    }
+    f.G[5][c] += f.h_b * ((Ex[idx3(g, i, jp, k)] - ex) - (Ey[idx3(g, ip, j, k)] - ey));
+    const int slot = k == 0 ? 0 : k == 1 ? 1 : k == g.nz - 1 ? 2 : k == g.nz ? 3 : -1;
+    if (save && slot >= 0) {
+        const size_t q = (size_t)j * g.nx + i;
+        f.save[slot * plane + q] = ex;
+        f.save[(4 + slot) * plane + q] = ey;
+    }
+}
+
+__device__ __forceinline__ float ex3_new(const Field3& f, int i, int j, int k, float old)
+{
+    const Geo3& g = f.g;
+    const size_t c = idx3(g, i, j, k);
+    const int jm = j == 0 ? g.ny - 1 : j - 1;
+    float v = old + f.h_e * ((f.G[5][c] - f.G[5][idx3(g, i, jm, k)]) - (f.G[4][c] - f.G[4][idx3(g, i, j, k - 1)])) -
+              f.cj * (float)(long long)f.J[0][c];
+    if (k == f.k_ant) {
+        const size_t q = (size_t)j * g.nx + i;
+        v += f.antc[q] * f.ant[0] + f.ants[q] * f.ant[1];
+    }
+    return v;
+}
+__device__ __forceinline__ float ey3_new(const Field3& f, int i, int j, int k, float old)
+{
+    const Geo3& g = f.g;
+    const size_t c = idx3(g, i, j, k);
+    const int im = i == 0 ? g.nx - 1 : i - 1;
+    return old + f.h_e * ((f.G[3][c] - f.G[3][idx3(g, i, j, k - 1)]) - (f.G[5][c] - f.G[5][idx3(g, im, j, k)])) -
+           f.cj * (float)(long long)f.J[1][c];
+}
+
+__global__ void k_E3(const __grid_constant__ Field3 f)
+{
+    const Geo3& g = f.g;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y, k = blockIdx.z;
+    float s = 0.0f;
+    if (i < g.nx) {
+        const size_t c = idx3(g, i, j, k), plane = (size_t)g.nx * g.ny, q = (size_t)j * g.nx + i;
+        if (k > 0 && k < g.nz) {
+            const float ex0 = f.G[0][c], ey0 = f.G[1][c];
+            const float ex1 = ex3_new(f, i, j, k, ex0), ey1 = ey3_new(f, i, j, k, ey0);
+            f.G[0][c] = ex1;
+            f.G[1][c] = ey1;
+            if (k == f.k_flux)
+                s = 0.25f * ((ex0 + ex1) * (f.G[4][c - plane] + f.G[4][c]) - (ey0 + ey1) * (f.G[3][c - plane] + f.G[3][c]));
+        } else {
+            const int w = k == 0 ? 0 : 3, b = k == 0 ? 1 : 2, kb = k == 0 ? 1 : g.nz - 1;
+            const float x0 = f.save[w * plane + q], x1 = f.save[b * plane + q];
+            const float y0 = f.save[(4 + w) * plane + q], y1 = f.save[(4 + b) * plane + q];
+            f.G[0][c] = x1 + f.mur * (ex3_new(f, i, j, kb, x1) - x0);
+            f.G[1][c] = y1 + f.mur * (ey3_new(f, i, j, kb, y1) - y0);
+        }
+        if (k < g.nz) {
+            const int im = i == 0 ? g.nx - 1 : i - 1, jm = j == 0 ? g.ny - 1 : j - 1;
+            f.G[2][c] += f.h_e * ((f.G[4][c] - f.G[4][idx3(g, im, j, k)]) - (f.G[3][c] - f.G[3][idx3(g, i, jm, k)])) -
+                         f.cj * (float)(long long)f.J[2][c];
+        }
+    }
+    if (k != f.k_flux) return;
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0 && s != 0.0f) atomicAdd(f.flux, (double)s);
+}
+
 void launch_fields3(Ctx& c, cudaStream_t st, int64_t step, int64_t* launches)
 {
     Field3 f;
@@ -1005,7 +1084,8 @@ void launch_fields3(Ctx& c, cudaStream_t st, int64_t step, int64_t* launches)
     f.next = (long long)step + 1;
     f.ant_next = c.ant + 2 * ((step + 1) & 1);
     for (int q = 0; q < 6; q++) f.F[q] = c.F[q];
-    for (int q = 0; q < 6; q++) f.G[q] = c.Fn[q];
+    for (int q = 0; q < 6; q++) f.G[q] = c.Fn[q] ? c.Fn[q] : c.F[q];
+    f.save = c.mur_save;
     for (int q = 0; q < 3; q++) f.J[q] = c.J[q];
     for (int q = 0; q < 3; q++) f.Z[q] = c.Jn[q];
     f.rho = c.rho[c.cur];
@@ -1014,6 +1094,14 @@ void launch_fields3(Ctx& c, cudaStream_t st, int64_t step, int64_t* launches)
     f.ants = c.ant_s;
     f.k_flux = c.k_ant - 1 >= 1 ? c.k_ant - 1 : -1;
     f.flux = c.red_out + 5;
+    if (!c.Fn[0]) {
+        const dim3 block(256), grid((c.nx + 255) / 256, c.ny, c.nz + 1);
+        k_half_B3<<<grid, block, 0, st>>>(f, 1);
+        k_E3<<<grid, block, 0, st>>>(f);
+        k_half_B3<<<grid, block, 0, st>>>(f, 0);
+        if (launches) *launches += 3;
+        return;
+    }
     // 16 planes per block (every segment repeats about two), fewer where that leaves under four blocks per SM
     // (90 x 80 x 60 cells: 56 us at 16 planes, 29 at 4; 37 x 27 x 32: 29, 15, 11 at 2); the last segment takes the remainder, at least `seg` planes
     f.bx = (c.nx + kCols3 - 1) / kCols3;

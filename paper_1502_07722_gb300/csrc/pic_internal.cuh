@@ -147,8 +147,9 @@ struct Ctx {
     u64* J[3];            // currents of the last step
     u64* rho[2];
     int32_t cur;          // rho[cur] holds the node density at the current positions
-    float* Fn[6];         // full mode: the fields the next update writes (swapped with F after it)
-    u64* Jn[3];           // full mode: the currents the next step deposits into
+    float* Fn[6];         // full mode: the fields the next update writes (swapped with F after it); NULL with one set
+    u64* Jn[3];           // full mode: the currents the next step deposits into; NULL with one set
+    float* mur_save;      // one set of grids: 8 planes of nx ny, the tangential E beside the walls before the E step
     int32_t prepared;     // Jn is clear and rho[1 - cur] equals rho[cur]
     WorkItem* items;      // 2D: work items of the particle kernel, from the tile offsets
     int32_t* nitems;
@@ -195,7 +196,8 @@ struct FieldArgs {
     float cjy;           // J6y -> dt J_y / eps0
     float mur;           // (c dt - dx) / (c dt + dx)
     const float* F[6];   // read
-    float* G[6];         // written
+    float* G[6];         // written (the same grids with one set)
+    float* save;         // one set: 8 rows of nx
     const u64* J[3];     // this step's currents
     u64* Z[3];           // cleared for the next step
     const u64* rho;      // node density after this step's moves
@@ -251,6 +253,8 @@ struct FieldBatch {
     int rb[kMaxFieldSlabs + 1];      // first block of each slab
     int n;
 };
+void launch_fields_one_set(const FieldArgs& f, cudaStream_t st);
+void launch_step_done(long long* step_dev, int n, cudaStream_t st);
 void launch_fields_batch(const FieldBatch& P, const AntennaParams* ap_dev, long long* step_dev, float* ant_next,
                          cudaStream_t st);
 void launch_antenna(const Ctx& c, cudaStream_t st, int64_t step);
@@ -265,6 +269,10 @@ void launch_work_items(const Ctx& c, int slab, int chunk, WorkItem* items, int* 
 int particle_slots(int nsm, int full, int batch, int W);
 int item_chunk(int64_t n, int slots);
 int64_t work_item_cap_of(const pic_config* cfg);     // 0 for an invalid configuration
+// Workspace of a context with two sets of grids (full mode, *twin on input, while the size allows; *twin says) or one.
+constexpr size_t kTwinBytes = (size_t)112 << 30;
+int workspace_bytes(const pic_config* cfg, bool* twin, size_t* bytes);
+int init_context(const pic_config* cfg, void* workspace, size_t bytes, void* stream, pic_ctx** out, bool twin);
 size_t particle_smem_bytes(int W);
 void launch_particle_step3(Ctx& c, cudaStream_t st);
 void launch_deposit_density3(Ctx& c, u64* out, cudaStream_t st);
