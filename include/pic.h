@@ -170,9 +170,11 @@ typedef struct pic_ctx pic_ctx;
  * against it. Host only; no errors. (Not a step of the paper's method.) */
 PIC_API size_t pic_config_bytes(void);
 
-/* Bytes of device workspace pic_init needs for cfg. Returns PIC_EINVAL for an invalid cfg and
- * PIC_EOVERFLOW for a slab whose particles per cell exceed the fixed-point range (see above);
- * makes no CUDA call. */
+/* Bytes of device workspace pic_init needs for cfg. With fields that is two sets of the field and current grids (112
+ * bytes per node, the update writes one and reads the other) while the whole stays within 112 GiB, else one set (64
+ * bytes per node, the update in place, the same results); a batch goes by its slabs' sum. Returns
+ * PIC_EINVAL for an invalid cfg and PIC_EOVERFLOW for a slab whose particles per cell exceed the
+ * fixed-point range (see above); makes no CUDA call. */
 PIC_API int pic_workspace_size(const pic_config* cfg, size_t* bytes);
 
 /* Create a simulation on the current device: generate the initial slab (paper: the damage
@@ -214,7 +216,8 @@ PIC_API int pic_crater_profile(pic_ctx* ctx, const int64_t* dev_rho0, double* de
  * in K (u = gamma v / c; the spread about the cell's mean flow); cells with fewer than two
  * particles get 0. dev_T: double[ncell], ncell = nz*nx (2D, index k*nx + i) or nz*ny*nx (3D,
  * (k*ny + j)*nx + i); dev_work: caller-owned scratch of 5*ncell doubles. FP64 per-cell sums by
- * atomics (the last bits depend on their order). Asynchronous on the context's stream.
+ * atomics of single particles or of runs of them, which are summed as three FP32 numbers (about 70 bits;
+ * the last bits depend on the atomics' order). Asynchronous on the context's stream.
  * Errors: PIC_EINVAL (NULL pointers, species not present). */
 PIC_API int pic_cell_temperature(pic_ctx* ctx, int32_t species, double* dev_work, double* dev_T);
 

@@ -464,6 +464,9 @@ __global__ void __launch_bounds__(256) k_adj_feT(const MaxAdjArgs a)
     }
 }
 
+// Resident CTAs of the particle transposes: 3 at 80 registers, although the ions' instance then spills 288 bytes and the
+// electrons' 112. ms per reverse step of the 7.3 M-particle slab: 0.624 at 3, 0.645 at 2 (128 registers, 104 and 8
+// bytes), 0.653 at 4 (64, 396 and 164): latency counts for more than the spills.
 constexpr int kAdjCtas = 3;
 
 struct FullAdjArgs {

@@ -4,10 +4,10 @@
 //   k_particles_batch    one persistent launch over the tiles of every slab
 //   k_fields_batch       the field update of every slab, which also prepares the next step (clears
 //                        its currents, starts its node density, evaluates its antenna scalars)
-// (the transport stage, and slabs with one set of grids, have k_prepare_batch in front instead) and is recorded once as a CUDA graph
-// per parity of the double-buffered grids, then replayed. The per-slab arguments live in device memory (copied into a constant-memory table in
-// front of the particle kernel), so a cell sort (host-driven, every
-// sort_every steps) only refreshes them; the graphs stay valid.
+// (the transport stage, and slabs with one set of grids, have k_prepare_batch in front instead) and is
+// recorded once as a CUDA graph per parity of the double-buffered grids, then replayed. The per-slab
+// arguments live in device memory (copied into a constant-memory table in front of the particle kernel), so
+// a cell sort (host-driven, every sort_every steps) only refreshes them; the graphs stay valid.
 #include <cstring>
 #include <new>
 #include <vector>

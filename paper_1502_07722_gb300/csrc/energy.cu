@@ -132,8 +132,8 @@ __global__ void __launch_bounds__(32 * kSlots) k_energy_final(const double* __re
     if (lane == 0) out[s] = r;
 }
 
-// Sums of FP32 terms by two-sum and the FP64 conversions kept off the common way: 482 -> 277 us for the
-// 33.5 M particles and 1 M nodes of the 1024^2 slab (8 FP64-pipe instructions per particle were its bound).
+// Sums of FP32 terms in three FP32 numbers (LongSum) and the FP64 conversions kept off the common way: a call on the
+// 33.5 M particles and 1 M nodes of the 1024^2 slab 520 -> 287 us (8 FP64-pipe instructions per particle were its bound).
 // Small states take as many blocks as give every thread a particle or a node: each block costs its share of
 // FP64 adds at the end (64^2 cells, 16384 ions: 23.1 us with every block and shuffle trees, 7.2 now; the final sum
 // 8.4 -> 2.3). Returns the blocks taken, at most `most`.

@@ -11,7 +11,8 @@
 //
 // What bounds it: memory traffic on the large grids, the launch on the small ones. Against three
 // in-place passes (B half, E, B half) with a copy/clear kernel and a one-thread antenna kernel, a
-// node moves 112 bytes instead of 172 and a step has two launches instead of six.
+// node moves 112 bytes instead of 172 and a step has two launches instead of six. (The largest states have no room
+// for a second set and keep the three passes: k_half_B, k_E.)
 #include "pic_device.cuh"
 #include "pic_internal.cuh"
 

@@ -37,9 +37,12 @@
 namespace gbpic {
 
 constexpr int kMargin = 2;              // cells a particle may drift out of its tile between sorts
-constexpr int kBlock = 128;                // threads per CTA (8 CTAs per SM)
+constexpr int kBlock = 128;             // threads per CTA
 // Resident CTAs: with fields 9 (56 registers; 8 at 64: 1.74 against 1.70 ms per launch on the 2048^2
-// slab), the transport stage 8 (9: 0.129 against 0.116 ms on the crater slab).
+// slab), the transport stage 8 (9: 0.129 against 0.116 ms on the crater slab). The Morse, altered, HCP and embedded-atom
+// instances spill up to 24 bytes (embedded atom 72) at 56 registers and still take 14 to 19 % less per step than the 64
+// registers and 8 CTAs of the kernel before (33.5 M particles, ms a step: Morse 0.634 -> 0.533, altered 0.589 -> 0.497, HCP 0.610 ->
+// 0.536, embedded atom 0.936 -> 0.805; tiles of 20 cells 0.648 -> 0.559, 0.611 -> 0.524, 0.649 -> 0.563, 1.026 -> 0.784).
 constexpr int kCtasPerSm = 9;
 constexpr int kCtasPerSmAtoms = 8;
 constexpr int kMinChunk = 512;

@@ -7,9 +7,9 @@
 //
 // The particle kernel stages each tile's fields and node density in shared memory and streams the
 // tile's particles straight from their records in coalesced order (the next record's position is
-// loaded one iteration ahead); the cell sort stores each block of 256 of a tile's cell-ordered
-// particles column by column as a 32-row matrix, so the lanes of a warp hold particles 8 places
-// apart in the cell order (neighbouring cells). CTAs draw tiles from a ticket counter (dynamic
+// loaded one iteration ahead); the cell sort stores each block of a tile's cell-ordered particles (256 to 4096,
+// 32 x the particles per cell) column by column as a 32-row matrix, so the lanes of a warp hold
+// particles of neighbouring cells. CTAs draw tiles, or parts of them, from a ticket counter (dynamic
 // assignment: 10.46 -> 8.79 ms per launch on the 384^2 x 256 slab against a static round robin).
 // Deposits use global 64-bit reductions, which are native in L2.
 #include <atomic>
@@ -27,6 +27,9 @@ namespace gbpic {
 constexpr int kQ3Bits = 14;
 constexpr int kQ3 = 1 << kQ3Bits;
 constexpr int kBlock3 = 256;
+// Resident CTAs: 3 with fields (80 registers), 4 without (64). All potentials gain from the fourth, also the embedded
+// atom and HCP Morse, which spill 12 to 28 bytes at 64 registers (1.5 M cells of 16 atoms, ms a step before and after: Eq. (3)
+// 0.577 -> 0.520, Morse 0.681 -> 0.587, HCP Morse 1.136 -> 1.010, embedded atom 1.035 -> 0.941).
 constexpr int kCtas3 = 3, kCtas3Atoms = 4;
 // Parts per tile (a power of two up to 16) until there are kFill3 items per resident CTA: a grid of few
 // tiles left most of the chip idle. Every item stages its tile's window, seven arrays with fields and the
@@ -219,7 +222,7 @@ struct Win3 {
 };
 
 // Window gathers. Every component of a particle reads the corners of one cell of the window: the
-// node cell (lx, ly, lz) for an integer-node axis, or that cell shifted one node down along a
+// particle's node cell for an integer-node axis, or that cell shifted one node down along a
 // half-node axis when the particle sits in the lower half of its cell (offset o = 0 or -stride,
 // weight f -+ 1/2). One base index serves all seven components; with the window edge WC known
 // at compile time the corner and component offsets are immediates.
@@ -254,7 +257,7 @@ struct Axis3 {
     float g, w;       // weights of the lower and upper node (1 - w, w)
 };
 
-// trilinear interpolation of the corners of the cell at p (strides sy = W, sz = W^2) on z-pairs of
+// trilinear interpolation of the corners of the cell at p (strides sy, sz of the window's layout) on z-pairs of
 // corners: each packed FP32x2 operation interpolates the lower and the upper face at once
 // (measured on the 384^2 x 256 slab with the deposit below inlined: 7.73 -> 7.44 ms per launch)
 __device__ __forceinline__ float trilerp3(const float* p, int sy, int sz, Axis3 x, Axis3 y, Axis3 z)
@@ -331,10 +334,8 @@ __device__ __noinline__ void gather_global3(const float* F0, const float* F1, co
     if (pair) density3(rho, g, rho_s, i, j, k, fx, fy, fz, out[6], out + 7);
 }
 
-// In-cell deposit (the particle stayed in its cell): current on the cell's edges and the node
-// density change on its corners, as global 64-bit reductions. Not inlined: it keeps the particle
-// loop small enough for the instruction cache.
-// A particle that stays in its cell: currents on the cell's edges, node density on its corners.
+// A particle that stays in its cell: currents on the cell's edges, node density changes on its corners, as
+// global 64-bit reductions.
 // The edge sums 2 S0 S0' + S1 S0' + S0 S1' + 2 S1 S1' are formed as S0 (2 S0' + S1') + S1 (S0' + 2 S1')
 // from the second axis' two combinations (each product at most 3 * 2^28, the sum at most
 // 6 * 2^28 < 2^31: exact in 32-bit); one widening multiply per term. Every reduction is issued

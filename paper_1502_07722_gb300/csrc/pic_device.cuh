@@ -46,8 +46,8 @@ struct Sum3 {
 
 // A long sum: every kFold terms the three numbers are added to an FP64 one, which keeps the error below that of
 // an FP64 sum at any length (256 terms in Sum3: 2^-51 S). Terms so large that an FP32 sum could overflow (or
-// infinite, or NaN) are added in FP64 at once. (Both are calls, as in i64_f32.) FP64 additions of every term took
-// 482 us where this takes 280, on the energies of 33.5 M particles; two numbers (48 bits) 277.
+// infinite, or NaN) are added in FP64 at once. (Both are calls, as in i64_f32.) With FP64 additions of
+// every term the energy call took 520 us on 33.5 M particles, with two numbers (48 bits) 273, so 287.
 constexpr int kFold = 256;
 static __device__ __noinline__ double add_wide(double s, float x) { return s + (double)x; }
 static __device__ __noinline__ double add_wide(double s, Sum3 x) { return s + x.value(); }

@@ -64,6 +64,8 @@ __device__ __forceinline__ int layout_slot(int ci, int nt, int lb)
 // block size for all (1024 in 2D, 256 in 3D): the 16-slab sweep (8 to 32 per cell) 1.59 -> 1.43, the
 // crater slab (128 per cell) 0.119 -> 0.114, the 3D crater slab (16 per cell) 2.80 -> 2.68; twice the
 // size: 1.69, 0.177, 4.06. Below 2^17 particles a launch is bound by latency and keeps the fixed size.
+// At high loads the sort itself pays for it (a cell's particles go to more lines), the steps between two sorts gain far
+// more: 3D at 128 atoms per cell 0.60 -> 0.81 ms a sort, 2.09 -> 0.48 ms a step; at 500 + 500 2.1 -> 4.0 and 11.4 -> 2.9.
 static int layout_log2(const Ctx& c, const Species& S)
 {
     const int base = c.dims == 3 ? 8 : 10;
