@@ -419,6 +419,8 @@ PIC_API int pic_checkpoint_restore(pic_ctx* ctx, const void* buf, int32_t on_hos
  *   context saved with its present particle counts (the context itself need not be at step t and is left
  *   as it is; dev_ckpt is 256-byte aligned as for pic_checkpoint_save). The checkpoint's header is read back
  *   first: PIC_EINVAL for a buffer that holds no checkpoint, or one of other species or particle counts.
+ * pic_adjoint_steps_at: n such steps in a row, the states in the order of dev_ckpts (a host array; a reverse
+ *   sweep lists the latest first). All headers are checked before the first step, with one wait.
  * All return PIC_ESTATE outside 2D, sort_every = 0 and pot_mode 0. */
 typedef struct {
     float* lam_pos[2];
@@ -434,6 +436,8 @@ PIC_API int pic_adjoint_seed(pic_ctx* ctx, double kin, const double* dev_weights
                              double* host_dLdr0);
 PIC_API int pic_adjoint_step(pic_ctx* ctx, const pic_adjoint_buffers* bufs);
 PIC_API int pic_adjoint_step_at(pic_ctx* ctx, const void* dev_ckpt, const pic_adjoint_buffers* bufs);
+PIC_API int pic_adjoint_steps_at(pic_ctx* ctx, int32_t n, const void* const* dev_ckpts,
+                                 const pic_adjoint_buffers* bufs);
 
 /* Static text for a return code. */
 PIC_API const char* pic_strerror(int code);

@@ -116,6 +116,7 @@ _SIGNATURES = {
                                         ctypes.POINTER(ctypes.c_double)]),
     "pic_adjoint_step": (ctypes.c_int, [_VP, ctypes.POINTER(pic_adjoint_buffers)]),
     "pic_adjoint_step_at": (ctypes.c_int, [_VP, _VP, ctypes.POINTER(pic_adjoint_buffers)]),
+    "pic_adjoint_steps_at": (ctypes.c_int, [_VP, _I32, ctypes.POINTER(_VP), ctypes.POINTER(pic_adjoint_buffers)]),
 }
 
 _lib = None
@@ -367,6 +368,11 @@ def pic_adjoint_step(h, bufs):
 
 def pic_adjoint_step_at(h, ckpt_ptr, bufs):
     _check(load_library().pic_adjoint_step_at(h, ckpt_ptr, ctypes.byref(bufs)), "pic_adjoint_step_at")
+
+
+def pic_adjoint_steps_at(h, ckpt_ptrs, bufs):
+    ptrs = (ctypes.c_void_p * len(ckpt_ptrs))(*ckpt_ptrs)
+    _check(load_library().pic_adjoint_steps_at(h, len(ckpt_ptrs), ptrs, ctypes.byref(bufs)), "pic_adjoint_steps_at")
 
 
 # ---- convenience wrapper: torch owns the workspace and the stream -----------------------------

@@ -967,21 +967,10 @@ int pic_adjoint_step(pic_ctx* h, const pic_adjoint_buffers* b)
 
 // The reverse step reads the state where the checkpoint holds it: a copy of the context whose particle,
 // field and density pointers lie in the buffer. (Restoring each state first moved it once more, 191 MB
-// and 54 us on the differentiable slab.) A buffer without this context's header, or with other particle counts,
-// is refused as pic_checkpoint_restore would: its cells would index outside the grids.
-int pic_adjoint_step_at(pic_ctx* h, const void* ckpt, const pic_adjoint_buffers* b)
+// and 54 us on the differentiable slab.)
+static int adjoint_step_in(Ctx c, const void* ckpt, int64_t step, const pic_adjoint_buffers* b)
 {
-    if (!h || !b || !ckpt || ((uintptr_t)ckpt & 255)) return PIC_EINVAL;
-    int r = adjoint_ok(h->c, b);
-    if (r) return r;
-    Ctx c = h->c;
-    CkptHeader hd;
-    CK(cudaMemcpyAsync(&hd, ckpt, sizeof(hd), cudaMemcpyDeviceToHost, c.stream));
-    CK(cudaStreamSynchronize(c.stream));
-    if (hd.magic != kCkptMagic || hd.nsp != c.nsp) return PIC_EINVAL;
-    for (int s = 0; s < c.nsp; s++)
-        if (hd.n[s] != c.sp[s].n) return PIC_EINVAL;
-    c.step = hd.step;
+    c.step = step;
     char* buf = (char*)const_cast<void*>(ckpt);
     size_t osp[2], otl[2], of, orho, oj;
     ckpt_layout(c, osp, otl, &of, &orho, &oj);
@@ -1000,6 +989,51 @@ int pic_adjoint_step_at(pic_ctx* h, const void* ckpt, const pic_adjoint_buffers*
         launch_adjoint_step(c, b->lam_pos[0], b->lam_u[0], b->lam_nodes, b->grads, c.stream);
     CK(cudaGetLastError());
     return PIC_OK;
+}
+
+// A buffer without this context's header, or with other particle counts, is refused as
+// pic_checkpoint_restore would: its cells would index outside the grids. The headers are gathered in the
+// energies' scratch and read back at once, so that the host waits for the stream once for all the steps (once
+// per step: 17 us each, 5.15 -> 5.49 ms for 18 steps on 111 x 282 cells).
+int pic_adjoint_steps_at(pic_ctx* h, int32_t n, const void* const* ckpt, const pic_adjoint_buffers* b)
+{
+    if (!h || !b || n < 0 || (n > 0 && !ckpt)) return PIC_EINVAL;
+    for (int q = 0; q < n; q++)
+        if (!ckpt[q] || ((uintptr_t)ckpt[q] & 255)) return PIC_EINVAL;
+    Ctx& c = h->c;
+    int r = adjoint_ok(c, b);
+    if (r) return r;
+    struct Slot {
+        CkptHeader hd;
+        char pad[48 - sizeof(CkptHeader)];
+    };
+    constexpr int kMost = 8 * 5 * kMaxEnergyBlocks / sizeof(Slot);
+    std::vector<Slot> hd(n);
+    for (int q0 = 0; q0 < n; q0 += kMost) {
+        const int m = n - q0 < kMost ? n - q0 : kMost;
+        std::vector<CopySeg> segs;
+        for (int q = 0; q < m; q++)
+            segs.push_back(CopySeg{ckpt[q0 + q], (char*)c.partials + q * sizeof(Slot), sizeof(CkptHeader)});
+        launch_copy_segments(c, segs.data(), m, c.stream);
+        CK(cudaMemcpyAsync(hd.data() + q0, c.partials, m * sizeof(Slot), cudaMemcpyDeviceToHost, c.stream));
+        CK(cudaStreamSynchronize(c.stream));
+    }
+    for (int q = 0; q < n; q++) {
+        const CkptHeader& k = hd[q].hd;
+        if (k.magic != kCkptMagic || k.nsp != c.nsp) return PIC_EINVAL;
+        for (int s = 0; s < c.nsp; s++)
+            if (k.n[s] != c.sp[s].n) return PIC_EINVAL;
+    }
+    for (int q = 0; q < n; q++) {
+        r = adjoint_step_in(c, ckpt[q], hd[q].hd.step, b);
+        if (r) return r;
+    }
+    return PIC_OK;
+}
+
+int pic_adjoint_step_at(pic_ctx* h, const void* ckpt, const pic_adjoint_buffers* b)
+{
+    return pic_adjoint_steps_at(h, 1, &ckpt, b);
 }
 
 const char* pic_strerror(int code)

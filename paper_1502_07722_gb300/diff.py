@@ -22,7 +22,7 @@ from __future__ import annotations
 import torch
 
 from . import (PIC_MODE_FULL, Simulation, pic_adjoint_buffers, pic_adjoint_seed, pic_adjoint_step,
-               pic_adjoint_step_at, pic_checkpoint_restore, pic_checkpoint_save, pic_checkpoint_size,
+               pic_adjoint_steps_at, pic_checkpoint_restore, pic_checkpoint_save, pic_checkpoint_size,
                pic_node_functional)
 
 QE = 1.602176634e-19
@@ -113,8 +113,8 @@ class DiffRun:
                 if j + 1 < m:
                     pic_checkpoint_save(self.sim.h, seg_states[j - 1].data_ptr())
             pic_adjoint_step(self.sim.h, bufs)
-            for j in range(m - 2, -1, -1):
-                pic_adjoint_step_at(self.sim.h, (seg_states[j - 1] if j else self.checkpoints[si]).data_ptr(), bufs)
+            states = [self.checkpoints[si]] + seg_states[:max(0, m - 2)]
+            pic_adjoint_steps_at(self.sim.h, [b.data_ptr() for b in reversed(states[:m - 1])], bufs)
         if self.checkpoints:
             pic_checkpoint_restore(self.sim.h, self.checkpoints[0].data_ptr())
         torch.cuda.current_stream().synchronize()

@@ -27,9 +27,11 @@ def test_reverse_step_from_a_foreign_buffer(gb):  # noqa: F811
         bad.append(b)
     torch.cuda.synchronize()
     for b in bad:
-        with pytest.raises(gb.PicError) as e:
-            gb.pic_adjoint_step_at(run.sim.h, b.data_ptr(), bufs)
-        assert e.value.code == gb.PIC_EINVAL
+        for call in (lambda: gb.pic_adjoint_step_at(run.sim.h, b.data_ptr(), bufs),
+                     lambda: gb.pic_adjoint_steps_at(run.sim.h, [good.data_ptr(), b.data_ptr()], bufs)):
+            with pytest.raises(gb.PicError) as e:
+                call()
+            assert e.value.code == gb.PIC_EINVAL
     torch.cuda.synchronize()
     for a, b in zip(before, run._keep):
         assert torch.equal(bits(a), bits(b))
